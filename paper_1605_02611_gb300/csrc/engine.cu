@@ -143,26 +143,49 @@ void GemmBuilder::term(const double* A, int lda, const double* B, int ldb, int k
 
 void GemmBuilder::end() {
   GemmTask& t = tasks.back();
-  if (t.t1 == t.t0) {
-    tasks.pop_back();
-    return;
-  }
-  int idx = (int)tasks.size() - 1;
-  for (int r0 = 0; r0 < t.m; r0 += GEMM_TM)
-    for (int c0 = 0; c0 < t.n; c0 += GEMM_TN) tiles.push_back({idx, r0, c0});
+  if (t.t1 == t.t0) tasks.pop_back();
 }
 
-void GemmPlan::upload(const std::vector<GemmTile>& ti, const std::vector<GemmTask>& ta,
-                      const std::vector<GemmTerm>& te, cudaStream_t s) {
-  tiles.upload(ti, s);
-  tasks.upload(ta, s);
-  terms.upload(te, s);
-  ntiles = (int)ti.size();
+// Tiles in the order of decreasing work where the list is short enough for its last
+// tiles to matter (and for the sort to be cheap), else in task order.
+int GemmBuilder::cut() {
+  long nt[3] = {0, 0, 0};
+  int max_dim = 0;
+  for (const GemmTask& t : tasks) {
+    max_dim = std::max(max_dim, std::max(t.m, t.n));
+    for (int i = 0; i < 3; ++i) nt[i] += (long)gemm_parts(t.m, GEMM_CAPS[i]) * gemm_parts(t.n, GEMM_CAPS[i]);
+  }
+  const int cap = gemm_pick_cap(max_dim, nt);
+  std::vector<int> order(tasks.size());
+  std::iota(order.begin(), order.end(), 0);
+  if (tasks.size() <= 16384) {
+    std::vector<long> work(tasks.size());
+    for (size_t i = 0; i < tasks.size(); ++i) {
+      const GemmTask& t = tasks[i];
+      long k = 0;
+      for (int j = t.t0; j < t.t1; ++j) k += terms[(size_t)j].k;
+      work[i] = k * std::min(t.m, cap) * std::min(t.n, cap);
+    }
+    std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return work[a] > work[b]; });
+  }
+  tiles.clear();
+  for (int i : order)
+    for (int ri = 0; ri < gemm_parts(tasks[i].m, cap); ++ri)
+      for (int ci = 0; ci < gemm_parts(tasks[i].n, cap); ++ci) tiles.push_back({i, ri, ci});
+  return cap;
+}
+
+void GemmPlan::upload(GemmBuilder& g, cudaStream_t s) {
+  cap = g.cut();
+  tiles.upload(g.tiles, s);
+  tasks.upload(g.tasks, s);
+  terms.upload(g.terms, s);
+  ntiles = (int)g.tiles.size();
 }
 
 void GemmPlan::run(cudaStream_t s) const {
   if (ntiles == 0) return;
-  launch_gemm(tiles.p, ntiles, tasks.p, terms.p, s);
+  launch_gemm(tiles.p, ntiles, tasks.p, terms.p, cap, s);
   cuda_check(cudaGetLastError(), "gemm launch");
 }
 
@@ -170,7 +193,7 @@ static void run_builder(Context& c, GemmBuilder& g) {
   if (g.tasks.empty()) return;
   c.other_flops_total += g.flops;
   GemmPlan p;
-  p.upload(g.tiles, g.tasks, g.terms, c.stream);
+  p.upload(g, c.stream);
   p.run(c.stream);
   // host vectors must outlive the async upload: synchronise before they go
   cuda_check(cudaStreamSynchronize(c.stream), "sync");
@@ -897,9 +920,9 @@ void build_sigma_plan(Context& c, Tilde& lt, Tilde& rt, int k, SigmaPlan& plan) 
       g2.end();
     }
     plan.stage1.emplace_back();
-    plan.stage1.back().upload(g1.tiles, g1.tasks, g1.terms, c.stream);
+    plan.stage1.back().upload(g1, c.stream);
     plan.stage2.emplace_back();
-    plan.stage2.back().upload(g2.tiles, g2.tasks, g2.terms, c.stream);
+    plan.stage2.back().upload(g2, c.stream);
     plan.flops += g1.flops + g2.flops;
     cuda_check(cudaStreamSynchronize(c.stream), "sync");
   }

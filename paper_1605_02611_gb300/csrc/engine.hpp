@@ -140,14 +140,14 @@ struct Tilde {
 };
 
 // Device-side work list of one grouped GEMM launch.
+struct GemmBuilder;
 struct GemmPlan {
   DArr<GemmTile> tiles;
   DArr<GemmTask> tasks;
   DArr<GemmTerm> terms;
-  int ntiles = 0;
+  int ntiles = 0, cap = 32;
   double flops = 0;
-  void upload(const std::vector<GemmTile>& ti, const std::vector<GemmTask>& ta,
-              const std::vector<GemmTerm>& te, cudaStream_t s);
+  void upload(GemmBuilder& g, cudaStream_t s);
   void run(cudaStream_t s) const;
 };
 struct GemmBuilder {
@@ -157,7 +157,8 @@ struct GemmBuilder {
   double flops = 0;
   int begin(double* C, int ldc, int m, int n, int beta);  // returns task index
   void term(const double* A, int lda, const double* B, int ldb, int k, int flags, double alpha, int m, int n);
-  void end();  // emits tiles of the last task if it has terms (or beta == 0)
+  void end();  // drops the last task if it has no terms
+  int cut();   // cuts the tasks into tiles; returns the tile edge
   bool empty() const { return tasks.empty(); }
   void clear() { tiles.clear(); tasks.clear(); terms.clear(); flops = 0; }
 };

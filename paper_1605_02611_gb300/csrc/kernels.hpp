@@ -23,11 +23,19 @@ struct GemmTask {
   int beta;
   int t0, t1;
 };
+// One tile of an output block.  A block of m rows is cut into gemm_parts(m, cap) nearly
+// equal row ranges (no range longer than cap, lengths differing by at most one), and its
+// columns likewise; ri, ci count the ranges.
 struct GemmTile {
-  int task, r0, c0;
+  int task, ri, ci;
 };
 
-constexpr int GEMM_TM = 64, GEMM_TN = 64, GEMM_TK = 16;
+// tile edges of the FP64 grouped GEMM (the largest row or column count of a tile)
+constexpr int GEMM_CAPS[3] = {8, 16, 32};
+__host__ __device__ inline int gemm_parts(int n, int cap) { return (n + cap - 1) / cap; }
+// The edge for a launch whose blocks are at most max_dim in either direction, given the
+// number of tiles ntiles[i] it has with each GEMM_CAPS[i]: see launch_gemm.
+int gemm_pick_cap(int max_dim, const long ntiles[3]);
 
 // Linear combination of operators with a common block layout:
 //   out_j[e] = sum_{t in [c0_j, c1_j)} coef_t * in_t[e],  e < nnz_j
@@ -54,8 +62,10 @@ long launch_count();
 // adds kernel launches made outside this file to the count
 void count_launches(long n);
 
+// cap: the tile edge the tiles were cut with (one of GEMM_CAPS), or 64: then every listed
+// tile is taken by four thread blocks, one per quarter (a list of a quarter of the length)
 void launch_gemm(const GemmTile* d_tiles, int ntiles, const GemmTask* d_tasks,
-                 const GemmTerm* d_terms, cudaStream_t s);
+                 const GemmTerm* d_terms, int cap, cudaStream_t s);
 void launch_combo(const ComboOut* d_outs, int nouts, long max_nnz, const ComboTerm* d_terms,
                   cudaStream_t s);
 void launch_copy(const CopyJob* d_jobs, int njobs, int max_elems, cudaStream_t s);

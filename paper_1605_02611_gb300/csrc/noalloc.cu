@@ -38,6 +38,8 @@ static __device__ __align__(256) unsigned char g_noalloc_scratch[NOALLOC_SCRATCH
 namespace {
 
 constexpr int kMaxDevices = 64;
+// listed tiles of 64 x 64, each taken by four thread blocks: the list stays short
+constexpr int TILE_CAP = 64;
 std::mutex g_setup_mu;
 void* g_scratch_dev[kMaxDevices] = {nullptr};
 // held by a call from staging its work lists until its GPU work has finished
@@ -104,7 +106,7 @@ void compute_diag_noalloc(Context& c, double* diag) {
   }
   size_t nblk = P.blocks.size(), ntiles = 0;
   for (const Block& b : P.blocks)
-    ntiles += (size_t)((b.rows + GEMM_TM - 1) / GEMM_TM) * ((b.cols + GEMM_TN - 1) / GEMM_TN);
+    ntiles += (size_t)gemm_parts(b.rows, TILE_CAP) * gemm_parts(b.cols, TILE_CAP);
   const size_t dl_bytes = align256((size_t)4 * Lb.total * nz * sizeof(double));
   const size_t dr_bytes = align256((size_t)4 * Rb.total * nz * sizeof(double));
   const size_t jobs_bytes = align256(njobs * sizeof(DiagJob));
@@ -159,15 +161,15 @@ void compute_diag_noalloc(Context& c, double* diag) {
     hk[pb] = {diag + ob.off, ob.cols, ob.rows, ob.cols, 0, (int)pb, (int)pb + 1};
     hm[pb] = {DL + ((size_t)n1 * Lb.total + Lb.off[ob.rs]) * nz, DR + ((size_t)n2 * Rb.total + Rb.off[ob.cs]) * nz, nz,
               nz, nz, 0, 1.0};
-    for (int r0 = 0; r0 < ob.rows; r0 += GEMM_TM)
-      for (int c0 = 0; c0 < ob.cols; c0 += GEMM_TN) ht[t++] = {(int)pb, r0, c0};
+    for (int ri = 0; ri < gemm_parts(ob.rows, TILE_CAP); ++ri)
+      for (int ci = 0; ci < gemm_parts(ob.cols, TILE_CAP); ++ci) ht[t++] = {(int)pb, ri, ci};
   }
   const size_t dsc_bytes = jobs_bytes + tile_bytes + task_bytes + term_bytes;
   cuda_check(cudaMemcpyAsync(dsc, g_stage, dsc_bytes, cudaMemcpyHostToDevice, c.stream), "h2d");
   launch_diag_extract((const DiagJob*)dsc, (int)njobs, mx, c.stream);
   cuda_check(cudaGetLastError(), "diag extract");
   launch_gemm((const GemmTile*)(dsc + jobs_bytes), (int)ntiles, (const GemmTask*)(dsc + jobs_bytes + tile_bytes),
-              (const GemmTerm*)(dsc + jobs_bytes + tile_bytes + task_bytes), c.stream);
+              (const GemmTerm*)(dsc + jobs_bytes + tile_bytes + task_bytes), TILE_CAP, c.stream);
   cuda_check(cudaGetLastError(), "gemm launch");
   // the host staging buffer is reused by the next call: wait for the copy and the kernels
   cuda_check(cudaStreamSynchronize(c.stream), "sync");
