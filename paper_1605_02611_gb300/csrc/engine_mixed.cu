@@ -78,6 +78,53 @@ __global__ void conv_kernel(const ConvJob* __restrict__ jobs) {
   }
 }
 
+// FP64 block -> nsl BF16 slices in the column-group layout of the TMA-staged matrices (8
+// columns of consecutive rows contiguous): element (i, j) of slice s goes to
+// dst[s * slice_stride + (j / 8) * group + i * 8 + j % 8], columns [cols, wcols) are zero
+// (wcols a multiple of 8).
+struct GroupJob {
+  const double* src;
+  __nv_bfloat16* dst;
+  long slice_stride, group;
+  int rows, cols, lds, wcols;
+  double scale;
+};
+
+// Memory-bound (8 bytes read, 2 written per slice and element): a thread takes 8 columns
+// of one row, 64 contiguous bytes of the source, and writes 16 bytes per slice; consecutive
+// threads take consecutive rows, so a warp writes 512 contiguous bytes.  Each value is split
+// as in conv_element.  src is read `shift` elements further than the job says (the jobs of
+// psi are made for one vector and serve any).
+template <int NSL>
+__global__ void conv_groups_kernel(const GroupJob* __restrict__ jobs, long shift) {
+  const GroupJob jb = jobs[blockIdx.y];
+  const int ng = jb.wcols >> 3;
+  const unsigned n = (unsigned)jb.rows * (unsigned)ng;
+  for (unsigned e = blockIdx.x * blockDim.x + threadIdx.x; e < n; e += gridDim.x * blockDim.x) {
+    const int q = (int)(e / (unsigned)jb.rows), i = (int)(e - (unsigned)q * (unsigned)jb.rows);
+    const double* s = jb.src + shift + (long)i * jb.lds + q * 8;
+    const int nc = jb.cols - q * 8;
+    uint32_t w[NSL][4];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const double y = u < nc ? jb.scale * s[u] : 0.0;
+      float a = __double2float_rn(y);
+      const float lo = NSL > 1 ? __double2float_rn(y - (double)a) : 0.0f;
+#pragma unroll
+      for (int sl = 0; sl < NSL; ++sl) {
+        const __nv_bfloat16 h = __float2bfloat16_rn(sl + 1 == NSL ? a + lo : a);
+        const uint32_t b = (uint32_t)__bfloat16_as_ushort(h);
+        w[sl][u / 2] = (u & 1) ? (w[sl][u / 2] | (b << 16)) : b;
+        a -= __bfloat162float(h);
+      }
+    }
+    __nv_bfloat16* d = jb.dst + (long)q * jb.group + (long)i * 8;
+#pragma unroll
+    for (int sl = 0; sl < NSL; ++sl)
+      *reinterpret_cast<uint4*>(d + sl * jb.slice_stride) = make_uint4(w[sl][0], w[sl][1], w[sl][2], w[sl][3]);
+  }
+}
+
 // transposed gather FP32 -> FP64: dst[i * cols + j] = src[j * lds + i]
 struct UnconvJob {
   const float* src;
@@ -85,12 +132,13 @@ struct UnconvJob {
   int rows, cols, lds;
 };
 
-__global__ void unconv_kernel(const UnconvJob* __restrict__ jobs) {
+// dst is written `shift` elements further than the job says
+__global__ void unconv_kernel(const UnconvJob* __restrict__ jobs, long shift) {
   const UnconvJob jb = jobs[blockIdx.y];
   const long n = (long)jb.rows * jb.cols;
   for (long e = (long)blockIdx.x * blockDim.x + threadIdx.x; e < n; e += (long)gridDim.x * blockDim.x) {
     const int i = (int)(e / jb.cols), j = (int)(e % jb.cols);
-    jb.dst[e] = (double)jb.src[(long)j * jb.lds + i];
+    jb.dst[shift + e] = (double)jb.src[(long)j * jb.lds + i];
   }
 }
 
@@ -102,29 +150,32 @@ static long job_blocks(int njobs, long maxel) {
   return std::min<long>(std::max<long>(1, (maxel + 255) / 256), 64);
 }
 
-void launch_unconv(const UnconvJob* jobs, int njobs, long maxel, cudaStream_t s) {
+void launch_unconv(const UnconvJob* jobs, int njobs, long maxel, cudaStream_t s, long shift = 0) {
   for (int o0 = 0; o0 < njobs; o0 += 65535) {
     int no = std::min(65535, njobs - o0);
     const long g = job_blocks(njobs, maxel);
-    unconv_kernel<<<dim3((unsigned)g, no), 256, 0, s>>>(jobs + o0);
+    unconv_kernel<<<dim3((unsigned)g, no), 256, 0, s>>>(jobs + o0, shift);
     count_launches(1);
   }
   cuda_check(cudaGetLastError(), "unconv launch");
 }
 
-// zero n elements at p + s * stride for every slice s < nsl
+// zero n elements at p + s * stride + r * pitch for every slice s < nsl and r < reps
 struct ZeroJob {
   __nv_bfloat16* p;
   long n, stride;
   int nsl;
+  int reps = 1;
+  long pitch = 0;
 };
 
 __global__ void zero_kernel(const ZeroJob* __restrict__ jobs) {
   const ZeroJob jb = jobs[blockIdx.y];
   const __nv_bfloat16 z = __float2bfloat16_rn(0.0f);
   for (int sl = 0; sl < jb.nsl; ++sl)
-    for (long e = (long)blockIdx.x * blockDim.x + threadIdx.x; e < jb.n; e += (long)gridDim.x * blockDim.x)
-      jb.p[sl * jb.stride + e] = z;
+    for (int r = 0; r < jb.reps; ++r)
+      for (long e = (long)blockIdx.x * blockDim.x + threadIdx.x; e < jb.n; e += (long)gridDim.x * blockDim.x)
+        jb.p[sl * jb.stride + r * jb.pitch + e] = z;
 }
 
 void launch_zero(const ZeroJob* jobs, int njobs, long maxel, cudaStream_t s) {
@@ -142,6 +193,22 @@ void launch_conv(const DArr<ConvJob>& jobs, int njobs, long maxel, cudaStream_t 
     int no = std::min(65535, njobs - o0);
     const long g = job_blocks(njobs, maxel);
     conv_kernel<<<dim3((unsigned)g, no), 256, 0, s>>>(jobs.p + o0);
+    count_launches(1);
+  }
+  cuda_check(cudaGetLastError(), "conv launch");
+}
+
+void launch_conv_groups(const DArr<GroupJob>& jobs, int njobs, int nsl, long maxel, cudaStream_t s, long shift = 0) {
+  for (int o0 = 0; o0 < njobs; o0 += 65535) {
+    const int no = std::min(65535, njobs - o0);
+    const dim3 g((unsigned)job_blocks(njobs, maxel / 8), no);
+    const GroupJob* j = jobs.p + o0;
+    if (nsl == 1)
+      conv_groups_kernel<1><<<g, 256, 0, s>>>(j, shift);
+    else if (nsl == 2)
+      conv_groups_kernel<2><<<g, 256, 0, s>>>(j, shift);
+    else
+      conv_groups_kernel<3><<<g, 256, 0, s>>>(j, shift);
     count_launches(1);
   }
   cuda_check(cudaGetLastError(), "conv launch");
@@ -747,10 +814,9 @@ int mixed_error(Context& c, SigmaPlan& plan) {
 struct TmaPlan {
   int nsl = 1;  // BF16 slices per operand (1: one pass; 2 or 3: slice products i + j < nsl)
   DArr<__nv_bfloat16> psi_b, a1, xt, lmir;
-  long x_stride = 0;  // slice stride of the X intermediates
   DArr<float> sig_t;
   long sig_total = 0;
-  DArr<ConvJob> psi_jobs, a1_jobs, l_jobs;
+  DArr<GroupJob> psi_jobs, a1_jobs, l_jobs;
   int n_psi_jobs = 0, n_a1_jobs = 0, n_l_jobs = 0;
   long psi_maxel = 0, a1_maxel = 0, l_maxel = 0;
   DArr<UnconvJob> sig_jobs;
@@ -758,7 +824,6 @@ struct TmaPlan {
   long sig_maxel = 0;
   DArr<CUtensorMap> maps;
   DArr<long> rowmap;
-  DArr<int2> cbtab;  // (first column, width) of the column blocks of every input group
   // device copies of a launch's copy lists
   struct Lists {
     DArr<int> cta_stage, sorder, tpiece0;
@@ -769,9 +834,9 @@ struct TmaPlan {
     long total = 0;
     // the stage counts on the host (reduce mode: sets the tiles' stages and segments,
     // so it comes before the tiles are uploaded); throws on a malformed term
-    void plan(int mode, std::vector<TmTile>& tiles, const std::vector<TmTerm>& terms, cudaStream_t s) {
+    void plan(int mode, int nsl, std::vector<TmTile>& tiles, const std::vector<TmTerm>& terms, cudaStream_t s) {
       TmListPlan lp;
-      if (!tma_plan_lists(mode, tiles, terms, lp)) throw Error(ST_ECUDA, "internal: malformed TMA term list");
+      if (!tma_plan_lists(mode, nsl, tiles, terms, lp)) throw Error(ST_ECUDA, "internal: malformed TMA term list");
       grid = lp.grid;
       total = lp.total;
       cta_stage.upload(lp.cta_stage, s);
@@ -779,11 +844,11 @@ struct TmaPlan {
       sfirst.upload(lp.sfirst, s);
       tpiece0.upload(lp.tpiece0, s);
       stages.alloc((size_t)std::max<long>(lp.total, 1), s);
-      pieces.alloc((size_t)std::max<long>(lp.total, 1) * tma_pieces(mode), s);
+      pieces.alloc((size_t)std::max<long>(lp.total, 1) * tma_pieces(mode, nsl), s);
     }
     // the lists themselves, on the device, from the uploaded tiles and terms
-    void fill(int mode, const TmTile* d_tiles, int ntiles, const TmTerm* d_terms, cudaStream_t s) {
-      cuda_check(launch_fill_lists(mode, d_tiles, ntiles, d_terms, tpiece0.p, sorder.p, sfirst.p, total, stages.p,
+    void fill(int mode, int nsl, const TmTile* d_tiles, int ntiles, const TmTerm* d_terms, cudaStream_t s) {
+      cuda_check(launch_fill_lists(mode, nsl, d_tiles, ntiles, d_terms, tpiece0.p, sorder.p, sfirst.p, total, stages.p,
                                    pieces.p, s),
                  "list fill");
     }
@@ -813,27 +878,14 @@ namespace {
 inline int pad16(int x) { return (x + 15) & ~15; }
 }  // namespace
 
-// conversion jobs must write inside their destination buffer
-static void check_conv_jobs(const std::vector<ConvJob>& jobs, const DArr<__nv_bfloat16>& buf) {
-  for (const ConvJob& j : jobs)
-    if (j.rows < 1 || j.wcols < j.cols || j.ldd < j.wcols || j.dst < buf.p ||
-        j.dst + (long)(j.rows - 1) * j.ldd + j.wcols > buf.p + buf.n)
+// conversion jobs must write inside their destination buffer, in whole 16-byte groups
+static void check_group_jobs(const std::vector<GroupJob>& jobs, int nsl, const DArr<__nv_bfloat16>& buf) {
+  for (const GroupJob& j : jobs)
+    if (j.rows < 1 || j.wcols < j.cols || j.wcols % 8 || (long)j.rows * (j.wcols / 8) >= (1L << 31) || j.dst < buf.p ||
+        (j.dst - buf.p) % 8 || j.group % 8 || j.slice_stride % 8 ||
+        j.dst + (nsl - 1) * j.slice_stride + (j.wcols / 8 - 1) * j.group + (long)j.rows * 8 > buf.p + buf.n)
       throw Error(ST_ECUDA, "internal: conversion job outside its buffer");
 }
-
-namespace {
-// stages of a reduce-mode tile: its pieces (ceil(k / TM_PACK_COLS) per slice pair of every
-// term) packed TM_PACK_SLOTS to a stage
-long packed_stages(const std::vector<TmTerm>& m, int t0, int t1) {
-  long pieces = 0;
-  for (int t = t0; t < t1; ++t) {
-    const int nsl = std::max(1, (m[t].neg >> 4) & 15);
-    pieces += (long)((m[t].k + TM_PACK_COLS - 1) / TM_PACK_COLS) * (nsl * (nsl + 1) / 2);
-  }
-  return (pieces + TM_PACK_SLOTS - 1) / TM_PACK_SLOTS;
-}
-
-}  // namespace
 
 void build_tma_plan(Context& c, Tilde& lt, Tilde& rt, int k, SigmaPlan& plan, int nsl) {
   const auto& mid = c.mpo.bonds[k + 1];
@@ -848,7 +900,7 @@ void build_tma_plan(Context& c, Tilde& lt, Tilde& rt, int k, SigmaPlan& plan, in
   tp->nsl = nsl;
   const int nL = Lb.nsec(), nR = Rb.nsec();
   const int nmid = (int)mid.size();
-  // slice pairs (i, j), i + j < nsl, per term (expanded by the kernel, level by level)
+  // slice pairs (i, j), i + j < nsl, multiplied per piece
   const int npair = nsl == 1 ? 1 : nsl == 2 ? 3 : 6;
   // ---- groups of the cut: rows (ql, n1) and columns (n2, qr), blocks padded to 16
   std::map<std::pair<int, int>, int> gidx;
@@ -911,7 +963,7 @@ void build_tma_plan(Context& c, Tilde& lt, Tilde& rt, int k, SigmaPlan& plan, in
   tp->sig_total = std::max<long>(stot, 4);
   tp->sig_t.alloc(tp->sig_total, c.stream);
   {
-    std::vector<ConvJob> pj;
+    std::vector<GroupJob> pj;
     std::vector<UnconvJob> sj;
     for (size_t b = 0; b < P.blocks.size(); ++b) {
       const Block& B = P.blocks[b];
@@ -919,13 +971,14 @@ void build_tma_plan(Context& c, Tilde& lt, Tilde& rt, int k, SigmaPlan& plan, in
       const auto cp = cpos[B.cs * 4 + P.b2[b]];
       if (rp[0] < 0 || rp[0] != cp[0]) throw Error(ST_ECUDA, "internal: psi block outside its group");
       const int g = rp[0];
-      pj.push_back({plan.in.p + B.off, tp->psi_b.p + goff[g] + (long)rp[1] * gC[g] + cp[1], std::max<long>(ptot, 8),
-                    B.rows, B.cols, B.cols, gC[g], nsl, 1.0, pad16(B.cols)});
+      // Psi_g: gR rows x gC columns in column groups of 8, slices one after another
+      pj.push_back({plan.in.p + B.off, tp->psi_b.p + goff[g] * nsl + (long)cp[1] * gR[g] + (long)rp[1] * 8,
+                    (long)gR[g] * gC[g], (long)gR[g] * 8, B.rows, B.cols, B.cols, pad16(B.cols), 1.0});
       tp->psi_maxel = std::max<long>(tp->psi_maxel, (long)B.rows * pad16(B.cols));
       sj.push_back({tp->sig_t.p + sgoff[g] + (long)cp[1] * gR[g] + rp[1], plan.out.p + B.off, B.rows, B.cols, gR[g]});
       tp->sig_maxel = std::max<long>(tp->sig_maxel, (long)B.rows * B.cols);
     }
-    check_conv_jobs(pj, tp->psi_b);
+    check_group_jobs(pj, nsl, tp->psi_b);
     for (const UnconvJob& u : sj)
       if (u.src < tp->sig_t.p || u.src + (long)(u.cols - 1) * u.lds + u.rows > tp->sig_t.p + tp->sig_total)
         throw Error(ST_ECUDA, "internal: gather job outside sigma^T");
@@ -984,7 +1037,8 @@ void build_tma_plan(Context& c, Tilde& lt, Tilde& rt, int k, SigmaPlan& plan, in
   std::vector<int> chunk_of(nmid, 0);
   for (int ci = 0; ci < nch; ++ci)
     for (int b = chunks[ci].first; b < chunks[ci].second; ++b) chunk_of[b] = ci;
-  // X^T layout per chunk: regions per g' (Sum_beta C_g(beta) rows x R_g' columns);
+  // X^T layout per chunk: regions per g' (Sum_beta C_g(beta) rows x R_g' columns in column
+  // groups of 8, the region's slices one after another: element offsets below count one slice);
   // xrow[beta][g'] = first row of beta's block in its region
   std::vector<std::vector<long>> xreg(nch, std::vector<long>(ng, 0)), xregrows(nch, std::vector<long>(ng, 0));
   std::vector<long> xrow((size_t)nmid * ng, -1);
@@ -1004,8 +1058,7 @@ void build_tma_plan(Context& c, Tilde& lt, Tilde& rt, int k, SigmaPlan& plan, in
     }
     maxchunk = std::max(maxchunk, (size_t)off);
   }
-  tp->x_stride = (long)std::max<size_t>(maxchunk, 8);
-  tp->xt.alloc((size_t)tp->x_stride * nsl, c.stream);
+  tp->xt.alloc(std::max<size_t>(maxchunk, 8) * nsl, c.stream);
   cuda_check(cudaMemsetAsync(tp->xt.p, 0, tp->xt.n * sizeof(__nv_bfloat16), c.stream), "memset");
   // ---- A1 per g': row blocks sorted by (chunk, mask), beta order kept inside a run
   for (int gp = 0; gp < ng; ++gp)
@@ -1013,17 +1066,23 @@ void build_tma_plan(Context& c, Tilde& lt, Tilde& rt, int k, SigmaPlan& plan, in
       if (chunk_of[a.beta] != chunk_of[b.beta]) return chunk_of[a.beta] < chunk_of[b.beta];
       return a.mask < b.mask;
     });
+  // (a run starts on a row group of 16, as the boxes of its tiles have to)
   std::vector<long> a1off(ng), a1rows(ng);
   long a1tot = 0;
   for (int gp = 0; gp < ng; ++gp) {
     long rows = 0;
-    for (const RowBlk& x : rb[gp]) rows += x.rows;
+    const RowBlk* prev = nullptr;
+    for (const RowBlk& x : rb[gp]) {
+      if (prev && (chunk_of[prev->beta] != chunk_of[x.beta] || prev->mask != x.mask)) rows = (rows + 15) / 16 * 16;
+      rows += x.rows;
+      prev = &x;
+    }
+    rows = (rows + 15) / 16 * 16;
     a1off[gp] = a1tot;
     a1rows[gp] = rows;
     a1tot += rows * gC[gp];
   }
-  const long a1s = std::max<long>(a1tot, 8);
-  tp->a1.alloc(a1s * nsl, c.stream);
+  tp->a1.alloc(std::max<long>(a1tot, 8) * nsl, c.stream);
   cuda_check(cudaMemsetAsync(tp->a1.p, 0, tp->a1.n * sizeof(__nv_bfloat16), c.stream), "memset");
   struct Run {
     int chunk, mask;
@@ -1033,14 +1092,16 @@ void build_tma_plan(Context& c, Tilde& lt, Tilde& rt, int k, SigmaPlan& plan, in
   // per A1 row: its row in the X^T region of its chunk (columns: blocks of g', each its
   // own submatrix of the region)
   std::vector<std::vector<long>> rowdst(ng);
-  std::vector<ConvJob> aconv;
+  std::vector<GroupJob> aconv;
   for (int gp = 0; gp < ng; ++gp) {
     long row = 0;
     rowdst[gp].assign((size_t)a1rows[gp], -1);
     for (const RowBlk& x : rb[gp]) {
       const int ci = chunk_of[x.beta];
-      if (runs[gp].empty() || runs[gp].back().chunk != ci || runs[gp].back().mask != x.mask)
+      if (runs[gp].empty() || runs[gp].back().chunk != ci || runs[gp].back().mask != x.mask) {
+        row = (row + 15) / 16 * 16;
         runs[gp].push_back({ci, x.mask, row, row});
+      }
       runs[gp].back().r1 = row + x.rows;
       const long xr0 = xrow[(size_t)x.beta * ng + gp] + (long)cpos[x.qr * 4 + x.n2][1];
       for (int i = 0; i < x.rows; ++i) rowdst[gp][(size_t)(row + i)] = xr0 + i;
@@ -1048,22 +1109,21 @@ void build_tma_plan(Context& c, Tilde& lt, Tilde& rt, int k, SigmaPlan& plan, in
         if (!((x.mask >> n2p) & 1)) continue;
         const TRef& r = rt.ref[x.beta][x.n2 * 4 + n2p];
         const Block& B = Renv.cls[r.cls].blocks[x.bl[n2p]];
-        // the K block (n2', qr') of g': submatrix of a1rows x pad16(d(qr')) at column offset coff
+        // the K block (n2', qr') of g': columns coff .. coff + pad16(d(qr')) of A1
         const int coff = cpos[B.cs * 4 + n2p][1];
-        const int w = pad16(B.cols);
-        aconv.push_back({r.p + B.off, tp->a1.p + a1off[gp] + a1rows[gp] * coff + row * w, a1s, B.rows, B.cols, B.cols,
-                         w, nsl, r.coef, w});
+        aconv.push_back({r.p + B.off, tp->a1.p + a1off[gp] * nsl + a1rows[gp] * coff + row * 8, a1rows[gp] * gC[gp],
+                         a1rows[gp] * 8, B.rows, B.cols, B.cols, pad16(B.cols), r.coef});
         tp->a1_maxel = std::max<long>(tp->a1_maxel, (long)B.rows * pad16(B.cols));
       }
       row += x.rows;
     }
   }
-  check_conv_jobs(aconv, tp->a1);
+  check_group_jobs(aconv, nsl, tp->a1);
   tp->a1_jobs.upload(aconv, c.stream);
   tp->n_a1_jobs = (int)aconv.size();
   // ---- left mirror: every distinct (operator, scale) referenced by Lt, all its blocks,
   // each padded to 16 rows and columns; blocks of one padded width w share one matrix of
-  // w columns (a box past the width then reads zeros without touching memory)
+  // w columns
   std::map<int, int> wcls;  // padded width -> class
   std::vector<int> wcls_w;
   for (const OpLayout& L : Lenv.cls)
@@ -1128,15 +1188,15 @@ void build_tma_plan(Context& c, Tilde& lt, Tilde& rt, int k, SigmaPlan& plan, in
   const long ls = std::max<long>(ltot, 8);
   tp->lmir.alloc(ls * nsl, c.stream);
   cuda_check(cudaMemsetAsync(tp->lmir.p, 0, tp->lmir.n * sizeof(__nv_bfloat16), c.stream), "memset");
-  std::vector<ConvJob> lconv;
+  std::vector<GroupJob> lconv;
   lconv.reserve(lpend.size());
   for (const PendL& pl : lpend) {
     const int w = wcls_w[pl.cls];
-    lconv.push_back({pl.src, tp->lmir.p + lbase[pl.cls] + pl.crow * w, ls, pl.rows, pl.cols, pl.cols, w, nsl, pl.scale,
-                     w});
+    lconv.push_back({pl.src, tp->lmir.p + lbase[pl.cls] * nsl + pl.crow * 8, lrows_c[pl.cls] * w,
+                     lrows_c[pl.cls] * 8, pl.rows, pl.cols, pl.cols, w, pl.scale});
     tp->l_maxel = std::max<long>(tp->l_maxel, (long)pl.rows * w);
   }
-  check_conv_jobs(lconv, tp->lmir);
+  check_group_jobs(lconv, nsl, tp->lmir);
   tp->l_jobs.upload(lconv, c.stream);
   tp->n_l_jobs = (int)lconv.size();
   // ---- tensor maps
@@ -1145,72 +1205,46 @@ void build_tma_plan(Context& c, Tilde& lt, Tilde& rt, int k, SigmaPlan& plan, in
   // but the extent itself is trusted by the hardware)
   struct MapInfo {
     long rows, cols;
-    int box, boxc;
+    int box;
   };
   std::vector<MapInfo> minfo;
-  // one map per slice, at consecutive indices (slice i of a map m is m + i)
-  auto add_map = [&](const DArr<__nv_bfloat16>& buf, long off, long stride, long rows, long cols, long ld,
-                     int box_rows, int box_cols) {
-    const int first = (int)maps.size();
-    for (int sl = 0; sl < nsl; ++sl) {
-      const long o = off + sl * stride;
-      if (o < 0 || rows < 1 || cols < 1 || ld < cols || ld % 8 != 0 || o % 8 != 0 ||
-          (size_t)(o + (rows - 1) * ld + cols) > buf.n)
-        throw Error(ST_ECUDA, "internal: tensor map outside its buffer");
-      CUtensorMap m;
-      if (!encode_bf16_map(&m, buf.p + o, (uint64_t)rows, (uint64_t)cols, (uint64_t)ld, (uint32_t)box_rows,
-                           (uint32_t)box_cols))
-        throw Error(ST_ECUDA, "cuTensorMapEncodeTiled failed");
-      maps.push_back(m);
-      minfo.push_back({rows, cols, box_rows, box_cols});
-    }
-    return first;
+  // a matrix of rows x cols in the column-group layout, its nsl slices from element off
+  auto add_map = [&](const DArr<__nv_bfloat16>& buf, long off, long rows, long cols, int box_rows) {
+    if (off < 0 || rows < 1 || cols < 1 || rows % 16 != 0 || cols % 16 != 0 || off % 8 != 0 ||
+        (size_t)(off + nsl * rows * cols) > buf.n)
+      throw Error(ST_ECUDA, "internal: tensor map outside its buffer");
+    CUtensorMap m;
+    if (!encode_slice_map(&m, buf.p + off, (uint64_t)rows, (uint64_t)cols, nsl, (uint32_t)box_rows))
+      throw Error(ST_ECUDA, "cuTensorMapEncodeTiled failed");
+    maps.push_back(m);
+    minfo.push_back({rows, cols, box_rows});
+    return (int)maps.size() - 1;
   };
   const int n1max = tma_max_n(TM_MODE_STORE_BF16), n2max = tma_max_n(TM_MODE_REDUCE_F32);
-  const int bc1 = tma_box_cols(TM_MODE_STORE_BF16), bc2 = tma_box_cols(TM_MODE_REDUCE_F32);
   std::vector<std::vector<std::array<int, 3>>> nt1(ng);  // per g': (row0, width, Psi map) of the stage-1 N tiles
-  // A1 of g': one map per K block (column block of g', a1rows x its padded width)
-  std::vector<std::vector<int>> a1map(ng);
+  std::vector<int> a1map(ng, -1);
   for (int gp = 0; gp < ng; ++gp) {
     if (a1rows[gp] == 0) continue;
     const int parts = (gR[gp] + n1max - 1) / n1max;
     int r0 = 0;
     for (int p = 0; p < parts; ++p) {
       const int w = std::min(gR[gp] - r0, pad16((gR[gp] - r0 + (parts - p) - 1) / (parts - p)));
-      nt1[gp].push_back(
-          {r0, w, add_map(tp->psi_b, goff[gp], std::max<long>(ptot, 8), gR[gp], gC[gp], gC[gp], w, bc1)});
+      nt1[gp].push_back({r0, w, add_map(tp->psi_b, goff[gp] * nsl, gR[gp], gC[gp], w)});
       r0 += w;
     }
-    for (const auto& cc : gcol[gp]) {
-      const int w = pad16(Rb.dim[cc[1]]);
-      a1map[gp].push_back(add_map(tp->a1, a1off[gp] + a1rows[gp] * cc[2], a1s, a1rows[gp], w, w, 128, bc1));
-    }
+    a1map[gp] = add_map(tp->a1, a1off[gp] * nsl, a1rows[gp], gC[gp], 128);
   }
-  // X^T region of (chunk, g'): one submatrix (and map) per column block (ql', n1') of g',
-  // xrows x its padded width; the table cbtab lists (first column, width) per g'
-  std::vector<std::vector<std::vector<int>>> xtmap(nch, std::vector<std::vector<int>>(ng));
-  std::vector<int2> cbtab;
-  std::vector<int> cbt0(ng), cbt1(ng);
-  for (int gp = 0; gp < ng; ++gp) {
-    cbt0[gp] = (int)cbtab.size();
-    for (const auto& rr : grow[gp]) cbtab.push_back(make_int2(rr[2], pad16(Lb.dim[rr[0]])));
-    cbt1[gp] = (int)cbtab.size();
-  }
+  // X^T region of (chunk, g')
+  std::vector<std::vector<int>> xtmap(nch, std::vector<int>(ng, -1));
   for (int ci = 0; ci < nch; ++ci)
     for (int gp = 0; gp < ng; ++gp)
-      if (xregrows[ci][gp] > 0)
-        for (const auto& rr : grow[gp]) {
-          const int w = pad16(Lb.dim[rr[0]]);
-          xtmap[ci][gp].push_back(add_map(tp->xt, xreg[ci][gp] + xregrows[ci][gp] * rr[2], tp->x_stride,
-                                          xregrows[ci][gp], w, w, 128, bc2));
-        }
+      if (xregrows[ci][gp] > 0) xtmap[ci][gp] = add_map(tp->xt, xreg[ci][gp] * nsl, xregrows[ci][gp], gR[gp], 128);
   // left mirror: per width class one map per box height
   std::vector<std::vector<int>> lmap(nwc, std::vector<int>(n2max / 16 + 1, -1));
   for (int wc = 0; wc < nwc; ++wc)
     if (lrows_c[wc] > 0)
       for (int h = 16; h <= n2max; h += 16)
-        lmap[wc][h / 16] = add_map(tp->lmir, lbase[wc], ls, lrows_c[wc], wcls_w[wc], wcls_w[wc], h, bc2);
-  tp->cbtab.upload(cbtab, c.stream);
+        lmap[wc][h / 16] = add_map(tp->lmir, lbase[wc] * nsl, lrows_c[wc], wcls_w[wc], h);
   tp->maps.alloc(std::max<size_t>(maps.size(), 1), c.stream);
   if (!maps.empty())
     cuda_check(cudaMemcpyAsync(tp->maps.p, maps.data(), maps.size() * sizeof(CUtensorMap), cudaMemcpyHostToDevice,
@@ -1242,19 +1276,15 @@ void build_tma_plan(Context& c, Tilde& lt, Tilde& rt, int k, SigmaPlan& plan, in
               // the K block of n2': the column block (n2', qr') of g'
               const int qrp = Rb.find(gq[gp].first + LQA[n2p], gq[gp].second + LQB[n2p]);
               const int coff = cpos[qrp * 4 + n2p][1];
-              const int cbi = cpos[qrp * 4 + n2p][2];
               const int kk = pad16(Rb.dim[qrp]);
-              // one term for all slice pairs (expanded by the kernel)
-              m1.push_back({a1map[gp][cbi], nt[2], 0, (int)r0, coff, nt[0], kk, nsl << 4});
+              m1.push_back({a1map[gp], nt[2], coff, (int)r0, coff, nt[0], kk, nsl << 4});
               ksum += kk * npair;
-              st1_steps += (kk + 63) / 64 * npair;
+              st1_steps += kk / TM_PIECE_COLS;
             }
             tl.t1 = (int)m1.size();
             tl.nseg = 1;
-            tl.xbase = xreg[ci][gp];
+            tl.xbase = xreg[ci][gp] * nsl;
             tl.xrows = xregrows[ci][gp];
-            tl.cb0 = cbt0[gp];
-            tl.cb1 = cbt1[gp];
             tl.n = nt[1];
             tl.m_valid = 128;
             tl.ldo = gR[gp];
@@ -1277,12 +1307,10 @@ void build_tma_plan(Context& c, Tilde& lt, Tilde& rt, int k, SigmaPlan& plan, in
           const int g = gout[(size_t)beta * ng + gp];
           for (const auto& cb : gcol[g]) {
             if (written.count(((long)beta * 4 + cb[0]) * nR + cb[1])) continue;
-            const long r0 = xrow[(size_t)beta * ng + gp] + cb[2];
-            for (const auto& rr : grow[gp]) {
-              const int w = pad16(Lb.dim[rr[0]]);
-              const long e0 = xreg[ci][gp] + xregrows[ci][gp] * rr[2] + r0 * w;
-              zj.push_back({tp->xt.p + e0, (long)pad16(Rb.dim[cb[1]]) * w, tp->x_stride, nsl});
-            }
+            // the block's rows in every column group
+            const long r0 = xrow[(size_t)beta * ng + gp] + cb[2], rows = xregrows[ci][gp];
+            zj.push_back({tp->xt.p + xreg[ci][gp] * nsl + r0 * 8, (long)pad16(Rb.dim[cb[1]]) * 8, rows * gR[gp], nsl,
+                          gR[gp] / 8, rows * 8});
           }
         }
       }
@@ -1318,14 +1346,14 @@ void build_tma_plan(Context& c, Tilde& lt, Tilde& rt, int k, SigmaPlan& plan, in
               if (rpp[0] != gp) continue;
               const int mid_ = lmid[beta][n1 * 4 + n1p];
               const int wc = wcls[pad16(Lb.dim[qlp])];
-              base.push_back({xtmap[ci][gp][rpp[2]], lmap[wc][nw / 16], 0, (int)xrow[(size_t)beta * ng + gp], 0,
+              base.push_back({xtmap[ci][gp], lmap[wc][nw / 16], rpp[1], (int)xrow[(size_t)beta * ng + gp], 0,
                               (int)(mblk_row[mid_][bl] + c0), pad16(Lb.dim[qlp]), (int)lneg[beta][n1 * 4 + n1p]});
             }
           }
           if (base.empty()) continue;
-          for (TmTerm& t : base) t.neg |= nsl << 4;  // all slice pairs, expanded by the kernel
-          long steps = 0;  // pieces (stage 2 packs TM_PACK_SLOTS per K step)
-          for (const TmTerm& t : base) steps += (t.k + bc2 - 1) / bc2 * npair;
+          for (TmTerm& t : base) t.neg |= nsl << 4;
+          long steps = 0;  // pieces
+          for (const TmTerm& t : base) steps += t.k / TM_PIECE_COLS;
           for (int r0 = 0; r0 < gC[g]; r0 += 128) {
             Pending pd;
             pd.tl = TmTile{};
@@ -1346,7 +1374,7 @@ void build_tma_plan(Context& c, Tilde& lt, Tilde& rt, int k, SigmaPlan& plan, in
       long acc = 0;
       size_t t0 = 0;
       for (size_t t = 0; t < pd.terms.size(); ++t) {
-        acc += (pd.terms[t].k + bc2 - 1) / bc2 * npair;
+        acc += pd.terms[t].k / TM_PIECE_COLS;
         if (acc >= target || t + 1 == pd.terms.size()) {
           TmTile tl = pd.tl;
           tl.t0 = (int)m2.size();
@@ -1356,7 +1384,7 @@ void build_tma_plan(Context& c, Tilde& lt, Tilde& rt, int k, SigmaPlan& plan, in
             ks += (long)pd.terms[u].k * npair;
           }
           tl.t1 = (int)m2.size();
-          const long stages = packed_stages(m2, tl.t0, tl.t1);
+          const long stages = (ks / npair / TM_PIECE_COLS + tm_slots(nsl) - 1) / tm_slots(nsl);
           if (stages > (1L << 30)) throw Error(ST_ECUDA, "internal: stage-2 tile too long");
           t2.push_back(tl);
           st2_steps += stages;
@@ -1385,78 +1413,50 @@ void build_tma_plan(Context& c, Tilde& lt, Tilde& rt, int k, SigmaPlan& plan, in
     order(t2, m2);
     // the copy lists of both launches (stage 2: sets every tile's stages and segments);
     // their pieces follow from the terms checked below
-    ch.l1.plan(TM_MODE_STORE_BF16, t1, m1, c.stream);
-    ch.l2.plan(TM_MODE_REDUCE_F32, t2, m2, c.stream);
+    ch.l1.plan(TM_MODE_STORE_BF16, nsl, t1, m1, c.stream);
+    ch.l2.plan(TM_MODE_REDUCE_F32, nsl, t2, m2, c.stream);
     st1_tiles += (double)t1.size();
     st2_tiles += (double)t2.size();
     // every access of the kernels checked against its buffer before anything runs:
     // operand boxes (their coordinates, alignment and widths), the rows stage 1 stores
     // through the row map and the blocks stage 2 reduces into
-    auto check_terms = [&](const std::vector<TmTile>& tt, const std::vector<TmTerm>& mm, int nmax, int bc) {
+    auto check_terms = [&](const std::vector<TmTile>& tt, const std::vector<TmTerm>& mm, int nmax) {
       for (const TmTile& tl : tt) {
         if (tl.n < 16 || tl.n > nmax || tl.n % 16 || tl.t0 < 0 || tl.t1 <= tl.t0 || tl.t1 > (int)mm.size())
           throw Error(ST_ECUDA, "internal: malformed TMA tile");
         for (int t = tl.t0; t < tl.t1; ++t) {
           const TmTerm& m = mm[t];
-          if (((m.neg >> 4) & 15) != nsl || m.amap < 0 || m.amap + nsl > (int)minfo.size() || m.bmap < 0 ||
-              m.bmap + nsl > (int)minfo.size() ||
-              minfo[m.amap].box != 128 || minfo[m.bmap].box != tl.n || minfo[m.amap].boxc != bc ||
-              minfo[m.bmap].boxc != bc || m.k < 16 || m.k % 16 || m.ax % 16 || m.bx % 16 || m.ax < 0 || m.bx < 0 ||
-              m.ay < 0 || m.by < 0 || m.ax + m.k > minfo[m.amap].cols + bc - 1 ||
-              m.bx + m.k > minfo[m.bmap].cols + bc - 1)
+          if (((m.neg >> 4) & 15) != nsl || m.amap < 0 || m.amap >= (int)minfo.size() || m.bmap < 0 ||
+              m.bmap >= (int)minfo.size() || minfo[m.amap].box != 128 || minfo[m.bmap].box != tl.n || m.k < 16 ||
+              m.k % 16 || m.ax % 8 || m.bx % 8 || m.ay % 16 || m.by % 16 || m.ax < 0 || m.bx < 0 || m.ay < 0 ||
+              m.by < 0 || m.ay >= minfo[m.amap].rows || m.by >= minfo[m.bmap].rows ||
+              m.ax + m.k > minfo[m.amap].cols || m.bx + m.k > minfo[m.bmap].cols)
             throw Error(ST_ECUDA, "internal: malformed TMA term");
         }
       }
     };
-    check_terms(t1, m1, n1max, bc1);
-    check_terms(t2, m2, n2max, bc2);
+    check_terms(t1, m1, n1max);
+    check_terms(t2, m2, n2max);
+    // stage-1 stores: every row inside its region, every region (all slices) inside X
+    for (const long d : rowmap)
+      if (d < -1) throw Error(ST_ECUDA, "internal: stage-1 row map");
     {
-      // the column blocks of every input group in increasing, disjoint column order, so
-      // that a chunk's block is found by binary search (the kernel takes the one block
-      // that holds the chunk)
-      for (int gp = 0; gp < ng; ++gp)
-        for (int e = cbt0[gp] + 1; e < cbt1[gp]; ++e)
-          if (cbtab[(size_t)e].x < cbtab[(size_t)e - 1].x + cbtab[(size_t)e - 1].y)
-            throw Error(ST_ECUDA, "internal: overlapping column blocks");
       std::atomic<int> bad{0}, next{0};
       auto check_range = [&]() {
         for (int i0 = next.fetch_add(1024); i0 < (int)t1.size() && !bad.load(); i0 = next.fetch_add(1024))
           for (int ti = i0; ti < std::min<int>((int)t1.size(), i0 + 1024); ++ti) {
             const TmTile& tl = t1[(size_t)ti];
-            if (tl.rowmap_off < 0 || tl.rowmap_off + 128 > (long)rowmap.size() || tl.cb0 < 0 ||
-                tl.cb1 > (int)cbtab.size() || tl.cb0 >= tl.cb1) {
-              bad = 1;  // row map or column blocks out of range
+            if (tl.rowmap_off < 0 || tl.rowmap_off + 128 > (long)rowmap.size() || tl.out_off < 0 || tl.out_off % 8 ||
+                tl.ldo % 8 || tl.out_off + tl.n > tl.ldo || tl.xbase < 0 || tl.xbase % 8 || tl.xrows < 1 ||
+                (size_t)(tl.xbase + nsl * tl.xrows * tl.ldo) > tp->xt.n) {
+              bad = 1;  // row map, columns or region out of range
               return;
             }
-            long dmax = -1;
-            for (int r = 0; r < 128; ++r) {
-              const long d = rowmap[(size_t)(tl.rowmap_off + r)];
-              if (d < -1 || d >= tl.xrows) {
+            for (int r = 0; r < 128; ++r)
+              if (rowmap[(size_t)(tl.rowmap_off + r)] >= tl.xrows) {
                 bad = 2;  // row outside its X region
                 return;
               }
-              dmax = std::max(dmax, d);
-            }
-            // every 8-column chunk of the tile lies in one column block; its highest row
-            // stays inside the buffer (addresses grow with the row)
-            for (int cc = 0; cc < tl.n; cc += 8) {
-              const long col = tl.out_off + cc;
-              int lo = tl.cb0, hi = tl.cb1 - 1;  // the last block starting at or before col
-              while (lo < hi) {
-                const int mid = (lo + hi + 1) / 2;
-                if (cbtab[(size_t)mid].x <= col) lo = mid; else hi = mid - 1;
-              }
-              const int2 cb = cbtab[(size_t)lo];
-              if (!(col >= cb.x && col + 8 <= cb.x + cb.y)) {
-                bad = 3;  // column outside the column blocks
-                return;
-              }
-              const long a0 = tl.xbase + tl.xrows * cb.x + (col - cb.x);
-              if (a0 < 0 || a0 % 8 || cb.y % 8 || (dmax >= 0 && a0 + dmax * cb.y + 8 > tp->x_stride)) {
-                bad = 4;  // store outside the X buffer
-                return;
-              }
-            }
           }
       };
       const int nth = (int)std::max(1u, std::min(16u, std::thread::hardware_concurrency()));
@@ -1467,8 +1467,10 @@ void build_tma_plan(Context& c, Tilde& lt, Tilde& rt, int k, SigmaPlan& plan, in
       if (bad) throw Error(ST_ECUDA, "internal: stage-1 tile check failed (" + std::to_string(bad.load()) + ")");
     }
     for (const TmTile& tl : t2) {
-      const long stages = packed_stages(m2, tl.t0, tl.t1);
-      if (tl.pad != stages || stages < 1 || tl.nseg != (int)((stages + TM_SEG_KSTEPS - 1) / TM_SEG_KSTEPS))
+      long pieces = 0;
+      for (int t = tl.t0; t < tl.t1; ++t) pieces += m2[(size_t)t].k / TM_PIECE_COLS;
+      const long stages = (pieces + tm_slots(nsl) - 1) / tm_slots(nsl);
+      if (tl.pad != stages || stages < 1 || tl.nseg != (int)((stages + tm_seg_stages(nsl) - 1) / tm_seg_stages(nsl)))
         throw Error(ST_ECUDA, "internal: stage-2 stage or segment count");
     }
 
@@ -1477,7 +1479,7 @@ void build_tma_plan(Context& c, Tilde& lt, Tilde& rt, int k, SigmaPlan& plan, in
           tl.out_off + (long)(tl.m_valid - 1) * tl.ldo + tl.n > tp->sig_total)
         throw Error(ST_ECUDA, "internal: stage-2 reduction outside sigma^T");
     for (const ZeroJob& z : zj)
-      if (z.p < tp->xt.p || z.p + (long)(z.nsl - 1) * z.stride + z.n > tp->xt.p + tp->xt.n)
+      if (z.p < tp->xt.p || z.p + (long)(z.nsl - 1) * z.stride + (z.reps - 1) * z.pitch + z.n > tp->xt.p + tp->xt.n)
         throw Error(ST_ECUDA, "internal: zero job outside X");
     ch.t1.upload(t1, c.stream);
     ch.m1.upload(m1, c.stream);
@@ -1485,8 +1487,8 @@ void build_tma_plan(Context& c, Tilde& lt, Tilde& rt, int k, SigmaPlan& plan, in
     ch.t2.upload(t2, c.stream);
     ch.m2.upload(m2, c.stream);
     ch.n2 = (int)t2.size();
-    ch.l1.fill(TM_MODE_STORE_BF16, ch.t1.p, ch.n1, ch.m1.p, c.stream);
-    ch.l2.fill(TM_MODE_REDUCE_F32, ch.t2.p, ch.n2, ch.m2.p, c.stream);
+    ch.l1.fill(TM_MODE_STORE_BF16, nsl, ch.t1.p, ch.n1, ch.m1.p, c.stream);
+    ch.l2.fill(TM_MODE_REDUCE_F32, nsl, ch.t2.p, ch.n2, ch.m2.p, c.stream);
     ch.nz = (int)zj.size();
     for (const ZeroJob& z : zj) ch.zmax = std::max(ch.zmax, z.n);
     ch.z.upload(zj, c.stream);
@@ -1494,8 +1496,8 @@ void build_tma_plan(Context& c, Tilde& lt, Tilde& rt, int k, SigmaPlan& plan, in
   }
   tp->rowmap.upload(rowmap, c.stream);
   // the operator stacks depend only on the environments: filled once per plan
-  if (tp->n_a1_jobs) launch_conv(tp->a1_jobs, tp->n_a1_jobs, tp->a1_maxel, c.stream);
-  if (tp->n_l_jobs) launch_conv(tp->l_jobs, tp->n_l_jobs, tp->l_maxel, c.stream);
+  if (tp->n_a1_jobs) launch_conv_groups(tp->a1_jobs, tp->n_a1_jobs, nsl, tp->a1_maxel, c.stream);
+  if (tp->n_l_jobs) launch_conv_groups(tp->l_jobs, tp->n_l_jobs, nsl, tp->l_maxel, c.stream);
   tp->err.alloc(1, c.stream);
   cuda_check(cudaMemsetAsync(tp->err.p, 0, sizeof(int), c.stream), "memset");
   cuda_check(cudaStreamSynchronize(c.stream), "sync");
@@ -1513,21 +1515,19 @@ void build_tma_plan(Context& c, Tilde& lt, Tilde& rt, int k, SigmaPlan& plan, in
 
 void run_tma_sigma(Context& c, SigmaPlan& plan, const double* x, double* y) {
   TmaPlan& tp = *plan.tm;
-  const size_t n = plan.psi.nnz;
-  if (x != plan.in.p) cuda_check(cudaMemcpyAsync(plan.in.p, x, n * sizeof(double), cudaMemcpyDeviceToDevice, c.stream), "d2d");
-  if (tp.n_psi_jobs) launch_conv(tp.psi_jobs, tp.n_psi_jobs, tp.psi_maxel, c.stream);
+  // the conversions read x and write y themselves (their jobs are made for plan.in and plan.out)
+  if (tp.n_psi_jobs) launch_conv_groups(tp.psi_jobs, tp.n_psi_jobs, tp.nsl, tp.psi_maxel, c.stream, x - plan.in.p);
   cuda_check(cudaMemsetAsync(tp.sig_t.p, 0, tp.sig_total * sizeof(float), c.stream), "memset");
   for (auto& ch : tp.chunks) {
     if (ch.nz) launch_zero(ch.z.p, ch.nz, ch.zmax, c.stream);
-    cuda_check(launch_gemm_tma(TM_MODE_STORE_BF16, ch.t1.p, ch.n1, ch.m1.p, tp.maps.p, tp.rowmap.p, tp.cbtab.p,
-                               tp.xt.p, tp.nsl, tp.x_stride, tp.err.p, c.stream, ch.l1.dev()),
+    cuda_check(launch_gemm_slices(TM_MODE_STORE_BF16, tp.nsl, ch.t1.p, ch.n1, tp.maps.p, tp.rowmap.p, tp.xt.p, tp.err.p,
+                                  c.stream, ch.l1.dev()),
                "tma stage 1");
-    cuda_check(launch_gemm_tma(TM_MODE_REDUCE_F32, ch.t2.p, ch.n2, ch.m2.p, tp.maps.p, tp.rowmap.p, tp.cbtab.p,
-                               tp.sig_t.p, 1, 0, tp.err.p, c.stream, ch.l2.dev()),
+    cuda_check(launch_gemm_slices(TM_MODE_REDUCE_F32, tp.nsl, ch.t2.p, ch.n2, tp.maps.p, nullptr, tp.sig_t.p, tp.err.p,
+                                  c.stream, ch.l2.dev()),
                "tma stage 2");
   }
-  if (tp.n_sig_jobs) launch_unconv(tp.sig_jobs.p, tp.n_sig_jobs, tp.sig_maxel, c.stream);
-  if (y != plan.out.p) cuda_check(cudaMemcpyAsync(y, plan.out.p, n * sizeof(double), cudaMemcpyDeviceToDevice, c.stream), "d2d");
+  if (tp.n_sig_jobs) launch_unconv(tp.sig_jobs.p, tp.n_sig_jobs, tp.sig_maxel, c.stream, y - plan.out.p);
 }
 
 int plan_error(Context& c, SigmaPlan& plan) {
@@ -2230,12 +2230,11 @@ void env_update_exact(Context& c, Tilde& t, const SiteT& A, int site, Env& out, 
     // copy lists of every launch; each piece reads through one of this update's maps
     // copy lists of every launch (their pieces follow from the terms checked above)
     TmaPlan::Lists dl1;
-    dl1.plan(TM_MODE_EXACT_F64, e1t, e1m, c.stream);
+    dl1.plan(TM_MODE_EXACT_F64, 1, e1t, e1m, c.stream);
     d1t.upload(e1t, c.stream);
     d1m.upload(e1m, c.stream);
-    dl1.fill(TM_MODE_EXACT_F64, d1t.p, (int)e1t.size(), d1m.p, c.stream);
-    cuda_check(launch_gemm_tma(TM_MODE_EXACT_F64, d1t.p, (int)e1t.size(), d1m.p, dmaps.p, nullptr, nullptr, T64.p, 1, 0,
-                               err.p, c.stream, dl1.dev(), expo.p),
+    dl1.fill(TM_MODE_EXACT_F64, 1, d1t.p, (int)e1t.size(), d1m.p, c.stream);
+    cuda_check(launch_gemm_exact(d1t.p, (int)e1t.size(), d1m.p, dmaps.p, T64.p, err.p, c.stream, dl1.dev(), expo.p),
                "exact stage 1");
     DArr<SplitJob> dj2;
     dj2.upload(split2, c.stream);
@@ -2245,11 +2244,11 @@ void env_update_exact(Context& c, Tilde& t, const SiteT& A, int site, Env& out, 
     std::vector<TmaPlan::Lists> dl2(out.cls.size());
     for (size_t ci = 0; ci < out.cls.size(); ++ci) {
       if (e2t[ci].empty()) continue;
-      dl2[ci].plan(TM_MODE_EXACT_F64, e2t[ci], e2m, c.stream);
+      dl2[ci].plan(TM_MODE_EXACT_F64, 1, e2t[ci], e2m, c.stream);
       d2t[ci].upload(e2t[ci], c.stream);
-      dl2[ci].fill(TM_MODE_EXACT_F64, d2t[ci].p, (int)e2t[ci].size(), d2m.p, c.stream);
-      cuda_check(launch_gemm_tma(TM_MODE_EXACT_F64, d2t[ci].p, (int)e2t[ci].size(), d2m.p, dmaps.p, nullptr, nullptr,
-                                 out.data[ci].p, 1, 0, err.p, c.stream, dl2[ci].dev(), expo.p),
+      dl2[ci].fill(TM_MODE_EXACT_F64, 1, d2t[ci].p, (int)e2t[ci].size(), d2m.p, c.stream);
+      cuda_check(launch_gemm_exact(d2t[ci].p, (int)e2t[ci].size(), d2m.p, dmaps.p, out.data[ci].p, err.p, c.stream,
+                                   dl2[ci].dev(), expo.p),
                  "exact stage 2");
     }
     // the host lists and the chunk's buffers must outlive the launches

@@ -1,18 +1,16 @@
 // TMA-staged tensor-core grouped GEMM (tcgen05, sm_103a): BF16 operands, FP32
 // accumulation in tensor memory.
 //
-// The operands of the sigma vector live in a few large row-major BF16 matrices (per
+// The operands of the sigma vector live in a few large BF16 matrices (per
 // quantum-number group of the cut: the stacked two-site wavefunction Psi_g, the stacked
-// right operators, the X intermediates; one matrix for all left-operator blocks), each
-// described by one tensor map.  A stage of the ring is one or more pieces, each a pair of
-// TMA box copies (A: 128 rows, B: n rows; 64 columns with 128-byte swizzle, or in the
-// reduce mode up to four 16-column pieces with 32-byte swizzle) that complete on the
-// stage's mbarrier by transaction count; zero fill outside the matrix covers ragged edges.
-// The tiles' terms are expanded before the launch into per-CTA copy lists (stage word,
-// expected bytes, box coordinates: fill_lists_kernel), so the producer does no term
-// arithmetic.
+// right operators, the X intermediates; one matrix per width for the left-operator blocks),
+// each described by one tensor map per box height.  A stage of the ring is one or more
+// pieces, each a pair of TMA box copies that complete on the stage's mbarrier by transaction
+// count; zero fill outside the matrix covers ragged edges.  The tiles' terms are expanded
+// before the launch into per-CTA copy lists (stage word, expected bytes, box coordinates:
+// fill_lists_kernel), so the producer does no term arithmetic.
 //
-// Persistent and warp-specialised, one CTA per SM (up to 212 KB of shared memory,
+// Persistent and warp-specialised, one CTA per SM (up to 221 KB of shared memory,
 // all 512 tensor-memory columns):
 //   warp 0     fetches its CTA's copy lists 32 stages at a time into shared memory
 //              (1D bulk copies, double-buffered); per stage lane 0 waits for the ring
@@ -21,15 +19,24 @@
 //   warp 1     one thread issues tcgen05.mma (M = 128, N = n, K = 16 per instruction)
 //              and commits to the stage's empty barrier / the accumulator's full
 //              barrier
-//   warps 2-5  epilogue: tcgen05.ld of their 32 tensor-memory lanes; BF16 rows
-//              (X intermediates, up to three slices) written with 16-byte stores to
-//              the rows a row map gives, FP32 vector reductions (sigma^T, several
-//              tiles may add into one block) of per-segment partial sums, or (exact
-//              mode) two-float sums of exact integer segments stored in FP64
+//   warps 2-5  epilogue: tcgen05.ld of their 32 tensor-memory lanes; BF16 slices of the X
+//              intermediates, FP32 vector reductions (sigma^T, several tiles may add into
+//              one block) of per-segment partial sums, or (exact mode) two-float sums of
+//              exact integer segments stored in FP64
 // Two (store mode, N <= 256), four (reduce mode, N <= 128) or eight (exact mode, N <=
 // 64) accumulators let the epilogue of one tile overlap the MMAs of the next.  Every
 // wait is bounded: on timeout the CTA raises a shared abort flag, records an error,
 // waits (bounded) for the copies it issued, frees its tensor memory and returns.
+//
+// gemm_slices_kernel (sigma): what bounds it is the operand traffic into shared memory, not
+// the tensor cores: a 128 x n tile of one K=16 product needs 32 (128 + n) bytes through L2
+// for n / 2 tensor clocks.  With two or three slices the products s_i t_j, i + j < nsl, share
+// their operands, so a piece brings every slice of both operands once (3 + 3 boxes' worth of
+// bytes for six products instead of 6 + 6) in two copies instead of twelve, and the
+// column-group layout lets each copy move 256-byte runs instead of 32-byte rows.
+// Measured against one pair of swizzled boxes per slice product (16-column boxes in the
+// reduce mode): three slices at K=24, M=512 3.18 -> 1.61 ms per sigma, K=40, M=1200 23.1 ->
+// 11.3 ms; one pass at K=32, M=1024 2.71 -> 1.79 ms.
 #include "kernels_tma.hpp"
 
 #include <cuda_bf16.h>
@@ -48,31 +55,25 @@ void count_tc_launches(long n);
 namespace {
 
 constexpr int TM_THREADS = 192;
-constexpr int TM_BOX_K = 64;                       // columns per box (128 bytes)
-constexpr int TM_A_BYTES = 128 * TM_BOX_K * 2;     // 16 KB
-constexpr int TM_SLOT_A = 128 * TM_PACK_COLS * 2;  // packed mode: one piece of A (or B, n <= 128)
+constexpr int TM_BOX_K = 64;                    // exact mode: columns per box (128 bytes)
+constexpr int TM_A_BYTES = 128 * TM_BOX_K * 2;  // 16 KB
 constexpr long TM_WAIT_LIMIT = 1L << 24;
 constexpr int TM_REC_BATCH = 32;  // stages of the copy lists fetched per bulk copy
 
-template <int MODE>
+template <int MODE, int NSL>
 struct TmCfg {
   static constexpr bool STORE = MODE == TM_MODE_STORE_BF16;
   static constexpr bool EXACT = MODE == TM_MODE_EXACT_F64;
-  // reduce mode: a stage holds up to TM_PACK_SLOTS pieces of 16 columns (32-byte swizzled
-  // boxes), from any terms of the tile, one K=16 instruction each
-  static constexpr bool PACK = MODE == TM_MODE_REDUCE_F32;
   // exact mode: 64 columns, so that the two-float sums (128 registers) fit
   static constexpr int NMAX = STORE ? 256 : (EXACT ? 64 : 128);
   static constexpr int NACC = 512 / NMAX;
-  static constexpr int B_BYTES = NMAX * TM_BOX_K * 2;
-  static constexpr int STAGE_BYTES = TM_A_BYTES + B_BYTES;
-  // store mode: each epilogue warp stages its 32 rows in shared memory (rows padded
-  // by 16 bytes against bank conflicts) and writes them row by row with coalesced
-  // 16-byte stores
-  static constexpr int STAGE_LD = NMAX + 8;  // elements per staged row
-  static constexpr int STAGING = STORE ? 128 * STAGE_LD * 2 : 0;
-  static constexpr int STAGES = STORE ? 3 : (EXACT ? 8 : 6);
-  static constexpr int SMEM = STAGES * STAGE_BYTES + STAGING + 1024;
+  static constexpr int SLOTS = EXACT ? 1 : tm_slots(NSL);
+  // bytes of one piece of A and of the largest piece of B (all slices)
+  static constexpr int A_BYTES = EXACT ? TM_A_BYTES : 128 * TM_PIECE_COLS * 2 * NSL;
+  static constexpr int B_BYTES = EXACT ? NMAX * TM_BOX_K * 2 : NMAX * TM_PIECE_COLS * 2 * NSL;
+  static constexpr int STAGE_BYTES = SLOTS * (A_BYTES + B_BYTES);
+  static constexpr int STAGES = EXACT ? 8 : (STORE ? (NSL == 3 ? 6 : 4) : (NSL == 3 ? 8 : 6));
+  static constexpr int SMEM = STAGES * STAGE_BYTES + 1024;
 };
 constexpr int TM_MAX_STAGES = 8, TM_MAX_ACC = 8;
 
@@ -89,16 +90,14 @@ __device__ __forceinline__ uint64_t sdesc(uint32_t saddr) {
   return d;
 }
 
-// the same for the packed pieces: K-major rows of TM_PACK_COLS columns, swizzled over
-// their width (32 columns: 64-byte swizzle, 8-row groups 512 B apart; 16 columns: 32-byte
-// swizzle, 256 B apart)
-__device__ __forceinline__ uint64_t sdesc_pack(uint32_t saddr) {
+// the same for the column-group layout: K-major without swizzle, core matrices of 8 rows x
+// 16 bytes contiguous along the rows (128 B apart), the second 8 columns `rows` rows further
+__device__ __forceinline__ uint64_t sdesc_groups(uint32_t saddr, int rows) {
   uint64_t d = 0;
   d |= (uint64_t)((saddr >> 4) & 0x3FFFu);
-  d |= (uint64_t)1 << 16;
-  d |= (uint64_t)((8 * TM_PACK_COLS * 2) >> 4) << 32;
+  d |= (uint64_t)(uint32_t)rows << 16;  // (rows * 16) >> 4
+  d |= (uint64_t)(128 >> 4) << 32;
   d |= (uint64_t)1 << 46;
-  d |= (uint64_t)(TM_PACK_COLS == 32 ? 4 : 6) << 61;
   return d;
 }
 
@@ -138,6 +137,15 @@ __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map
       : "memory");
 }
 
+// box of a column-group map: all of dimension 0, row group y, column group x, every slice
+__device__ __forceinline__ void tma_load_groups(uint32_t dst, const CUtensorMap* map, int x, int y, uint64_t* bar) {
+  asm volatile(
+      "cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %2}], "
+      "[%5];\n" ::"r"(dst),
+      "l"(map), "r"(0), "r"(y), "r"(x), "r"(smem_u32(bar))
+      : "memory");
+}
+
 // 1D bulk copy global -> shared (16-byte aligned addresses, size a multiple of 16), completing on bar
 __device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_t bytes, uint64_t* bar) {
   asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n" ::"r"(dst),
@@ -164,19 +172,13 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&v)[32]) {
   asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
 }
 
-__device__ __forceinline__ uint32_t pack_bf16x2(uint32_t lo, uint32_t hi) {
-  const __nv_bfloat162 h = __floats2bfloat162_rn(__uint_as_float(lo), __uint_as_float(hi));
-  return *reinterpret_cast<const uint32_t*>(&h);
-}
-
-template <int MODE>
+template <int MODE, int NSL>
 __global__ void __launch_bounds__(TM_THREADS, 1)
     gemm_tma_kernel(const TmTile* __restrict__ tiles, int ntiles, const TmTerm* __restrict__ terms,
-                    const CUtensorMap* __restrict__ maps, const long* __restrict__ rowmap,
-                    const int2* __restrict__ cbtab, void* __restrict__ out, int out_slices, long slice_stride,
+                    const CUtensorMap* __restrict__ maps, const long* __restrict__ rowmap, void* __restrict__ out,
                     int* __restrict__ err, const int* __restrict__ expo, const int* __restrict__ cta_stage,
                     const TmStage* __restrict__ stg, const TmPiece* __restrict__ pcs) {
-  using Cfg = TmCfg<MODE>;
+  using Cfg = TmCfg<MODE, NSL>;
   constexpr int S = Cfg::STAGES;
   constexpr int STAGE_BYTES = Cfg::STAGE_BYTES;
   constexpr int NACC = Cfg::NACC;
@@ -188,19 +190,15 @@ __global__ void __launch_bounds__(TM_THREADS, 1)
       tempty_b[TM_MAX_ACC];
   __shared__ uint32_t tmem_base_sh;
   __shared__ int abort_sh;
-  // per stage: instruction descriptor, K=16 steps, first K step of a segment, last K
-  // step of a segment, last K step of the tile
-  // (packed into one 64-bit word: low half the instruction descriptor, high half the
-  // K=16 steps in bits 0-2 and the flags first / segment end / last in bits 3-5)
+  // per stage: the stage word (TmStage)
   __shared__ uint64_t meta[TM_MAX_STAGES];
   // copy lists of the producer: batches of TM_REC_BATCH stages, double-buffered, each
   // landing by bulk copy on rec_b[buffer]
-  constexpr int PCS = Cfg::PACK ? TM_PACK_SLOTS : 1;
+  constexpr int PCS = Cfg::SLOTS;
   __shared__ __align__(16) TmStage rec_stage[2][TM_REC_BATCH];
   __shared__ __align__(16) TmPiece rec_piece[2][TM_REC_BATCH * PCS];
   __shared__ __align__(8) uint64_t rec_b[2];
   const uint32_t base = (smem_u32(dsm) + 1023u) & ~1023u;
-  uint8_t* const base_ptr = dsm + (base - smem_u32(dsm));
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
   if (warp == 2) {  // an epilogue warp (all lanes take the same path) owns the tensor memory
@@ -234,7 +232,6 @@ __global__ void __launch_bounds__(TM_THREADS, 1)
     // stage lane 0 waits until the ring slot is free and posts the stage word and the
     // expected bytes, then lane p < np issues the two box copies of piece p.
     constexpr int PIECES = PCS;
-    constexpr uint32_t A_BOX = 128u * (Cfg::PACK ? TM_PACK_COLS : TM_BOX_K) * 2;
     constexpr unsigned FULL = 0xffffffffu;
     long j = 0;            // stages issued
     int st = 0;            // ring slot of the next one (j % S)
@@ -278,8 +275,14 @@ __global__ void __launch_bounds__(TM_THREADS, 1)
         if (lane < h.np) {
           const TmPiece q = rec_piece[b & 1][i * PIECES + lane];
           const uint32_t sa = base + st * STAGE_BYTES;
-          tma_load_2d(sa + lane * A_BOX, maps + q.amap, q.ax, q.ay, &full_b[st]);
-          tma_load_2d(sa + PIECES * A_BOX + lane * A_BOX, maps + q.bmap, q.bx, q.by, &full_b[st]);
+          const uint32_t da = sa + lane * Cfg::A_BYTES, db = sa + PIECES * Cfg::A_BYTES + lane * Cfg::B_BYTES;
+          if constexpr (EXACT) {
+            tma_load_2d(da, maps + q.amap, q.ax, q.ay, &full_b[st]);
+            tma_load_2d(db, maps + q.bmap, q.bx, q.by, &full_b[st]);
+          } else {
+            tma_load_groups(da, maps + q.amap, q.ax, q.ay, &full_b[st]);
+            tma_load_groups(db, maps + q.bmap, q.bx, q.by, &full_b[st]);
+          }
         }
         ++j;
         if (++st == S) {
@@ -309,11 +312,11 @@ __global__ void __launch_bounds__(TM_THREADS, 1)
       uint32_t par = 0;      // its round's parity
       int sg = 0;  // segments issued
       bool ok = true;
-      // shared-memory descriptors of stage 0's operands; stage s and K=16 step kk add
-      // (s * STAGE_BYTES + kk * 32) / 16 to the 14-bit address field (no carry: shared
+      // shared-memory descriptors of stage 0's operands; later stages, slots, slices and K
+      // steps add their byte offsets / 16 to the 14-bit address field (no carry: shared
       // addresses stay below 256 KB)
-      const uint64_t ad0 = Cfg::PACK ? sdesc_pack(base) : sdesc(base);
-      const uint64_t bd0 = Cfg::PACK ? sdesc_pack(base + TM_PACK_SLOTS * TM_SLOT_A) : sdesc(base + TM_A_BYTES);
+      const uint64_t ad0 = EXACT ? sdesc(base) : sdesc_groups(base, 128);
+      const uint64_t bd0 = EXACT ? sdesc(base + TM_A_BYTES) : sdesc_groups(base + Cfg::SLOTS * Cfg::A_BYTES, 0);
       for (int ti = blockIdx.x; ti < ntiles && ok; ti += gridDim.x) {
         bool tile_done = false;
         while (!tile_done && ok) {
@@ -334,21 +337,28 @@ __global__ void __launch_bounds__(TM_THREADS, 1)
             const uint32_t id = (uint32_t)mw, fl = (uint32_t)(mw >> 32);
             const int nk = (int)(fl & 7u);
             const uint64_t off = (uint64_t)((st * STAGE_BYTES) >> 4);
-            // (packed) slot sl: A at sl * TM_SLOT_A, B at TM_PACK_SLOTS * TM_SLOT_A + sl *
-            // TM_SLOT_A of the stage, its K=16 steps 32 bytes apart along the row
-            const int nslot = Cfg::PACK ? nk : 1;
-            int m = 0;
-            for (int sl = 0; sl < nslot; ++sl) {
-              const int nks = Cfg::PACK ? (int)((fl >> (12 + 2 * sl)) & 3u) : nk;
-              const uint32_t idk = Cfg::PACK ? (id | (((fl >> (8 + sl)) & 1u) << 13)) : id;
-              const uint64_t so = Cfg::PACK ? (uint64_t)((sl * TM_SLOT_A) >> 4) : 0;
-              for (int kk = 0; kk < nks; ++kk, ++m) {
-                const uint64_t ad = ad0 + off + so + (uint64_t)(kk * 2), bd = bd0 + off + so + (uint64_t)(kk * 2);
-                const uint32_t accum = ((fl & 8u) && m == 0) ? 0u : 1u;
-                asm volatile(
-                    "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-                    " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(dacc),
-                    "l"(ad), "l"(bd), "r"(idk), "r"(accum));
+            uint32_t accum = (fl & 8u) ? 0u : 1u;
+            auto mma = [&](uint64_t ad, uint64_t bd, uint32_t idk) {
+              asm volatile(
+                  "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
+                  " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(dacc),
+                  "l"(ad), "l"(bd), "r"(idk), "r"(accum));
+              accum = 1u;
+            };
+            if constexpr (EXACT) {
+              for (int kk = 0; kk < nk; ++kk)
+                mma(ad0 + off + (uint64_t)(kk * 2), bd0 + off + (uint64_t)(kk * 2), id);
+            } else {
+              const uint32_t n = ((id >> 17) & 63u) << 3;  // rows of B: 8 columns are n * 16 bytes, a slice n * 32
+              const uint64_t bdn = bd0 + ((uint64_t)n << 16);
+              for (int sl = 0; sl < nk; ++sl) {
+                const uint32_t idk = id | (((fl >> (8 + sl)) & 1u) << 13);
+                const uint64_t ad = ad0 + off + (uint64_t)((sl * Cfg::A_BYTES) >> 4);
+                const uint64_t bd = bdn + off + (uint64_t)((sl * Cfg::B_BYTES) >> 4);
+#pragma unroll
+                for (int l = 0; l < NSL; ++l)
+#pragma unroll
+                  for (int i = 0; i <= l; ++i) mma(ad + (uint64_t)(i * 256), bd + (uint64_t)((l - i) * 2 * n), idk);
               }
             }
             asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(
@@ -373,12 +383,10 @@ __global__ void __launch_bounds__(TM_THREADS, 1)
     // ---------------- epilogue (warps 2-5: tensor-memory lanes 32 * (warp % 4) ...)
     const int sub = warp & 3;
     const int r = sub * 32 + lane;  // row of the tile
-    __nv_bfloat16* const srow =
-        reinterpret_cast<__nv_bfloat16*>(base_ptr + S * STAGE_BYTES) + (STORE ? r * Cfg::STAGE_LD : 0);
     int sg = 0;
     bool ok = true;
-    // the next tile's descriptor is loaded one tile ahead; in store mode the row map and
-    // column blocks of a tile are read before its accumulator is waited for
+    // the next tile's descriptor is loaded one tile ahead; in store mode the row map of a
+    // tile is read before its accumulator is waited for
     TmTile tl_next{};
     if ((int)blockIdx.x < ntiles) tl_next = tiles[blockIdx.x];
     for (int ti = blockIdx.x; ti < ntiles && ok; ti += gridDim.x) {
@@ -387,88 +395,38 @@ __global__ void __launch_bounds__(TM_THREADS, 1)
       if constexpr (STORE) {
         const int acc = sg % NACC;
         const long row_own = rowmap[tl.rowmap_off + r];
-        // this lane's 8-column chunk of every row: its column block, base and width
-        long lane_base = -1;
-        int lane_w = 0;
-        if (lane * 8 < tl.n) {
-          const long col = tl.out_off + lane * 8;
-          for (int e = tl.cb0; e < tl.cb1; ++e) {
-            const int2 cb = cbtab[e];
-            if (col >= cb.x && col < cb.x + cb.y) {
-              lane_base = tl.xbase + tl.xrows * cb.x + (col - cb.x);
-              lane_w = cb.y;
-            }
-          }
-        }
         ok = mbar_wait(&tfull_b[acc], (uint32_t)((sg / NACC) & 1), abort_flag);
         ok = __all_sync(0xffffffffu, ok);
         if (!ok) break;
         asm volatile("tcgen05.fence::after_thread_sync;\n" ::);
-        __nv_bfloat16* const wrows =
-            reinterpret_cast<__nv_bfloat16*>(base_ptr + S * STAGE_BYTES) + sub * 32 * Cfg::STAGE_LD;
-        if (out_slices == 1) {
-          // one pass: this thread's row into the staging rows of its warp, then the warp
-          // writes its 32 rows one after another, each as one contiguous run of 16-byte
-          // stores across the lanes (up to 512 bytes per instruction)
+        // per 8 columns one 16-byte store per slice, x = s0 + s1 + s2 from one read of each
+        // value; the lanes' rows are mostly consecutive, so a warp writes contiguous runs.
+        // The tensor-memory loads (32 columns, one wait) are warp-wide.
+        __nv_bfloat16* g = reinterpret_cast<__nv_bfloat16*>(out) + tl.xbase + tl.out_off * tl.xrows + row_own * 8;
+        const long slice = tl.xrows * tl.ldo;
 #pragma unroll 1
-          for (int c0 = 0; c0 < tl.n; c0 += 32) {
-            uint32_t v[32];
-            tmem_ld32(tmem + ((uint32_t)(sub * 32) << 16) + (uint32_t)(acc * NMAX + c0), v);
+        for (int c0 = 0; c0 < tl.n; c0 += 32) {
+          uint32_t v[32];
+          tmem_ld32(tmem + ((uint32_t)(sub * 32) << 16) + (uint32_t)(acc * NMAX + c0), v);
 #pragma unroll
-            for (int u = 0; u < 32; u += 8) {
-              uint4 w;
-              w.x = pack_bf16x2(v[u], v[u + 1]);
-              w.y = pack_bf16x2(v[u + 2], v[u + 3]);
-              w.z = pack_bf16x2(v[u + 4], v[u + 5]);
-              w.w = pack_bf16x2(v[u + 6], v[u + 7]);
-              if (c0 + u < tl.n) *reinterpret_cast<uint4*>(srow + c0 + u) = w;
-            }
-          }
-          __syncwarp();
-#pragma unroll 1
-          for (int rr = 0; rr < 32; ++rr) {
-            const long d = __shfl_sync(0xffffffffu, row_own, rr);
-            if (d >= 0 && lane_base >= 0) {
-              const uint4 w = *reinterpret_cast<const uint4*>(wrows + rr * Cfg::STAGE_LD + lane * 8);
-              *reinterpret_cast<uint4*>(reinterpret_cast<__nv_bfloat16*>(out) + lane_base + d * lane_w) = w;
-            }
-          }
-          __syncwarp();
-        } else {
-          // two or three slices x = s0 + s1 + s2 from one read of each value, stored
-          // directly: per 8 columns one 16-byte store per slice into this row.  The
-          // tensor-memory loads (32 columns, one wait) are warp-wide, the stores only for
-          // rows that exist; the column block of 8-column chunk c is lane c's (above)
-#pragma unroll 1
-          for (int c0 = 0; c0 < tl.n; c0 += 32) {
-            uint32_t v[32];
-            tmem_ld32(tmem + ((uint32_t)(sub * 32) << 16) + (uint32_t)(acc * NMAX + c0), v);
+          for (int u8 = 0; u8 < 32; u8 += 8) {
+            if (c0 + u8 >= tl.n || row_own < 0) continue;
+            uint32_t w[NSL][4];
 #pragma unroll
-            for (int u8 = 0; u8 < 32; u8 += 8) {
-              const int ch = (c0 + u8) >> 3;  // < NMAX / 8 <= 32
-              const long cb_base = __shfl_sync(0xffffffffu, lane_base, ch);
-              const int cb_w = __shfl_sync(0xffffffffu, lane_w, ch);
-              if (c0 + u8 >= tl.n) break;
-              uint32_t w[3][4];
+            for (int u = 0; u < 8; u += 2) {
+              float a = __uint_as_float(v[u8 + u]), b = __uint_as_float(v[u8 + u + 1]);
 #pragma unroll
-              for (int u = 0; u < 8; u += 2) {
-                float a = __uint_as_float(v[u8 + u]), b = __uint_as_float(v[u8 + u + 1]);
-#pragma unroll
-                for (int sl = 0; sl < 3; ++sl) {
-                  const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
-                  w[sl][u / 2] = *reinterpret_cast<const uint32_t*>(&h);
-                  a -= __low2float(h);
-                  b -= __high2float(h);
-                }
+              for (int sl = 0; sl < NSL; ++sl) {
+                const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
+                w[sl][u / 2] = *reinterpret_cast<const uint32_t*>(&h);
+                a -= __low2float(h);
+                b -= __high2float(h);
               }
-              if (cb_base < 0 || row_own < 0) continue;
-              __nv_bfloat16* g = reinterpret_cast<__nv_bfloat16*>(out) + cb_base + row_own * cb_w;
-#pragma unroll
-              for (int sl = 0; sl < 3; ++sl)
-                if (sl < out_slices)
-                  *reinterpret_cast<uint4*>(g + sl * slice_stride) =
-                      make_uint4(w[sl][0], w[sl][1], w[sl][2], w[sl][3]);
             }
+            __nv_bfloat16* q = g + (long)(c0 + u8) * tl.xrows;
+#pragma unroll
+            for (int sl = 0; sl < NSL; ++sl)
+              *reinterpret_cast<uint4*>(q + sl * slice) = make_uint4(w[sl][0], w[sl][1], w[sl][2], w[sl][3]);
           }
         }
         asm volatile("tcgen05.fence::before_thread_sync;\n" ::);
@@ -572,20 +530,20 @@ __global__ void __launch_bounds__(TM_THREADS, 1)
   }
 }
 
-template <int MODE>
+template <int MODE, int NSL>
 cudaError_t launch_mode(const TmTile* d_tiles, int ntiles, const TmTerm* d_terms, const CUtensorMap* d_maps,
-                        const long* d_rowmap, const int2* d_cbtab, void* out, int out_slices, long slice_stride,
-                        int* d_err, cudaStream_t s, const int* d_expo, const TmListsDev& lists) {
-  static const bool attr_ok = cudaFuncSetAttribute(gemm_tma_kernel<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                   TmCfg<MODE>::SMEM) == cudaSuccess;
+                        const long* d_rowmap, void* out, int* d_err, cudaStream_t s, const int* d_expo,
+                        const TmListsDev& lists) {
+  static const bool attr_ok =
+      cudaFuncSetAttribute(gemm_tma_kernel<MODE, NSL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           TmCfg<MODE, NSL>::SMEM) == cudaSuccess;
   if (!attr_ok) return cudaErrorInvalidValue;
   // the lists were built for this grid: every CTA's tiles and stages
   if (lists.grid != tma_grid(ntiles) || !lists.cta_stage || !lists.stages || !lists.pieces)
     return cudaErrorInvalidValue;
   count_tc_launches(1);
-  gemm_tma_kernel<MODE><<<lists.grid, TM_THREADS, TmCfg<MODE>::SMEM, s>>>(
-      d_tiles, ntiles, d_terms, d_maps, d_rowmap, d_cbtab, out, out_slices, slice_stride, d_err, d_expo,
-      lists.cta_stage, lists.stages, lists.pieces);
+  gemm_tma_kernel<MODE, NSL><<<lists.grid, TM_THREADS, TmCfg<MODE, NSL>::SMEM, s>>>(
+      d_tiles, ntiles, d_terms, d_maps, d_rowmap, out, d_err, d_expo, lists.cta_stage, lists.stages, lists.pieces);
   return cudaGetLastError();
 }
 
@@ -675,26 +633,29 @@ cudaError_t launch_split_exact(const SplitJob* d_jobs, int njobs, int nsl, int* 
 }
 
 int tma_max_n(int mode) { return mode == TM_MODE_STORE_BF16 ? 256 : (mode == TM_MODE_EXACT_F64 ? 64 : 128); }
-int tma_box_cols(int mode) { return mode == TM_MODE_REDUCE_F32 ? TM_PACK_COLS : TM_BOX_K; }
 
-cudaError_t launch_gemm_tma(int mode, const TmTile* d_tiles, int ntiles, const TmTerm* d_terms,
-                            const CUtensorMap* d_maps, const long* d_rowmap, const int2* d_cbtab, void* out,
-                            int out_slices, long slice_stride, int* d_err, cudaStream_t s, const TmListsDev& lists,
-                            const int* d_expo) {
+cudaError_t launch_gemm_slices(int mode, int nsl, const TmTile* d_tiles, int ntiles, const CUtensorMap* d_maps,
+                               const long* d_rowmap, void* out, int* d_err, cudaStream_t s, const TmListsDev& lists) {
   if (ntiles <= 0) return cudaSuccess;
-  if (out_slices < 1 || out_slices > 3) return cudaErrorInvalidValue;
-  if (mode == TM_MODE_STORE_BF16)
-    return launch_mode<TM_MODE_STORE_BF16>(d_tiles, ntiles, d_terms, d_maps, d_rowmap, d_cbtab, out, out_slices,
-                                           slice_stride, d_err, s, nullptr, lists);
-  if (mode == TM_MODE_REDUCE_F32)
-    return launch_mode<TM_MODE_REDUCE_F32>(d_tiles, ntiles, d_terms, d_maps, d_rowmap, d_cbtab, out, 1, 0, d_err, s,
-                                           nullptr, lists);
-  if (mode == TM_MODE_EXACT_F64) {
-    if (!d_expo || !d_terms) return cudaErrorInvalidValue;
-    return launch_mode<TM_MODE_EXACT_F64>(d_tiles, ntiles, d_terms, d_maps, d_rowmap, d_cbtab, out, 1, 0, d_err, s,
-                                          d_expo, lists);
+  auto go = [&](auto fn) { return fn(d_tiles, ntiles, nullptr, d_maps, d_rowmap, out, d_err, s, nullptr, lists); };
+  if (mode == TM_MODE_STORE_BF16) {
+    if (nsl == 1) return go(launch_mode<TM_MODE_STORE_BF16, 1>);
+    if (nsl == 2) return go(launch_mode<TM_MODE_STORE_BF16, 2>);
+    if (nsl == 3) return go(launch_mode<TM_MODE_STORE_BF16, 3>);
+  }
+  if (mode == TM_MODE_REDUCE_F32) {
+    if (nsl == 1) return go(launch_mode<TM_MODE_REDUCE_F32, 1>);
+    if (nsl == 2) return go(launch_mode<TM_MODE_REDUCE_F32, 2>);
+    if (nsl == 3) return go(launch_mode<TM_MODE_REDUCE_F32, 3>);
   }
   return cudaErrorInvalidValue;
+}
+
+cudaError_t launch_gemm_exact(const TmTile* d_tiles, int ntiles, const TmTerm* d_terms, const CUtensorMap* d_maps,
+                              double* out, int* d_err, cudaStream_t s, const TmListsDev& lists, const int* d_expo) {
+  if (ntiles <= 0) return cudaSuccess;
+  if (!d_expo || !d_terms) return cudaErrorInvalidValue;
+  return launch_mode<TM_MODE_EXACT_F64, 1>(d_tiles, ntiles, d_terms, d_maps, nullptr, out, d_err, s, d_expo, lists);
 }
 
 int tma_grid(int ntiles) {
@@ -708,30 +669,32 @@ int tma_grid(int ntiles) {
   return ntiles < nsm ? ntiles : nsm;
 }
 
-int tma_pieces(int mode) { return mode == TM_MODE_REDUCE_F32 ? TM_PACK_SLOTS : 1; }
+int tma_pieces(int mode, int nsl) { return mode == TM_MODE_EXACT_F64 ? 1 : tm_slots(nsl); }
 
 namespace {
-__host__ __device__ inline long term_pieces(const TmTerm& m, int bc) {
+// pieces of a term: 16 columns each, or (exact mode) 64 columns of every slice pair
+__host__ __device__ inline long term_pieces(const TmTerm& m, bool exact) {
+  if (!exact) return m.k / TM_PIECE_COLS;
   const int nsl = ((m.neg >> 4) & 15) > 1 ? ((m.neg >> 4) & 15) : 1;
-  return (long)((m.k + bc - 1) / bc) * (nsl * (nsl + 1) / 2);
+  return (long)((m.k + TM_BOX_K - 1) / TM_BOX_K) * (nsl * (nsl + 1) / 2);
 }
 
 // One thread per stage.  It finds its tile (stages in the launch order: sorder[i] has
 // the stages from sfirst[i]) and the term of its first piece (tpiece0: a term's first
-// piece within its tile), then walks the stage's pieces: a term's pieces are its slice
-// pairs (i, j), i + j < nsl, in level order, each its boxes along K.  Segments: store mode
-// one per tile; reduce mode TM_SEG_KSTEPS stages each (the products accumulate in tensor
-// memory over a segment only and the epilogue adds the segments in FP32 with
+// piece within its tile), then walks the stage's pieces.  Exact mode: a term's pieces are its
+// slice pairs (i, j), i + j < nsl, in level order, each its boxes along K.  Segments: store
+// mode one per tile; reduce mode tm_seg_stages(nsl) stages each (the products accumulate in
+// tensor memory over a segment only and the epilogue adds the segments in FP32 with
 // round-to-nearest, so the rounding toward zero of the tensor-core accumulation acts on
 // short sums); exact mode one per level of every term.
-__global__ void fill_lists_kernel(int mode, const TmTile* __restrict__ tiles, int ntiles,
+__global__ void fill_lists_kernel(int mode, int nslices, const TmTile* __restrict__ tiles, int ntiles,
                                   const TmTerm* __restrict__ terms, const int* __restrict__ tpiece0,
                                   const int* __restrict__ sorder, const long* __restrict__ sfirst, long total,
                                   TmStage* __restrict__ stages, TmPiece* __restrict__ pieces) {
   const long g = (long)blockIdx.x * blockDim.x + threadIdx.x;
   if (g >= total) return;
-  const bool pack = mode == TM_MODE_REDUCE_F32, exact = mode == TM_MODE_EXACT_F64;
-  const int bc = pack ? TM_PACK_COLS : TM_BOX_K, P = pack ? TM_PACK_SLOTS : 1;
+  const bool exact = mode == TM_MODE_EXACT_F64;
+  const int bc = exact ? TM_BOX_K : TM_PIECE_COLS, P = exact ? 1 : tm_slots(nslices);
   int lo = 0, hi = ntiles - 1;  // the last tile (in stage order) starting at or before g
   while (lo < hi) {
     const int mid = (lo + hi + 1) >> 1;
@@ -746,17 +709,23 @@ __global__ void fill_lists_kernel(int mode, const TmTile* __restrict__ tiles, in
     const int mid = (t + th + 1) >> 1;
     if (tpiece0[mid] <= p0) t = mid; else th = mid - 1;
   }
-  const long tile_pieces = tpiece0[tl.t1 - 1] + term_pieces(terms[tl.t1 - 1], bc);
+  const long tile_pieces = tpiece0[tl.t1 - 1] + term_pieces(terms[tl.t1 - 1], exact);
   const int np = (int)min((long)P, tile_pieces - p0);
-  const uint32_t a_box = 128u * bc * 2, b_box = (uint32_t)tl.n * bc * 2;
+  const uint32_t piece_bytes = (uint32_t)(128 + tl.n) * bc * 2 * (exact ? 1 : nslices);
   const bool last = sl == nst - 1;
   TmTerm m = terms[t];
   long r = p0 - tpiece0[t];
-  uint32_t negm = 0, nkm = 0, fl = 0, id = 0;
+  uint32_t negm = 0, fl = 0, id = 0;
   for (int slot = 0; slot < np; ++slot, ++r) {
-    if (r >= term_pieces(m, bc)) {
+    if (r >= term_pieces(m, exact)) {
       m = terms[++t];
       r = 0;
+    }
+    if (!exact) {
+      const int k0 = (int)r * bc;
+      pieces[g * P + slot] = TmPiece{m.amap, (m.ax + k0) / 8, m.ay / 16, m.bmap, (m.bx + k0) / 8, m.by / 16, 0, 0};
+      negm |= (uint32_t)(m.neg & 1) << slot;
+      continue;
     }
     const int nsl = max(1, (m.neg >> 4) & 15);
     const int kp = (m.k + bc - 1) / bc;
@@ -768,39 +737,30 @@ __global__ void fill_lists_kernel(int mode, const TmTile* __restrict__ tiles, in
       ++l;
     }
     const int i = q, k0 = kk * bc;
-    const int nk = min(bc / 16, (m.k - k0) / 16);
     pieces[g * P + slot] = TmPiece{m.amap + i, m.ax + k0, m.ay, m.bmap + (l - i), m.bx + k0, m.by, 0, 0};
-    negm |= (uint32_t)(m.neg & 1) << slot;
-    nkm |= (uint32_t)nk << (12 + 2 * slot);
-    if (!pack) {
-      fl = (uint32_t)nk;
-      if (exact) {
-        fl |= (i == 0 && kk == 0) ? 8u : 0u;
-        fl |= (i == l && kk == kp - 1) ? 16u : 0u;
-      } else {
-        fl |= sl == 0 ? 8u : 0u;
-        fl |= last ? 16u : 0u;
-      }
-      id = tm_idesc_bf16(tl.n, (m.neg & 1) != 0);
-    }
+    fl = (uint32_t)min(bc / 16, (m.k - k0) / 16);
+    fl |= (i == 0 && kk == 0) ? 8u : 0u;
+    fl |= (i == l && kk == kp - 1) ? 16u : 0u;
+    id = tm_idesc_bf16(tl.n, (m.neg & 1) != 0);
   }
   for (int p = np; p < P; ++p) pieces[g * P + p] = TmPiece{0, 0, 0, 0, 0, 0, 0, 0};
-  if (pack) {
-    const long seg_pos = sl % TM_SEG_KSTEPS;
-    fl = (uint32_t)np | (negm << 8) | nkm;
-    fl |= seg_pos == 0 ? 8u : 0u;
-    fl |= (last || seg_pos == TM_SEG_KSTEPS - 1) ? 16u : 0u;
+  if (!exact) {
+    const long seg = mode == TM_MODE_REDUCE_F32 ? tm_seg_stages(nslices) : nst;
+    fl = (uint32_t)np | (negm << 8);
+    fl |= sl % seg == 0 ? 8u : 0u;
+    fl |= (last || sl % seg == seg - 1) ? 16u : 0u;
     id = tm_idesc_bf16(tl.n, false);
   }
   fl |= last ? 32u : 0u;
-  stages[g] = TmStage{(uint64_t)id | ((uint64_t)fl << 32), (uint32_t)np * (a_box + b_box), np};
+  stages[g] = TmStage{(uint64_t)id | ((uint64_t)fl << 32), (uint32_t)np * piece_bytes, np};
 }
 }  // namespace
 
-bool tma_plan_lists(int mode, std::vector<TmTile>& tiles, const std::vector<TmTerm>& terms, TmListPlan& out) {
+bool tma_plan_lists(int mode, int nsl, std::vector<TmTile>& tiles, const std::vector<TmTerm>& terms, TmListPlan& out) {
   const int ntiles = (int)tiles.size();
   const int grid = ntiles > 0 ? tma_grid(ntiles) : 0;
-  const int bc = tma_box_cols(mode), P = tma_pieces(mode);
+  const bool exact = mode == TM_MODE_EXACT_F64;
+  const int P = tma_pieces(mode, nsl);
   for (const TmTerm& m : terms)
     if (m.k < 16 || m.k % 16) return false;
   // every term belongs to one tile; its first piece within the tile
@@ -813,7 +773,7 @@ bool tma_plan_lists(int mode, std::vector<TmTile>& tiles, const std::vector<TmTe
     for (int t = tl.t0; t < tl.t1; ++t) {
       if (out.tpiece0[(size_t)t] >= 0 || pc >= (1L << 31)) return false;
       out.tpiece0[(size_t)t] = (int)pc;
-      pc += term_pieces(terms[(size_t)t], bc);
+      pc += term_pieces(terms[(size_t)t], exact);
     }
     tst[(size_t)ti] = (pc + P - 1) / P;
   }
@@ -837,36 +797,48 @@ bool tma_plan_lists(int mode, std::vector<TmTile>& tiles, const std::vector<TmTe
   if (mode == TM_MODE_REDUCE_F32)
     for (int ti = 0; ti < ntiles; ++ti) {
       tiles[(size_t)ti].pad = (int)tst[(size_t)ti];
-      tiles[(size_t)ti].nseg = (int)((tst[(size_t)ti] + TM_SEG_KSTEPS - 1) / TM_SEG_KSTEPS);
+      tiles[(size_t)ti].nseg = (int)((tst[(size_t)ti] + tm_seg_stages(nsl) - 1) / tm_seg_stages(nsl));
     }
   return true;
 }
 
-cudaError_t launch_fill_lists(int mode, const TmTile* d_tiles, int ntiles, const TmTerm* d_terms, const int* d_tpiece0,
-                              const int* d_sorder, const long* d_sfirst, long total, TmStage* d_stages,
-                              TmPiece* d_pieces, cudaStream_t s) {
+cudaError_t launch_fill_lists(int mode, int nsl, const TmTile* d_tiles, int ntiles, const TmTerm* d_terms,
+                              const int* d_tpiece0, const int* d_sorder, const long* d_sfirst, long total,
+                              TmStage* d_stages, TmPiece* d_pieces, cudaStream_t s) {
   if (ntiles <= 0 || total <= 0) return cudaSuccess;
   count_tc_launches(1);
-  fill_lists_kernel<<<(unsigned)((total + 255) / 256), 256, 0, s>>>(mode, d_tiles, ntiles, d_terms, d_tpiece0, d_sorder,
-                                                                    d_sfirst, total, d_stages, d_pieces);
+  fill_lists_kernel<<<(unsigned)((total + 255) / 256), 256, 0, s>>>(mode, nsl, d_tiles, ntiles, d_terms, d_tpiece0,
+                                                                    d_sorder, d_sfirst, total, d_stages, d_pieces);
   return cudaGetLastError();
 }
 
 bool encode_bf16_map(CUtensorMap* out, const void* base, uint64_t rows, uint64_t cols, uint64_t ld,
-                     uint32_t box_rows, uint32_t box_cols) {
+                     uint32_t box_rows) {
   EncodeTiledFn fn = encoder();
   if (!fn || rows == 0 || cols == 0 || (ld * 2) % 16 != 0 || ((uintptr_t)base & 15) != 0 || box_rows == 0 ||
-      box_rows > 256 || (box_cols != 16 && box_cols != 32 && box_cols != (uint32_t)TM_BOX_K))
+      box_rows > 256)
     return false;
   const cuuint64_t dims[2] = {cols, rows};
   const cuuint64_t strides[1] = {ld * 2};
-  const cuuint32_t box[2] = {box_cols, box_rows};
+  const cuuint32_t box[2] = {(cuuint32_t)TM_BOX_K, box_rows};
   const cuuint32_t estr[2] = {1, 1};
   return fn(out, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims, strides, box, estr,
-            CU_TENSOR_MAP_INTERLEAVE_NONE,
-            box_cols == 16 ? CU_TENSOR_MAP_SWIZZLE_32B
-                           : (box_cols == 32 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B),
-            CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+bool encode_slice_map(CUtensorMap* out, const void* base, uint64_t rows, uint64_t cols, int nsl, uint32_t box_rows) {
+  EncodeTiledFn fn = encoder();
+  if (!fn || rows == 0 || rows % 16 != 0 || cols == 0 || cols % 8 != 0 || nsl < 1 || nsl > 3 ||
+      ((uintptr_t)base & 15) != 0 || box_rows == 0 || box_rows % 16 != 0 || box_rows > 256)
+    return false;
+  const cuuint64_t dims[4] = {128, rows / 16, cols / 8, (cuuint64_t)nsl};
+  const cuuint64_t strides[3] = {256, rows * 16, rows * cols * 2};
+  const cuuint32_t box[4] = {128, box_rows / 16, TM_PIECE_COLS / 8, (cuuint32_t)nsl};
+  const cuuint32_t estr[4] = {1, 1, 1, 1};
+  return fn(out, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(base), dims, strides, box, estr,
+            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
 }  // namespace gbdmrg

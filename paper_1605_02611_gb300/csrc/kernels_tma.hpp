@@ -10,13 +10,19 @@
 
 namespace gbdmrg {
 
+// Operand layout of the sigma modes (store and reduce): every BF16 matrix of rows x cols
+// is kept in column groups of 8, [slice][cols / 8][rows][8], rows a multiple of 16.  Eight
+// columns of consecutive rows are contiguous, so a box copy moves runs of 256 bytes
+// (16 rows), lands in shared memory in the K-major layout that the tensor cores read without
+// swizzle, and a warp that owns 32 rows writes 512 contiguous bytes.  Its tensor map has
+// four dimensions, (8 columns x 16 rows, row groups, column groups, slices).
+//
 // One term of an output tile: C[128 x n] (-)= A[128 x k] B[n x k]^T (neg bit 0), where A is the
 // box of rows [ay, ay + 128) and columns [ax, ax + k) of tensor map amap and B the
-// rows [by, by + n) and columns [bx, bx + k) of tensor map bmap (both BF16,
-// row-major, 128-byte swizzled boxes of 64 columns; rows or columns outside a
-// map's extent read as zero).  k is a multiple of 16; columns of a 64-wide box
-// past k are loaded but never multiplied.  The B map's box height must be the
-// tile's n.
+// rows [by, by + n) and columns [bx, bx + k) of tensor map bmap; rows outside a map's
+// extent read as zero.  ay, by and k are multiples of 16, ax and bx of 8.  A piece, 16
+// columns of a term, is one copy per operand that brings all its slices.  The B map's box
+// height must be the tile's n.
 //
 // Exact mode (TM_MODE_EXACT_F64): the operands are integer slices (|x| <= 128, exact in
 // BF16) of blocks scaled by powers of two, so every product sum is an exact integer in
@@ -33,20 +39,15 @@ struct TmTerm {
 
 // Output tile over the terms [t0, t1).  n: MMA width (multiple of 16, <= the
 // kernel's maximum).
-//   reduce mode (packed): the tensor maps of the tile's terms have boxes of TM_PACK_COLS
-//     columns, and a K step (stage) holds up to TM_PACK_SLOTS consecutive pieces of the
-//     tile (a term has ceil(k / TM_PACK_COLS) pieces per slice pair); pad = the tile's
-//     stages, ceil(pieces / TM_PACK_SLOTS).
-//   store mode (X intermediates, BF16): the output matrix is split by columns into
-//     column blocks, each its own row-major submatrix of xrows rows: block e of
-//     cbtab[cb0..cb1) = (first column c0, width w) starts at element
-//     xbase + xrows * c0 and holds column c at (c - c0) of its rows.  Row r of the
-//     tile is row rowmap[rowmap_off + r] of the submatrices (< 0: skipped); its
-//     columns are out_off .. out_off + n (every 8-column chunk inside one block).
+//   store mode (X intermediates, BF16 slices): the output matrix has xrows rows and ldo
+//     columns in the layout above, slice 0 from element xbase, slices xrows * ldo apart.
+//     Row r of the tile is its row rowmap[rowmap_off + r] (< 0: skipped), its columns are
+//     out_off .. out_off + n.
 //   reduce mode (sigma^T, FP32): rows r < m_valid are added (vector reductions) to
 //     out + out_off + r * ldo, columns [0, n).
-//   nseg (reduce mode): segments of the tile, ceil(stages / TM_SEG_KSTEPS); each segment
-//     accumulates in tensor memory on its own and the epilogue adds the segments in FP32.
+//   pad, nseg (reduce mode): the tile's stages and segments, ceil(stages /
+//     tm_seg_stages(nsl)); each segment accumulates in tensor memory on its own and the
+//     epilogue adds the segments in FP32.
 struct TmTile {
   int t0, t1;
   int n, m_valid;
@@ -54,8 +55,7 @@ struct TmTile {
   long out_off;
   long rowmap_off;
   long xbase, xrows;
-  int cb0, cb1;
-  int nvalid, pad;  // exact mode: valid columns of the output block; reduce mode: pad = pieces
+  int nvalid, pad;  // exact mode: valid columns of the output block; reduce mode: pad = stages
 };
 
 //   exact mode (FP64): rows r < m_valid, columns c < nvalid of
@@ -64,29 +64,31 @@ struct TmTile {
 constexpr int TM_MODE_STORE_BF16 = 1, TM_MODE_REDUCE_F32 = 2, TM_MODE_EXACT_F64 = 3;
 // bits of the slices of the exact mode
 constexpr int TM_EXACT_BITS = 7;
-// K steps (stages of up to TM_PACK_SLOTS 16-column pieces) accumulated in tensor memory
-// before the reduce-mode epilogue takes the partial sum over
-constexpr int TM_SEG_KSTEPS = 16;
-constexpr int TM_PACK_SLOTS = 4;  // pieces per stage of the reduce mode
-constexpr int TM_PACK_COLS = 16;  // their width (32-byte swizzled boxes), one K=16 instruction each
+constexpr int TM_PIECE_COLS = 16;  // columns of a piece in the sigma modes: one K=16 instruction per product
+// pieces per stage of the sigma modes, so that a stage is 24 to 48 KB whatever the slices
+__host__ __device__ constexpr int tm_slots(int nsl) { return nsl == 1 ? 4 : nsl == 2 ? 2 : 1; }
+// stages accumulated in tensor memory before the reduce-mode epilogue takes the partial
+// sum over (60 to 64 instructions: the tensor cores round their running sum toward zero)
+__host__ __device__ constexpr int tm_seg_stages(int nsl) { return nsl == 1 ? 16 : 10; }
 
-// Copy lists.  The tiles' terms are expanded on the host into stages, each holding up
-// to tma_pieces(mode) pieces (a piece: one A box and one B box, both of tma_box_cols(mode)
-// columns; store and exact modes one piece of 64 columns, reduce mode up to
-// TM_PACK_SLOTS consecutive pieces of TM_PACK_COLS columns).  A term expands into its slice pairs
-// (i, j), i + j < nsl, in the order of the level l = i + j (A map amap + i, B map
-// bmap + j), each into its boxes along K.  CTA c of a launch of `grid` CTAs takes the
-// tiles c, c + grid, ... and issues the stages [cta_stage[c], cta_stage[c + 1]), stage s
-// with the pieces pieces[s * tma_pieces(mode) + p], p < np.
+// Copy lists.  The tiles' terms are expanded before the launch into stages, each holding
+// up to tma_pieces(mode, nsl) pieces.  In the sigma modes a piece is 16 columns of one term
+// with all slices of both operands: the slice products i + j < nsl come from one pair of
+// copies.  In the exact mode a term expands into its slice pairs (i, j), i + j < nsl, in the
+// order of the level l = i + j (A map amap + i, B map bmap + j), each into boxes of 64
+// columns along K, one to a stage.  CTA c of a launch of `grid` CTAs takes the tiles c,
+// c + grid, ... and issues the stages [cta_stage[c], cta_stage[c + 1]), stage s with the
+// pieces pieces[s * tma_pieces(mode, nsl) + p], p < np.
+// A piece's coordinates are columns and rows in the exact mode, column groups (8) and row
+// groups (16) in the sigma modes.
 struct TmPiece {  // 32 bytes, so that any run of pieces is a bulk copy of 16-byte multiples
   int amap, ax, ay, bmap, bx, by, pad0, pad1;
 };
 // word: the stage word the MMA issuer reads, the instruction descriptor (negation of A in
-// the store and exact modes) in the low half, in the high half the K=16 instructions
-// (store and exact modes; the pieces in the reduce mode) in bits 0-2, flags first of a
-// segment (bit 3), end of a segment (4), last stage of the tile (5), and in the reduce
-// mode the negation of slot p in bit 8 + p and its K=16 instructions in bits 12 + 2p and
-// 13 + 2p.  bytes: the stage's expected copy bytes.
+// the exact mode) in the low half, in the high half the K=16 instructions (exact mode) or
+// the pieces (sigma modes) in bits 0-2, flags first of a segment (bit 3), end of a segment
+// (4), last stage of the tile (5), and in the sigma modes the negation of slot p in bit
+// 8 + p.  bytes: the stage's expected copy bytes.
 struct TmStage {
   uint64_t word;
   uint32_t bytes;
@@ -123,31 +125,31 @@ __host__ __device__ inline uint32_t tm_idesc_bf16(int n, bool negA) {
   return d;
 }
 
-// Host: the stage counts of a launch of `mode` over these tiles (for the grid the launch
-// will use, tma_grid(tiles.size())); reduce mode: sets every tile's pad (its stages) and
-// nseg.  Returns false if a term is malformed (k not a positive multiple of 16), belongs
-// to two tiles, or the lists would be too long.
-bool tma_plan_lists(int mode, std::vector<TmTile>& tiles, const std::vector<TmTerm>& terms, TmListPlan& out);
-// Device: fills the copy lists (stages: total entries, pieces: total * tma_pieces(mode)),
-// one thread per stage, from the tiles and terms the plan was made from and the plan's
+// Host: the stage counts of a launch of `mode` (operands of nsl slices) over these tiles
+// (for the grid the launch will use, tma_grid(tiles.size())); reduce mode: sets every
+// tile's pad (its stages) and nseg.  Returns false if a term is malformed (k not a positive
+// multiple of 16), belongs to two tiles, or the lists would be too long.
+bool tma_plan_lists(int mode, int nsl, std::vector<TmTile>& tiles, const std::vector<TmTerm>& terms, TmListPlan& out);
+// Device: fills the copy lists (stages: total entries, pieces: total * tma_pieces(mode,
+// nsl)), one thread per stage, from the tiles and terms the plan was made from and the plan's
 // tpiece0, sorder and sfirst (all on the device).
-cudaError_t launch_fill_lists(int mode, const TmTile* d_tiles, int ntiles, const TmTerm* d_terms, const int* d_tpiece0,
-                              const int* d_sorder, const long* d_sfirst, long total, TmStage* d_stages,
-                              TmPiece* d_pieces, cudaStream_t s);
+cudaError_t launch_fill_lists(int mode, int nsl, const TmTile* d_tiles, int ntiles, const TmTerm* d_terms,
+                              const int* d_tpiece0, const int* d_sorder, const long* d_sfirst, long total,
+                              TmStage* d_stages, TmPiece* d_pieces, cudaStream_t s);
 // CTAs of a launch over ntiles tiles (min(ntiles, SMs of the current device))
 int tma_grid(int ntiles);
-int tma_pieces(int mode);
+int tma_pieces(int mode, int nsl);
 
-// maps: device array of encoded tensor maps (64-byte aligned).  Store mode:
-// out_slices (1-3) BF16 slices x = s0 + s1 + ... of every FP32 result, written
-// slice_stride elements apart.  err: set to 1 if a bounded wait ran out (the CTA
-// then stops, lets its copies land and frees its tensor memory).  lists: the copy lists
-// of these tiles (tma_plan_lists, launch_fill_lists), on the device.  d_terms: read by the exact mode's
-// epilogue only.
-cudaError_t launch_gemm_tma(int mode, const TmTile* d_tiles, int ntiles, const TmTerm* d_terms,
-                            const CUtensorMap* d_maps, const long* d_rowmap, const int2* d_cbtab, void* out,
-                            int out_slices, long slice_stride, int* d_err, cudaStream_t s, const TmListsDev& lists,
-                            const int* d_expo = nullptr);
+// maps: device array of encoded tensor maps (64-byte aligned).  nsl: BF16 slices of the
+// operands (1-3; store mode: also of the results, x = s0 + s1 + ... of every FP32 value).
+// err: set to 1 if a bounded wait ran out (the CTA then stops, lets its copies land and frees
+// its tensor memory).  lists: the copy lists of these tiles (tma_plan_lists,
+// launch_fill_lists), on the device.
+cudaError_t launch_gemm_slices(int mode, int nsl, const TmTile* d_tiles, int ntiles, const CUtensorMap* d_maps,
+                               const long* d_rowmap, void* out, int* d_err, cudaStream_t s, const TmListsDev& lists);
+// the exact mode (d_terms and d_expo: read by its epilogue)
+cudaError_t launch_gemm_exact(const TmTile* d_tiles, int ntiles, const TmTerm* d_terms, const CUtensorMap* d_maps,
+                              double* out, int* d_err, cudaStream_t s, const TmListsDev& lists, const int* d_expo);
 
 // Exact splitting of FP64 blocks for the exact mode: per job, e = the smallest
 // exponent with |scale * x| < 2^e over the block, then nsl (1 to 6) integer slices d_s
@@ -166,15 +168,14 @@ struct SplitJob {
 cudaError_t launch_split_exact(const SplitJob* d_jobs, int njobs, int nsl, int* d_expo, cudaStream_t s);
 // maximum MMA width of a mode (256 for the BF16 store mode, 128 for the reduce mode)
 int tma_max_n(int mode);
-// box width in columns of the tensor maps a mode reads (TM_PACK_COLS for the reduce mode,
-// else 64)
-int tma_box_cols(int mode);
 
-// Host: encode a 2D BF16 tensor map over a row-major matrix (rows x cols, leading
-// dimension ld elements, ld * 2 a multiple of 16 bytes, base 16-byte aligned), box
-// of box_cols columns x box_rows rows: 64, 32 or 16 columns with 128-, 64- or 32-byte
-// swizzle.  Returns false on failure.
-bool encode_bf16_map(CUtensorMap* out, const void* base, uint64_t rows, uint64_t cols, uint64_t ld,
-                     uint32_t box_rows, uint32_t box_cols = 64);
+// Host: encode a 2D BF16 tensor map of the exact mode over a row-major matrix (rows x cols,
+// leading dimension ld elements, ld * 2 a multiple of 16 bytes, base 16-byte aligned), boxes
+// of 64 columns (128-byte swizzle) x box_rows rows.  Returns false on failure.
+bool encode_bf16_map(CUtensorMap* out, const void* base, uint64_t rows, uint64_t cols, uint64_t ld, uint32_t box_rows);
+// Host: encode the 4D map of a matrix in the layout of the sigma modes (rows a multiple of
+// 16, cols of 8, nsl slices one after another), boxes of box_rows rows (a multiple of 16, at
+// most 256), TM_PIECE_COLS columns and all slices.  Returns false on failure.
+bool encode_slice_map(CUtensorMap* out, const void* base, uint64_t rows, uint64_t cols, int nsl, uint32_t box_rows);
 
 }  // namespace gbdmrg
