@@ -971,9 +971,9 @@ void build_tma_plan(Context& c, Tilde& lt, Tilde& rt, int k, SigmaPlan& plan, in
       const auto cp = cpos[B.cs * 4 + P.b2[b]];
       if (rp[0] < 0 || rp[0] != cp[0]) throw Error(ST_ECUDA, "internal: psi block outside its group");
       const int g = rp[0];
-      // Psi_g: gR rows x gC columns in column groups of 8, slices one after another
-      pj.push_back({plan.in.p + B.off, tp->psi_b.p + goff[g] * nsl + (long)cp[1] * gR[g] + (long)rp[1] * 8,
-                    (long)gR[g] * gC[g], (long)gR[g] * 8, B.rows, B.cols, B.cols, pad16(B.cols), 1.0});
+      // Psi_g: gR rows x gC columns in column groups of 8
+      pj.push_back({plan.in.p + B.off, tp->psi_b.p + (goff[g] + (long)cp[1] * gR[g]) * nsl + (long)rp[1] * 8,
+                    (long)gR[g] * 8, (long)gR[g] * 8 * nsl, B.rows, B.cols, B.cols, pad16(B.cols), 1.0});
       tp->psi_maxel = std::max<long>(tp->psi_maxel, (long)B.rows * pad16(B.cols));
       sj.push_back({tp->sig_t.p + sgoff[g] + (long)cp[1] * gR[g] + rp[1], plan.out.p + B.off, B.rows, B.cols, gR[g]});
       tp->sig_maxel = std::max<long>(tp->sig_maxel, (long)B.rows * B.cols);
@@ -1038,7 +1038,7 @@ void build_tma_plan(Context& c, Tilde& lt, Tilde& rt, int k, SigmaPlan& plan, in
   for (int ci = 0; ci < nch; ++ci)
     for (int b = chunks[ci].first; b < chunks[ci].second; ++b) chunk_of[b] = ci;
   // X^T layout per chunk: regions per g' (Sum_beta C_g(beta) rows x R_g' columns in column
-  // groups of 8, the region's slices one after another: element offsets below count one slice);
+  // groups of 8; element offsets below count one slice);
   // xrow[beta][g'] = first row of beta's block in its region
   std::vector<std::vector<long>> xreg(nch, std::vector<long>(ng, 0)), xregrows(nch, std::vector<long>(ng, 0));
   std::vector<long> xrow((size_t)nmid * ng, -1);
@@ -1111,8 +1111,8 @@ void build_tma_plan(Context& c, Tilde& lt, Tilde& rt, int k, SigmaPlan& plan, in
         const Block& B = Renv.cls[r.cls].blocks[x.bl[n2p]];
         // the K block (n2', qr') of g': columns coff .. coff + pad16(d(qr')) of A1
         const int coff = cpos[B.cs * 4 + n2p][1];
-        aconv.push_back({r.p + B.off, tp->a1.p + a1off[gp] * nsl + a1rows[gp] * coff + row * 8, a1rows[gp] * gC[gp],
-                         a1rows[gp] * 8, B.rows, B.cols, B.cols, pad16(B.cols), r.coef});
+        aconv.push_back({r.p + B.off, tp->a1.p + (a1off[gp] + a1rows[gp] * coff) * nsl + row * 8, a1rows[gp] * 8,
+                         a1rows[gp] * 8 * nsl, B.rows, B.cols, B.cols, pad16(B.cols), r.coef});
         tp->a1_maxel = std::max<long>(tp->a1_maxel, (long)B.rows * pad16(B.cols));
       }
       row += x.rows;
@@ -1192,8 +1192,8 @@ void build_tma_plan(Context& c, Tilde& lt, Tilde& rt, int k, SigmaPlan& plan, in
   lconv.reserve(lpend.size());
   for (const PendL& pl : lpend) {
     const int w = wcls_w[pl.cls];
-    lconv.push_back({pl.src, tp->lmir.p + lbase[pl.cls] * nsl + pl.crow * 8, lrows_c[pl.cls] * w,
-                     lrows_c[pl.cls] * 8, pl.rows, pl.cols, pl.cols, w, pl.scale});
+    lconv.push_back({pl.src, tp->lmir.p + lbase[pl.cls] * nsl + pl.crow * 8, lrows_c[pl.cls] * 8,
+                     lrows_c[pl.cls] * 8 * nsl, pl.rows, pl.cols, pl.cols, w, pl.scale});
     tp->l_maxel = std::max<long>(tp->l_maxel, (long)pl.rows * w);
   }
   check_group_jobs(lconv, nsl, tp->lmir);
@@ -1208,7 +1208,7 @@ void build_tma_plan(Context& c, Tilde& lt, Tilde& rt, int k, SigmaPlan& plan, in
     int box;
   };
   std::vector<MapInfo> minfo;
-  // a matrix of rows x cols in the column-group layout, its nsl slices from element off
+  // a matrix of rows x cols in the column-group layout from element off
   auto add_map = [&](const DArr<__nv_bfloat16>& buf, long off, long rows, long cols, int box_rows) {
     if (off < 0 || rows < 1 || cols < 1 || rows % 16 != 0 || cols % 16 != 0 || off % 8 != 0 ||
         (size_t)(off + nsl * rows * cols) > buf.n)
@@ -1309,8 +1309,8 @@ void build_tma_plan(Context& c, Tilde& lt, Tilde& rt, int k, SigmaPlan& plan, in
             if (written.count(((long)beta * 4 + cb[0]) * nR + cb[1])) continue;
             // the block's rows in every column group
             const long r0 = xrow[(size_t)beta * ng + gp] + cb[2], rows = xregrows[ci][gp];
-            zj.push_back({tp->xt.p + xreg[ci][gp] * nsl + r0 * 8, (long)pad16(Rb.dim[cb[1]]) * 8, rows * gR[gp], nsl,
-                          gR[gp] / 8, rows * 8});
+            zj.push_back({tp->xt.p + xreg[ci][gp] * nsl + r0 * 8, (long)pad16(Rb.dim[cb[1]]) * 8, rows * 8, nsl,
+                          gR[gp] / 8, rows * 8 * nsl});
           }
         }
       }

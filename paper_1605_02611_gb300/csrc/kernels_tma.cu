@@ -66,7 +66,10 @@ struct TmCfg {
   static constexpr bool EXACT = MODE == TM_MODE_EXACT_F64;
   // exact mode: 64 columns, so that the two-float sums (128 registers) fit
   static constexpr int NMAX = STORE ? 256 : (EXACT ? 64 : 128);
-  static constexpr int NACC = 512 / NMAX;
+  // tensor-memory columns of an accumulator: in the reduce mode with slices two blocks of n
+  // columns, one for the products with slice 0 of B and one for the others
+  static constexpr int PARTS = !STORE && !EXACT && NSL > 1 ? 2 : 1;
+  static constexpr int NACC = 512 / (NMAX * PARTS);
   static constexpr int SLOTS = EXACT ? 1 : tm_slots(NSL);
   // bytes of one piece of A and of the largest piece of B (all slices)
   static constexpr int A_BYTES = EXACT ? TM_A_BYTES : 128 * TM_PIECE_COLS * 2 * NSL;
@@ -91,13 +94,12 @@ __device__ __forceinline__ uint64_t sdesc(uint32_t saddr) {
 }
 
 // the same for the column-group layout: K-major without swizzle, core matrices of 8 rows x
-// 16 bytes contiguous along the rows (128 B apart), the second 8 columns `rows` rows further
-__device__ __forceinline__ uint64_t sdesc_groups(uint32_t saddr, int rows) {
-  uint64_t d = 0;
-  d |= (uint64_t)((saddr >> 4) & 0x3FFFu);
-  d |= (uint64_t)(uint32_t)rows << 16;  // (rows * 16) >> 4
-  d |= (uint64_t)(128 >> 4) << 32;
-  d |= (uint64_t)1 << 46;
+// 16 bytes contiguous along the rows (128 B apart), the second 8 columns `rows` rows further.
+// lo: address and rows in 16-byte units, (saddr >> 4) | rows << 16.
+__device__ __forceinline__ uint64_t sdesc_groups(uint32_t lo) {
+  constexpr uint32_t hi = (128u >> 4) | (1u << (46 - 32));
+  uint64_t d;
+  asm("mov.b64 %0, {%1, %2};\n" : "=l"(d) : "r"(lo), "r"(hi));
   return d;
 }
 
@@ -140,7 +142,7 @@ __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map
 // box of a column-group map: all of dimension 0, row group y, column group x, every slice
 __device__ __forceinline__ void tma_load_groups(uint32_t dst, const CUtensorMap* map, int x, int y, uint64_t* bar) {
   asm volatile(
-      "cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %2}], "
+      "cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %2, %4}], "
       "[%5];\n" ::"r"(dst),
       "l"(map), "r"(0), "r"(y), "r"(x), "r"(smem_u32(bar))
       : "memory");
@@ -185,6 +187,7 @@ __global__ void __launch_bounds__(TM_THREADS, 1)
   constexpr int NMAX = Cfg::NMAX;
   constexpr bool STORE = Cfg::STORE;
   constexpr bool EXACT = Cfg::EXACT;
+  constexpr int PARTS = Cfg::PARTS;
   extern __shared__ uint8_t dsm[];
   __shared__ __align__(8) uint64_t full_b[TM_MAX_STAGES], empty_b[TM_MAX_STAGES], tfull_b[TM_MAX_ACC],
       tempty_b[TM_MAX_ACC];
@@ -315,8 +318,9 @@ __global__ void __launch_bounds__(TM_THREADS, 1)
       // shared-memory descriptors of stage 0's operands; later stages, slots, slices and K
       // steps add their byte offsets / 16 to the 14-bit address field (no carry: shared
       // addresses stay below 256 KB)
-      const uint64_t ad0 = EXACT ? sdesc(base) : sdesc_groups(base, 128);
-      const uint64_t bd0 = EXACT ? sdesc(base + TM_A_BYTES) : sdesc_groups(base + Cfg::SLOTS * Cfg::A_BYTES, 0);
+      const uint64_t ad0 = sdesc(base), bd0 = sdesc(base + TM_A_BYTES);
+      const uint32_t al0 = (base >> 4) | (uint32_t)(NSL * 128) << 16;
+      const uint32_t bl0 = (base + Cfg::SLOTS * Cfg::A_BYTES) >> 4;
       for (int ti = blockIdx.x; ti < ntiles && ok; ti += gridDim.x) {
         bool tile_done = false;
         while (!tile_done && ok) {
@@ -326,7 +330,7 @@ __global__ void __launch_bounds__(TM_THREADS, 1)
             break;
           }
           asm volatile("tcgen05.fence::after_thread_sync;\n" ::);
-          const uint32_t dacc = tmem + (uint32_t)(acc * NMAX);
+          const uint32_t dacc = tmem + (uint32_t)(acc * NMAX * PARTS);
           for (;;) {
             if (!mbar_wait(&full_b[st], par, abort_flag)) {
               ok = false;
@@ -336,29 +340,47 @@ __global__ void __launch_bounds__(TM_THREADS, 1)
             const uint64_t mw = meta[st];
             const uint32_t id = (uint32_t)mw, fl = (uint32_t)(mw >> 32);
             const int nk = (int)(fl & 7u);
-            const uint64_t off = (uint64_t)((st * STAGE_BYTES) >> 4);
+            const uint32_t off = (uint32_t)((st * STAGE_BYTES) >> 4);
             uint32_t accum = (fl & 8u) ? 0u : 1u;
-            auto mma = [&](uint64_t ad, uint64_t bd, uint32_t idk) {
+            auto mma = [&](uint32_t d, uint64_t ad, uint64_t bd, uint32_t idk) {
               asm volatile(
                   "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-                  " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(dacc),
+                  " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d),
                   "l"(ad), "l"(bd), "r"(idk), "r"(accum));
-              accum = 1u;
             };
             if constexpr (EXACT) {
-              for (int kk = 0; kk < nk; ++kk)
-                mma(ad0 + off + (uint64_t)(kk * 2), bd0 + off + (uint64_t)(kk * 2), id);
+              for (int kk = 0; kk < nk; ++kk) {
+                mma(dacc, ad0 + off + (uint64_t)(kk * 2), bd0 + off + (uint64_t)(kk * 2), id);
+                accum = 1u;
+              }
             } else {
-              const uint32_t n = ((id >> 17) & 63u) << 3;  // rows of B: 8 columns are n * 16 bytes, a slice n * 32
-              const uint64_t bdn = bd0 + ((uint64_t)n << 16);
+              // rows of B: 8 columns of one slice are n * 16 bytes, of all NSL * n * 16
+              const uint32_t nf = id & (63u << 17), n = nf >> 14;
+              const uint32_t bl = bl0 + off + ((n * NSL) << 16), al = al0 + off;
               for (int sl = 0; sl < nk; ++sl) {
                 const uint32_t idk = id | (((fl >> (8 + sl)) & 1u) << 13);
-                const uint64_t ad = ad0 + off + (uint64_t)((sl * Cfg::A_BYTES) >> 4);
-                const uint64_t bd = bdn + off + (uint64_t)((sl * Cfg::B_BYTES) >> 4);
+                const uint32_t a = al + (uint32_t)((sl * Cfg::A_BYTES) >> 4), b = bl + (uint32_t)((sl * Cfg::B_BYTES) >> 4);
+                if constexpr (PARTS == 2) {
+                  // the two blocks of the accumulator start from the first product, of both
+                  // slices of B at once (2 n columns)
+                  mma(dacc, sdesc_groups(a), sdesc_groups(b), idk + nf);
+                  accum = 1u;
+                  if constexpr (NSL == 2) {
+                    mma(dacc, sdesc_groups(a + 128u), sdesc_groups(b), idk);
+                  } else {
+                    mma(dacc, sdesc_groups(a + 128u), sdesc_groups(b), idk + nf);
+                    mma(dacc + n, sdesc_groups(a), sdesc_groups(b + 2 * n), idk);
+                    mma(dacc, sdesc_groups(a + 256u), sdesc_groups(b), idk);
+                  }
+                } else {
 #pragma unroll
-                for (int l = 0; l < NSL; ++l)
+                  for (int l = 0; l < NSL; ++l)
 #pragma unroll
-                  for (int i = 0; i <= l; ++i) mma(ad + (uint64_t)(i * 256), bd + (uint64_t)((l - i) * 2 * n), idk);
+                    for (int i = 0; i <= l; ++i) {
+                      mma(dacc, sdesc_groups(a + (uint32_t)(i * 128)), sdesc_groups(b + (uint32_t)(l - i) * n), idk);
+                      accum = 1u;
+                    }
+                }
               }
             }
             asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(
@@ -402,8 +424,7 @@ __global__ void __launch_bounds__(TM_THREADS, 1)
         // per 8 columns one 16-byte store per slice, x = s0 + s1 + s2 from one read of each
         // value; the lanes' rows are mostly consecutive, so a warp writes contiguous runs.
         // The tensor-memory loads (32 columns, one wait) are warp-wide.
-        __nv_bfloat16* g = reinterpret_cast<__nv_bfloat16*>(out) + tl.xbase + tl.out_off * tl.xrows + row_own * 8;
-        const long slice = tl.xrows * tl.ldo;
+        __nv_bfloat16* g = reinterpret_cast<__nv_bfloat16*>(out) + tl.xbase + tl.out_off * NSL * tl.xrows + row_own * 8;
 #pragma unroll 1
         for (int c0 = 0; c0 < tl.n; c0 += 32) {
           uint32_t v[32];
@@ -423,10 +444,10 @@ __global__ void __launch_bounds__(TM_THREADS, 1)
                 b -= __high2float(h);
               }
             }
-            __nv_bfloat16* q = g + (long)(c0 + u8) * tl.xrows;
+            __nv_bfloat16* q = g + (long)(c0 + u8) * NSL * tl.xrows;
 #pragma unroll
             for (int sl = 0; sl < NSL; ++sl)
-              *reinterpret_cast<uint4*>(q + sl * slice) = make_uint4(w[sl][0], w[sl][1], w[sl][2], w[sl][3]);
+              *reinterpret_cast<uint4*>(q + sl * tl.xrows * 8) = make_uint4(w[sl][0], w[sl][1], w[sl][2], w[sl][3]);
           }
         }
         asm volatile("tcgen05.fence::before_thread_sync;\n" ::);
@@ -491,14 +512,17 @@ __global__ void __launch_bounds__(TM_THREADS, 1)
           for (int cc = 0; cc < NMAX / 32; ++cc) {
             const int c0 = cc * 32;
             if (c0 < tl.n) {
-              uint32_t v[32];
-              tmem_ld32(tmem + ((uint32_t)(sub * 32) << 16) + (uint32_t)(acc * NMAX + c0), v);
-              if (q == 0) {
 #pragma unroll
-                for (int u = 0; u < 32; ++u) run[cc][u] = __uint_as_float(v[u]);
-              } else {
+              for (int part = 0; part < PARTS; ++part) {
+                uint32_t v[32];
+                tmem_ld32(tmem + ((uint32_t)(sub * 32) << 16) + (uint32_t)(acc * NMAX * PARTS + part * tl.n + c0), v);
+                if (q == 0 && part == 0) {
 #pragma unroll
-                for (int u = 0; u < 32; ++u) run[cc][u] += __uint_as_float(v[u]);
+                  for (int u = 0; u < 32; ++u) run[cc][u] = __uint_as_float(v[u]);
+                } else {
+#pragma unroll
+                  for (int u = 0; u < 32; ++u) run[cc][u] += __uint_as_float(v[u]);
+                }
               }
             }
           }
@@ -832,9 +856,9 @@ bool encode_slice_map(CUtensorMap* out, const void* base, uint64_t rows, uint64_
   if (!fn || rows == 0 || rows % 16 != 0 || cols == 0 || cols % 8 != 0 || nsl < 1 || nsl > 3 ||
       ((uintptr_t)base & 15) != 0 || box_rows == 0 || box_rows % 16 != 0 || box_rows > 256)
     return false;
-  const cuuint64_t dims[4] = {128, rows / 16, cols / 8, (cuuint64_t)nsl};
-  const cuuint64_t strides[3] = {256, rows * 16, rows * cols * 2};
-  const cuuint32_t box[4] = {128, box_rows / 16, TM_PIECE_COLS / 8, (cuuint32_t)nsl};
+  const cuuint64_t dims[4] = {128, rows / 16, (cuuint64_t)nsl, cols / 8};
+  const cuuint64_t strides[3] = {256, rows * 16, rows * 16 * nsl};
+  const cuuint32_t box[4] = {128, box_rows / 16, (cuuint32_t)nsl, TM_PIECE_COLS / 8};
   const cuuint32_t estr[4] = {1, 1, 1, 1};
   return fn(out, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(base), dims, strides, box, estr,
             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,

@@ -11,11 +11,13 @@
 namespace gbdmrg {
 
 // Operand layout of the sigma modes (store and reduce): every BF16 matrix of rows x cols
-// is kept in column groups of 8, [slice][cols / 8][rows][8], rows a multiple of 16.  Eight
+// is kept in column groups of 8, [cols / 8][slice][rows][8], rows a multiple of 16.  Eight
 // columns of consecutive rows are contiguous, so a box copy moves runs of 256 bytes
 // (16 rows), lands in shared memory in the K-major layout that the tensor cores read without
-// swizzle, and a warp that owns 32 rows writes 512 contiguous bytes.  Its tensor map has
-// four dimensions, (8 columns x 16 rows, row groups, column groups, slices).
+// swizzle, and a warp that owns 32 rows writes 512 contiguous bytes.  The slices of a box
+// follow one another like further rows, so that one instruction can multiply by several
+// slices of B.  The tensor map has four dimensions, (8 columns x 16 rows, row groups, slices,
+// column groups).
 //
 // One term of an output tile: C[128 x n] (-)= A[128 x k] B[n x k]^T (neg bit 0), where A is the
 // box of rows [ay, ay + 128) and columns [ax, ax + k) of tensor map amap and B the
@@ -40,7 +42,7 @@ struct TmTerm {
 // Output tile over the terms [t0, t1).  n: MMA width (multiple of 16, <= the
 // kernel's maximum).
 //   store mode (X intermediates, BF16 slices): the output matrix has xrows rows and ldo
-//     columns in the layout above, slice 0 from element xbase, slices xrows * ldo apart.
+//     columns in the layout above, from element xbase.
 //     Row r of the tile is its row rowmap[rowmap_off + r] (< 0: skipped), its columns are
 //     out_off .. out_off + n.
 //   reduce mode (sigma^T, FP32): rows r < m_valid are added (vector reductions) to
@@ -174,7 +176,7 @@ int tma_max_n(int mode);
 // of 64 columns (128-byte swizzle) x box_rows rows.  Returns false on failure.
 bool encode_bf16_map(CUtensorMap* out, const void* base, uint64_t rows, uint64_t cols, uint64_t ld, uint32_t box_rows);
 // Host: encode the 4D map of a matrix in the layout of the sigma modes (rows a multiple of
-// 16, cols of 8, nsl slices one after another), boxes of box_rows rows (a multiple of 16, at
+// 16, cols of 8, nsl slices), boxes of box_rows rows (a multiple of 16, at
 // most 256), TM_PIECE_COLS columns and all slices.  Returns false on failure.
 bool encode_slice_map(CUtensorMap* out, const void* base, uint64_t rows, uint64_t cols, int nsl, uint32_t box_rows);
 
