@@ -10,8 +10,8 @@
 // before the launch into per-CTA copy lists (stage word, expected bytes, box coordinates:
 // fill_lists_kernel), so the producer does no term arithmetic.
 //
-// Persistent and warp-specialised, one CTA per SM (up to 221 KB of shared memory,
-// all 512 tensor-memory columns):
+// Persistent and warp-specialised, two CTAs per SM in the sigma modes (up to 113 KB of shared
+// memory and 256 tensor-memory columns each), one in the exact mode:
 //   warp 0     fetches its CTA's copy lists 32 stages at a time into shared memory
 //              (1D bulk copies, double-buffered); per stage lane 0 waits for the ring
 //              slot and posts the stage word and the expected bytes, then lane p issues
@@ -23,9 +23,9 @@
 //              intermediates, FP32 vector reductions (sigma^T, several tiles may add into
 //              one block) of per-segment partial sums, or (exact mode) two-float sums of
 //              exact integer segments stored in FP64
-// Two (store mode, N <= 256), four (reduce mode, N <= 128) or eight (exact mode, N <=
-// 64) accumulators let the epilogue of one tile overlap the MMAs of the next.  Every
-// wait is bounded: on timeout the CTA raises a shared abort flag, records an error,
+// One (sigma modes; two for one slice in the reduce mode) or eight (exact mode, N <= 64)
+// accumulators.  In the sigma modes the two CTAs of an SM overlap each other's epilogues,
+// products and copies.  Every wait is bounded: on timeout the CTA raises a shared abort flag, records an error,
 // waits (bounded) for the copies it issued, frees its tensor memory and returns.
 //
 // gemm_slices_kernel (sigma): what bounds it is the operand traffic into shared memory, not
@@ -35,8 +35,12 @@
 // bytes for six products instead of 6 + 6) in two copies instead of twelve, and the
 // column-group layout lets each copy move 256-byte runs instead of 32-byte rows.
 // Measured against one pair of swizzled boxes per slice product (16-column boxes in the
-// reduce mode): three slices at K=24, M=512 3.18 -> 1.61 ms per sigma, K=40, M=1200 23.1 ->
-// 11.3 ms; one pass at K=32, M=1024 2.71 -> 1.79 ms.
+// reduce mode): three slices at K=24, M=512 3.18 -> 1.54 ms per sigma, K=40, M=1200 23.1 ->
+// 11.2 ms; one pass at K=32, M=1024 2.71 -> 1.79 ms.  What then bounded one CTA per SM was
+// the chain inside a tile (parts removed in turn, K=24: stage 2 880 us, without products 700,
+// without copies 820; stage 1 580 us, without stores 350): two CTAs per SM overlap them,
+// 1.54 -> 1.27 ms, 11.2 -> 9.2 ms and 1.79 -> 1.60 ms.  The X intermediates' round trip and the
+// stacked operators, 6.3 GB at K=24, take 0.93 ms of that at the measured copy rate.
 #include "kernels_tma.hpp"
 
 #include <cuda_bf16.h>
@@ -69,13 +73,17 @@ struct TmCfg {
   // tensor-memory columns of an accumulator: in the reduce mode with slices two blocks of n
   // columns, one for the products with slice 0 of B and one for the others
   static constexpr int PARTS = !STORE && !EXACT && NSL > 1 ? 2 : 1;
-  static constexpr int NACC = 512 / (NMAX * PARTS);
+  // the sigma modes run two CTAs per SM, each with half of the tensor memory: one CTA's
+  // copies, products and epilogue fill the gaps of the other's
+  static constexpr int CTAS = EXACT ? 1 : 2;
+  static constexpr int TMEM = 512 / CTAS;
+  static constexpr int NACC = TMEM / (NMAX * PARTS);
   static constexpr int SLOTS = EXACT ? 1 : tm_slots(NSL);
   // bytes of one piece of A and of the largest piece of B (all slices)
   static constexpr int A_BYTES = EXACT ? TM_A_BYTES : 128 * TM_PIECE_COLS * 2 * NSL;
   static constexpr int B_BYTES = EXACT ? NMAX * TM_BOX_K * 2 : NMAX * TM_PIECE_COLS * 2 * NSL;
   static constexpr int STAGE_BYTES = SLOTS * (A_BYTES + B_BYTES);
-  static constexpr int STAGES = EXACT ? 8 : (STORE ? (NSL == 3 ? 6 : 4) : (NSL == 3 ? 8 : 6));
+  static constexpr int STAGES = EXACT ? 8 : (STORE ? (NSL == 3 ? 3 : 4) : (NSL == 3 ? 4 : 6));
   static constexpr int SMEM = STAGES * STAGE_BYTES + 1024;
 };
 constexpr int TM_MAX_STAGES = 8, TM_MAX_ACC = 8;
@@ -174,8 +182,18 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&v)[32]) {
   asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
 }
 
+// 16 of them
+__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&v)[16]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];\n"
+      : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
+        "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
+      : "r"(taddr));
+  asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
+}
+
 template <int MODE, int NSL>
-__global__ void __launch_bounds__(TM_THREADS, 1)
+__global__ void __launch_bounds__(TM_THREADS, TmCfg<MODE, NSL>::CTAS)
     gemm_tma_kernel(const TmTile* __restrict__ tiles, int ntiles, const TmTerm* __restrict__ terms,
                     const CUtensorMap* __restrict__ maps, const long* __restrict__ rowmap, void* __restrict__ out,
                     int* __restrict__ err, const int* __restrict__ expo, const int* __restrict__ cta_stage,
@@ -206,7 +224,7 @@ __global__ void __launch_bounds__(TM_THREADS, 1)
 
   if (warp == 2) {  // an epilogue warp (all lanes take the same path) owns the tensor memory
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(smem_u32(&tmem_base_sh)),
-                 "r"(512));
+                 "r"(Cfg::TMEM));
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::);
   }
   if (tid == 0) {
@@ -501,7 +519,7 @@ __global__ void __launch_bounds__(TM_THREADS, 1)
             if (c < tl.nvalid) p[c] = (double)hi[c] + (double)lo[c];
         }
       } else {
-        float run[NMAX / 32][32];  // the tile's running FP32 sum (row r)
+        float run[NMAX / 16][16];  // the tile's running FP32 sum (row r)
         for (int q = 0; q < tl.nseg; ++q, ++sg) {
           const int acc = sg % NACC;
           ok = mbar_wait(&tfull_b[acc], (uint32_t)((sg / NACC) & 1), abort_flag);
@@ -509,19 +527,19 @@ __global__ void __launch_bounds__(TM_THREADS, 1)
           if (!ok) break;
           asm volatile("tcgen05.fence::after_thread_sync;\n" ::);
 #pragma unroll
-          for (int cc = 0; cc < NMAX / 32; ++cc) {
-            const int c0 = cc * 32;
+          for (int cc = 0; cc < NMAX / 16; ++cc) {
+            const int c0 = cc * 16;
             if (c0 < tl.n) {
 #pragma unroll
               for (int part = 0; part < PARTS; ++part) {
-                uint32_t v[32];
-                tmem_ld32(tmem + ((uint32_t)(sub * 32) << 16) + (uint32_t)(acc * NMAX * PARTS + part * tl.n + c0), v);
+                uint32_t v[16];
+                tmem_ld16(tmem + ((uint32_t)(sub * 32) << 16) + (uint32_t)(acc * NMAX * PARTS + part * tl.n + c0), v);
                 if (q == 0 && part == 0) {
 #pragma unroll
-                  for (int u = 0; u < 32; ++u) run[cc][u] = __uint_as_float(v[u]);
+                  for (int u = 0; u < 16; ++u) run[cc][u] = __uint_as_float(v[u]);
                 } else {
 #pragma unroll
-                  for (int u = 0; u < 32; ++u) run[cc][u] += __uint_as_float(v[u]);
+                  for (int u = 0; u < 16; ++u) run[cc][u] += __uint_as_float(v[u]);
                 }
               }
             }
@@ -533,12 +551,12 @@ __global__ void __launch_bounds__(TM_THREADS, 1)
         if (r < tl.m_valid) {
           float* p = reinterpret_cast<float*>(out) + tl.out_off + (long)r * tl.ldo;
 #pragma unroll
-          for (int cc = 0; cc < NMAX / 32; ++cc)
+          for (int cc = 0; cc < NMAX / 16; ++cc)
+            if (cc * 16 < tl.n) {
 #pragma unroll
-            for (int u = 0; u < 32; u += 4) {
-              if (cc * 32 + u >= tl.n) break;
-              red_add_v4(p + cc * 32 + u, __float_as_uint(run[cc][u]), __float_as_uint(run[cc][u + 1]),
-                         __float_as_uint(run[cc][u + 2]), __float_as_uint(run[cc][u + 3]));
+              for (int u = 0; u < 16; u += 4)
+                red_add_v4(p + cc * 16 + u, __float_as_uint(run[cc][u]), __float_as_uint(run[cc][u + 1]),
+                           __float_as_uint(run[cc][u + 2]), __float_as_uint(run[cc][u + 3]));
             }
         }
       }
@@ -550,7 +568,7 @@ __global__ void __launch_bounds__(TM_THREADS, 1)
   if (warp == 2) {
     __syncwarp();
     asm volatile("tcgen05.fence::after_thread_sync;\n" ::);
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(512));
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(Cfg::TMEM));
   }
 }
 
@@ -563,7 +581,7 @@ cudaError_t launch_mode(const TmTile* d_tiles, int ntiles, const TmTerm* d_terms
                            TmCfg<MODE, NSL>::SMEM) == cudaSuccess;
   if (!attr_ok) return cudaErrorInvalidValue;
   // the lists were built for this grid: every CTA's tiles and stages
-  if (lists.grid != tma_grid(ntiles) || !lists.cta_stage || !lists.stages || !lists.pieces)
+  if (lists.grid != tma_grid(MODE, ntiles) || !lists.cta_stage || !lists.stages || !lists.pieces)
     return cudaErrorInvalidValue;
   count_tc_launches(1);
   gemm_tma_kernel<MODE, NSL><<<lists.grid, TM_THREADS, TmCfg<MODE, NSL>::SMEM, s>>>(
@@ -682,7 +700,7 @@ cudaError_t launch_gemm_exact(const TmTile* d_tiles, int ntiles, const TmTerm* d
   return launch_mode<TM_MODE_EXACT_F64, 1>(d_tiles, ntiles, d_terms, d_maps, nullptr, out, d_err, s, d_expo, lists);
 }
 
-int tma_grid(int ntiles) {
+int tma_grid(int mode, int ntiles) {
   static const int nsm = [] {
     int dev = 0, n = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) !=
@@ -690,7 +708,8 @@ int tma_grid(int ntiles) {
       return 148;
     return n > 0 ? n : 148;
   }();
-  return ntiles < nsm ? ntiles : nsm;
+  const int n = mode == TM_MODE_EXACT_F64 ? nsm : 2 * nsm;
+  return ntiles < n ? ntiles : n;
 }
 
 int tma_pieces(int mode, int nsl) { return mode == TM_MODE_EXACT_F64 ? 1 : tm_slots(nsl); }
@@ -782,7 +801,7 @@ __global__ void fill_lists_kernel(int mode, int nslices, const TmTile* __restric
 
 bool tma_plan_lists(int mode, int nsl, std::vector<TmTile>& tiles, const std::vector<TmTerm>& terms, TmListPlan& out) {
   const int ntiles = (int)tiles.size();
-  const int grid = ntiles > 0 ? tma_grid(ntiles) : 0;
+  const int grid = ntiles > 0 ? tma_grid(mode, ntiles) : 0;
   const bool exact = mode == TM_MODE_EXACT_F64;
   const int P = tma_pieces(mode, nsl);
   for (const TmTerm& m : terms)

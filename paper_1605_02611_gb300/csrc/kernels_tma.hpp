@@ -67,11 +67,11 @@ constexpr int TM_MODE_STORE_BF16 = 1, TM_MODE_REDUCE_F32 = 2, TM_MODE_EXACT_F64 
 // bits of the slices of the exact mode
 constexpr int TM_EXACT_BITS = 7;
 constexpr int TM_PIECE_COLS = 16;  // columns of a piece in the sigma modes: one K=16 instruction per product
-// pieces per stage of the sigma modes, so that a stage is 24 to 48 KB whatever the slices
-__host__ __device__ constexpr int tm_slots(int nsl) { return nsl == 1 ? 4 : nsl == 2 ? 2 : 1; }
+// pieces per stage of the sigma modes, so that a stage is 16 to 36 KB whatever the slices
+__host__ __device__ constexpr int tm_slots(int nsl) { return nsl == 1 ? 2 : 1; }
 // stages accumulated in tensor memory before the reduce-mode epilogue takes the partial
-// sum over (60 to 64 instructions: the tensor cores round their running sum toward zero)
-__host__ __device__ constexpr int tm_seg_stages(int nsl) { return nsl == 1 ? 16 : 10; }
+// sum over (about 64 products: the tensor cores round their running sum toward zero)
+__host__ __device__ constexpr int tm_seg_stages(int nsl) { return nsl == 1 ? 32 : nsl == 2 ? 20 : 10; }
 
 // Copy lists.  The tiles' terms are expanded before the launch into stages, each holding
 // up to tma_pieces(mode, nsl) pieces.  In the sigma modes a piece is 16 columns of one term
@@ -128,7 +128,7 @@ __host__ __device__ inline uint32_t tm_idesc_bf16(int n, bool negA) {
 }
 
 // Host: the stage counts of a launch of `mode` (operands of nsl slices) over these tiles
-// (for the grid the launch will use, tma_grid(tiles.size())); reduce mode: sets every
+// (for the grid the launch will use, tma_grid(mode, tiles.size())); reduce mode: sets every
 // tile's pad (its stages) and nseg.  Returns false if a term is malformed (k not a positive
 // multiple of 16), belongs to two tiles, or the lists would be too long.
 bool tma_plan_lists(int mode, int nsl, std::vector<TmTile>& tiles, const std::vector<TmTerm>& terms, TmListPlan& out);
@@ -138,8 +138,9 @@ bool tma_plan_lists(int mode, int nsl, std::vector<TmTile>& tiles, const std::ve
 cudaError_t launch_fill_lists(int mode, int nsl, const TmTile* d_tiles, int ntiles, const TmTerm* d_terms,
                               const int* d_tpiece0, const int* d_sorder, const long* d_sfirst, long total,
                               TmStage* d_stages, TmPiece* d_pieces, cudaStream_t s);
-// CTAs of a launch over ntiles tiles (min(ntiles, SMs of the current device))
-int tma_grid(int ntiles);
+// CTAs of a launch over ntiles tiles (at most one per SM of the current device in the exact
+// mode, two in the sigma modes)
+int tma_grid(int mode, int ntiles);
 int tma_pieces(int mode, int nsl);
 
 // maps: device array of encoded tensor maps (64-byte aligned).  nsl: BF16 slices of the
