@@ -42,6 +42,7 @@
 // 1.54 -> 1.27 ms, 11.2 -> 9.2 ms and 1.79 -> 1.60 ms.  The X intermediates' round trip and the
 // stacked operators, 6.3 GB at K=24, take 0.93 ms of that at the measured copy rate.
 #include "kernels_tma.hpp"
+#include "ptx.cuh"
 
 #include <cuda_bf16.h>
 
@@ -61,7 +62,6 @@ namespace {
 constexpr int TM_THREADS = 192;
 constexpr int TM_BOX_K = 64;                    // exact mode: columns per box (128 bytes)
 constexpr int TM_A_BYTES = 128 * TM_BOX_K * 2;  // 16 KB
-constexpr long TM_WAIT_LIMIT = 1L << 24;
 constexpr int TM_REC_BATCH = 32;  // stages of the copy lists fetched per bulk copy
 
 template <int MODE, int NSL>
@@ -88,8 +88,6 @@ struct TmCfg {
 };
 constexpr int TM_MAX_STAGES = 8, TM_MAX_ACC = 8;
 
-__device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-
 // shared-memory matrix descriptor: K-major, 128-byte swizzle, 8-row groups 1024 B apart
 __device__ __forceinline__ uint64_t sdesc(uint32_t saddr) {
   uint64_t d = 0;
@@ -99,44 +97,6 @@ __device__ __forceinline__ uint64_t sdesc(uint32_t saddr) {
   d |= (uint64_t)1 << 46;
   d |= (uint64_t)2 << 61;
   return d;
-}
-
-// the same for the column-group layout: K-major without swizzle, core matrices of 8 rows x
-// 16 bytes contiguous along the rows (128 B apart), the second 8 columns `rows` rows further.
-// lo: address and rows in 16-byte units, (saddr >> 4) | rows << 16.
-__device__ __forceinline__ uint64_t sdesc_groups(uint32_t lo) {
-  constexpr uint32_t hi = (128u >> 4) | (1u << (46 - 32));
-  uint64_t d;
-  asm("mov.b64 %0, {%1, %2};\n" : "=l"(d) : "r"(lo), "r"(hi));
-  return d;
-}
-
-__device__ __forceinline__ void mbar_init(uint64_t* b, int count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(smem_u32(b)), "r"(count));
-}
-__device__ __forceinline__ void mbar_arrive(uint64_t* b) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(smem_u32(b)) : "memory");
-}
-__device__ __forceinline__ void mbar_arrive_expect_tx(uint64_t* b, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(smem_u32(b)), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ bool mbar_test(uint64_t* b, uint32_t parity) {
-  uint32_t done;
-  asm volatile(
-      "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
-      : "=r"(done)
-      : "r"(smem_u32(b)), "r"(parity)
-      : "memory");
-  return done != 0;
-}
-// bounded parity wait; gives up when the CTA-wide abort flag is raised
-__device__ __forceinline__ bool mbar_wait(uint64_t* b, uint32_t parity, volatile int* abort_flag) {
-  for (long it = 0; it < TM_WAIT_LIMIT; ++it) {
-    if (mbar_test(b, parity)) return true;
-    if ((it & 1023) == 1023 && *abort_flag) return false;
-  }
-  *abort_flag = 1;
-  return false;
 }
 
 __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map, int x, int y, uint64_t* bar) {
@@ -167,19 +127,6 @@ __device__ __forceinline__ void red_add_v4(float* p, uint32_t a, uint32_t b, uin
   asm volatile("red.relaxed.gpu.global.add.v4.f32 [%0], {%1, %2, %3, %4};\n" ::"l"(p), "f"(__uint_as_float(a)),
                "f"(__uint_as_float(b)), "f"(__uint_as_float(c)), "f"(__uint_as_float(d))
                : "memory");
-}
-
-// 32 consecutive FP32 columns of this warp's 32 tensor-memory lanes
-__device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&v)[32]) {
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
-      "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];\n"
-      : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
-        "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15]),
-        "=r"(v[16]), "=r"(v[17]), "=r"(v[18]), "=r"(v[19]), "=r"(v[20]), "=r"(v[21]), "=r"(v[22]), "=r"(v[23]),
-        "=r"(v[24]), "=r"(v[25]), "=r"(v[26]), "=r"(v[27]), "=r"(v[28]), "=r"(v[29]), "=r"(v[30]), "=r"(v[31])
-      : "r"(taddr));
-  asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
 }
 
 // 16 of them
@@ -319,11 +266,11 @@ __global__ void __launch_bounds__(TM_THREADS, TmCfg<MODE, NSL>::CTAS)
       // the last record batch fetched
       for (long qq = j - 1; qq >= 0 && qq >= j - S; --qq) {
         const int s2 = (int)(qq % S);
-        for (long it = 0; it < TM_WAIT_LIMIT && !mbar_test(&full_b[s2], (uint32_t)((qq / S) & 1)); ++it) {
+        for (long it = 0; it < WAIT_LIMIT && !mbar_test(&full_b[s2], (uint32_t)((qq / S) & 1)); ++it) {
         }
       }
       for (int b = max(0, fetched - 2); b < fetched; ++b)
-        for (long it = 0; it < TM_WAIT_LIMIT && !mbar_test(&rec_b[b & 1], (uint32_t)((b >> 1) & 1)); ++it) {
+        for (long it = 0; it < WAIT_LIMIT && !mbar_test(&rec_b[b & 1], (uint32_t)((b >> 1) & 1)); ++it) {
         }
     }
   } else if (warp == 1) {

@@ -16,7 +16,7 @@
 //
 // Numerics: training runs in FP32 on the CUDA cores with the weights rounded to
 // BF16 in the forward pass (FP32 master copy, straight-through gradient).
-// Inference stores h1 in BF16 and runs the 256 x 256 layer on the tensor cores
+// Inference rounds h1 to BF16 and runs the 256 x 256 layer on the tensor cores
 // (tcgen05, FP32 accumulation); the rest is FP32, the correction FP64.
 #pragma once
 #include <cuda_bf16.h>
@@ -25,7 +25,6 @@
 #include <cstdint>
 
 #include "engine.hpp"
-#include "kernels_tc.hpp"
 
 namespace gbdmrg {
 
@@ -49,7 +48,8 @@ struct Mlp {
   DArr<int> err;                 // tensor-core kernel wait flag
   // training scratch, sized for `cap` samples
   long cap = 0;
-  DArr<float> Fb, Pb, Tb, A1, H1, A2, H2, G, dA2, dH1;
+  DArr<float> H1, dA2, G;
+  DArr<float> part;  // partial sums of dL/dW2
   DArr<double> acc;
   ~Mlp();
 };
@@ -74,18 +74,12 @@ struct MlpScratch {
   DArr<long> boff;        // nb + 1 block offsets of psi
   DArr<double> bsum;      // per block: sum of r^2
   DArr<double> bmean;     // per block: mean of the diagonal
-  long chunk = 0;
-  DArr<__nv_bfloat16> H1; // chunk x 256
-  DArr<float> Z;          // chunk x 256
-  DArr<TcTile> tiles;     // tiles of a full chunk, then those of the last chunk
-  DArr<TcTask> tasks;     // [0] full chunk, [1] last chunk
-  DArr<TcTerm> terms;     // [0]: H1 x W2^T
-  int ntiles_full = 0, ntiles_last = 0;
+  bool network = false;   // built for inference, not for pair generation alone
   DArr<int> flag;
   DArr<double> tmp;       // n: tau for pair generation
 };
 
-// m == nullptr: pair generation only (no inference buffers)
+// m == nullptr: pair generation only
 void mlp_scratch_build(MlpScratch& s, const Mlp* m, const PsiLayout& P, cudaStream_t st);
 // block means of the diagonal (once per diagonal)
 void mlp_scratch_set_diag(MlpScratch& s, const double* d, cudaStream_t st);
