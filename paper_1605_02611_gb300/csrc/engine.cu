@@ -169,9 +169,13 @@ int GemmBuilder::cut() {
     std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return work[a] > work[b]; });
   }
   tiles.clear();
-  for (int i : order)
-    for (int ri = 0; ri < gemm_parts(tasks[i].m, cap); ++ri)
-      for (int ci = 0; ci < gemm_parts(tasks[i].n, cap); ++ci) tiles.push_back({i, ri, ci});
+  tiles.reserve((size_t)nt[cap == GEMM_CAPS[0] ? 0 : cap == GEMM_CAPS[1] ? 1 : 2]);
+  for (int i : order) {
+    const int m = tasks[i].m, n = tasks[i].n, pm = gemm_parts(m, cap), pn = gemm_parts(n, cap);
+    if (m >= 1 << 24 || n >= 1 << 24) throw Error(ST_EINVAL, "block dimension too large");
+    for (int ri = 0; ri < pm; ++ri)
+      for (int ci = 0; ci < pn; ++ci) tiles.push_back({i, gemm_range(m, pm, ri), gemm_range(n, pn, ci)});
+  }
   return cap;
 }
 

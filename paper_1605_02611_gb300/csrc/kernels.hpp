@@ -25,14 +25,20 @@ struct GemmTask {
 };
 // One tile of an output block.  A block of m rows is cut into gemm_parts(m, cap) nearly
 // equal row ranges (no range longer than cap, lengths differing by at most one), and its
-// columns likewise; ri, ci count the ranges.
+// columns likewise.  rows, cols: the first row or column in the low 24 bits, the length
+// (at most 64) above them.
 struct GemmTile {
-  int task, ri, ci;
+  int task, rows, cols;
 };
 
 // tile edges of the FP64 grouped GEMM (the largest row or column count of a tile)
 constexpr int GEMM_CAPS[3] = {8, 16, 32};
-__host__ __device__ inline int gemm_parts(int n, int cap) { return (n + cap - 1) / cap; }
+inline int gemm_parts(int n, int cap) { return (n + cap - 1) / cap; }
+// range i of the `parts` ranges of n (n < 2^24)
+inline int gemm_range(int n, int parts, int i) {
+  const int a = (int)((long)n * i / parts), b = (int)((long)n * (i + 1) / parts);
+  return a | (b - a) << 24;
+}
 // The edge for a launch whose blocks are at most max_dim in either direction, given the
 // number of tiles ntiles[i] it has with each GEMM_CAPS[i]: see launch_gemm.
 int gemm_pick_cap(int max_dim, const long ntiles[3]);

@@ -300,25 +300,26 @@ __global__ void __launch_bounds__(TR_THREADS, 1)
       }
     }
   }
-  if constexpr (!GRAD) return;
+  if constexpr (GRAD) {
 #pragma unroll
-  for (int c = 0; c < 4; ++c) {
-    const int j = half * 128 + c * 32 + lane, k = half * 128 + lane * 4 + c;
-    atomicAdd(grad + MLP_OFF_W3 + j, sw3[c]);
-    atomicAdd(grad + MLP_OFF_B2 + j, sb2[c]);
-    atomicAdd(grad + MLP_OFF_B1 + k, sb1[c]);
+    for (int c = 0; c < 4; ++c) {
+      const int j = half * 128 + c * 32 + lane, k = half * 128 + lane * 4 + c;
+      atomicAdd(grad + MLP_OFF_W3 + j, sw3[c]);
+      atomicAdd(grad + MLP_OFF_B2 + j, sb2[c]);
+      atomicAdd(grad + MLP_OFF_B1 + k, sb1[c]);
 #pragma unroll
-    for (int q = 0; q < MLP_F; ++q) atomicAdd(grad + MLP_OFF_W1 + k * MLP_F + q, sw1[c][q]);
-  }
-  if (warp == 0) {
-#pragma unroll
-    for (int o = 16; o; o >>= 1) {
-      lsum += __shfl_xor_sync(0xffffffffu, lsum, o);
-      gsum += __shfl_xor_sync(0xffffffffu, gsum, o);
+      for (int q = 0; q < MLP_F; ++q) atomicAdd(grad + MLP_OFF_W1 + k * MLP_F + q, sw1[c][q]);
     }
-    if (lane == 0) {
-      atomicAdd(loss, lsum * scale);
-      atomicAdd(grad + MLP_OFF_B3, gsum);
+    if (warp == 0) {
+#pragma unroll
+      for (int o = 16; o; o >>= 1) {
+        lsum += __shfl_xor_sync(0xffffffffu, lsum, o);
+        gsum += __shfl_xor_sync(0xffffffffu, gsum, o);
+      }
+      if (lane == 0) {
+        atomicAdd(loss, lsum * scale);
+        atomicAdd(grad + MLP_OFF_B3, gsum);
+      }
     }
   }
 }

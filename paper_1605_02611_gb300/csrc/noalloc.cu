@@ -161,8 +161,9 @@ void compute_diag_noalloc(Context& c, double* diag) {
     hk[pb] = {diag + ob.off, ob.cols, ob.rows, ob.cols, 0, (int)pb, (int)pb + 1};
     hm[pb] = {DL + ((size_t)n1 * Lb.total + Lb.off[ob.rs]) * nz, DR + ((size_t)n2 * Rb.total + Rb.off[ob.cs]) * nz, nz,
               nz, nz, 0, 1.0};
-    for (int ri = 0; ri < gemm_parts(ob.rows, TILE_CAP); ++ri)
-      for (int ci = 0; ci < gemm_parts(ob.cols, TILE_CAP); ++ci) ht[t++] = {(int)pb, ri, ci};
+    const int pm = gemm_parts(ob.rows, TILE_CAP), pn = gemm_parts(ob.cols, TILE_CAP);
+    for (int ri = 0; ri < pm; ++ri)
+      for (int ci = 0; ci < pn; ++ci) ht[t++] = {(int)pb, gemm_range(ob.rows, pm, ri), gemm_range(ob.cols, pn, ci)};
   }
   const size_t dsc_bytes = jobs_bytes + tile_bytes + task_bytes + term_bytes;
   cuda_check(cudaMemcpyAsync(dsc, g_stage, dsc_bytes, cudaMemcpyHostToDevice, c.stream), "h2d");
