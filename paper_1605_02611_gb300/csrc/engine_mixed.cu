@@ -830,7 +830,7 @@ struct TmaPlan {
     DArr<long> sfirst;
     DArr<TmStage> stages;
     DArr<TmPiece> pieces;
-    int grid = 0;
+    int grid = 0, ctas = 1, slots = 0, slot_bytes = 0;
     long total = 0;
     // the stage counts on the host (reduce mode: sets the tiles' stages and segments,
     // so it comes before the tiles are uploaded); throws on a malformed term
@@ -838,6 +838,9 @@ struct TmaPlan {
       TmListPlan lp;
       if (!tma_plan_lists(mode, nsl, tiles, terms, lp)) throw Error(ST_ECUDA, "internal: malformed TMA term list");
       grid = lp.grid;
+      ctas = lp.ctas;
+      slots = lp.slots;
+      slot_bytes = lp.slot_bytes;
       total = lp.total;
       cta_stage.upload(lp.cta_stage, s);
       sorder.upload(lp.sorder, s);
@@ -848,11 +851,11 @@ struct TmaPlan {
     }
     // the lists themselves, on the device, from the uploaded tiles and terms
     void fill(int mode, int nsl, const TmTile* d_tiles, int ntiles, const TmTerm* d_terms, cudaStream_t s) {
-      cuda_check(launch_fill_lists(mode, nsl, d_tiles, ntiles, d_terms, tpiece0.p, sorder.p, sfirst.p, total, stages.p,
+      cuda_check(launch_fill_lists(mode, nsl, slots, d_tiles, ntiles, d_terms, tpiece0.p, sorder.p, sfirst.p, total, stages.p,
                                    pieces.p, s),
                  "list fill");
     }
-    TmListsDev dev() const { return {grid, cta_stage.p, stages.p, pieces.p}; }
+    TmListsDev dev() const { return {grid, ctas, slots, slot_bytes, cta_stage.p, stages.p, pieces.p}; }
   };
   struct Chunk {
     DArr<TmTile> t1, t2;
@@ -1213,14 +1216,30 @@ void build_tma_plan(Context& c, Tilde& lt, Tilde& rt, int k, SigmaPlan& plan, in
     if (off < 0 || rows < 1 || cols < 1 || rows % 16 != 0 || cols % 16 != 0 || off % 8 != 0 ||
         (size_t)(off + nsl * rows * cols) > buf.n)
       throw Error(ST_ECUDA, "internal: tensor map outside its buffer");
-    CUtensorMap m;
-    if (!encode_slice_map(&m, buf.p + off, (uint64_t)rows, (uint64_t)cols, nsl, (uint32_t)box_rows))
-      throw Error(ST_ECUDA, "cuTensorMapEncodeTiled failed");
-    maps.push_back(m);
-    minfo.push_back({rows, cols, box_rows});
-    return (int)maps.size() - 1;
+    // boxes of all slices, then (two or three slices) of one
+    const int first = (int)maps.size();
+    for (int bs = nsl; bs >= 1; bs -= std::max(1, nsl - 1)) {
+      CUtensorMap m;
+      if (!encode_slice_map(&m, buf.p + off, (uint64_t)rows, (uint64_t)cols, nsl, (uint32_t)box_rows, bs))
+        throw Error(ST_ECUDA, "cuTensorMapEncodeTiled failed");
+      maps.push_back(m);
+      minfo.push_back({rows, cols, box_rows});
+    }
+    return first;
   };
-  const int n1max = tma_max_n(TM_MODE_STORE_BF16), n2max = tma_max_n(TM_MODE_REDUCE_F32);
+  // width of the stage-1 N tiles: with two or three slices the largest whose ring holds the longest
+  // term with two CTAs per SM (one CTA per SM is far slower)
+  int n1max = tm_max_n(TM_MODE_STORE_BF16, nsl);
+  const int n2max = tm_max_n(TM_MODE_REDUCE_F32, nsl);
+  if (nsl > 1) {
+    int kmax = 16;
+    for (int qr = 0; qr < nR; ++qr) kmax = std::max(kmax, pad16(Rb.dim[qr]));
+    for (int n = n1max; n >= 64; n -= 16)
+      if (tm_fit_slots(nsl, n, 2) >= kmax / TM_PIECE_COLS) {
+        n1max = n;
+        break;
+      }
+  }
   std::vector<std::vector<std::array<int, 3>>> nt1(ng);  // per g': (row0, width, Psi map) of the stage-1 N tiles
   std::vector<int> a1map(ng, -1);
   for (int gp = 0; gp < ng; ++gp) {
@@ -1352,8 +1371,8 @@ void build_tma_plan(Context& c, Tilde& lt, Tilde& rt, int k, SigmaPlan& plan, in
           }
           if (base.empty()) continue;
           for (TmTerm& t : base) t.neg |= nsl << 4;
-          long steps = 0;  // pieces
-          for (const TmTerm& t : base) steps += t.k / TM_PIECE_COLS;
+          long steps = 0;  // products
+          for (const TmTerm& t : base) steps += (long)t.k / TM_PIECE_COLS * npair;
           for (int r0 = 0; r0 < gC[g]; r0 += 128) {
             Pending pd;
             pd.tl = TmTile{};
@@ -1374,7 +1393,7 @@ void build_tma_plan(Context& c, Tilde& lt, Tilde& rt, int k, SigmaPlan& plan, in
       long acc = 0;
       size_t t0 = 0;
       for (size_t t = 0; t < pd.terms.size(); ++t) {
-        acc += pd.terms[t].k / TM_PIECE_COLS;
+        acc += (long)pd.terms[t].k / TM_PIECE_COLS * npair;
         if (acc >= target || t + 1 == pd.terms.size()) {
           TmTile tl = pd.tl;
           tl.t0 = (int)m2.size();
@@ -1384,10 +1403,9 @@ void build_tma_plan(Context& c, Tilde& lt, Tilde& rt, int k, SigmaPlan& plan, in
             ks += (long)pd.terms[u].k * npair;
           }
           tl.t1 = (int)m2.size();
-          const long stages = (ks / npair / TM_PIECE_COLS + tm_slots(nsl) - 1) / tm_slots(nsl);
-          if (stages > (1L << 30)) throw Error(ST_ECUDA, "internal: stage-2 tile too long");
+          if (ks / TM_PIECE_COLS > (1L << 30)) throw Error(ST_ECUDA, "internal: stage-2 tile too long");
           t2.push_back(tl);
-          st2_steps += stages;
+          st2_steps += (double)(ks / npair / TM_PIECE_COLS);
           st2_fl += 2.0 * 128 * tl.n * ks;
           t0 = t + 1;
           acc = 0;
@@ -1426,8 +1444,8 @@ void build_tma_plan(Context& c, Tilde& lt, Tilde& rt, int k, SigmaPlan& plan, in
           throw Error(ST_ECUDA, "internal: malformed TMA tile");
         for (int t = tl.t0; t < tl.t1; ++t) {
           const TmTerm& m = mm[t];
-          if (((m.neg >> 4) & 15) != nsl || m.amap < 0 || m.amap >= (int)minfo.size() || m.bmap < 0 ||
-              m.bmap >= (int)minfo.size() || minfo[m.amap].box != 128 || minfo[m.bmap].box != tl.n || m.k < 16 ||
+          if (((m.neg >> 4) & 15) != nsl || m.amap < 0 || m.amap + (nsl > 1) >= (int)minfo.size() || m.bmap < 0 ||
+              m.bmap + (nsl > 1) >= (int)minfo.size() || minfo[m.amap].box != 128 || minfo[m.bmap].box != tl.n || m.k < 16 ||
               m.k % 16 || m.ax % 8 || m.bx % 8 || m.ay % 16 || m.by % 16 || m.ax < 0 || m.bx < 0 || m.ay < 0 ||
               m.by < 0 || m.ay >= minfo[m.amap].rows || m.by >= minfo[m.bmap].rows ||
               m.ax + m.k > minfo[m.amap].cols || m.bx + m.k > minfo[m.bmap].cols)
@@ -1467,10 +1485,9 @@ void build_tma_plan(Context& c, Tilde& lt, Tilde& rt, int k, SigmaPlan& plan, in
       if (bad) throw Error(ST_ECUDA, "internal: stage-1 tile check failed (" + std::to_string(bad.load()) + ")");
     }
     for (const TmTile& tl : t2) {
-      long pieces = 0;
-      for (int t = tl.t0; t < tl.t1; ++t) pieces += m2[(size_t)t].k / TM_PIECE_COLS;
-      const long stages = (pieces + tm_slots(nsl) - 1) / tm_slots(nsl);
-      if (tl.pad != stages || stages < 1 || tl.nseg != (int)((stages + tm_seg_stages(nsl) - 1) / tm_seg_stages(nsl)))
+      long prod = 0;
+      for (int t = tl.t0; t < tl.t1; ++t) prod += (long)m2[(size_t)t].k / TM_PIECE_COLS * npair;
+      if (tl.pad < 1 || tl.nseg != (int)((prod + TM_SEG_PRODUCTS - 1) / TM_SEG_PRODUCTS))
         throw Error(ST_ECUDA, "internal: stage-2 stage or segment count");
     }
 
@@ -1901,7 +1918,7 @@ void env_update_exact(Context& c, Tilde& t, const SiteT& A, int site, Env& out, 
   const Bond& ib = left ? Lb : Rb;  // bond of the contracted index
   env_alloc(c, out, ob, st);
   const int no = ob.nsec();
-  const int nmax = tma_max_n(TM_MODE_EXACT_F64);
+  const int nmax = tm_max_n(TM_MODE_EXACT_F64, 1);
   std::vector<SplitJob> split1;  // site and operator blocks
   int nexpo = 0;
   // ---- site tensor: left At blocks [d(qr) x d(ql)], right B blocks [d(ql) x d(qr)]; K = columns

@@ -10,8 +10,8 @@
 // before the launch into per-CTA copy lists (stage word, expected bytes, box coordinates:
 // fill_lists_kernel), so the producer does no term arithmetic.
 //
-// Persistent and warp-specialised, two CTAs per SM in the sigma modes (up to 113 KB of shared
-// memory and 256 tensor-memory columns each), one in the exact mode:
+// Persistent and warp-specialised, one or two CTAs per SM in the sigma modes (256 tensor-memory
+// columns each), one in the exact mode:
 //   warp 0     fetches its CTA's copy lists 32 stages at a time into shared memory
 //              (1D bulk copies, double-buffered); per stage lane 0 waits for the ring
 //              slot and posts the stage word and the expected bytes, then lane p issues
@@ -23,24 +23,26 @@
 //              intermediates, FP32 vector reductions (sigma^T, several tiles may add into
 //              one block) of per-segment partial sums, or (exact mode) two-float sums of
 //              exact integer segments stored in FP64
-// One (sigma modes; two for one slice in the reduce mode) or eight (exact mode, N <= 64)
-// accumulators.  In the sigma modes the two CTAs of an SM overlap each other's epilogues,
-// products and copies.  Every wait is bounded: on timeout the CTA raises a shared abort flag, records an error,
+// One or two (sigma modes) or eight (exact mode, N <= 64) accumulators.  Two CTAs of an SM
+// overlap each other's epilogues, products and copies.  Every wait is bounded: on timeout the CTA raises a shared abort flag, records an error,
 // waits (bounded) for the copies it issued, frees its tensor memory and returns.
 //
-// gemm_slices_kernel (sigma): what bounds it is the operand traffic into shared memory, not
-// the tensor cores: a 128 x n tile of one K=16 product needs 32 (128 + n) bytes through L2
-// for n / 2 tensor clocks.  With two or three slices the products s_i t_j, i + j < nsl, share
-// their operands, so a piece brings every slice of both operands once (3 + 3 boxes' worth of
-// bytes for six products instead of 6 + 6) in two copies instead of twelve, and the
-// column-group layout lets each copy move 256-byte runs instead of 32-byte rows.
+// The sigma modes: what bounds them is the operand traffic into shared memory and the issuing
+// thread, not the tensor cores: a 128 x n tile of one K=16 product needs 32 (128 + n) bytes
+// through L2 for n / 2 tensor clocks.  With two or three slices the products s_i t_j, i + j < nsl,
+// share their operands, so a piece brings every slice of both operands once (3 + 3 boxes' worth
+// of bytes for six products instead of 6 + 6) in two copies instead of twelve, and the
+// column-group layout lets each copy move 256-byte runs instead of 32-byte rows.  The products
+// keep the order term, slice pair, column (they are rounded into the accumulator one by one, and
+// a Davidson solve magnifies another order's rounding), so a term's pieces stay in the ring until
+// its last pair.  Two CTAs per SM: with one, the copies, the products and the epilogue of a tile wait
+// for each other (K=24, one CTA: 3.1 ms).
 // Measured against one pair of swizzled boxes per slice product (16-column boxes in the
-// reduce mode): three slices at K=24, M=512 3.18 -> 1.54 ms per sigma, K=40, M=1200 23.1 ->
-// 11.2 ms; one pass at K=32, M=1024 2.71 -> 1.79 ms.  What then bounded one CTA per SM was
-// the chain inside a tile (parts removed in turn, K=24: stage 2 880 us, without products 700,
-// without copies 820; stage 1 580 us, without stores 350): two CTAs per SM overlap them,
-// 1.54 -> 1.27 ms, 11.2 -> 9.2 ms and 1.79 -> 1.60 ms.  The X intermediates' round trip and the
-// stacked operators, 6.3 GB at K=24, take 0.93 ms of that at the measured copy rate.
+// reduce mode), one CTA per SM: three slices at K=24, M=512 3.19 -> 1.53 ms per sigma, K=40, M=1200
+// 23.1 -> 12.6 ms, K=10, M=150 0.240 -> 0.144 ms; one pass at K=32, M=1024 2.71 -> 1.60 ms.  (Without
+// the fixed order, four instructions of up to 2 n columns per piece and slots released piece by
+// piece: 1.27 and 9.2 ms.)  The X intermediates' round trip and the stacked operators, 6.3 GB at
+// K=24, take 0.93 ms of that at the measured copy rate.
 #include "kernels_tma.hpp"
 #include "ptx.cuh"
 
@@ -51,6 +53,7 @@
 #include <cstdint>
 #include <mutex>
 #include <thread>
+#include <type_traits>
 
 namespace gbdmrg {
 
@@ -64,29 +67,28 @@ constexpr int TM_BOX_K = 64;                    // exact mode: columns per box (
 constexpr int TM_A_BYTES = 128 * TM_BOX_K * 2;  // 16 KB
 constexpr int TM_REC_BATCH = 32;  // stages of the copy lists fetched per bulk copy
 
-template <int MODE, int NSL>
+// CTAS: CTAs per SM the launch is made for (the sigma modes; the exact mode has one)
+template <int MODE, int NSL, int CTAS>
 struct TmCfg {
   static constexpr bool STORE = MODE == TM_MODE_STORE_BF16;
   static constexpr bool EXACT = MODE == TM_MODE_EXACT_F64;
-  // exact mode: 64 columns, so that the two-float sums (128 registers) fit
-  static constexpr int NMAX = STORE ? 256 : (EXACT ? 64 : 128);
-  // tensor-memory columns of an accumulator: in the reduce mode with slices two blocks of n
-  // columns, one for the products with slice 0 of B and one for the others
-  static constexpr int PARTS = !STORE && !EXACT && NSL > 1 ? 2 : 1;
-  // the sigma modes run two CTAs per SM, each with half of the tensor memory: one CTA's
-  // copies, products and epilogue fill the gaps of the other's
-  static constexpr int CTAS = EXACT ? 1 : 2;
-  static constexpr int TMEM = 512 / CTAS;
-  static constexpr int NACC = TMEM / (NMAX * PARTS);
+  // two or three slices: a term's 16-column pieces, one per ring slot, stay until all slice
+  // products of the term have been issued
+  static constexpr bool CHAIN = !EXACT && NSL > 1;
+  static constexpr int NMAX = tm_max_n(MODE, NSL);
+  static constexpr int TMEM = EXACT ? 512 : 256;
+  static constexpr int NACC = TMEM / NMAX;
   static constexpr int SLOTS = EXACT ? 1 : tm_slots(NSL);
   // bytes of one piece of A and of the largest piece of B (all slices)
   static constexpr int A_BYTES = EXACT ? TM_A_BYTES : 128 * TM_PIECE_COLS * 2 * NSL;
   static constexpr int B_BYTES = EXACT ? NMAX * TM_BOX_K * 2 : NMAX * TM_PIECE_COLS * 2 * NSL;
-  static constexpr int STAGE_BYTES = SLOTS * (A_BYTES + B_BYTES);
-  static constexpr int STAGES = EXACT ? 8 : (STORE ? (NSL == 3 ? 3 : 4) : (NSL == 3 ? 4 : 6));
-  static constexpr int SMEM = STAGES * STAGE_BYTES + 1024;
+  static constexpr int STAGE_BYTES = SLOTS * (A_BYTES + B_BYTES);  // (chains: a launch's own slot size)
+  static constexpr int STAGES = EXACT ? 8 : (STORE ? 4 : 6);       // (chains: a launch's own count)
+  static constexpr int SMEM = (CHAIN ? tm_ring_bytes(CTAS) : STAGES * STAGE_BYTES) + 1024;
 };
-constexpr int TM_MAX_STAGES = 8, TM_MAX_ACC = 8;
+constexpr int TM_MAX_STAGES = TM_MAX_SLOTS, TM_MAX_ACC = 8;
+constexpr int TM_TERMS = 32;  // term barriers of the chains (a power of two, more than twice the slots)
+static_assert(TM_TERMS > 2 * TM_MAX_SLOTS, "a ring's terms need distinct barriers");
 
 // shared-memory matrix descriptor: K-major, 128-byte swizzle, 8-row groups 1024 B apart
 __device__ __forceinline__ uint64_t sdesc(uint32_t saddr) {
@@ -107,12 +109,13 @@ __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map
       : "memory");
 }
 
-// box of a column-group map: all of dimension 0, row group y, column group x, every slice
-__device__ __forceinline__ void tma_load_groups(uint32_t dst, const CUtensorMap* map, int x, int y, uint64_t* bar) {
+// box of a column-group map: all of dimension 0, row group y, slices from sl, column group x
+__device__ __forceinline__ void tma_load_groups(uint32_t dst, const CUtensorMap* map, int x, int y, int sl,
+                                                uint64_t* bar) {
   asm volatile(
-      "cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %2, %4}], "
-      "[%5];\n" ::"r"(dst),
-      "l"(map), "r"(0), "r"(y), "r"(x), "r"(smem_u32(bar))
+      "cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5}], "
+      "[%6];\n" ::"r"(dst),
+      "l"(map), "r"(0), "r"(y), "r"(sl), "r"(x), "r"(smem_u32(bar))
       : "memory");
 }
 
@@ -139,23 +142,25 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&v)[16]) {
   asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
 }
 
-template <int MODE, int NSL>
-__global__ void __launch_bounds__(TM_THREADS, TmCfg<MODE, NSL>::CTAS)
+template <int MODE, int NSL, int CTAS>
+__global__ void __launch_bounds__(TM_THREADS, CTAS)
     gemm_tma_kernel(const TmTile* __restrict__ tiles, int ntiles, const TmTerm* __restrict__ terms,
                     const CUtensorMap* __restrict__ maps, const long* __restrict__ rowmap, void* __restrict__ out,
                     int* __restrict__ err, const int* __restrict__ expo, const int* __restrict__ cta_stage,
-                    const TmStage* __restrict__ stg, const TmPiece* __restrict__ pcs) {
-  using Cfg = TmCfg<MODE, NSL>;
-  constexpr int S = Cfg::STAGES;
-  constexpr int STAGE_BYTES = Cfg::STAGE_BYTES;
+                    const TmStage* __restrict__ stg, const TmPiece* __restrict__ pcs, int ring_slots,
+                    int slot_bytes) {
+  using Cfg = TmCfg<MODE, NSL, CTAS>;
+  constexpr bool CHAIN = Cfg::CHAIN;
+  const int S = CHAIN ? ring_slots : Cfg::STAGES;
+  const int STAGE_BYTES = CHAIN ? slot_bytes : Cfg::STAGE_BYTES;
   constexpr int NACC = Cfg::NACC;
   constexpr int NMAX = Cfg::NMAX;
   constexpr bool STORE = Cfg::STORE;
   constexpr bool EXACT = Cfg::EXACT;
-  constexpr int PARTS = Cfg::PARTS;
   extern __shared__ uint8_t dsm[];
   __shared__ __align__(8) uint64_t full_b[TM_MAX_STAGES], empty_b[TM_MAX_STAGES], tfull_b[TM_MAX_ACC],
       tempty_b[TM_MAX_ACC];
+  __shared__ __align__(8) uint64_t term_b[CHAIN ? TM_TERMS : 1];
   __shared__ uint32_t tmem_base_sh;
   __shared__ int abort_sh;
   // per stage: the stage word (TmStage)
@@ -179,6 +184,8 @@ __global__ void __launch_bounds__(TM_THREADS, TmCfg<MODE, NSL>::CTAS)
       mbar_init(&full_b[s], 1);  // the producer's arrive (with the expected bytes)
       mbar_init(&empty_b[s], 1);
     }
+    if (CHAIN)
+      for (int t = 0; t < TM_TERMS; ++t) mbar_init(&term_b[t], 1);
     for (int a = 0; a < NACC; ++a) {
       mbar_init(&tfull_b[a], 1);
       mbar_init(&tempty_b[a], 128);
@@ -202,6 +209,9 @@ __global__ void __launch_bounds__(TM_THREADS, TmCfg<MODE, NSL>::CTAS)
     constexpr int PIECES = PCS;
     constexpr unsigned FULL = 0xffffffffu;
     long j = 0;            // stages issued
+    long freed = 0;        // (chains) stages released, by the terms before `th`; terms issued
+    int th = 0, tq = 0, left = 0;  // pieces of the current term still to come
+    __shared__ unsigned char term_size[CHAIN ? TM_TERMS : 1];
     int st = 0;            // ring slot of the next one (j % S)
     uint32_t par = 0;      // its round's parity ((j / S) & 1)
     bool wrapped = false;  // j >= S
@@ -232,7 +242,21 @@ __global__ void __launch_bounds__(TM_THREADS, TmCfg<MODE, NSL>::CTAS)
       for (int i = 0; i < n && ok; ++i) {
         const TmStage h = rec_stage[b & 1][i];
         if (lane == 0) {
-          if (wrapped && !mbar_wait(&empty_b[st], par ^ 1u, abort_flag)) ok = false;
+          if constexpr (CHAIN) {
+            if (left == 0) {  // first piece of a term
+              left = (int)((uint32_t)(h.word >> 32) & 255u);
+              term_size[tq++ & (TM_TERMS - 1)] = (unsigned char)left;
+            }
+            --left;
+            // at most S <= TM_TERMS / 2 terms are in the ring, so their barriers and sizes are distinct
+            while (ok && j - freed >= S) {
+              ok = mbar_wait(&term_b[th & (TM_TERMS - 1)], (uint32_t)((th / TM_TERMS) & 1), abort_flag);
+              freed += term_size[th & (TM_TERMS - 1)];
+              ++th;
+            }
+          } else {
+            if (wrapped && !mbar_wait(&empty_b[st], par ^ 1u, abort_flag)) ok = false;
+          }
           if (ok) {
             meta[st] = h.word;
             mbar_arrive_expect_tx(&full_b[st], h.bytes);
@@ -248,8 +272,8 @@ __global__ void __launch_bounds__(TM_THREADS, TmCfg<MODE, NSL>::CTAS)
             tma_load_2d(da, maps + q.amap, q.ax, q.ay, &full_b[st]);
             tma_load_2d(db, maps + q.bmap, q.bx, q.by, &full_b[st]);
           } else {
-            tma_load_groups(da, maps + q.amap, q.ax, q.ay, &full_b[st]);
-            tma_load_groups(db, maps + q.bmap, q.bx, q.by, &full_b[st]);
+            tma_load_groups(da, maps + q.amap, q.ax, q.ay, q.as, &full_b[st]);
+            tma_load_groups(db, maps + q.bmap, q.bx, q.by, q.bs, &full_b[st]);
           }
         }
         ++j;
@@ -280,89 +304,201 @@ __global__ void __launch_bounds__(TM_THREADS, TmCfg<MODE, NSL>::CTAS)
       uint32_t par = 0;      // its round's parity
       int sg = 0;  // segments issued
       bool ok = true;
+      auto mma = [&](uint32_t d, uint64_t ad, uint64_t bd, uint32_t idk, uint32_t accum) {
+        asm volatile(
+            "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
+            " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d),
+            "l"(ad), "l"(bd), "r"(idk), "r"(accum));
+      };
+      auto commit = [&](uint64_t* bar) {
+        asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(smem_u32(bar)));
+      };
       // shared-memory descriptors of stage 0's operands; later stages, slots, slices and K
       // steps add their byte offsets / 16 to the 14-bit address field (no carry: shared
       // addresses stay below 256 KB)
       const uint64_t ad0 = sdesc(base), bd0 = sdesc(base + TM_A_BYTES);
-      const uint32_t al0 = (base >> 4) | (uint32_t)(NSL * 128) << 16;
-      const uint32_t bl0 = (base + Cfg::SLOTS * Cfg::A_BYTES) >> 4;
-      for (int ti = blockIdx.x; ti < ntiles && ok; ti += gridDim.x) {
-        bool tile_done = false;
-        while (!tile_done && ok) {
+      const uint32_t al0 = base >> 4, bl0 = (base + Cfg::SLOTS * Cfg::A_BYTES) >> 4;
+      if constexpr (CHAIN) {
+        // A term's products in the order of the slice pairs (i, j), by level i + j, each over all
+        // 16-column pieces of the term: the order in which they are rounded into the
+        // accumulator.  The pieces' slots are released during the last pair.
+        // One thread issues them all and needs several clocks per instruction, so what it executes
+        // per product bounds the kernel once its loops, branches and commits outnumber the products.
+        // Terms of up to six pieces (96 columns) that end inside the open segment are straight-line
+        // code with one commit for all their slots (term barriers, in order), short ones that cross
+        // its end too, with a check per product; the others go product by product in a loop.
+        // Measured at K=24, M=512 (stage 2): all in loops 1.20-1.50 ms, whatever was moved out of
+        // them, straight-line 0.80 ms.
+        constexpr int SEG = STORE ? 0x7fffffff : TM_SEG_PRODUCTS;
+        constexpr int NPAIR = NSL == 2 ? 3 : 6;
+        constexpr uint32_t PAIR_I = 0x210100u, PAIR_J = 0x012010u;  // slices of pair q in the nibble q
+        const uint32_t step = (uint32_t)(STAGE_BYTES >> 4);
+        int cnt = 0;        // products in the open segment
+        uint32_t dacc = 0;  // its accumulator
+        int tm = 0;         // terms released
+        auto open = [&]() -> bool {
           const int acc = sg % NACC;
-          if (sg >= NACC && !mbar_wait(&tempty_b[acc], (uint32_t)(((sg / NACC) - 1) & 1), abort_flag)) {
-            ok = false;
-            break;
-          }
+          if (sg >= NACC && !mbar_wait(&tempty_b[acc], (uint32_t)(((sg / NACC) - 1) & 1), abort_flag)) return false;
           asm volatile("tcgen05.fence::after_thread_sync;\n" ::);
-          const uint32_t dacc = tmem + (uint32_t)(acc * NMAX * PARTS);
-          for (;;) {
-            if (!mbar_wait(&full_b[st], par, abort_flag)) {
+          dacc = tmem + (uint32_t)(acc * NMAX);
+          return true;
+        };
+        auto close = [&]() {
+          commit(&tfull_b[sg % NACC]);
+          ++sg;
+          cnt = 0;
+        };
+        for (int ti = blockIdx.x; ti < ntiles && ok; ti += gridDim.x) {
+          for (bool tile_done = false; !tile_done && ok;) {
+            ok = mbar_wait(&full_b[st], par, abort_flag);
+            if (!ok) break;
+            const uint64_t mw = meta[st];
+            const uint32_t fl = (uint32_t)(mw >> 32), id = (uint32_t)mw | ((fl >> 9 & 1u) << 13);
+            const uint32_t n = ((uint32_t)mw >> 17 & 63u) << 3;  // rows of B: 8 columns of a slice are n * 16 bytes
+            const bool single = (fl & 256u) != 0;  // one slice of each operand
+            tile_done = (fl & 1024u) != 0;
+            const int kp = (int)(fl & 255u), npair = single ? 1 : NPAIR;
+            const uint32_t a0 = al0 | (uint32_t)(single ? 128 : 128 * NSL) << 16, b0 = bl0 | (single ? n : n * NSL) << 16;
+            // the term's pieces: slot offsets of the first six, and their arrival
+            uint32_t off[6];
+            {
+              int s2 = st;
+              uint32_t p2 = par;
+#pragma unroll 1
+              for (int c = 0; c < kp; ++c) {
+                if (c > 0 && !(ok = mbar_wait(&full_b[s2], p2, abort_flag))) break;
+                if (++s2 == S) {
+                  s2 = 0;
+                  p2 ^= 1u;
+                }
+              }
+              if (!ok) break;
+#pragma unroll
+              for (int c = 0; c < 6; ++c) off[c] = (uint32_t)(st + c < S ? st + c : st + c - S) * step;
+            }
+            asm volatile("tcgen05.fence::after_thread_sync;\n" ::);
+            if (cnt == 0 && !(ok = open())) break;
+            const int after = cnt + kp * NPAIR;
+            auto term = [&](auto len, auto check) {
+              constexpr int K = decltype(len)::value;
+              uint32_t accum = cnt > 0;
+#pragma unroll
+              for (int l = 0; l < NSL; ++l)
+#pragma unroll
+                for (int i = 0; i <= l; ++i)
+#pragma unroll
+                  for (int c = 0; c < K; ++c) {
+                    mma(dacc, sdesc_groups(a0 + off[c] + (uint32_t)(i * 128)),
+                        sdesc_groups(b0 + off[c] + (uint32_t)(l - i) * n), id, accum);
+                    accum = 1u;
+                    if constexpr (decltype(check)::value) {
+                      const bool last = l == NSL - 1 && i == l && c == K - 1;
+                      if (++cnt == SEG && !last) {
+                        close();
+                        ok = ok && open();
+                        accum = 0u;
+                      }
+                    }
+                  }
+            };
+            using std::integral_constant;
+            if (!single && kp <= 6 && after <= SEG) {
+              const integral_constant<bool, false> no{};
+              switch (kp) {
+                case 1: term(integral_constant<int, 1>{}, no); break;
+                case 2: term(integral_constant<int, 2>{}, no); break;
+                case 3: term(integral_constant<int, 3>{}, no); break;
+                case 4: term(integral_constant<int, 4>{}, no); break;
+                case 5: term(integral_constant<int, 5>{}, no); break;
+                default: term(integral_constant<int, 6>{}, no); break;
+              }
+              cnt = after;
+              if (cnt == SEG || tile_done) close();
+            } else if (!single && kp <= 3) {
+              const integral_constant<bool, true> yes{};
+              switch (kp) {
+                case 1: term(integral_constant<int, 1>{}, yes); break;
+                case 2: term(integral_constant<int, 2>{}, yes); break;
+                default: term(integral_constant<int, 3>{}, yes); break;
+              }
+              if (!ok) break;
+              if (cnt == SEG || tile_done) close();
+            } else {
+#pragma unroll 1
+              for (int q = 0; q < npair && ok; ++q) {
+                uint32_t a = a0 + off[0] + (PAIR_I >> (4 * q) & 15u) * 128u, b = b0 + off[0] + (PAIR_J >> (4 * q) & 15u) * n;
+                int s2 = st;
+#pragma unroll 1
+                for (int c = 0; c < kp; ++c) {
+                  if (cnt == 0 && !(ok = open())) break;
+                  mma(dacc, sdesc_groups(a), sdesc_groups(b), id, cnt > 0);
+                  if (++cnt == SEG || (tile_done && q == npair - 1 && c == kp - 1)) close();
+                  a += step;
+                  b += step;
+                  if (++s2 == S) {
+                    s2 = 0;
+                    a -= (uint32_t)S * step;
+                    b -= (uint32_t)S * step;
+                  }
+                }
+              }
+              if (!ok) break;
+            }
+            commit(&term_b[tm & (TM_TERMS - 1)]);
+            ++tm;
+            st += kp;
+            if (st >= S) {
+              st -= S;
+              par ^= 1u;
+            }
+          }
+        }
+      } else {
+        for (int ti = blockIdx.x; ti < ntiles && ok; ti += gridDim.x) {
+          bool tile_done = false;
+          while (!tile_done && ok) {
+            const int acc = sg % NACC;
+            if (sg >= NACC && !mbar_wait(&tempty_b[acc], (uint32_t)(((sg / NACC) - 1) & 1), abort_flag)) {
               ok = false;
               break;
             }
             asm volatile("tcgen05.fence::after_thread_sync;\n" ::);
-            const uint64_t mw = meta[st];
-            const uint32_t id = (uint32_t)mw, fl = (uint32_t)(mw >> 32);
-            const int nk = (int)(fl & 7u);
-            const uint32_t off = (uint32_t)((st * STAGE_BYTES) >> 4);
-            uint32_t accum = (fl & 8u) ? 0u : 1u;
-            auto mma = [&](uint32_t d, uint64_t ad, uint64_t bd, uint32_t idk) {
-              asm volatile(
-                  "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-                  " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d),
-                  "l"(ad), "l"(bd), "r"(idk), "r"(accum));
-            };
-            if constexpr (EXACT) {
+            const uint32_t dacc = tmem + (uint32_t)(acc * NMAX);
+            for (;;) {
+              if (!mbar_wait(&full_b[st], par, abort_flag)) {
+                ok = false;
+                break;
+              }
+              asm volatile("tcgen05.fence::after_thread_sync;\n" ::);
+              const uint64_t mw = meta[st];
+              const uint32_t id = (uint32_t)mw, fl = (uint32_t)(mw >> 32);
+              const int nk = (int)(fl & 7u);
+              const uint32_t off = (uint32_t)((st * STAGE_BYTES) >> 4);
+              uint32_t accum = (fl & 8u) ? 0u : 1u;
+              const uint32_t n = (id >> 17 & 63u) << 3;
               for (int kk = 0; kk < nk; ++kk) {
-                mma(dacc, ad0 + off + (uint64_t)(kk * 2), bd0 + off + (uint64_t)(kk * 2), id);
+                if constexpr (EXACT)
+                  mma(dacc, ad0 + off + (uint64_t)(kk * 2), bd0 + off + (uint64_t)(kk * 2), id, accum);
+                else
+                  mma(dacc, sdesc_groups((al0 + off + (uint32_t)((kk * Cfg::A_BYTES) >> 4)) | 128u << 16),
+                      sdesc_groups((bl0 + off + (uint32_t)((kk * Cfg::B_BYTES) >> 4)) | n << 16),
+                      id | (((fl >> (8 + kk)) & 1u) << 13), accum);
                 accum = 1u;
               }
-            } else {
-              // rows of B: 8 columns of one slice are n * 16 bytes, of all NSL * n * 16
-              const uint32_t nf = id & (63u << 17), n = nf >> 14;
-              const uint32_t bl = bl0 + off + ((n * NSL) << 16), al = al0 + off;
-              for (int sl = 0; sl < nk; ++sl) {
-                const uint32_t idk = id | (((fl >> (8 + sl)) & 1u) << 13);
-                const uint32_t a = al + (uint32_t)((sl * Cfg::A_BYTES) >> 4), b = bl + (uint32_t)((sl * Cfg::B_BYTES) >> 4);
-                if constexpr (PARTS == 2) {
-                  // the two blocks of the accumulator start from the first product, of both
-                  // slices of B at once (2 n columns)
-                  mma(dacc, sdesc_groups(a), sdesc_groups(b), idk + nf);
-                  accum = 1u;
-                  if constexpr (NSL == 2) {
-                    mma(dacc, sdesc_groups(a + 128u), sdesc_groups(b), idk);
-                  } else {
-                    mma(dacc, sdesc_groups(a + 128u), sdesc_groups(b), idk + nf);
-                    mma(dacc + n, sdesc_groups(a), sdesc_groups(b + 2 * n), idk);
-                    mma(dacc, sdesc_groups(a + 256u), sdesc_groups(b), idk);
-                  }
-                } else {
-#pragma unroll
-                  for (int l = 0; l < NSL; ++l)
-#pragma unroll
-                    for (int i = 0; i <= l; ++i) {
-                      mma(dacc, sdesc_groups(a + (uint32_t)(i * 128)), sdesc_groups(b + (uint32_t)(l - i) * n), idk);
-                      accum = 1u;
-                    }
-                }
+              commit(&empty_b[st]);
+              if (++st == S) {
+                st = 0;
+                par ^= 1u;
+              }
+              if (fl & 16u) {
+                tile_done = (fl & 32u) != 0;
+                break;
               }
             }
-            asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(
-                smem_u32(&empty_b[st])));
-            if (++st == S) {
-              st = 0;
-              par ^= 1u;
-            }
-            if (fl & 16u) {
-              tile_done = (fl & 32u) != 0;
-              break;
-            }
+            if (!ok) break;
+            commit(&tfull_b[acc]);
+            ++sg;
           }
-          if (!ok) break;
-          asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(
-              smem_u32(&tfull_b[acc])));
-          ++sg;
         }
       }
     }
@@ -477,17 +613,14 @@ __global__ void __launch_bounds__(TM_THREADS, TmCfg<MODE, NSL>::CTAS)
           for (int cc = 0; cc < NMAX / 16; ++cc) {
             const int c0 = cc * 16;
             if (c0 < tl.n) {
+              uint32_t v[16];
+              tmem_ld16(tmem + ((uint32_t)(sub * 32) << 16) + (uint32_t)(acc * NMAX + c0), v);
+              if (q == 0) {
 #pragma unroll
-              for (int part = 0; part < PARTS; ++part) {
-                uint32_t v[16];
-                tmem_ld16(tmem + ((uint32_t)(sub * 32) << 16) + (uint32_t)(acc * NMAX * PARTS + part * tl.n + c0), v);
-                if (q == 0 && part == 0) {
+                for (int u = 0; u < 16; ++u) run[cc][u] = __uint_as_float(v[u]);
+              } else {
 #pragma unroll
-                  for (int u = 0; u < 16; ++u) run[cc][u] = __uint_as_float(v[u]);
-                } else {
-#pragma unroll
-                  for (int u = 0; u < 16; ++u) run[cc][u] += __uint_as_float(v[u]);
-                }
+                for (int u = 0; u < 16; ++u) run[cc][u] += __uint_as_float(v[u]);
               }
             }
           }
@@ -519,20 +652,25 @@ __global__ void __launch_bounds__(TM_THREADS, TmCfg<MODE, NSL>::CTAS)
   }
 }
 
-template <int MODE, int NSL>
+template <int MODE, int NSL, int CTAS>
 cudaError_t launch_mode(const TmTile* d_tiles, int ntiles, const TmTerm* d_terms, const CUtensorMap* d_maps,
                         const long* d_rowmap, void* out, int* d_err, cudaStream_t s, const int* d_expo,
                         const TmListsDev& lists) {
+  using Cfg = TmCfg<MODE, NSL, CTAS>;
   static const bool attr_ok =
-      cudaFuncSetAttribute(gemm_tma_kernel<MODE, NSL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           TmCfg<MODE, NSL>::SMEM) == cudaSuccess;
+      cudaFuncSetAttribute(gemm_tma_kernel<MODE, NSL, CTAS>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::SMEM) ==
+      cudaSuccess;
   if (!attr_ok) return cudaErrorInvalidValue;
-  // the lists were built for this grid: every CTA's tiles and stages
-  if (lists.grid != tma_grid(MODE, ntiles) || !lists.cta_stage || !lists.stages || !lists.pieces)
+  // the lists were built for this grid (every CTA's tiles and stages) and ring
+  if (lists.grid != tma_grid(CTAS, ntiles) || !lists.cta_stage || !lists.stages || !lists.pieces)
+    return cudaErrorInvalidValue;
+  if (Cfg::CHAIN && (lists.slots < 1 || lists.slots > TM_MAX_SLOTS || lists.slot_bytes % 1024 != 0 ||
+                     lists.slots * lists.slot_bytes > tm_ring_bytes(CTAS)))
     return cudaErrorInvalidValue;
   count_tc_launches(1);
-  gemm_tma_kernel<MODE, NSL><<<lists.grid, TM_THREADS, TmCfg<MODE, NSL>::SMEM, s>>>(
-      d_tiles, ntiles, d_terms, d_maps, d_rowmap, out, d_err, d_expo, lists.cta_stage, lists.stages, lists.pieces);
+  gemm_tma_kernel<MODE, NSL, CTAS><<<lists.grid, TM_THREADS, Cfg::SMEM, s>>>(
+      d_tiles, ntiles, d_terms, d_maps, d_rowmap, out, d_err, d_expo, lists.cta_stage, lists.stages, lists.pieces,
+      lists.slots, lists.slot_bytes);
   return cudaGetLastError();
 }
 
@@ -621,21 +759,20 @@ cudaError_t launch_split_exact(const SplitJob* d_jobs, int njobs, int nsl, int* 
   return cudaGetLastError();
 }
 
-int tma_max_n(int mode) { return mode == TM_MODE_STORE_BF16 ? 256 : (mode == TM_MODE_EXACT_F64 ? 64 : 128); }
-
 cudaError_t launch_gemm_slices(int mode, int nsl, const TmTile* d_tiles, int ntiles, const CUtensorMap* d_maps,
                                const long* d_rowmap, void* out, int* d_err, cudaStream_t s, const TmListsDev& lists) {
   if (ntiles <= 0) return cudaSuccess;
   auto go = [&](auto fn) { return fn(d_tiles, ntiles, nullptr, d_maps, d_rowmap, out, d_err, s, nullptr, lists); };
+  const bool two = lists.ctas == 2;
   if (mode == TM_MODE_STORE_BF16) {
-    if (nsl == 1) return go(launch_mode<TM_MODE_STORE_BF16, 1>);
-    if (nsl == 2) return go(launch_mode<TM_MODE_STORE_BF16, 2>);
-    if (nsl == 3) return go(launch_mode<TM_MODE_STORE_BF16, 3>);
+    if (nsl == 1) return go(launch_mode<TM_MODE_STORE_BF16, 1, 2>);
+    if (nsl == 2) return two ? go(launch_mode<TM_MODE_STORE_BF16, 2, 2>) : go(launch_mode<TM_MODE_STORE_BF16, 2, 1>);
+    if (nsl == 3) return two ? go(launch_mode<TM_MODE_STORE_BF16, 3, 2>) : go(launch_mode<TM_MODE_STORE_BF16, 3, 1>);
   }
   if (mode == TM_MODE_REDUCE_F32) {
-    if (nsl == 1) return go(launch_mode<TM_MODE_REDUCE_F32, 1>);
-    if (nsl == 2) return go(launch_mode<TM_MODE_REDUCE_F32, 2>);
-    if (nsl == 3) return go(launch_mode<TM_MODE_REDUCE_F32, 3>);
+    if (nsl == 1) return go(launch_mode<TM_MODE_REDUCE_F32, 1, 2>);
+    if (nsl == 2) return two ? go(launch_mode<TM_MODE_REDUCE_F32, 2, 2>) : go(launch_mode<TM_MODE_REDUCE_F32, 2, 1>);
+    if (nsl == 3) return two ? go(launch_mode<TM_MODE_REDUCE_F32, 3, 2>) : go(launch_mode<TM_MODE_REDUCE_F32, 3, 1>);
   }
   return cudaErrorInvalidValue;
 }
@@ -644,10 +781,10 @@ cudaError_t launch_gemm_exact(const TmTile* d_tiles, int ntiles, const TmTerm* d
                               double* out, int* d_err, cudaStream_t s, const TmListsDev& lists, const int* d_expo) {
   if (ntiles <= 0) return cudaSuccess;
   if (!d_expo || !d_terms) return cudaErrorInvalidValue;
-  return launch_mode<TM_MODE_EXACT_F64, 1>(d_tiles, ntiles, d_terms, d_maps, nullptr, out, d_err, s, d_expo, lists);
+  return launch_mode<TM_MODE_EXACT_F64, 1, 1>(d_tiles, ntiles, d_terms, d_maps, nullptr, out, d_err, s, d_expo, lists);
 }
 
-int tma_grid(int mode, int ntiles) {
+int tma_grid(int ctas, int ntiles) {
   static const int nsm = [] {
     int dev = 0, n = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) !=
@@ -655,29 +792,44 @@ int tma_grid(int mode, int ntiles) {
       return 148;
     return n > 0 ? n : 148;
   }();
-  const int n = mode == TM_MODE_EXACT_F64 ? nsm : 2 * nsm;
-  return ntiles < n ? ntiles : n;
+  return ntiles < ctas * nsm ? ntiles : ctas * nsm;
 }
 
 int tma_pieces(int mode, int nsl) { return mode == TM_MODE_EXACT_F64 ? 1 : tm_slots(nsl); }
 
 namespace {
-// pieces of a term: 16 columns each, or (exact mode) 64 columns of every slice pair
-__host__ __device__ inline long term_pieces(const TmTerm& m, bool exact) {
-  if (!exact) return m.k / TM_PIECE_COLS;
+__host__ __device__ inline int slice_pairs(int nsl) { return nsl * (nsl + 1) / 2; }
+
+// pieces of a term: 16 columns each; 16 columns of every slice pair where a term of two or three
+// slices has more pieces than the ring has slots; or (exact mode) 64 columns of every slice pair
+__host__ __device__ inline long term_pieces(const TmTerm& m, bool exact, int nslices, int slots) {
+  if (!exact) {
+    const int kp = m.k / TM_PIECE_COLS;
+    return nslices > 1 && kp > slots ? (long)kp * slice_pairs(nslices) : kp;
+  }
   const int nsl = ((m.neg >> 4) & 15) > 1 ? ((m.neg >> 4) & 15) : 1;
-  return (long)((m.k + TM_BOX_K - 1) / TM_BOX_K) * (nsl * (nsl + 1) / 2);
+  return (long)((m.k + TM_BOX_K - 1) / TM_BOX_K) * slice_pairs(nsl);
+}
+
+// slice pair number q in level order: its level and first index
+__device__ __forceinline__ void slice_pair(int q, int& l, int& i) {
+  l = 0;
+  while (q > l) {
+    q -= l + 1;
+    ++l;
+  }
+  i = q;
 }
 
 // One thread per stage.  It finds its tile (stages in the launch order: sorder[i] has
 // the stages from sfirst[i]) and the term of its first piece (tpiece0: a term's first
 // piece within its tile), then walks the stage's pieces.  Exact mode: a term's pieces are its
 // slice pairs (i, j), i + j < nsl, in level order, each its boxes along K.  Segments: store
-// mode one per tile; reduce mode tm_seg_stages(nsl) stages each (the products accumulate in
+// mode one per tile; reduce mode TM_SEG_PRODUCTS products each (they accumulate in
 // tensor memory over a segment only and the epilogue adds the segments in FP32 with
 // round-to-nearest, so the rounding toward zero of the tensor-core accumulation acts on
 // short sums); exact mode one per level of every term.
-__global__ void fill_lists_kernel(int mode, int nslices, const TmTile* __restrict__ tiles, int ntiles,
+__global__ void fill_lists_kernel(int mode, int nslices, int slots, const TmTile* __restrict__ tiles, int ntiles,
                                   const TmTerm* __restrict__ terms, const int* __restrict__ tpiece0,
                                   const int* __restrict__ sorder, const long* __restrict__ sfirst, long total,
                                   TmStage* __restrict__ stages, TmPiece* __restrict__ pieces) {
@@ -699,34 +851,39 @@ __global__ void fill_lists_kernel(int mode, int nslices, const TmTile* __restric
     const int mid = (t + th + 1) >> 1;
     if (tpiece0[mid] <= p0) t = mid; else th = mid - 1;
   }
-  const long tile_pieces = tpiece0[tl.t1 - 1] + term_pieces(terms[tl.t1 - 1], exact);
+  const long tile_pieces = tpiece0[tl.t1 - 1] + term_pieces(terms[tl.t1 - 1], exact, nslices, slots);
   const int np = (int)min((long)P, tile_pieces - p0);
-  const uint32_t piece_bytes = (uint32_t)(128 + tl.n) * bc * 2 * (exact ? 1 : nslices);
+  uint32_t piece_bytes = (uint32_t)(128 + tl.n) * bc * 2 * (exact ? 1 : nslices);
   const bool last = sl == nst - 1;
   TmTerm m = terms[t];
   long r = p0 - tpiece0[t];
   uint32_t negm = 0, fl = 0, id = 0;
   for (int slot = 0; slot < np; ++slot, ++r) {
-    if (r >= term_pieces(m, exact)) {
+    if (r >= term_pieces(m, exact, nslices, slots)) {
       m = terms[++t];
       r = 0;
     }
     if (!exact) {
-      const int k0 = (int)r * bc;
-      pieces[g * P + slot] = TmPiece{m.amap, (m.ax + k0) / 8, m.ay / 16, m.bmap, (m.bx + k0) / 8, m.by / 16, 0, 0};
+      const int kp = m.k / bc, q = (int)r / kp, k0 = ((int)r - q * kp) * bc;
+      const bool single = nslices > 1 && kp > slots;  // one slice of each operand: the maps after the term's
+      int l = 0, i = 0;
+      if (single) slice_pair(q, l, i);
+      pieces[g * P + slot] = TmPiece{m.amap + single, (m.ax + k0) / 8, m.ay / 16, m.bmap + single, (m.bx + k0) / 8,
+                                     m.by / 16, i, l - i};
       negm |= (uint32_t)(m.neg & 1) << slot;
+      if (nslices > 1) {
+        const bool term_last = t == tl.t1 - 1;
+        if (single) piece_bytes = (uint32_t)(128 + tl.n) * bc * 2;
+        fl = (single ? 256u + 1u : (uint32_t)kp) | (negm & 1u) << 9;
+        fl |= (single ? last : term_last) ? 1024u : 0u;
+      }
       continue;
     }
     const int nsl = max(1, (m.neg >> 4) & 15);
     const int kp = (m.k + bc - 1) / bc;
-    int q = (int)(r / kp);
-    const int kk = (int)(r - (long)q * kp);
-    int l = 0;
-    while (q > l) {
-      q -= l + 1;
-      ++l;
-    }
-    const int i = q, k0 = kk * bc;
+    const int q = (int)(r / kp), kk = (int)(r - (long)q * kp), k0 = kk * bc;
+    int l, i;
+    slice_pair(q, l, i);
     pieces[g * P + slot] = TmPiece{m.amap + i, m.ax + k0, m.ay, m.bmap + (l - i), m.bx + k0, m.by, 0, 0};
     fl = (uint32_t)min(bc / 16, (m.k - k0) / 16);
     fl |= (i == 0 && kk == 0) ? 8u : 0u;
@@ -734,38 +891,55 @@ __global__ void fill_lists_kernel(int mode, int nslices, const TmTile* __restric
     id = tm_idesc_bf16(tl.n, (m.neg & 1) != 0);
   }
   for (int p = np; p < P; ++p) pieces[g * P + p] = TmPiece{0, 0, 0, 0, 0, 0, 0, 0};
-  if (!exact) {
-    const long seg = mode == TM_MODE_REDUCE_F32 ? tm_seg_stages(nslices) : nst;
+  if (!exact) id = tm_idesc_bf16(tl.n, false);
+  if (!exact && nslices == 1) {
+    const long seg = mode == TM_MODE_REDUCE_F32 ? TM_SEG_PRODUCTS / tm_slots(1) : nst;
     fl = (uint32_t)np | (negm << 8);
     fl |= sl % seg == 0 ? 8u : 0u;
     fl |= (last || sl % seg == seg - 1) ? 16u : 0u;
-    id = tm_idesc_bf16(tl.n, false);
   }
-  fl |= last ? 32u : 0u;
+  if (exact || nslices == 1) fl |= last ? 32u : 0u;
   stages[g] = TmStage{(uint64_t)id | ((uint64_t)fl << 32), (uint32_t)np * piece_bytes, np};
 }
 }  // namespace
 
 bool tma_plan_lists(int mode, int nsl, std::vector<TmTile>& tiles, const std::vector<TmTerm>& terms, TmListPlan& out) {
   const int ntiles = (int)tiles.size();
-  const int grid = ntiles > 0 ? tma_grid(mode, ntiles) : 0;
-  const bool exact = mode == TM_MODE_EXACT_F64;
+  const bool exact = mode == TM_MODE_EXACT_F64, chain = !exact && nsl > 1;
   const int P = tma_pieces(mode, nsl);
-  for (const TmTerm& m : terms)
+  int max_n = 16, max_k = 16;
+  for (const TmTile& tl : tiles) max_n = std::max(max_n, tl.n);
+  for (const TmTerm& m : terms) {
     if (m.k < 16 || m.k % 16) return false;
+    max_k = std::max(max_k, m.k);
+  }
+  // ring of a launch with two or three slices: slots of one piece of all slices.  Two CTAs per SM
+  // where the longest term fits the ring of each, else one with a ring twice as large (and terms
+  // that do not fit that go slice pair by slice pair).
+  out.ctas = exact ? 1 : 2;
+  out.slots = 0;
+  out.slot_bytes = 0;
+  if (chain) {
+    out.slot_bytes = tm_slot_bytes(nsl, max_n);
+    if (tm_fit_slots(nsl, max_n, 2) < max_k / TM_PIECE_COLS) out.ctas = 1;
+    out.slots = tm_fit_slots(nsl, max_n, out.ctas);
+  }
+  const int grid = ntiles > 0 ? tma_grid(out.ctas, ntiles) : 0;
   // every term belongs to one tile; its first piece within the tile
   out.tpiece0.assign(terms.size(), -1);
-  std::vector<long> tst((size_t)ntiles);
+  std::vector<long> tst((size_t)ntiles), tprod((size_t)ntiles);
   for (int ti = 0; ti < ntiles; ++ti) {
     const TmTile& tl = tiles[(size_t)ti];
     if (tl.t0 < 0 || tl.t1 <= tl.t0 || tl.t1 > (int)terms.size()) return false;
-    long pc = 0;
+    long pc = 0, pr = 0;
     for (int t = tl.t0; t < tl.t1; ++t) {
       if (out.tpiece0[(size_t)t] >= 0 || pc >= (1L << 31)) return false;
       out.tpiece0[(size_t)t] = (int)pc;
-      pc += term_pieces(terms[(size_t)t], exact);
+      pc += term_pieces(terms[(size_t)t], exact, nsl, out.slots);
+      pr += (long)terms[(size_t)t].k / TM_PIECE_COLS * slice_pairs(nsl);
     }
     tst[(size_t)ti] = (pc + P - 1) / P;
+    tprod[(size_t)ti] = pr;
   }
   // stages in launch order: CTA c takes the tiles c, c + grid, ...
   out.grid = grid;
@@ -787,17 +961,17 @@ bool tma_plan_lists(int mode, int nsl, std::vector<TmTile>& tiles, const std::ve
   if (mode == TM_MODE_REDUCE_F32)
     for (int ti = 0; ti < ntiles; ++ti) {
       tiles[(size_t)ti].pad = (int)tst[(size_t)ti];
-      tiles[(size_t)ti].nseg = (int)((tst[(size_t)ti] + tm_seg_stages(nsl) - 1) / tm_seg_stages(nsl));
+      tiles[(size_t)ti].nseg = (int)((tprod[(size_t)ti] + TM_SEG_PRODUCTS - 1) / TM_SEG_PRODUCTS);
     }
   return true;
 }
 
-cudaError_t launch_fill_lists(int mode, int nsl, const TmTile* d_tiles, int ntiles, const TmTerm* d_terms,
+cudaError_t launch_fill_lists(int mode, int nsl, int slots, const TmTile* d_tiles, int ntiles, const TmTerm* d_terms,
                               const int* d_tpiece0, const int* d_sorder, const long* d_sfirst, long total,
                               TmStage* d_stages, TmPiece* d_pieces, cudaStream_t s) {
   if (ntiles <= 0 || total <= 0) return cudaSuccess;
   count_tc_launches(1);
-  fill_lists_kernel<<<(unsigned)((total + 255) / 256), 256, 0, s>>>(mode, nsl, d_tiles, ntiles, d_terms, d_tpiece0,
+  fill_lists_kernel<<<(unsigned)((total + 255) / 256), 256, 0, s>>>(mode, nsl, slots, d_tiles, ntiles, d_terms, d_tpiece0,
                                                                     d_sorder, d_sfirst, total, d_stages, d_pieces);
   return cudaGetLastError();
 }
@@ -817,14 +991,15 @@ bool encode_bf16_map(CUtensorMap* out, const void* base, uint64_t rows, uint64_t
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-bool encode_slice_map(CUtensorMap* out, const void* base, uint64_t rows, uint64_t cols, int nsl, uint32_t box_rows) {
+bool encode_slice_map(CUtensorMap* out, const void* base, uint64_t rows, uint64_t cols, int nsl, uint32_t box_rows,
+                      int box_slices) {
   EncodeTiledFn fn = encoder();
-  if (!fn || rows == 0 || rows % 16 != 0 || cols == 0 || cols % 8 != 0 || nsl < 1 || nsl > 3 ||
+  if (!fn || rows == 0 || rows % 16 != 0 || cols == 0 || cols % 8 != 0 || nsl < 1 || nsl > 3 || box_slices < 1 || box_slices > nsl ||
       ((uintptr_t)base & 15) != 0 || box_rows == 0 || box_rows % 16 != 0 || box_rows > 256)
     return false;
   const cuuint64_t dims[4] = {128, rows / 16, (cuuint64_t)nsl, cols / 8};
   const cuuint64_t strides[3] = {256, rows * 16, rows * 16 * nsl};
-  const cuuint32_t box[4] = {128, box_rows / 16, (cuuint32_t)nsl, TM_PIECE_COLS / 8};
+  const cuuint32_t box[4] = {128, box_rows / 16, (cuuint32_t)box_slices, TM_PIECE_COLS / 8};
   const cuuint32_t estr[4] = {1, 1, 1, 1};
   return fn(out, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(base), dims, strides, box, estr,
             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,

@@ -47,8 +47,8 @@ struct TmTerm {
 //     out_off .. out_off + n.
 //   reduce mode (sigma^T, FP32): rows r < m_valid are added (vector reductions) to
 //     out + out_off + r * ldo, columns [0, n).
-//   pad, nseg (reduce mode): the tile's stages and segments, ceil(stages /
-//     tm_seg_stages(nsl)); each segment accumulates in tensor memory on its own and the
+//   pad, nseg (reduce mode): the tile's stages and segments, ceil(products /
+//     TM_SEG_PRODUCTS); each segment accumulates in tensor memory on its own and the
 //     epilogue adds the segments in FP32.
 struct TmTile {
   int t0, t1;
@@ -67,16 +67,31 @@ constexpr int TM_MODE_STORE_BF16 = 1, TM_MODE_REDUCE_F32 = 2, TM_MODE_EXACT_F64 
 // bits of the slices of the exact mode
 constexpr int TM_EXACT_BITS = 7;
 constexpr int TM_PIECE_COLS = 16;  // columns of a piece in the sigma modes: one K=16 instruction per product
-// pieces per stage of the sigma modes, so that a stage is 16 to 36 KB whatever the slices
+// pieces per stage of the sigma modes: several in one pass; one, with all its slices, for two or
+// three slices
 __host__ __device__ constexpr int tm_slots(int nsl) { return nsl == 1 ? 2 : 1; }
-// stages accumulated in tensor memory before the reduce-mode epilogue takes the partial
-// sum over (about 64 products: the tensor cores round their running sum toward zero)
-__host__ __device__ constexpr int tm_seg_stages(int nsl) { return nsl == 1 ? 32 : nsl == 2 ? 20 : 10; }
+// K=16 products accumulated in tensor memory before the reduce-mode epilogue takes the partial
+// sum over (the tensor cores round their running sum toward zero)
+constexpr int TM_SEG_PRODUCTS = 64;
+// ring of two or three slices: at most TM_MAX_SLOTS slots of one piece in tm_ring_bytes(CTAs per SM)
+constexpr int TM_MAX_SLOTS = 12;
+constexpr int tm_ring_bytes(int ctas) { return ctas == 2 ? 108 * 1024 : 216 * 1024; }
+constexpr int tm_slot_bytes(int nsl, int n) { return ((128 + n) * TM_PIECE_COLS * 2 * nsl + 1023) / 1024 * 1024; }
+constexpr int tm_fit_slots(int nsl, int n, int ctas) {
+  return tm_ring_bytes(ctas) / tm_slot_bytes(nsl, n) < TM_MAX_SLOTS ? tm_ring_bytes(ctas) / tm_slot_bytes(nsl, n)
+                                                                     : TM_MAX_SLOTS;
+}
+// maximum MMA width of a mode
+constexpr int tm_max_n(int mode, int nsl) {
+  return mode == TM_MODE_EXACT_F64 ? 64 : mode == TM_MODE_STORE_BF16 && nsl == 1 ? 256 : 128;
+}
 
 // Copy lists.  The tiles' terms are expanded before the launch into stages, each holding
 // up to tma_pieces(mode, nsl) pieces.  In the sigma modes a piece is 16 columns of one term
 // with all slices of both operands: the slice products i + j < nsl come from one pair of
-// copies.  In the exact mode a term expands into its slice pairs (i, j), i + j < nsl, in the
+// copies, and a term's pieces stay in the ring until all its products have been issued (slice pair
+// by slice pair, each over all pieces).  A term with more pieces than the ring has slots
+// expands into 16 columns of one slice of each operand instead, pair by pair.  In the exact mode a term expands into its slice pairs (i, j), i + j < nsl, in the
 // order of the level l = i + j (A map amap + i, B map bmap + j), each into boxes of 64
 // columns along K, one to a stage.  CTA c of a launch of `grid` CTAs takes the tiles c,
 // c + grid, ... and issues the stages [cta_stage[c], cta_stage[c + 1]), stage s with the
@@ -84,29 +99,31 @@ __host__ __device__ constexpr int tm_seg_stages(int nsl) { return nsl == 1 ? 32 
 // A piece's coordinates are columns and rows in the exact mode, column groups (8) and row
 // groups (16) in the sigma modes.
 struct TmPiece {  // 32 bytes, so that any run of pieces is a bulk copy of 16-byte multiples
-  int amap, ax, ay, bmap, bx, by, pad0, pad1;
+  int amap, ax, ay, bmap, bx, by, as, bs;  // as, bs: first slice (sigma modes)
 };
 // word: the stage word the MMA issuer reads, the instruction descriptor (negation of A in
-// the exact mode) in the low half, in the high half the K=16 instructions (exact mode) or
-// the pieces (sigma modes) in bits 0-2, flags first of a segment (bit 3), end of a segment
-// (4), last stage of the tile (5), and in the sigma modes the negation of slot p in bit
-// 8 + p.  bytes: the stage's expected copy bytes.
+// the exact mode) in the low half.  High half, exact mode and one slice: the K=16 instructions
+// (exact) or pieces in bits 0-2, flags first of a segment (bit 3), end of a segment (4), last
+// stage of the tile (5), with one slice the negation of slot p in bit 8 + p.  Two or three slices:
+// the term's pieces in bits 0-7 (read from its first), a piece of single slices (bit 8),
+// negation (9), last term (or single-slice piece) of the tile (10).  bytes: the stage's expected
+// copy bytes.
 struct TmStage {
   uint64_t word;
   uint32_t bytes;
   int np;
 };
 struct TmListsDev {  // device copies, kept alive by the caller for the launches
-  int grid = 0;
+  int grid = 0, ctas = 1, slots = 0, slot_bytes = 0;
   const int* cta_stage = nullptr;
   const TmStage* stages = nullptr;
   const TmPiece* pieces = nullptr;
 };
-// host side of a launch's lists: its grid, every CTA's first stage (grid + 1 entries),
+// host side of a launch's lists: its grid, CTAs per SM and (two or three slices) ring, every CTA's first stage (grid + 1 entries),
 // the tiles in stage order (sorder) with their first stages (sfirst), and every term's
 // first piece within its tile (tpiece0; a term belongs to one tile)
 struct TmListPlan {
-  int grid = 0;
+  int grid = 0, ctas = 1, slots = 0, slot_bytes = 0;
   long total = 0;
   std::vector<int> cta_stage;
   std::vector<int> sorder;
@@ -128,19 +145,18 @@ __host__ __device__ inline uint32_t tm_idesc_bf16(int n, bool negA) {
 }
 
 // Host: the stage counts of a launch of `mode` (operands of nsl slices) over these tiles
-// (for the grid the launch will use, tma_grid(mode, tiles.size())); reduce mode: sets every
+// (for the grid the launch will use); reduce mode: sets every
 // tile's pad (its stages) and nseg.  Returns false if a term is malformed (k not a positive
 // multiple of 16), belongs to two tiles, or the lists would be too long.
 bool tma_plan_lists(int mode, int nsl, std::vector<TmTile>& tiles, const std::vector<TmTerm>& terms, TmListPlan& out);
 // Device: fills the copy lists (stages: total entries, pieces: total * tma_pieces(mode,
 // nsl)), one thread per stage, from the tiles and terms the plan was made from and the plan's
 // tpiece0, sorder and sfirst (all on the device).
-cudaError_t launch_fill_lists(int mode, int nsl, const TmTile* d_tiles, int ntiles, const TmTerm* d_terms,
+cudaError_t launch_fill_lists(int mode, int nsl, int slots, const TmTile* d_tiles, int ntiles, const TmTerm* d_terms,
                               const int* d_tpiece0, const int* d_sorder, const long* d_sfirst, long total,
                               TmStage* d_stages, TmPiece* d_pieces, cudaStream_t s);
-// CTAs of a launch over ntiles tiles (at most one per SM of the current device in the exact
-// mode, two in the sigma modes)
-int tma_grid(int mode, int ntiles);
+// CTAs of a launch over ntiles tiles (at most ctas per SM of the current device)
+int tma_grid(int ctas, int ntiles);
 int tma_pieces(int mode, int nsl);
 
 // maps: device array of encoded tensor maps (64-byte aligned).  nsl: BF16 slices of the
@@ -169,16 +185,14 @@ struct SplitJob {
   double scale;
 };
 cudaError_t launch_split_exact(const SplitJob* d_jobs, int njobs, int nsl, int* d_expo, cudaStream_t s);
-// maximum MMA width of a mode (256 for the BF16 store mode, 128 for the reduce mode)
-int tma_max_n(int mode);
-
 // Host: encode a 2D BF16 tensor map of the exact mode over a row-major matrix (rows x cols,
 // leading dimension ld elements, ld * 2 a multiple of 16 bytes, base 16-byte aligned), boxes
 // of 64 columns (128-byte swizzle) x box_rows rows.  Returns false on failure.
 bool encode_bf16_map(CUtensorMap* out, const void* base, uint64_t rows, uint64_t cols, uint64_t ld, uint32_t box_rows);
 // Host: encode the 4D map of a matrix in the layout of the sigma modes (rows a multiple of
 // 16, cols of 8, nsl slices), boxes of box_rows rows (a multiple of 16, at
-// most 256), TM_PIECE_COLS columns and all slices.  Returns false on failure.
-bool encode_slice_map(CUtensorMap* out, const void* base, uint64_t rows, uint64_t cols, int nsl, uint32_t box_rows);
+// most 256), TM_PIECE_COLS columns and box_slices slices.  Returns false on failure.
+bool encode_slice_map(CUtensorMap* out, const void* base, uint64_t rows, uint64_t cols, int nsl, uint32_t box_rows,
+                      int box_slices);
 
 }  // namespace gbdmrg
