@@ -129,8 +129,9 @@ gbdmrg_status gbdmrg_set_env_precision(gbdmrg_ctx* ctx, int32_t precision);
  * default).  EINVAL for precision outside -1..6 or max_iters < 1. */
 gbdmrg_status gbdmrg_set_refinement(gbdmrg_ctx* ctx, int32_t precision, int32_t max_iters);
 /* Work-list statistics of the prepared precision 4-6 H_eff.psi (zeros for other
- * precisions): out[0] stage-1 tiles, [1] stage-1 64-wide K steps, [2] stage-2
- * tiles, [3] stage-2 K steps, [4] stage-1 and [5] stage-2 tensor-core flops as
+ * precisions): out[0] stage-1 tiles, [1] stage-1 64-wide K steps over all slice
+ * products, [2] stage-2 tiles, [3] the same for stage 2 with the terms of a tile
+ * packed, [4] stage-1 and [5] stage-2 tensor-core flops as
  * executed (128-row tiles, blocks padded to 16), [6] bytes of the X
  * intermediates per chunk, [7] bytes of the stacked right operators, [8] chunks. */
 gbdmrg_status gbdmrg_plan_stats(gbdmrg_ctx* ctx, double* out);
@@ -172,14 +173,9 @@ void gbdmrg_batch_destroy(gbdmrg_batch* b);
  * Default 8.  Every value gives the same sigma up to the order of the FP32
  * additions.  EINVAL for a null context or a non-finite value. */
 gbdmrg_status gbdmrg_set_split(gbdmrg_ctx* ctx, double tiles_per_sm);
-/* Stage-1 decomposition of the tensor-core H_eff.psi for work lists built by
- * later gbdmrg_prepare / gbdmrg_plan calls.  stacked = 0 (default): one task per
- * (bond state, group of psi columns, output sector) with up to four site-block
- * terms.  stacked = 1: one task per (bond state, group) whose operand is the
- * W-contracted right operator over all four x four site blocks of the two groups,
- * built once per work list in BF16 slices with absent blocks zero (fewer, deeper
- * tiles; more memory and more padded products).  Same sigma up to the order of
- * the FP32 additions.  EINVAL for a null context. */
+/* Accepted and without effect: every tensor-core H_eff.psi runs stage 1 over
+ * stacked right operators that hold only the site blocks present.  EINVAL for a
+ * null context. */
 gbdmrg_status gbdmrg_set_stage1_stacked(gbdmrg_ctx* ctx, int32_t stacked);
 /* W-contracted operator sums on the tensor cores.  on != 0: a blocking sum of
  * Eq. prenormrule type with at least min_terms terms in total, built for later
@@ -207,8 +203,8 @@ gbdmrg_status gbdmrg_get_plan_params(gbdmrg_ctx* ctx, double* tiles_per_sm, int3
  * their work lists rebuilt with it (a batch created earlier must be created
  * again).  splits == NULL: {32, 8, 2, 0.5, 0.125, 0.03125, 0}; budgets_mb ==
  * NULL: the current budget of ctxs[0].  EINVAL for empty lists, non-positive
- * budgets or reps; ESTATE if a context is not prepared in a tensor-core
- * precision.  Errors are reported through gbdmrg_last_error(ctxs[0]); after an
+ * budgets or reps; ESTATE if a context is not prepared in precision 1,
+ * 2 or 3.  Errors are reported through gbdmrg_last_error(ctxs[0]); after an
  * error during timing the contexts keep their previous parameters and must be
  * prepared again. */
 gbdmrg_status gbdmrg_autotune(int32_t n, gbdmrg_ctx* const* ctxs, int32_t reps, const double* splits,

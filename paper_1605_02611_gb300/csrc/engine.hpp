@@ -163,11 +163,6 @@ struct GemmBuilder {
   void clear() { tiles.clear(); tasks.clear(); terms.clear(); flops = 0; }
 };
 
-struct MixedPlan;
-void mixed_plan_free(MixedPlan* p);
-struct MixedDeleter {
-  void operator()(MixedPlan* p) const { mixed_plan_free(p); }
-};
 struct TmaPlan;
 void tma_plan_free(TmaPlan* p);
 struct TmaDeleter {
@@ -175,16 +170,15 @@ struct TmaDeleter {
 };
 
 // Work lists of H_eff.psi for one two-site problem: FP64 grouped GEMMs, or
-// (mx set) the tensor-core mixed-precision plan of engine_mixed.cu.
+// (tm set) the tensor-core plan of engine_mixed.cu.
 struct SigmaPlan {
   PsiLayout psi;
   DArr<double> in, out, X;
   std::vector<GemmPlan> stage1, stage2;
-  std::unique_ptr<MixedPlan, MixedDeleter> mx;
-  // tensor-core plan with TMA-staged operands (precisions 4-6)
+  // tensor-core plan with TMA-staged operands (precisions 1-6)
   std::unique_ptr<TmaPlan, TmaDeleter> tm;
   double flops = 0;
-  bool tensor() const { return mx != nullptr || tm != nullptr; }
+  bool tensor() const { return tm != nullptr; }
 };
 
 struct Context;
@@ -249,10 +243,6 @@ struct Context {
   // is cut into parts of about (k-steps of the whole stage) / (split_tps x 152), i.e.
   // about split_tps tiles per SM; <= 0: no split
   double split_tps = 8.0;
-  // stage 1 of the tensor-core sigma with stacked right operands: one task per
-  // (bond state, group) whose operand is the W-contracted right operator over all
-  // four x four site blocks of the two groups (absent blocks zero)
-  bool stage1_stacked = false;
   // blocking sums with at least tc_combo_min_terms terms that feed only the
   // tensor-core sigma and the H_eff diagonal are formed on the tensor cores
   // (three BF16 slices, FP32 accumulation) instead of the FP64 units
@@ -260,9 +250,8 @@ struct Context {
   long tc_combo_min_terms = 100000;
   // 0: FP64 grouped GEMMs; 1: tensor cores, one BF16 pass; 2: tensor cores,
   // three BF16 slices (six products, about FP32 accuracy); 3: two BF16 slices
-  // (three products); 4, 5, 6: tensor cores on the TMA-staged plan (stage 1 as
-  // one dense GEMM per group over the stacked right operators) with one BF16
-  // pass, three slices and two slices
+  // (three products); 4, 5, 6: the same three with the X intermediates in the
+  // budget of tma_budget_mb instead of chunk_budget_mb, and not for batches
   int precision = 0;
   // Davidson refinement of the tensor-core steps: after the solve with the
   // operator of `precision`, its Ritz vector starts a solve with the operator of
@@ -316,9 +305,6 @@ void env_update_right(Context& c, Tilde& rt, const SiteT& B, int site, Env& out)
 
 void build_sigma_plan(Context& c, Tilde& lt, Tilde& rt, int k, SigmaPlan& plan);
 void run_sigma(Context& c, SigmaPlan& plan, const double* x, double* y);
-void build_mixed_plan(Context& c, Tilde& lt, Tilde& rt, int k, SigmaPlan& plan, int nslices);
-void run_mixed_sigma(Context& c, SigmaPlan& plan, const double* x, double* y);
-int mixed_error(Context& c, SigmaPlan& plan);
 void build_tma_plan(Context& c, Tilde& lt, Tilde& rt, int k, SigmaPlan& plan, int nslices);
 void run_tma_sigma(Context& c, SigmaPlan& plan, const double* x, double* y);
 // non-zero if a tensor-core launch of the plan reported a bounded wait that ran out

@@ -1,8 +1,8 @@
-// Mixed-precision sigma vector on the tensor cores (tcgen05, BF16 operands,
-// FP32 accumulation).  Same two-stage contraction as the FP64 plan:
+// Sigma vector and environment updates on the tensor cores (tcgen05, BF16 operands, FP32
+// accumulation).  The sigma is the same two-stage contraction as the FP64 plan:
 //   stage 1: X_beta^T[qr, ql'] = sum_{n2'} Rt_beta^{n2 n2'}[qr, qr'] psi[ql', n1', n2', qr']^T
 //   stage 2: sigma[ql, qr]   += sum_{beta, n1'} Lt_beta^{n1 n1'}[ql, ql'] X_beta^T[qr, ql']^T
-// with every operand stored as 1 or 3 BF16 slices (x = s0 + s1 + s2, each the
+// with every operand stored as 1 to 3 BF16 slices (x = s0 + s1 + s2, each the
 // BF16 rounding of the remainder).  With 3 slices the products s_i t_j with
 // i + j <= 2 are summed (6 tensor-core products), which carries the operands
 // to about 2^-24 relative accuracy; with 1 slice it is a single BF16 pass.
@@ -240,47 +240,6 @@ struct TcBuilder {
 
 }  // namespace
 
-struct TcPlan {
-  DArr<TcTile> tiles;
-  DArr<TcTask> tasks;
-  DArr<TcTerm> terms;
-  int ntiles = 0;
-  // host copies, kept when the plan may be fused into a batched launch
-  std::vector<TcTile> htiles;
-  std::vector<TcTask> htasks;
-  std::vector<TcTerm> hterms;
-  // regions of the shared X buffer to clear before this launch (stage 1 of a
-  // multi-chunk plan: blocks of X that no term of this chunk writes)
-  DArr<ZeroJob> zeros;
-  std::vector<ZeroJob> hzeros;
-  int nzeros = 0;
-  long zmax = 0;
-};
-
-void run_zeros(const TcPlan& tp, cudaStream_t s) {
-  if (tp.nzeros) launch_zero(tp.zeros.p, tp.nzeros, tp.zmax, s);
-}
-
-struct MixedPlan {
-  int nsl = 1;
-  DArr<__nv_bfloat16> psi_b, X_b, mirror;
-  DArr<float> sig_f;
-  DArr<ConvJob> psi_jobs;
-  DArr<UnconvJob> sig_jobs;
-  std::vector<ConvJob> h_psi_jobs;
-  std::vector<UnconvJob> h_sig_jobs;
-  int n_psi_jobs = 0, n_sig_jobs = 0;
-  long psi_maxel = 0, sig_maxel = 0;
-  long sig_total = 0;
-  std::vector<TcPlan> stage1, stage2;
-  DArr<int> err;
-  // stacked right operands of stage 1 (stage1_stacked): nsl slices of rs_total elements
-  DArr<__nv_bfloat16> rstack;
-  long rs_total = 0;
-};
-
-void mixed_plan_free(MixedPlan* p) { delete p; }
-
 // padded BF16 layout of one operator class: per-block offsets (elements)
 static std::vector<long> padded_offsets(const OpLayout& L, long* total) {
   std::vector<long> off(L.blocks.size());
@@ -291,507 +250,6 @@ static std::vector<long> padded_offsets(const OpLayout& L, long* total) {
   }
   *total = t;
   return off;
-}
-
-namespace {
-
-// BF16 mirror of the operators referenced by a W-contracted side
-struct MirrorRef {
-  long off = -1;      // element offset of slice 0 in the mirror buffer
-  long stride = 0;    // slice stride
-  bool neg = false;
-  const std::vector<long>* boff = nullptr;  // padded block offsets of its class
-};
-
-}  // namespace
-
-void build_mixed_plan(Context& c, Tilde& lt, Tilde& rt, int k, SigmaPlan& plan, int nsl) {
-  const auto& mid = c.mpo.bonds[k + 1];
-  Env& Lenv = *lt.env;
-  Env& Renv = *rt.env;
-  const Bond& Lb = Lenv.bond;
-  const Bond& Rb = Renv.bond;
-  auto* mx = new MixedPlan();
-  plan.mx.reset(mx);
-  mx->nsl = nsl;
-  PsiLayout& P = plan.psi;
-  const int nL = Lb.nsec();
-  // ---- operator mirrors (one per distinct referenced operator and scale)
-  std::vector<std::vector<long>> loff(Lenv.cls.size()), roff(Renv.cls.size());
-  std::vector<long> lsz(Lenv.cls.size()), rsz(Renv.cls.size());
-  for (size_t i = 0; i < Lenv.cls.size(); ++i) loff[i] = padded_offsets(Lenv.cls[i], &lsz[i]);
-  for (size_t i = 0; i < Renv.cls.size(); ++i) roff[i] = padded_offsets(Renv.cls[i], &rsz[i]);
-  struct MirrorKeyHash {
-    size_t operator()(const std::pair<const double*, double>& k) const {
-      uint64_t b;
-      std::memcpy(&b, &k.second, sizeof b);
-      return std::hash<uint64_t>()((uint64_t)(uintptr_t)k.first * 0x9e3779b97f4a7c15ULL ^ b);
-    }
-  };
-  std::unordered_map<std::pair<const double*, double>, MirrorRef, MirrorKeyHash> mref;
-  long mtot = 0;
-  // mirrors in the order of their first reference: (operator, scale, class, side, offset)
-  struct NewMirror {
-    const double* p;
-    double scale;
-    int cls;
-    bool left;
-    long off;
-  };
-  std::vector<NewMirror> created;
-  std::vector<std::array<MirrorRef, 16>> lm(mid.size()), rm(mid.size());
-  auto mirror_of = [&](const TRef& r, bool left) -> MirrorRef {
-    const double a = std::fabs(r.coef);
-    const double scale = a == 1.0 ? 1.0 : r.coef;
-    auto key = std::make_pair(r.p, scale);
-    auto it = mref.find(key);
-    MirrorRef m;
-    if (it == mref.end()) {
-      const long sz = left ? lsz[r.cls] : rsz[r.cls];
-      m.off = mtot;
-      m.stride = sz;
-      m.boff = left ? &loff[r.cls] : &roff[r.cls];
-      mtot += sz * nsl;
-      mref.emplace(key, m);
-      created.push_back({r.p, scale, r.cls, left, m.off});
-    } else m = it->second;
-    m.neg = (a == 1.0 && r.coef < 0);
-    return m;
-  };
-  const bool stacked = c.stage1_stacked;
-  for (size_t beta = 0; beta < mid.size(); ++beta)
-    for (int nn = 0; nn < 16; ++nn) {
-      if (lt.ref[beta][nn].p) lm[beta][nn] = mirror_of(lt.ref[beta][nn], true);
-      if (rt.ref[beta][nn].p && !stacked) rm[beta][nn] = mirror_of(rt.ref[beta][nn], false);
-    }
-  // one conversion job per block of every mirror, filled on host threads (each mirror's
-  // jobs are contiguous, in the order the mirrors were first referenced)
-  mx->mirror.alloc(std::max<long>(mtot, 8), c.stream);
-  std::vector<size_t> jstart(created.size() + 1, 0);
-  for (size_t i = 0; i < created.size(); ++i)
-    jstart[i + 1] = jstart[i] + (created[i].left ? Lenv.cls[created[i].cls] : Renv.cls[created[i].cls]).blocks.size();
-  std::vector<ConvJob> conv(jstart.back());
-  long maxel = 0;
-  {
-    std::mutex mu;
-    auto fill = [&](size_t lo, size_t hi) {
-      long mymax = 0;
-      for (size_t i = lo; i < hi; ++i) {
-        const NewMirror& nm = created[i];
-        const OpLayout& L = nm.left ? Lenv.cls[nm.cls] : Renv.cls[nm.cls];
-        const long sz = nm.left ? lsz[nm.cls] : rsz[nm.cls];
-        const std::vector<long>& boff = nm.left ? loff[nm.cls] : roff[nm.cls];
-        for (size_t b = 0; b < L.blocks.size(); ++b) {
-          const Block& B = L.blocks[b];
-          conv[jstart[i] + b] = ConvJob{nm.p + B.off, mx->mirror.p + nm.off + boff[b], sz, B.rows, B.cols, B.cols,
-                                        pad8(B.cols), nsl, nm.scale, pad8(B.cols)};
-          mymax = std::max<long>(mymax, (long)B.rows * pad8(B.cols));
-        }
-      }
-      std::lock_guard<std::mutex> lk(mu);
-      maxel = std::max(maxel, mymax);
-    };
-    const size_t nt = std::max<size_t>(1, std::min<size_t>({std::max(1u, std::thread::hardware_concurrency()), 16,
-                                                             created.size() / 256 + 1}));
-    std::vector<std::thread> pool;
-    for (size_t t = 1; t < nt; ++t) pool.emplace_back(fill, created.size() * t / nt, created.size() * (t + 1) / nt);
-    fill(0, created.size() / nt);
-    for (auto& th : pool) th.join();
-  }
-  {
-    DArr<ConvJob> dj;
-    dj.upload(conv, c.stream);
-    if (!conv.empty()) launch_conv(dj, (int)conv.size(), maxel, c.stream);
-    cuda_check(cudaStreamSynchronize(c.stream), "sync");
-  }
-  // ---- group layout.  psi reshaped to (l n1) x (n2 r) is block diagonal in the
-  // quantum number g of the cut; per group the row blocks (ql, n1) and column
-  // blocks (n2, qr) are stacked (each padded to a multiple of 8) into one matrix
-  // Psi_g (R_g x C_g).  X_beta^T and sigma^T use the same stacked blocks, so the
-  // tensor-core tiles span a whole group instead of one small block.
-  std::map<std::pair<int, int>, int> gidx;
-  std::vector<std::pair<int, int>> gq;
-  std::vector<std::vector<std::array<int, 3>>> grow, gcol;  // (ql, n1, off), (n2, qr, off)
-  std::vector<int> gR, gC;
-  {
-    std::map<std::pair<int, int>, std::pair<std::vector<std::array<int, 3>>, std::vector<std::array<int, 3>>>> tmp;
-    for (int ql = 0; ql < nL; ++ql)
-      for (int n1 = 0; n1 < 4; ++n1) tmp[{Lb.qa[ql] + LQA[n1], Lb.qb[ql] + LQB[n1]}].first.push_back({ql, n1, 0});
-    for (int qr = 0; qr < Rb.nsec(); ++qr)
-      for (int n2 = 0; n2 < 4; ++n2) tmp[{Rb.qa[qr] - LQA[n2], Rb.qb[qr] - LQB[n2]}].second.push_back({n2, qr, 0});
-    for (auto& kv : tmp) {
-      if (kv.second.first.empty() || kv.second.second.empty()) continue;
-      gidx[kv.first] = (int)gq.size();
-      gq.push_back(kv.first);
-      auto rows = kv.second.first, cols = kv.second.second;
-      int R = 0, C = 0;
-      for (auto& r : rows) { r[2] = R; R += pad8(Lb.dim[r[0]]); }
-      for (auto& cc : cols) { cc[2] = C; C += pad8(Rb.dim[cc[1]]); }
-      grow.push_back(rows);
-      gcol.push_back(cols);
-      gR.push_back(R);
-      gC.push_back(C);
-    }
-  }
-  const int ng = (int)gq.size();
-  // (ql, n1) -> (group, row offset); (n2, qr) -> (group, col offset)
-  std::vector<std::array<int, 2>> rpos((size_t)nL * 4, {-1, 0}), cpos((size_t)Rb.nsec() * 4, {-1, 0});
-  for (int g = 0; g < ng; ++g) {
-    for (auto& r : grow[g]) rpos[r[0] * 4 + r[1]] = {g, r[2]};
-    for (auto& cc : gcol[g]) cpos[cc[1] * 4 + cc[0]] = {g, cc[2]};
-  }
-  auto group_of = [&](int a, int b) {
-    auto it = gidx.find({a, b});
-    return it == gidx.end() ? -1 : it->second;
-  };
-  std::vector<long> goff(ng), sgoff(ng);
-  long ptot = 0, stot = 0;
-  for (int g = 0; g < ng; ++g) {
-    goff[g] = ptot;
-    ptot += (long)gR[g] * gC[g];
-    sgoff[g] = stot;
-    stot += (long)gC[g] * gR[g];
-  }
-  mx->psi_b.alloc(std::max<long>(ptot * nsl, 8), c.stream);
-  cuda_check(cudaMemsetAsync(mx->psi_b.p, 0, mx->psi_b.n * sizeof(__nv_bfloat16), c.stream), "memset");
-  mx->sig_total = std::max<long>(stot, 1);
-  mx->sig_f.alloc(mx->sig_total, c.stream);
-  {
-    std::vector<ConvJob> pj;
-    std::vector<UnconvJob> sj;
-    for (size_t b = 0; b < P.blocks.size(); ++b) {
-      const Block& B = P.blocks[b];
-      const int n1 = P.b1[b], n2 = P.b2[b];
-      const auto rp = rpos[B.rs * 4 + n1];
-      const auto cp = cpos[B.cs * 4 + n2];
-      if (rp[0] < 0 || rp[0] != cp[0]) throw Error(ST_ECUDA, "internal: psi block outside its group");
-      const int g = rp[0];
-      pj.push_back({plan.in.p + B.off, mx->psi_b.p + goff[g] + (long)rp[1] * gC[g] + cp[1], ptot, B.rows, B.cols,
-                    B.cols, gC[g], nsl, 1.0, pad8(B.cols)});
-      mx->psi_maxel = std::max<long>(mx->psi_maxel, (long)B.rows * pad8(B.cols));
-      sj.push_back({mx->sig_f.p + sgoff[g] + (long)cp[1] * gR[g] + rp[1], plan.out.p + B.off, B.rows, B.cols, gR[g]});
-      mx->sig_maxel = std::max<long>(mx->sig_maxel, (long)B.rows * B.cols);
-    }
-    mx->psi_jobs.upload(pj, c.stream);
-    mx->n_psi_jobs = (int)pj.size();
-    mx->sig_jobs.upload(sj, c.stream);
-    mx->n_sig_jobs = (int)sj.size();
-    mx->h_psi_jobs = pj;
-    mx->h_sig_jobs = sj;
-  }
-  mx->err.alloc(1, c.stream);
-  cuda_check(cudaMemsetAsync(mx->err.p, 0, sizeof(int), c.stream), "memset");
-  // ---- stacked right operands (stage1_stacked): for every (beta, g') with g = g' + dQ_beta
-  // the matrix Rt_beta[(n2, qr) blocks of g, (n2', qr') blocks of g'] (C_g x C_g', the
-  // column layout of Psi_g'), absent site blocks and padding zero, scaled by the W
-  // coefficient of each block
-  std::vector<long> soff;
-  if (stacked) {
-    soff.assign(mid.size() * (size_t)ng, -1);
-    std::vector<ConvJob> sj;
-    long stot = 0, smax = 0;
-    for (size_t beta = 0; beta < mid.size(); ++beta)
-      for (int gp = 0; gp < ng; ++gp) {
-        const int g = group_of(gq[gp].first + mid[beta].dna, gq[gp].second + mid[beta].dnb);
-        if (g < 0) continue;
-        const size_t j0 = sj.size();
-        for (const auto& cb : gcol[g]) {
-          const int n2 = cb[0], qr = cb[1];
-          for (int n2p = 0; n2p < 4; ++n2p) {
-            const TRef& r = rt.ref[beta][n2 * 4 + n2p];
-            if (!r.p) continue;
-            const int qrp = Rb.find(gq[gp].first + LQA[n2p], gq[gp].second + LQB[n2p]);
-            if (qrp < 0) continue;
-            const auto cpp = cpos[qrp * 4 + n2p];
-            if (cpp[0] != gp) continue;
-            const OpLayout& Lay = Renv.cls[r.cls];
-            const int bl = Lay.blk_of_col[qrp];
-            if (bl < 0 || Lay.blocks[bl].rs != qr) continue;
-            const Block& B = Lay.blocks[bl];
-            // dst holds the element offset until the buffer exists
-            sj.push_back({r.p + B.off, (__nv_bfloat16*)(intptr_t)(stot + (long)cb[2] * gC[gp] + cpp[1]), 0, B.rows,
-                          B.cols, B.cols, gC[gp], nsl, r.coef, pad8(B.cols)});
-            smax = std::max<long>(smax, (long)B.rows * pad8(B.cols));
-          }
-        }
-        if (sj.size() > j0) {
-          soff[beta * ng + gp] = stot;
-          stot += (long)gC[g] * gC[gp];
-        }
-      }
-    mx->rs_total = std::max<long>(stot, 8);
-    mx->rstack.alloc((size_t)mx->rs_total * nsl, c.stream);
-    cuda_check(cudaMemsetAsync(mx->rstack.p, 0, mx->rstack.n * sizeof(__nv_bfloat16), c.stream), "memset");
-    for (auto& j : sj) {
-      j.dst = mx->rstack.p + (intptr_t)j.dst;
-      j.slice_stride = mx->rs_total;
-    }
-    DArr<ConvJob> dj;
-    dj.upload(sj, c.stream);
-    if (!sj.empty()) launch_conv(dj, (int)sj.size(), smax, c.stream);
-    cuda_check(cudaStreamSynchronize(c.stream), "sync");
-  }
-  // ---- X_beta^T per (beta, g'): C_g x R_g' with g = g' + dQ_beta; chunking over beta
-  std::vector<size_t> xsz(mid.size(), 0);
-  for (size_t beta = 0; beta < mid.size(); ++beta)
-    for (int gp = 0; gp < ng; ++gp) {
-      int g = group_of(gq[gp].first + mid[beta].dna, gq[gp].second + mid[beta].dnb);
-      if (g >= 0) xsz[beta] += (size_t)gC[g] * gR[gp];
-    }
-  const size_t budget = (size_t)c.chunk_budget_mb * (1u << 20) / (2 * nsl);
-  std::vector<std::pair<size_t, size_t>> chunks;
-  size_t maxchunk = 0;
-  {
-    size_t b0 = 0;
-    while (b0 < mid.size()) {
-      size_t b1 = b0, tot = 0;
-      while (b1 < mid.size() && (b1 == b0 || tot + xsz[b1] <= budget)) tot += xsz[b1++];
-      chunks.push_back({b0, b1});
-      maxchunk = std::max(maxchunk, tot);
-      b0 = b1;
-    }
-  }
-  mx->X_b.alloc(std::max<size_t>(maxchunk * nsl, 8), c.stream);
-  cuda_check(cudaMemsetAsync(mx->X_b.p, 0, mx->X_b.n * sizeof(__nv_bfloat16), c.stream), "memset");
-  const long xstride = (long)maxchunk;
-  const __nv_bfloat16* mir = mx->mirror.p;
-  const bool multi = chunks.size() > 1;
-  // the chunks' work lists are independent: built on host threads, uploaded in order
-  struct ChunkLists {
-    TcBuilder g1, g2;
-    std::vector<ZeroJob> zj;
-  };
-  auto build_chunk = [&](std::pair<size_t, size_t> ch, ChunkLists& out) {
-    TcBuilder& g1 = out.g1;
-    TcBuilder& g2 = out.g2;
-    std::vector<ZeroJob>& zj = out.zj;
-    size_t xoff = 0;
-    // X^T offsets of this chunk: [beta - b0][g'] (-1 if absent or never written)
-    std::vector<std::vector<long>> xpos(ch.second - ch.first, std::vector<long>(ng, -1));
-    for (size_t beta = ch.first; beta < ch.second; ++beta) {
-      auto& xp = xpos[beta - ch.first];
-      for (int gp = 0; gp < ng; ++gp) {
-        const int g = group_of(gq[gp].first + mid[beta].dna, gq[gp].second + mid[beta].dnb);
-        if (g < 0) continue;
-        const long base = (long)xoff;
-        if (stacked) {
-          // one task: X_beta^T (C_g x R_g') = (Psi_g' Rt_beta^T)^T over the whole group
-          const long so = soff[beta * ng + gp];
-          if (so < 0) continue;
-          TcTask t{};
-          t.Cb = mx->X_b.p + base;
-          t.slice_stride = xstride;
-          t.ldcb = gR[gp];
-          t.m = gR[gp];
-          t.n = gC[g];
-          t.nslices = nsl;
-          t.trans = 1;
-          g1.begin(t);
-          g1.term(mx->psi_b.p + goff[gp], ptot, gC[gp], mx->rstack.p + so, mx->rs_total, gC[gp], gC[gp], false, nsl);
-          g1.end();
-          xp[gp] = base;
-          xoff += (size_t)gC[g] * gR[gp];
-          continue;
-        }
-        bool any = false;
-        std::vector<ZeroJob> empty_cb;  // column blocks of X^T without a term
-        // stage 1: X_beta[rows of g', (n2, qr) block of g] = sum_{n2'} Psi_g'[:, (n2', qr')] Rt^{n2 n2'}[qr, qr']^T,
-        // stored transposed into X^T (rows (n2, qr) of g, columns = rows of g')
-        for (const auto& cb : gcol[g]) {
-          const int n2 = cb[0], qr = cb[1];
-          TcTask t{};
-          t.Cb = mx->X_b.p + base + (long)cb[2] * gR[gp];
-          t.slice_stride = xstride;
-          t.ldcb = gR[gp];
-          t.m = gR[gp];
-          t.n = Rb.dim[qr];
-          t.nslices = nsl;
-          t.trans = 1;
-          g1.begin(t);
-          for (int n2p = 0; n2p < 4; ++n2p) {
-            const TRef& r = rt.ref[beta][n2 * 4 + n2p];
-            if (!r.p) continue;
-            const int qrp = Rb.find(gq[gp].first + LQA[n2p], gq[gp].second + LQB[n2p]);
-            if (qrp < 0) continue;
-            const auto cpp = cpos[qrp * 4 + n2p];
-            if (cpp[0] != gp) continue;
-            const OpLayout& Lay = Renv.cls[r.cls];
-            const int bl = Lay.blk_of_col[qrp];
-            if (bl < 0 || Lay.blocks[bl].rs != qr) continue;
-            const MirrorRef& mr = rm[beta][n2 * 4 + n2p];
-            const int kk = Rb.dim[qrp];
-            g1.term(mx->psi_b.p + goff[gp] + cpp[1], ptot, gC[gp], mir + mr.off + (*mr.boff)[bl], mr.stride, pad8(kk),
-                    kk, mr.neg, nsl);
-          }
-          if (g1.end())
-            any = true;
-          else
-            empty_cb.push_back({mx->X_b.p + base + (long)cb[2] * gR[gp], (long)Rb.dim[qr] * gR[gp], xstride, nsl});
-        }
-        if (any) {
-          xp[gp] = base;
-          xoff += (size_t)gC[g] * gR[gp];
-          // with several chunks the X buffer is shared, so rows that stay exactly zero
-          // here may hold another chunk's values: clear them (one chunk: zero from the start)
-          if (multi) zj.insert(zj.end(), empty_cb.begin(), empty_cb.end());
-        }
-      }
-    }
-    // stage 2: sigma^T_g[:, (ql, n1) block] += sum_{beta, n1'} X_beta^T[:, (ql', n1')] Lt^{n1 n1'}[ql, ql']^T.
-    // Long term lists are split into parts that accumulate atomically (split-K), so
-    // that there are enough tiles for every resident CTA.
-    TcBuilder g2all;
-    for (int g = 0; g < ng; ++g)
-      for (const auto& rb : grow[g]) {
-        const int ql = rb[0], n1 = rb[1];
-        TcTask t{};
-        t.C = mx->sig_f.p + sgoff[g] + rb[2];
-        t.ldc = gR[g];
-        t.m = gC[g];
-        t.n = Lb.dim[ql];
-        t.beta = 2;
-        g2all.begin(t);
-        for (size_t beta = ch.first; beta < ch.second; ++beta) {
-          const int gp = group_of(gq[g].first - mid[beta].dna, gq[g].second - mid[beta].dnb);
-          if (gp < 0) continue;
-          const long xo = xpos[beta - ch.first][gp];
-          if (xo < 0) continue;
-          for (int n1p = 0; n1p < 4; ++n1p) {
-            const TRef& r = lt.ref[beta][n1 * 4 + n1p];
-            if (!r.p) continue;
-            const OpLayout& Lay = Lenv.cls[r.cls];
-            const int qlp = Lb.find(Lb.qa[ql] - Lay.da, Lb.qb[ql] - Lay.db);
-            if (qlp < 0) continue;
-            const int bl = Lay.blk_of_col[qlp];
-            if (bl < 0 || Lay.blocks[bl].rs != ql) continue;
-            const auto rpp = rpos[qlp * 4 + n1p];
-            if (rpp[0] != gp) continue;
-            const MirrorRef& mr = lm[beta][n1 * 4 + n1p];
-            const int kk = Lb.dim[qlp];
-            g2all.term(mx->X_b.p + xo + rpp[1], xstride, gR[gp], mir + mr.off + (*mr.boff)[bl], mr.stride, pad8(kk),
-                       kk, mr.neg, nsl);
-          }
-        }
-        g2all.end();
-      }
-    {
-      // k-steps per task and the split that gives about split_tps tiles per SM
-      long total = 0;
-      std::vector<long> w(g2all.tasks.size(), 0);
-      for (size_t i = 0; i < g2all.tasks.size(); ++i) {
-        for (int t = g2all.tasks[i].t0; t < g2all.tasks[i].t1; ++t) w[i] += (g2all.terms[t].k + 63) / 64;
-        total += w[i] * ((g2all.tasks[i].m + 127) / 128);
-      }
-      const long target = c.split_tps > 0
-                              ? std::max<long>(1, total / std::max<long>(1, std::lround(c.split_tps * 152)))
-                              : std::numeric_limits<long>::max();
-      for (size_t i = 0; i < g2all.tasks.size(); ++i) {
-        const TcTask& tk = g2all.tasks[i];
-        long acc = 0;
-        int t0 = tk.t0;
-        for (int t = tk.t0; t < tk.t1; ++t) {
-          acc += (g2all.terms[t].k + 63) / 64;
-          if (acc >= target || t + 1 == tk.t1) {
-            TcTask part = tk;
-            g2.begin(part);
-            for (int u = t0; u <= t; ++u) g2.terms.push_back(g2all.terms[u]);
-            g2.tasks.back().t1 = (int)g2.terms.size();
-            g2.end();
-            t0 = t + 1;
-            acc = 0;
-          }
-        }
-      }
-    }
-    // longest tiles first (static round-robin over persistent CTAs)
-    auto order = [&](TcBuilder& g) {
-      std::vector<long> w(g.tasks.size(), 0);
-      for (size_t i = 0; i < g.tasks.size(); ++i)
-        for (int t = g.tasks[i].t0; t < g.tasks[i].t1; ++t) w[i] += (g.terms[t].k + 63) / 64;
-      std::stable_sort(g.tiles.begin(), g.tiles.end(),
-                       [&](const TcTile& a, const TcTile& b) { return w[a.task] > w[b.task]; });
-    };
-    order(g2);
-  };
-  std::vector<ChunkLists> lists(chunks.size());
-  {
-    const unsigned hw = std::max(1u, std::thread::hardware_concurrency());
-    const size_t nth = std::min<size_t>(chunks.size(), std::min(hw, 16u));
-    std::atomic<size_t> next{0};
-    std::exception_ptr fail;
-    std::mutex fail_mu;
-    auto worker = [&] {
-      for (size_t i; (i = next.fetch_add(1)) < chunks.size();) {
-        try {
-          build_chunk(chunks[i], lists[i]);
-        } catch (...) {
-          std::lock_guard<std::mutex> lk(fail_mu);
-          if (!fail) fail = std::current_exception();
-        }
-      }
-    };
-    std::vector<std::thread> pool;
-    for (size_t t = 1; t < nth; ++t) pool.emplace_back(worker);
-    worker();
-    for (auto& th : pool) th.join();
-    if (fail) std::rethrow_exception(fail);
-  }
-  for (ChunkLists& cl : lists) {
-    TcBuilder& g1 = cl.g1;
-    TcBuilder& g2 = cl.g2;
-    std::vector<ZeroJob>& zj = cl.zj;
-    auto keep = [&](TcPlan& tp, TcBuilder& g) {
-      tp.tiles.upload(g.tiles, c.stream);
-      tp.tasks.upload(g.tasks, c.stream);
-      tp.terms.upload(g.terms, c.stream);
-      tp.ntiles = (int)g.tiles.size();
-      cuda_check(cudaStreamSynchronize(c.stream), "sync");
-      if (c.keep_host_plans) {
-        tp.htiles.swap(g.tiles);
-        tp.htasks.swap(g.tasks);
-        tp.hterms.swap(g.terms);
-      }
-    };
-    mx->stage1.emplace_back();
-    keep(mx->stage1.back(), g1);
-    {
-      TcPlan& tp = mx->stage1.back();
-      tp.nzeros = (int)zj.size();
-      for (const ZeroJob& z : zj) tp.zmax = std::max(tp.zmax, z.n);
-      tp.zeros.upload(zj, c.stream);
-      tp.hzeros = zj;
-      cuda_check(cudaStreamSynchronize(c.stream), "sync");
-    }
-    mx->stage2.emplace_back();
-    keep(mx->stage2.back(), g2);
-  }
-  plan.flops = count_sigma_flops(c.mpo, k, Lb, Rb);
-}
-
-void run_mixed_sigma(Context& c, SigmaPlan& plan, const double* x, double* y) {
-  MixedPlan& mx = *plan.mx;
-  const size_t n = plan.psi.nnz;
-  if (x != plan.in.p) cuda_check(cudaMemcpyAsync(plan.in.p, x, n * sizeof(double), cudaMemcpyDeviceToDevice, c.stream), "d2d");
-  if (mx.n_psi_jobs) launch_conv(mx.psi_jobs, mx.n_psi_jobs, mx.psi_maxel, c.stream);
-  cuda_check(cudaMemsetAsync(mx.sig_f.p, 0, mx.sig_total * sizeof(float), c.stream), "memset");
-  for (size_t i = 0; i < mx.stage1.size(); ++i) {
-    auto& s1 = mx.stage1[i];
-    auto& s2 = mx.stage2[i];
-    run_zeros(s1, c.stream);
-    cuda_check(launch_gemm_bf16_tc(s1.tiles.p, s1.ntiles, s1.tasks.p, s1.terms.p, mx.err.p, c.stream, mx.nsl),
-               "tc stage 1");
-    cuda_check(launch_gemm_bf16_tc(s2.tiles.p, s2.ntiles, s2.tasks.p, s2.terms.p, mx.err.p, c.stream, mx.nsl),
-               "tc stage 2");
-  }
-  if (mx.n_sig_jobs) launch_unconv(mx.sig_jobs.p, mx.n_sig_jobs, mx.sig_maxel, c.stream);
-  if (y != plan.out.p) cuda_check(cudaMemcpyAsync(y, plan.out.p, n * sizeof(double), cudaMemcpyDeviceToDevice, c.stream), "d2d");
-}
-
-int mixed_error(Context& c, SigmaPlan& plan) {
-  int h = 0;
-  cuda_check(cudaMemcpyAsync(&h, plan.mx->err.p, sizeof(int), cudaMemcpyDeviceToHost, c.stream), "d2h");
-  cuda_check(cudaStreamSynchronize(c.stream), "sync");
-  return h;
 }
 
 // ---------------------------------------------------------------- TMA-staged single-pass plan
@@ -812,6 +270,7 @@ int mixed_error(Context& c, SigmaPlan& plan) {
 // Every block is padded to 16 rows and columns with zeros, so a K step of 16 never
 // mixes two blocks and padding contributes exact zeros.
 struct TmaPlan {
+  int precision = 4;  // the context's precision when the plan was built
   int nsl = 1;  // BF16 slices per operand (1: one pass; 2 or 3: slice products i + j < nsl)
   DArr<__nv_bfloat16> psi_b, a1, xt, lmir;
   DArr<float> sig_t;
@@ -865,8 +324,17 @@ struct TmaPlan {
     DArr<ZeroJob> z;
     int nz = 0;
     long zmax = 0;
+    // host copies, kept when the plan may be fused into a batched launch
+    std::vector<TmTile> ht1, ht2;
+    std::vector<TmTerm> hm1, hm2;
+    std::vector<ZeroJob> hz;
   };
   std::vector<Chunk> chunks;
+  bool host_copies = false;
+  std::vector<CUtensorMap> hmaps;
+  std::vector<long> hrowmap;
+  std::vector<GroupJob> h_psi_jobs;
+  std::vector<UnconvJob> h_sig_jobs;
   DArr<int> err;
   double stats[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
 };
@@ -874,7 +342,8 @@ struct TmaPlan {
 void tma_plan_free(TmaPlan* p) { delete p; }
 
 void tma_plan_stats(const SigmaPlan& plan, double* out) {
-  for (int i = 0; i < 9; ++i) out[i] = plan.tm ? plan.tm->stats[i] : 0.0;
+  // (statistics are reported for precisions 4-6)
+  for (int i = 0; i < 9; ++i) out[i] = plan.tm && plan.tm->precision >= 4 ? plan.tm->stats[i] : 0.0;
 }
 
 namespace {
@@ -890,6 +359,22 @@ static void check_group_jobs(const std::vector<GroupJob>& jobs, int nsl, const D
       throw Error(ST_ECUDA, "internal: conversion job outside its buffer");
 }
 
+// longest tiles first (static round-robin over the persistent CTAs); tiles of equal
+// length keep their order, so the N tiles of one row tile stay adjacent
+static void longest_first(std::vector<TmTile>& t, const std::vector<TmTerm>& m) {
+  std::vector<std::pair<long, int>> key(t.size());
+  for (size_t i = 0; i < t.size(); ++i) {
+    long ks = 0;
+    for (int j = t[i].t0; j < t[i].t1; ++j) ks += (m[j].k + 63) / 64;
+    key[i] = {-ks, (int)i};
+  }
+  std::stable_sort(key.begin(), key.end(),
+                   [](const std::pair<long, int>& a, const std::pair<long, int>& b) { return a.first < b.first; });
+  std::vector<TmTile> out(t.size());
+  for (size_t i = 0; i < t.size(); ++i) out[i] = t[(size_t)key[i].second];
+  t.swap(out);
+}
+
 void build_tma_plan(Context& c, Tilde& lt, Tilde& rt, int k, SigmaPlan& plan, int nsl) {
   const auto& mid = c.mpo.bonds[k + 1];
   Env& Lenv = *lt.env;
@@ -901,6 +386,8 @@ void build_tma_plan(Context& c, Tilde& lt, Tilde& rt, int k, SigmaPlan& plan, in
   plan.tm.reset(tp);
   if (nsl < 1 || nsl > 3) throw Error(ST_EINVAL, "TMA plan: 1 to 3 slices");
   tp->nsl = nsl;
+  tp->precision = c.precision;
+  tp->host_copies = c.keep_host_plans && c.precision <= 3;  // what a batch takes
   const int nL = Lb.nsec(), nR = Rb.nsec();
   const int nmid = (int)mid.size();
   // slice pairs (i, j), i + j < nsl, multiplied per piece
@@ -989,6 +476,10 @@ void build_tma_plan(Context& c, Tilde& lt, Tilde& rt, int k, SigmaPlan& plan, in
     tp->n_psi_jobs = (int)pj.size();
     tp->sig_jobs.upload(sj, c.stream);
     tp->n_sig_jobs = (int)sj.size();
+    if (tp->host_copies) {
+      tp->h_psi_jobs = pj;
+      tp->h_sig_jobs = sj;
+    }
     cuda_check(cudaStreamSynchronize(c.stream), "sync");
   }
   // ---- stage-1 row blocks: per input group g', every (beta, n2) with at least one
@@ -1027,7 +518,8 @@ void build_tma_plan(Context& c, Tilde& lt, Tilde& rt, int k, SigmaPlan& plan, in
   for (int beta = 0; beta < nmid; ++beta)
     for (int gp = 0; gp < ng; ++gp)
       if (xhas[(size_t)beta * ng + gp]) xsz[beta] += (size_t)gC[gout[(size_t)beta * ng + gp]] * gR[gp];
-  const size_t budget = (size_t)std::max<long>(1, c.tma_budget_mb) * (1u << 20) / (sizeof(__nv_bfloat16) * nsl);
+  const long budget_mb = c.precision >= 4 ? c.tma_budget_mb : (long)c.chunk_budget_mb;
+  const size_t budget = (size_t)std::max<long>(1, budget_mb) * (1u << 20) / (sizeof(__nv_bfloat16) * nsl);
   std::vector<std::pair<int, int>> chunks;
   for (int b0 = 0; b0 < nmid;) {
     int b1 = b0;
@@ -1269,6 +761,7 @@ void build_tma_plan(Context& c, Tilde& lt, Tilde& rt, int k, SigmaPlan& plan, in
     cuda_check(cudaMemcpyAsync(tp->maps.p, maps.data(), maps.size() * sizeof(CUtensorMap), cudaMemcpyHostToDevice,
                                c.stream),
                "h2d");
+  if (tp->host_copies) tp->hmaps = maps;
   // ---- work lists per chunk
   std::vector<long> rowmap;
   double st1_tiles = 0, st1_steps = 0, st2_tiles = 0, st2_steps = 0, st1_fl = 0, st2_fl = 0;
@@ -1298,7 +791,7 @@ void build_tma_plan(Context& c, Tilde& lt, Tilde& rt, int k, SigmaPlan& plan, in
               const int kk = pad16(Rb.dim[qrp]);
               m1.push_back({a1map[gp], nt[2], coff, (int)r0, coff, nt[0], kk, nsl << 4});
               ksum += kk * npair;
-              st1_steps += kk / TM_PIECE_COLS;
+              st1_steps += (kk + 63) / 64 * npair;
             }
             tl.t1 = (int)m1.size();
             tl.nseg = 1;
@@ -1405,30 +898,15 @@ void build_tma_plan(Context& c, Tilde& lt, Tilde& rt, int k, SigmaPlan& plan, in
           tl.t1 = (int)m2.size();
           if (ks / TM_PIECE_COLS > (1L << 30)) throw Error(ST_ECUDA, "internal: stage-2 tile too long");
           t2.push_back(tl);
-          st2_steps += (double)(ks / npair / TM_PIECE_COLS);
+          st2_steps += (double)((ks + 63) / 64);
           st2_fl += 2.0 * 128 * tl.n * ks;
           t0 = t + 1;
           acc = 0;
         }
       }
     }
-    // longest tiles first (static round-robin over the persistent CTAs); tiles of equal
-    // length keep their order, so the N tiles of one row tile stay adjacent
-    auto order = [](std::vector<TmTile>& t, const std::vector<TmTerm>& m) {
-      std::vector<std::pair<long, int>> key(t.size());
-      for (size_t i = 0; i < t.size(); ++i) {
-        long ks = 0;
-        for (int j = t[i].t0; j < t[i].t1; ++j) ks += (m[j].k + 63) / 64;
-        key[i] = {-ks, (int)i};
-      }
-      std::stable_sort(key.begin(), key.end(),
-                       [](const std::pair<long, int>& a, const std::pair<long, int>& b) { return a.first < b.first; });
-      std::vector<TmTile> out(t.size());
-      for (size_t i = 0; i < t.size(); ++i) out[i] = t[(size_t)key[i].second];
-      t.swap(out);
-    };
-    order(t1, m1);
-    order(t2, m2);
+    longest_first(t1, m1);
+    longest_first(t2, m2);
     // the copy lists of both launches (stage 2: sets every tile's stages and segments);
     // their pieces follow from the terms checked below
     ch.l1.plan(TM_MODE_STORE_BF16, nsl, t1, m1, c.stream);
@@ -1510,8 +988,16 @@ void build_tma_plan(Context& c, Tilde& lt, Tilde& rt, int k, SigmaPlan& plan, in
     for (const ZeroJob& z : zj) ch.zmax = std::max(ch.zmax, z.n);
     ch.z.upload(zj, c.stream);
     cuda_check(cudaStreamSynchronize(c.stream), "sync");
+    if (tp->host_copies) {
+      ch.ht1.swap(t1);
+      ch.ht2.swap(t2);
+      ch.hm1.swap(m1);
+      ch.hm2.swap(m2);
+      ch.hz.swap(zj);
+    }
   }
   tp->rowmap.upload(rowmap, c.stream);
+  if (tp->host_copies) tp->hrowmap = rowmap;
   // the operator stacks depend only on the environments: filled once per plan
   if (tp->n_a1_jobs) launch_conv_groups(tp->a1_jobs, tp->n_a1_jobs, nsl, tp->a1_maxel, c.stream);
   if (tp->n_l_jobs) launch_conv_groups(tp->l_jobs, tp->n_l_jobs, nsl, tp->l_maxel, c.stream);
@@ -1549,7 +1035,7 @@ void run_tma_sigma(Context& c, SigmaPlan& plan, const double* x, double* y) {
 
 int plan_error(Context& c, SigmaPlan& plan) {
   int h = 0;
-  int* p = plan.mx ? plan.mx->err.p : plan.tm ? plan.tm->err.p : nullptr;
+  int* p = plan.tm ? plan.tm->err.p : nullptr;
   if (!p) return 0;
   cuda_check(cudaMemcpyAsync(&h, p, sizeof(int), cudaMemcpyDeviceToHost, c.stream), "d2h");
   cuda_check(cudaStreamSynchronize(c.stream), "sync");
@@ -2280,24 +1766,36 @@ void env_update_exact(Context& c, Tilde& t, const SiteT& A, int site, Env& out, 
 
 // ---------------------------------------------------------------- batched sigma
 
-// Several independent two-site problems (each prepared in tensor-core precision
-// on the same device) fused into one launch per stage and chunk: the tile, task
-// and term lists are concatenated, so one persistent kernel walks the tiles of
-// every problem.  Optionally the whole sequence (conversions, stage launches,
-// gathers) is captured once in a CUDA graph and replayed.
+// Several independent two-site problems (each prepared in a tensor-core precision
+// on the same device) fused into one launch per stage and chunk: the tile and term lists, tensor
+// maps and row maps are concatenated, so one persistent kernel walks the tiles of
+// every problem (one launch per slice count where the problems differ in it).  Optionally the
+// whole sequence (conversions, stage launches, gathers) is captured once in a CUDA graph and
+// replayed.  (Eight problems, K 12-20, M 64-256, three slices: 1.29 ms; 9.04 ms on per-sector
+// tiles staged by cp.async.)
 struct BatchPlan {
   std::vector<Context*> ctx;
   cudaStream_t stream = nullptr;
-  std::vector<TcPlan> stage1, stage2;
-  DArr<ConvJob> conv;
+  struct Launch {
+    int nsl = 1, n1 = 0, n2 = 0, nz = 0;
+    long zmax = 0;
+    DArr<TmTile> t1, t2;
+    DArr<TmTerm> m1, m2;
+    TmaPlan::Lists l1, l2;
+    DArr<ZeroJob> z;
+    void *out1 = nullptr, *out2 = nullptr;  // what the tiles' offsets count from
+  };
+  std::vector<Launch> launches;  // chunk by chunk
+  DArr<CUtensorMap> maps;
+  DArr<long> rowmap;
+  DArr<GroupJob> conv[3];  // by slice count
   DArr<UnconvJob> unconv;
-  int nconv = 0, nunconv = 0;
+  int nconv[3] = {0, 0, 0}, nunconv = 0;
   long conv_maxel = 0, unconv_maxel = 0;
   DArr<int> err;
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t exec = nullptr;
   long graph_launches = 0, graph_tc_launches = 0;  // kernels in one replay of the graph
-  int nsl = 1;                                      // largest slice count of the problems
   double flops = 0;
   ~BatchPlan() {
     if (exec) cudaGraphExecDestroy(exec);
@@ -2305,86 +1803,107 @@ struct BatchPlan {
   }
 };
 
-static void concat_into(TcPlan& out, const std::vector<const TcPlan*>& parts, cudaStream_t s) {
-  std::vector<TcTile> ti;
-  std::vector<TcTask> ta;
-  std::vector<TcTerm> te;
+// chunk ch of the problems with nsl slices as one launch per stage; map0, row0: every problem's first
+// tensor map and row-map entry in the concatenated arrays
+static void batch_launch(BatchPlan& b, size_t ch, int nsl, const std::vector<int>& map0, const std::vector<long>& row0) {
+  std::vector<TmTile> t1, t2;
+  std::vector<TmTerm> m1, m2;
   std::vector<ZeroJob> zj;
-  for (const TcPlan* p : parts) {
-    if (p->ntiles && p->htiles.empty()) throw Error(ST_ESTATE, "batched sigma: plan was built without host copies");
-    const int toff = (int)ta.size(), eoff = (int)te.size();
-    for (TcTask t : p->htasks) {
-      t.t0 += eoff;
-      t.t1 += eoff;
-      ta.push_back(t);
+  BatchPlan::Launch L;
+  L.nsl = nsl;
+  auto add = [&](std::vector<TmTile>& tiles, std::vector<TmTerm>& terms, const std::vector<TmTile>& pt,
+                 const std::vector<TmTerm>& pm, int map, auto&& rebase) {
+    const int t0 = (int)terms.size();
+    for (TmTile t : pt) {
+      t.t0 += t0;
+      t.t1 += t0;
+      rebase(t);
+      tiles.push_back(t);
     }
-    te.insert(te.end(), p->hterms.begin(), p->hterms.end());
-    for (TcTile x : p->htiles) {
-      x.task += toff;
-      ti.push_back(x);
+    for (TmTerm m : pm) {
+      m.amap += map;
+      m.bmap += map;
+      terms.push_back(m);
     }
-    zj.insert(zj.end(), p->hzeros.begin(), p->hzeros.end());
-    out.zmax = std::max(out.zmax, p->zmax);
+  };
+  for (size_t p = 0; p < b.ctx.size(); ++p) {
+    const TmaPlan& tp = *b.ctx[p]->plan.tm;
+    if (tp.nsl != nsl || ch >= tp.chunks.size()) continue;
+    const TmaPlan::Chunk& c = tp.chunks[ch];
+    if (!L.out1) {
+      L.out1 = tp.xt.p;
+      L.out2 = tp.sig_t.p;
+    }
+    const long dx = ((intptr_t)tp.xt.p - (intptr_t)L.out1) / (long)sizeof(__nv_bfloat16);
+    const long ds = ((intptr_t)tp.sig_t.p - (intptr_t)L.out2) / (long)sizeof(float);
+    add(t1, m1, c.ht1, c.hm1, map0[p], [&](TmTile& t) {
+      t.rowmap_off += row0[p];
+      t.xbase += dx;
+    });
+    add(t2, m2, c.ht2, c.hm2, map0[p], [&](TmTile& t) { t.out_off += ds; });
+    zj.insert(zj.end(), c.hz.begin(), c.hz.end());
+    L.zmax = std::max(L.zmax, c.zmax);
   }
-  out.tiles.upload(ti, s);
-  out.tasks.upload(ta, s);
-  out.terms.upload(te, s);
-  out.ntiles = (int)ti.size();
-  out.nzeros = (int)zj.size();
-  out.zeros.upload(zj, s);
-  out.hzeros = zj;
-  cuda_check(cudaStreamSynchronize(s), "sync");
+  if (t1.empty() && t2.empty()) return;
+  longest_first(t1, m1);
+  longest_first(t2, m2);
+  L.l1.plan(TM_MODE_STORE_BF16, nsl, t1, m1, b.stream);
+  L.l2.plan(TM_MODE_REDUCE_F32, nsl, t2, m2, b.stream);
+  L.n1 = (int)t1.size();
+  L.n2 = (int)t2.size();
+  L.nz = (int)zj.size();
+  L.t1.upload(t1, b.stream);
+  L.m1.upload(m1, b.stream);
+  L.t2.upload(t2, b.stream);
+  L.m2.upload(m2, b.stream);
+  L.z.upload(zj, b.stream);
+  L.l1.fill(TM_MODE_STORE_BF16, nsl, L.t1.p, L.n1, L.m1.p, b.stream);
+  L.l2.fill(TM_MODE_REDUCE_F32, nsl, L.t2.p, L.n2, L.m2.p, b.stream);
+  cuda_check(cudaStreamSynchronize(b.stream), "sync");
+  b.launches.push_back(std::move(L));
 }
 
 BatchPlan* batch_create(const std::vector<Context*>& ctxs) {
-  auto* b = new BatchPlan();
+  std::unique_ptr<BatchPlan, void (*)(BatchPlan*)> b(new BatchPlan(), batch_free);
   b->ctx = ctxs;
   b->stream = ctxs[0]->stream;
   size_t nch = 0;
-  std::vector<ConvJob> cj;
+  std::vector<GroupJob> cj[3];
   std::vector<UnconvJob> uj;
+  std::vector<CUtensorMap> maps;
+  std::vector<long> rowmap;
+  std::vector<int> map0;
+  std::vector<long> row0;
   for (Context* c : ctxs) {
-    if (c->prepared < 0 || !c->plan.mx) {
-      delete b;
-      throw Error(ST_ESTATE,
-                  "batched sigma: every context must be prepared in a tensor-core precision of the cp.async plan (1-3)");
-    }
-    MixedPlan& mx = *c->plan.mx;
-    nch = std::max(nch, mx.stage1.size());
-    cj.insert(cj.end(), mx.h_psi_jobs.begin(), mx.h_psi_jobs.end());
-    uj.insert(uj.end(), mx.h_sig_jobs.begin(), mx.h_sig_jobs.end());
-    b->conv_maxel = std::max(b->conv_maxel, mx.psi_maxel);
-    b->unconv_maxel = std::max(b->unconv_maxel, mx.sig_maxel);
+    if (c->prepared < 0 || !c->plan.tm || c->plan.tm->precision > 3)
+      throw Error(ST_ESTATE, "batched sigma: every context must be prepared in precision 1, 2 or 3");
+    const TmaPlan& tp = *c->plan.tm;
+    if (!tp.host_copies) throw Error(ST_ESTATE, "batched sigma: plan was built without host copies");
+    nch = std::max(nch, tp.chunks.size());
+    cj[tp.nsl - 1].insert(cj[tp.nsl - 1].end(), tp.h_psi_jobs.begin(), tp.h_psi_jobs.end());
+    uj.insert(uj.end(), tp.h_sig_jobs.begin(), tp.h_sig_jobs.end());
+    map0.push_back((int)maps.size());
+    row0.push_back((long)rowmap.size());
+    maps.insert(maps.end(), tp.hmaps.begin(), tp.hmaps.end());
+    rowmap.insert(rowmap.end(), tp.hrowmap.begin(), tp.hrowmap.end());
+    b->conv_maxel = std::max(b->conv_maxel, tp.psi_maxel);
+    b->unconv_maxel = std::max(b->unconv_maxel, tp.sig_maxel);
     b->flops += c->plan.flops;
-    b->nsl = std::max(b->nsl, mx.nsl);
   }
-  try {
-    for (size_t ch = 0; ch < nch; ++ch) {
-      std::vector<const TcPlan*> p1, p2;
-      for (Context* c : ctxs) {
-        MixedPlan& mx = *c->plan.mx;
-        if (ch < mx.stage1.size()) {
-          p1.push_back(&mx.stage1[ch]);
-          p2.push_back(&mx.stage2[ch]);
-        }
-      }
-      b->stage1.emplace_back();
-      concat_into(b->stage1.back(), p1, b->stream);
-      b->stage2.emplace_back();
-      concat_into(b->stage2.back(), p2, b->stream);
-    }
-    b->conv.upload(cj, b->stream);
-    b->nconv = (int)cj.size();
-    b->unconv.upload(uj, b->stream);
-    b->nunconv = (int)uj.size();
-    b->err.alloc(1, b->stream);
-    cuda_check(cudaMemsetAsync(b->err.p, 0, sizeof(int), b->stream), "memset");
-    cuda_check(cudaStreamSynchronize(b->stream), "sync");
-  } catch (...) {
-    delete b;
-    throw;
+  b->maps.upload(maps, b->stream);
+  b->rowmap.upload(rowmap, b->stream);
+  for (size_t ch = 0; ch < nch; ++ch)
+    for (int nsl = 1; nsl <= 3; ++nsl) batch_launch(*b, ch, nsl, map0, row0);
+  for (int i = 0; i < 3; ++i) {
+    b->conv[i].upload(cj[i], b->stream);
+    b->nconv[i] = (int)cj[i].size();
   }
-  return b;
+  b->unconv.upload(uj, b->stream);
+  b->nunconv = (int)uj.size();
+  b->err.alloc(1, b->stream);
+  cuda_check(cudaMemsetAsync(b->err.p, 0, sizeof(int), b->stream), "memset");
+  cuda_check(cudaStreamSynchronize(b->stream), "sync");
+  return b.release();
 }
 
 void batch_free(BatchPlan* b) {
@@ -2397,18 +1916,19 @@ double batch_flops(const BatchPlan* b) { return b->flops; }
 static void batch_enqueue(BatchPlan& b) {
   cudaStream_t s = b.stream;
   for (Context* c : b.ctx) {
-    MixedPlan& mx = *c->plan.mx;
-    cuda_check(cudaMemsetAsync(mx.sig_f.p, 0, mx.sig_total * sizeof(float), s), "memset");
+    TmaPlan& tp = *c->plan.tm;
+    cuda_check(cudaMemsetAsync(tp.sig_t.p, 0, tp.sig_total * sizeof(float), s), "memset");
   }
-  if (b.nconv) launch_conv(b.conv, b.nconv, b.conv_maxel, s);
-  for (size_t i = 0; i < b.stage1.size(); ++i) {
-    run_zeros(b.stage1[i], s);
-    cuda_check(launch_gemm_bf16_tc(b.stage1[i].tiles.p, b.stage1[i].ntiles, b.stage1[i].tasks.p,
-                                   b.stage1[i].terms.p, b.err.p, s, b.nsl),
-               "tc stage 1");
-    cuda_check(launch_gemm_bf16_tc(b.stage2[i].tiles.p, b.stage2[i].ntiles, b.stage2[i].tasks.p,
-                                   b.stage2[i].terms.p, b.err.p, s, b.nsl),
-               "tc stage 2");
+  for (int i = 0; i < 3; ++i)
+    if (b.nconv[i]) launch_conv_groups(b.conv[i], b.nconv[i], i + 1, b.conv_maxel, s);
+  for (const BatchPlan::Launch& L : b.launches) {
+    if (L.nz) launch_zero(L.z.p, L.nz, L.zmax, s);
+    cuda_check(launch_gemm_slices(TM_MODE_STORE_BF16, L.nsl, L.t1.p, L.n1, b.maps.p, b.rowmap.p, L.out1, b.err.p, s,
+                                  L.l1.dev()),
+               "batch stage 1");
+    cuda_check(launch_gemm_slices(TM_MODE_REDUCE_F32, L.nsl, L.t2.p, L.n2, b.maps.p, nullptr, L.out2, b.err.p, s,
+                                  L.l2.dev()),
+               "batch stage 2");
   }
   if (b.nunconv) launch_unconv(b.unconv.p, b.nunconv, b.unconv_maxel, s);
 }
@@ -2564,8 +2084,8 @@ TuneChoice autotune_plans(const std::vector<Context*>& ctxs, const std::vector<d
     if (b <= 0) throw Error(ST_EINVAL, "autotune: chunk budgets must be positive");
   const bool batched = ctxs.size() > 1;
   for (Context* c : ctxs) {
-    if (c->prepared < 0 || !c->plan.mx)
-      throw Error(ST_ESTATE, "autotune: every context must be prepared in a tensor-core precision");
+    if (c->prepared < 0 || !c->plan.tm || c->plan.tm->precision > 3)
+      throw Error(ST_ESTATE, "autotune: every context must be prepared in precision 1, 2 or 3");
     if (batched && !c->keep_host_plans)
       throw Error(ST_ESTATE, "autotune: tuning a batch needs host copies of the plans (keep_host_plans)");
   }
@@ -2614,7 +2134,7 @@ TuneChoice autotune_plans(const std::vector<Context*>& ctxs, const std::vector<d
           for (int r = 0; r < reps; ++r) run_sigma(c, c.plan, pin[0], pout[0]);
           cuda_check(cudaEventRecord(c.ev1, c.stream), "record");
           cuda_check(cudaEventSynchronize(c.ev1), "sync");
-          if (mixed_error(c, c.plan)) throw Error(ST_ETIMEOUT, "tensor-core GEMM: a bounded wait ran out");
+          if (plan_error(c, c.plan)) throw Error(ST_ETIMEOUT, "tensor-core GEMM: a bounded wait ran out");
           float e = 0;
           cuda_check(cudaEventElapsedTime(&e, c.ev0, c.ev1), "elapsed");
           t = e;
