@@ -187,9 +187,9 @@ void GemmPlan::upload(GemmBuilder& g, cudaStream_t s) {
   ntiles = (int)g.tiles.size();
 }
 
-void GemmPlan::run(cudaStream_t s) const {
+void GemmPlan::run(cudaStream_t s, long b_shift, long c_shift) const {
   if (ntiles == 0) return;
-  launch_gemm(tiles.p, ntiles, tasks.p, terms.p, cap, s);
+  launch_gemm(tiles.p, ntiles, tasks.p, terms.p, cap, s, b_shift, c_shift);
   cuda_check(cudaGetLastError(), "gemm launch");
 }
 
@@ -235,9 +235,9 @@ Context::~Context() {
   for (int i = 0; i < kAux; ++i) {
     if (aux_solver[i]) cusolverDnDestroy(aux_solver[i]);
     if (aux[i]) cudaStreamDestroy(aux[i]);
-  }
-  for (int i = 0; i <= kAux; ++i)
     if (aux_ev[i]) cudaEventDestroy(aux_ev[i]);
+  }
+  if (fork_ev) cudaEventDestroy(fork_ev);
   if (own_stream && stream) cudaStreamDestroy(stream);
 }
 
@@ -254,13 +254,7 @@ void ctx_init(Context& c) {
   cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &thr);
   cuda_check(cudaEventCreate(&c.ev0), "event");
   cuda_check(cudaEventCreate(&c.ev1), "event");
-  for (int i = 0; i < Context::kAux; ++i) {
-    cuda_check(cudaStreamCreateWithFlags(&c.aux[i], cudaStreamNonBlocking), "aux stream");
-    solver_check(cusolverDnCreate(&c.aux_solver[i]), "cusolverDnCreate");
-    solver_check(cusolverDnSetStream(c.aux_solver[i], c.aux[i]), "cusolverDnSetStream");
-  }
-  for (int i = 0; i <= Context::kAux; ++i)
-    cuda_check(cudaEventCreateWithFlags(&c.aux_ev[i], cudaEventDisableTiming), "aux event");
+  cuda_check(cudaEventCreateWithFlags(&c.fork_ev, cudaEventDisableTiming), "aux event");
   solver_check(cusolverDnCreate(&c.solver), "cusolverDnCreate");
   solver_check(cusolverDnSetStream(c.solver, c.stream), "cusolverDnSetStream");
   c.mpo = build_mpo(c.K, c.h1.data(), c.eri.data());
@@ -937,14 +931,18 @@ void run_sigma(Context& c, SigmaPlan& plan, const double* x, double* y) {
     run_tma_sigma(c, plan, x, y);
     return;
   }
+  // the work lists are made for plan.in and plan.out and serve any x and y that do not overlap
   const size_t bytes = plan.psi.nnz * sizeof(double);
-  if (x != plan.in.p) cuda_check(cudaMemcpyAsync(plan.in.p, x, bytes, cudaMemcpyDeviceToDevice, c.stream), "d2d");
-  cuda_check(cudaMemsetAsync(plan.out.p, 0, bytes, c.stream), "memset");
-  for (size_t i = 0; i < plan.stage1.size(); ++i) {
-    plan.stage1[i].run(c.stream);
-    plan.stage2[i].run(c.stream);
+  const uintptr_t xa = (uintptr_t)x, ya = (uintptr_t)y;
+  if (xa < ya + bytes && ya < xa + bytes) {
+    cuda_check(cudaMemcpyAsync(plan.in.p, x, bytes, cudaMemcpyDeviceToDevice, c.stream), "d2d");
+    x = plan.in.p;
   }
-  if (y != plan.out.p) cuda_check(cudaMemcpyAsync(y, plan.out.p, bytes, cudaMemcpyDeviceToDevice, c.stream), "d2d");
+  cuda_check(cudaMemsetAsync(y, 0, bytes, c.stream), "memset");
+  for (size_t i = 0; i < plan.stage1.size(); ++i) {
+    plan.stage1[i].run(c.stream, x - plan.in.p, 0);
+    plan.stage2[i].run(c.stream, 0, y - plan.out.p);
+  }
 }
 
 void compute_diag(Context& c, Tilde& lt, Tilde& rt, int k, const PsiLayout& P, double* diag) {
@@ -1055,22 +1053,16 @@ void prepare_two_site(Context& c, int k) {
 
 // ---------------------------------------------------------------- Davidson
 
-struct DotHelper {
-  DArr<double> part, out;
-  int nblk = 128;
-  std::vector<double> host;
-  void init(int maxm, cudaStream_t s) {
-    part.alloc((size_t)maxm * nblk, s);
-    out.alloc(maxm, s);
-    host.resize(maxm);
+// device workspace of the deterministic reductions (one launch at a time)
+struct DotBuf {
+  DArr<double> part;
+  DArr<unsigned> count;
+  void init(cudaStream_t s) {
+    part.alloc((size_t)DOT_MAX * DOT_BLOCKS, s);
+    count.alloc(1, s);
+    cuda_check(cudaMemsetAsync(count.p, 0, sizeof(unsigned), s), "memset");
   }
-  // dots of rows V[0..m) (stride ldv) with x, returned on host
-  const std::vector<double>& dots(Context& c, const double* V, long ldv, int m, const double* x, long n) {
-    launch_multidot(V, ldv, m, x, n, part.p, nblk, out.p, c.stream);
-    cuda_check(cudaMemcpyAsync(host.data(), out.p, m * sizeof(double), cudaMemcpyDeviceToHost, c.stream), "d2h");
-    cuda_check(cudaStreamSynchronize(c.stream), "sync");
-    return host;
-  }
+  DotWork work() const { return {part.p, count.p}; }
 };
 
 // Davidson on the device: the subspace vectors, their sigma vectors, the projected
@@ -1082,8 +1074,10 @@ struct DotHelper {
 double davidson(Context& c, SigmaPlan& plan, const double* diag, double* psi, const DavidsonOpts& o, int* iters) {
   const long n = plan.psi.nnz;
   const int ms = (int)std::max<long>(2, std::min<long>(std::min(o.max_sub, RR_MAX_SUB), n));
-  const int nblk = 128;
-  DArr<double> V, S, x, hx, r, t, coef, ocoef, G, part, scal;
+  DotBuf db;
+  db.init(c.stream);
+  const DotWork dw = db.work();
+  DArr<double> V, S, x, hx, r, t, coef, ocoef, ocoef2, G, scal;
   V.alloc((size_t)ms * n, c.stream);
   S.alloc((size_t)ms * n, c.stream);
   x.alloc(n, c.stream);
@@ -1092,8 +1086,8 @@ double davidson(Context& c, SigmaPlan& plan, const double* diag, double* psi, co
   t.alloc(n, c.stream);
   coef.alloc(ms, c.stream);
   ocoef.alloc(ms + 1, c.stream);
+  ocoef2.alloc(ms + 1, c.stream);
   G.alloc((size_t)ms * ms, c.stream);
-  part.alloc((size_t)(ms + 1) * nblk, c.stream);
   // scal: [0] Ritz value, [1] |r|^2, [2] |t|^2, [3] |psi|^2, [4] |x|^2
   scal.alloc(8, c.stream);
   cuda_check(cudaMemsetAsync(G.p, 0, G.n * sizeof(double), c.stream), "memset");
@@ -1125,15 +1119,13 @@ double davidson(Context& c, SigmaPlan& plan, const double* diag, double* psi, co
     cuda_check(cudaStreamSynchronize(c.stream), "sync");
   };
   auto dots = [&](const double* Vb, long ldv, int m, const double* y, double* out) {
-    launch_multidot(Vb, ldv, m, y, n, part.p, nblk, out, c.stream);
+    launch_multidot(Vb, ldv, m, y, n, dw, out, c.stream);
   };
   // two passes of classical Gram-Schmidt of t against V[0..m), then |t|^2
   auto orthogonalise = [&](int m) {
-    for (int pass = 0; pass < 2; ++pass) {
-      dots(V.p, n, m, t.p, ocoef.p);
-      launch_sub_combine(V.p, n, m, ocoef.p, n, t.p, c.stream);
-    }
-    dots(t.p, 0, 1, t.p, scal.p + 2);
+    dots(V.p, n, m, t.p, ocoef.p);
+    launch_project(V.p, n, m, ocoef.p, n, t.p, dw, ocoef2.p, c.stream);
+    launch_project_norm(V.p, n, m, ocoef2.p, n, t.p, dw, scal.p + 2, c.stream);
   };
   double h3[3] = {0, 0, 0};
   int it = 0;
@@ -1148,8 +1140,7 @@ double davidson(Context& c, SigmaPlan& plan, const double* diag, double* psi, co
     if (!(h3[0] > 0) || !std::isfinite(h3[0])) throw Error(ST_EINVAL, "Davidson: zero or non-finite start vector");
     launch_scale_rsqrt(n, psi, scal.p + 3, V.p, c.stream);
     sigma_of(V.p, S.p);
-    dots(V.p, 0, 1, S.p, ocoef.p);
-    launch_gcol(ocoef.p, 1, G.p, ms, 0, c.stream);
+    launch_multidot(V.p, 0, 1, S.p, n, dw, ocoef.p, c.stream, G.p, ms, 0);
     int m = 1;
     double best_rn = 1e300;
     int since_best = 0;
@@ -1163,11 +1154,7 @@ double davidson(Context& c, SigmaPlan& plan, const double* diag, double* psi, co
     for (; it < o.max_iter; ++it) {
       // Rayleigh-Ritz, Ritz vector, residual, diagonal correction
       if (!launch_rr(G.p, ms, m, coef.p, th_d, c.stream)) throw Error(ST_EINVAL, "Davidson: subspace too large");
-      launch_combine_vectors(V.p, n, m, coef.p, n, x.p, c.stream);
-      launch_combine_vectors(S.p, n, m, coef.p, n, hx.p, c.stream);
-      launch_resid(n, hx.p, x.p, th_d, r.p, c.stream);
-      dots(r.p, 0, 1, r.p, scal.p + 1);
-      launch_precond_dev(n, r.p, diag, th_d, 1e-8, t.p, c.stream);
+      launch_ritz(V.p, S.p, n, m, coef.p, n, th_d, diag, 1e-8, x.p, hx.p, r.p, t.p, dw, scal.p + 1, c.stream);
       // a full subspace restarts from the Ritz vector (harmless if this iteration
       // turns out converged: x and hx are kept)
       int mb = m;
@@ -1226,8 +1213,7 @@ double davidson(Context& c, SigmaPlan& plan, const double* diag, double* psi, co
       if (!(tn > 1e-14)) break;  // subspace exhausted: the Ritz pair is exact in it
       launch_scale_rsqrt(n, t.p, scal.p + 2, V.p + (size_t)m * n, c.stream);
       sigma_of(V.p + (size_t)m * n, S.p + (size_t)m * n);
-      dots(V.p, n, m + 1, S.p + (size_t)m * n, ocoef.p);
-      launch_gcol(ocoef.p, m + 1, G.p, ms, m, c.stream);
+      launch_multidot(V.p, n, m + 1, S.p + (size_t)m * n, n, dw, ocoef.p, c.stream, G.p, ms, m);
       ++m;
     }
     dots(x.p, 0, 1, x.p, scal.p + 4);
@@ -1273,10 +1259,16 @@ double expectation(Context& c) {
   make_psi(c, c.sites[k], c.sites[k + 1], plan.psi, psi.p);
   run_sigma(c, plan, psi.p, sig.p);
   if (plan.tensor() && plan_error(c, plan)) throw Error(ST_ETIMEOUT, "tensor-core GEMM: a bounded wait ran out");
-  DotHelper dh;
-  dh.init(1, c.stream);
-  const double num = dh.dots(c, psi.p, 0, 1, sig.p, n)[0];
-  const double den = dh.dots(c, psi.p, 0, 1, psi.p, n)[0];
+  DotBuf db;
+  db.init(c.stream);
+  DArr<double> d;
+  d.alloc(2, c.stream);
+  launch_multidot(psi.p, 0, 1, sig.p, n, db.work(), d.p, c.stream);
+  launch_multidot(psi.p, 0, 1, psi.p, n, db.work(), d.p + 1, c.stream);
+  double h[2];
+  cuda_check(cudaMemcpyAsync(h, d.p, 2 * sizeof(double), cudaMemcpyDeviceToHost, c.stream), "d2h");
+  cuda_check(cudaStreamSynchronize(c.stream), "sync");
+  const double num = h[0], den = h[1];
   if (!(den > 0)) throw Error(ST_ESTATE, "the MPS has zero norm at this position");
   return num / den + c.ecore;
 }
@@ -1354,36 +1346,56 @@ double decimate(Context& c, const PsiLayout& P, const double* psi, int M, int di
   size_t etot = 0;
   for (auto& g : groups) etot += direction == 0 ? g.nr : g.nc;
   evals.alloc(std::max<size_t>(etot, 1), c.stream);
-  int lwork = 0;
-  solver_check(cusolverDnDsyevd_bufferSize(c.solver, CUSOLVER_EIG_MODE_VECTOR, CUBLAS_FILL_MODE_UPPER, maxd, Gram.p,
-                                           maxd, evals.p, &lwork),
-               "syevd_bufferSize");
-  // the group eigenproblems are independent: spread them over the auxiliary
-  // streams (one workspace each), joined back into the context stream
-  const int na = Context::kAux;
-  DArr<double> work;
-  work.alloc((size_t)std::max(lwork, 1) * na, c.stream);
+  // The group eigenproblems are independent.  Small ones share one launch of the Jacobi kernel,
+  // a thread block each; the others are spread over auxiliary streams (one workspace each), all
+  // joined back into the context stream.  Measured (decimation of two K=6, M=64 sweeps / a K=16,
+  // M=128 step): no sector in the shared launch 13.0 / 5.0 ms, those up to 16 rows 7.7 / 4.4, up
+  // to 32 7.5 / 3.6, up to 48 28.7 / 3.8.  Streams (K=24, M=512 step): 4 23.3 ms, 8 16.1, 16 15.8.
   DArr<int> info;
   info.alloc(groups.size() + 1, c.stream);
-  cuda_check(cudaEventRecord(c.aux_ev[na], c.stream), "record");
-  for (int a = 0; a < na; ++a) cuda_check(cudaStreamWaitEvent(c.aux[a], c.aux_ev[na], 0), "wait");
+  cuda_check(cudaMemsetAsync(info.p, 0, info.n * sizeof(int), c.stream), "memset");
   size_t eo = 0;
   std::vector<size_t> eoff(groups.size());
-  std::vector<size_t> order(groups.size());
-  std::iota(order.begin(), order.end(), 0);
-  std::sort(order.begin(), order.end(), [&](size_t x, size_t y) {
-    int dx = direction == 0 ? groups[x].nr : groups[x].nc, dy = direction == 0 ? groups[y].nr : groups[y].nc;
-    return dx > dy;
-  });
   for (size_t gi = 0; gi < groups.size(); ++gi) {
     eoff[gi] = eo;
     eo += direction == 0 ? groups[gi].nr : groups[gi].nc;
   }
-  for (size_t q = 0; q < order.size(); ++q) {
-    const size_t gi = order[q];
+  auto dim_of = [&](size_t gi) { return direction == 0 ? groups[gi].nr : groups[gi].nc; };
+  std::vector<EighJob> small;
+  std::vector<size_t> large;
+  for (size_t gi = 0; gi < groups.size(); ++gi) {
+    if (dim_of(gi) <= EIGH_MAX)
+      small.push_back({Gram.p + groups[gi].goff, evals.p + eoff[gi], info.p + gi, dim_of(gi)});
+    else
+      large.push_back(gi);
+  }
+  std::sort(large.begin(), large.end(), [&](size_t x, size_t y) { return dim_of(x) > dim_of(y); });
+  const int na = (int)std::min<size_t>(Context::kAux, large.size());
+  int lwork = 0;
+  if (na > 0)
+    solver_check(cusolverDnDsyevd_bufferSize(c.solver, CUSOLVER_EIG_MODE_VECTOR, CUBLAS_FILL_MODE_UPPER, maxd, Gram.p,
+                                             maxd, evals.p, &lwork),
+                 "syevd_bufferSize");
+  DArr<double> work;
+  work.alloc((size_t)std::max(lwork, 1) * std::max(na, 1), c.stream);
+  cuda_check(cudaEventRecord(c.fork_ev, c.stream), "record");
+  for (int a = 0; a < na; ++a) {
+    if (!c.aux[a]) cuda_check(cudaStreamCreateWithFlags(&c.aux[a], cudaStreamNonBlocking), "aux stream");
+    if (!c.aux_ev[a]) cuda_check(cudaEventCreateWithFlags(&c.aux_ev[a], cudaEventDisableTiming), "aux event");
+    if (!c.aux_solver[a]) {
+      solver_check(cusolverDnCreate(&c.aux_solver[a]), "cusolverDnCreate");
+      solver_check(cusolverDnSetStream(c.aux_solver[a], c.aux[a]), "cusolverDnSetStream");
+    }
+    cuda_check(cudaStreamWaitEvent(c.aux[a], c.fork_ev, 0), "wait");
+  }
+  DArr<EighJob> dsmall;
+  dsmall.upload(small, c.stream);
+  launch_eigh(dsmall.p, (int)small.size(), c.stream);
+  cuda_check(cudaGetLastError(), "eigh launch");
+  for (size_t q = 0; q < large.size(); ++q) {
+    const size_t gi = large[q];
     auto& g = groups[gi];
-    int d = direction == 0 ? g.nr : g.nc;
-    const int a = (int)(q % na);
+    const int d = dim_of(gi), a = (int)(q % na);
     solver_check(cusolverDnDsyevd(c.aux_solver[a], CUSOLVER_EIG_MODE_VECTOR, CUBLAS_FILL_MODE_UPPER, d, Gram.p + g.goff, d,
                                   evals.p + eoff[gi], work.p + (size_t)a * std::max(lwork, 1), lwork, info.p + gi),
                  "syevd");

@@ -148,7 +148,7 @@ struct GemmPlan {
   int ntiles = 0, cap = 32;
   double flops = 0;
   void upload(GemmBuilder& g, cudaStream_t s);
-  void run(cudaStream_t s) const;
+  void run(cudaStream_t s, long b_shift = 0, long c_shift = 0) const;
 };
 struct GemmBuilder {
   std::vector<GemmTile> tiles;
@@ -229,10 +229,11 @@ struct Context {
   long sigma_calls = 0;
   cudaEvent_t ev0 = nullptr, ev1 = nullptr;
   // auxiliary streams/events for the independent per-sector eigenproblems of the decimation
-  static constexpr int kAux = 4;
-  cudaStream_t aux[kAux] = {nullptr, nullptr, nullptr, nullptr};
-  cusolverDnHandle_t aux_solver[kAux] = {nullptr, nullptr, nullptr, nullptr};
-  cudaEvent_t aux_ev[kAux + 1] = {nullptr, nullptr, nullptr, nullptr, nullptr};
+  // (created by the first decimation that needs them)
+  static constexpr int kAux = 8;
+  cudaStream_t aux[kAux] = {};
+  cusolverDnHandle_t aux_solver[kAux] = {};
+  cudaEvent_t aux_ev[kAux] = {}, fork_ev = nullptr;
   // wall seconds per phase of the two-site step (stream-synchronised):
   // 0 W-contracted operators, 1 sigma work lists, 2 diagonal, 3 Davidson,
   // 4 decimation, 5 environment update

@@ -69,9 +69,11 @@ long launch_count();
 void count_launches(long n);
 
 // cap: the tile edge the tiles were cut with (one of GEMM_CAPS), or 64: then every listed
-// tile is taken by four thread blocks, one per quarter (a list of a quarter of the length)
+// tile is taken by four thread blocks, one per quarter (a list of a quarter of the length).
+// Every B is read b_shift elements and every C written c_shift elements further than its
+// descriptor says (a plan made for one vector serves any).
 void launch_gemm(const GemmTile* d_tiles, int ntiles, const GemmTask* d_tasks,
-                 const GemmTerm* d_terms, int cap, cudaStream_t s);
+                 const GemmTerm* d_terms, int cap, cudaStream_t s, long b_shift = 0, long c_shift = 0);
 void launch_combo(const ComboOut* d_outs, int nouts, long max_nnz, const ComboTerm* d_terms,
                   cudaStream_t s);
 void launch_copy(const CopyJob* d_jobs, int njobs, int max_elems, cudaStream_t s);
@@ -80,12 +82,18 @@ void launch_fill(double* p, long n, double v, cudaStream_t s);
 // vector ops (FP64, length n)
 // y = a x + b y (b == 0: y is only written)
 void launch_axpby(long n, double a, const double* x, double b, double* y, cudaStream_t s);
+// Workspace of the reductions below: partial sums of up to DOT_MAX dots over DOT_BLOCKS blocks
+// and a counter (zero before the first use; every launch leaves it at zero).  One launch
+// at a time may use it.
+constexpr int DOT_MAX = 49, DOT_BLOCKS = 304;
+struct DotWork {
+  double* part;  // DOT_MAX * DOT_BLOCKS
+  unsigned* count;
+};
 // dots[j] = <V_j, x> for j < m, V row-major [m][n]; result written to d_out[m] (deterministic)
-void launch_multidot(const double* V, long ldv, int m, const double* x, long n, double* d_part,
-                     int nblk, double* d_out, cudaStream_t s);
-// y = sum_j c[j] V_j  (c on device)
-void launch_combine_vectors(const double* V, long ldv, int m, const double* d_c, long n, double* y,
-                            cudaStream_t s);
+// and, where G is given, to row and column `col` of G
+void launch_multidot(const double* V, long ldv, int m, const double* x, long n, DotWork w, double* d_out,
+                     cudaStream_t s, double* G = nullptr, int ldg = 0, int col = 0);
 // t = r / (theta - diag), |denominator| clamped to >= eps
 void launch_precond(long n, const double* r, const double* diag, double theta, double eps,
                     double* t, cudaStream_t s);
@@ -103,18 +111,32 @@ void launch_diag_extract(const DiagJob* d_jobs, int njobs, int max_rows, cudaStr
 // thread block; eigenvalue to scal[0], eigenvector to y[0..m).  false (nothing
 // launched) if m is outside [1, RR_MAX_SUB]
 constexpr int RR_MAX_SUB = 48;
+// Eigen-decompositions of symmetric d x d matrices (row-major, d <= EIGH_MAX), one thread block
+// each: w the eigenvalues in ascending order, row i of G the eigenvector of w[i]; *info is set to
+// 1 (and w to NaN) if the matrix is not finite
+constexpr int EIGH_MAX = 32;
+struct EighJob {
+  double* G;
+  double* w;
+  int* info;
+  int d;
+};
+void launch_eigh(const EighJob* d_jobs, int njobs, cudaStream_t s);
 bool launch_rr(const double* G, int ldg, int m, double* y, double* scal, cudaStream_t s);
-// r = hx - theta x (theta on device)
-void launch_resid(long n, const double* hx, const double* x, const double* d_theta, double* r, cudaStream_t s);
-// t = r / (theta - diag), theta on device
-void launch_precond_dev(long n, const double* r, const double* diag, const double* d_theta, double eps, double* t,
-                        cudaStream_t s);
-// t -= sum_j c[j] V_j (c on device)
-void launch_sub_combine(const double* V, long ldv, int m, const double* d_c, long n, double* t, cudaStream_t s);
+// One Davidson iteration's vectors from the subspace V, its sigma vectors S and the Ritz
+// coefficients c: x = sum_j c_j V_j, hx = sum_j c_j S_j, r = hx - theta x (theta on device), the
+// diagonal correction t = r / (theta - diag) with |denominator| >= eps, and *rr = |r|^2
+void launch_ritz(const double* V, const double* S, long ldv, int m, const double* d_c, long n, const double* d_theta,
+                 const double* diag, double eps, double* x, double* hx, double* r, double* t, DotWork w, double* rr,
+                 cudaStream_t s);
+// t -= sum_j c[j] V_j (c on device), then dots[j] = <V_j, t>
+void launch_project(const double* V, long ldv, int m, const double* d_c, long n, double* t, DotWork w, double* dots,
+                    cudaStream_t s);
+// t -= sum_j c[j] V_j (c on device), then *tt = |t|^2
+void launch_project_norm(const double* V, long ldv, int m, const double* d_c, long n, double* t, DotWork w, double* tt,
+                         cudaStream_t s);
 // y = x / sqrt(*nrm2)
 void launch_scale_rsqrt(long n, const double* x, const double* d_nrm2, double* y, cudaStream_t s);
-// G[i][col] = G[col][i] = dots[i], i < m1
-void launch_gcol(const double* dots, int m1, double* G, int ld, int col, cudaStream_t s);
 // G[0] = theta / xn2
 void launch_restart_g(double* G, const double* d_theta, const double* d_xn2, cudaStream_t s);
 
