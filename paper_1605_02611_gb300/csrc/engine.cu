@@ -3,6 +3,7 @@
 // in the kernels of kernels.cu (cuSOLVER syevd serves the dense symmetric
 // eigenproblems of the decimation step).
 #include <algorithm>
+#include <atomic>
 #include <cstdint>
 #include <cstdio>
 #include <chrono>
@@ -12,6 +13,7 @@
 #include <map>
 #include <mutex>
 #include <numeric>
+#include <system_error>
 #include <thread>
 #include <tuple>
 
@@ -812,6 +814,38 @@ void env_update_right(Context& c, Tilde& rt, const SiteT& B, int site, Env& out)
     run_builder(c, g2);
     b0 = b1;
   }
+}
+
+// ---------------------------------------------------------------- host threads
+
+void host_parallel(long n, long work, const std::function<void(long)>& f) {
+  const unsigned hw = std::max(1u, std::thread::hardware_concurrency());
+  const long nth = std::min({n, (long)std::min(16u, hw), work / 4000 + 1});
+  if (nth <= 1) {
+    for (long i = 0; i < n; ++i) f(i);
+    return;
+  }
+  std::atomic<long> next{0};
+  std::exception_ptr err;
+  std::mutex mu;
+  auto run = [&] {
+    try {
+      for (long i = next.fetch_add(1); i < n; i = next.fetch_add(1)) f(i);
+    } catch (...) {
+      next = n;
+      std::lock_guard<std::mutex> lk(mu);
+      if (!err) err = std::current_exception();
+    }
+  };
+  std::vector<std::thread> th;
+  try {
+    for (long w = 1; w < nth; ++w) th.emplace_back(run);
+  } catch (const std::system_error&) {
+    // no more threads to be had: the ones there are do it
+  }
+  run();
+  for (auto& t : th) t.join();
+  if (err) std::rethrow_exception(err);
 }
 
 // ---------------------------------------------------------------- sigma

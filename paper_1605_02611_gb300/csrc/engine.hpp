@@ -6,6 +6,7 @@
 
 #include <array>
 #include <cstdint>
+#include <functional>
 #include <memory>
 #include <stdexcept>
 #include <string>
@@ -306,6 +307,10 @@ void env_update_right(Context& c, Tilde& rt, const SiteT& B, int site, Env& out)
 
 void build_sigma_plan(Context& c, Tilde& lt, Tilde& rt, int k, SigmaPlan& plan);
 void run_sigma(Context& c, SigmaPlan& plan, const double* x, double* y);
+// f(0) .. f(n - 1) on the host threads, each index once in no fixed order; work: an estimate of
+// the steps in all (a thread costs about 20 us, so few of them run in the calling thread alone).
+// The first exception is thrown on to the caller after every thread has ended.
+void host_parallel(long n, long work, const std::function<void(long)>& f);
 void build_tma_plan(Context& c, Tilde& lt, Tilde& rt, int k, SigmaPlan& plan, int nslices);
 void run_tma_sigma(Context& c, SigmaPlan& plan, const double* x, double* y);
 // non-zero if a tensor-core launch of the plan reported a bounded wait that ran out
