@@ -145,8 +145,8 @@ __host__ __device__ inline uint32_t tm_idesc_bf16(int n, bool negA) {
 }
 
 // Host: the stage counts of a launch of `mode` (operands of nsl slices) over these tiles
-// (for the grid the launch will use); reduce mode: sets every
-// tile's pad (its stages) and nseg.  Returns false if a term is malformed (k not a positive
+// (for the grid the launch will use).  The tiles are put in an order that levels the work of the
+// CTAs; reduce mode: every tile's pad (its stages) and nseg are set.  Returns false if a term is malformed (k not a positive
 // multiple of 16), belongs to two tiles, or the lists would be too long.
 bool tma_plan_lists(int mode, int nsl, std::vector<TmTile>& tiles, const std::vector<TmTerm>& terms, TmListPlan& out);
 // Device: fills the copy lists (stages: total entries, pieces: total * tma_pieces(mode,
