@@ -250,8 +250,6 @@ def run_ours(args, rank, world, local_rank):
     stream = torch.cuda.Stream()
     ctx = G.Context(h, eri, N, w["two_sz"], stream=stream.cuda_stream)
     ctx.set_precision(args.precision)
-    if args.stage1_stacked:
-        ctx.set_stage1_stacked(True)
     if args.fp64_w_sums:
         ctx.set_tc_combos(False)
     if args.env_precision:
@@ -426,8 +424,7 @@ def run_ours(args, rank, world, local_rank):
         # cores actually execute for the slices are reported beside it, not in frac
         roof = {"bound": "tensor", "achieved": ach_k, "peak": peak, "unit": "TFLOP/s",
                 "frac": ach_k / peak, "traffic": TRAFFIC.get(args.precision) if args.workload == "k40_m2000" else None,
-                "kernel": ("gemm_tma_kernel<1>+<2> (sigma stages 1+2, TMA-staged)" if args.precision >= 4 else
-                           "gemm_bf16_tc_kernel (sigma stages 1+2)") + f", precision {args.precision}",
+                "kernel": f"gemm_tma_kernel<1>+<2> (sigma stages 1+2, TMA-staged), precision {args.precision}",
                 "executed_tflops": ach_k * nprod,
                 "products_per_multiply_add": nprod,
                 "peak_note": f"{src} bf16 dense, sustained (kernel timed inside a long step); achieved and frac "
@@ -440,7 +437,7 @@ def run_ours(args, rank, world, local_rank):
         "config": {"workload": workload_name(args, sig_calls / args.steps),
                    "psi_nnz": nnz, "parallelism": f"replicas{world}", "l2": "inputs larger than L2 (no flush)",
                    "setup_s": round(setup_s, 1), "setup_launches": int(setup_launches),
-                   "stage1": "stacked" if args.stage1_stacked else "per-sector",
+                   "stage1": "stacked",
                    "w_sums": "fp64" if args.fp64_w_sums else
                    (f"fp64 (tensor-core sums failed: {w_sums_failed})" if w_sums_failed else
                     "tensor cores (bf16x3) for sums of >= 1e5 terms that feed only the sigma, fp64 otherwise")},
@@ -614,7 +611,7 @@ def main():
     ap.add_argument("--batched", type=int, default=0,
                     help="> 0: batched H_eff.psi over this many independent problems instead of the step bench")
     ap.add_argument("--stage1-stacked", action="store_true",
-                    help="tensor-core sigma with stacked right operands in stage 1")
+                    help="no effect: stage 1 of the tensor-core sigma always runs on stacked right operands")
     ap.add_argument("--fp64-w-sums", action="store_true",
                     help="form every W-contracted sum on the FP64 units (default: large sums that feed only "
                          "the tensor-core sigma run on the tensor cores)")
