@@ -1,5 +1,5 @@
-// Tensor-core (tcgen05, sm_103a) grouped block GEMM for the mixed-precision
-// sigma vector: BF16 operands, FP32 accumulation in tensor memory.
+// Tensor-core (tcgen05, sm_103a) grouped block GEMM of the three-slice environment update and
+// the large W-contracted operator sums: BF16 operands, FP32 accumulation in tensor memory.
 //
 // Same work-list model as the FP64 kernel: an output tile (128 rows x up to 128
 // columns) of one output block is the sum over the block's term list (the
