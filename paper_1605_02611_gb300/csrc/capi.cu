@@ -433,7 +433,7 @@ gbdmrg_status gbdmrg_sigma(gbdmrg_ctx* ctx, const double* psi, double* sigma, in
     auto& plan = c.plan;
     const size_t bytes = plan.psi.nnz * sizeof(double);
     if (on_device) {
-      gbdmrg::run_sigma(c, plan, psi, sigma);
+      gbdmrg::run_sigma_caller(c, plan, psi, sigma);
     } else {
       gbdmrg::cuda_check(cudaMemcpyAsync(plan.in.p, psi, bytes, cudaMemcpyHostToDevice, c.stream), "h2d");
       gbdmrg::run_sigma(c, plan, plan.in.p, plan.out.p);
@@ -479,7 +479,7 @@ gbdmrg_status gbdmrg_sigma_timing(gbdmrg_ctx* ctx, int32_t reps, const double* p
     gbdmrg::cuda_check(cudaEventCreate(&e0), "event");
     gbdmrg::cuda_check(cudaEventCreate(&e1), "event");
     gbdmrg::cuda_check(cudaEventRecord(e0, c.stream), "record");
-    for (int r = 0; r < reps; ++r) gbdmrg::run_sigma(c, c.plan, psi_dev, sigma_dev);
+    for (int r = 0; r < reps; ++r) gbdmrg::run_sigma_caller(c, c.plan, psi_dev, sigma_dev);
     gbdmrg::cuda_check(cudaEventRecord(e1, c.stream), "record");
     gbdmrg::cuda_check(cudaEventSynchronize(e1), "sync");
     if (c.plan.tensor() && gbdmrg::plan_error(c, c.plan))

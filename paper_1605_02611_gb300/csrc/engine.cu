@@ -17,8 +17,11 @@
 #include <thread>
 #include <tuple>
 
+#include <cuda.h>  // types of cuMemGetAddressRange (reached through the runtime)
+
 #include "engine.hpp"
 #include "mlp.hpp"
+#include "vector_access.hpp"
 
 namespace gbdmrg {
 
@@ -977,6 +980,45 @@ void run_sigma(Context& c, SigmaPlan& plan, const double* x, double* y) {
     plan.stage1[i].run(c.stream, x - plan.in.p, 0);
     plan.stage2[i].run(c.stream, 0, y - plan.out.p);
   }
+}
+
+// the allocation that p lies in, if p is device memory of the current device
+static bool device_allocation(const void* p, uintptr_t* base, size_t* size) {
+  using RangeFn = CUresult (*)(CUdeviceptr*, size_t*, CUdeviceptr);
+  static const RangeFn range = [] {
+    void* f = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    if (cudaGetDriverEntryPointByVersion("cuMemGetAddressRange", &f, 12000, cudaEnableDefault, &q) != cudaSuccess ||
+        q != cudaDriverEntryPointSuccess)
+      return (RangeFn) nullptr;
+    return reinterpret_cast<RangeFn>(f);
+  }();
+  cudaPointerAttributes at;
+  int dev = -1;
+  if (cudaPointerGetAttributes(&at, p) != cudaSuccess || cudaGetDevice(&dev) != cudaSuccess) {
+    cudaGetLastError();  // the copy of the vector says what is wrong with it
+    return false;
+  }
+  CUdeviceptr b = 0;
+  if (!range || at.type != cudaMemoryTypeDevice || at.device != dev ||
+      range(&b, size, (CUdeviceptr)(uintptr_t)p) != CUDA_SUCCESS)
+    return false;
+  *base = (uintptr_t)b;
+  return true;
+}
+
+void run_sigma_caller(Context& c, SigmaPlan& plan, const double* x, double* y) {
+  const size_t bytes = plan.psi.nnz * sizeof(double);
+  auto direct = [&](const void* p) {
+    uintptr_t base = 0;
+    size_t size = 0;
+    const bool dev = device_allocation(p, &base, &size);
+    return direct_vector((uintptr_t)p, bytes, dev, base, size);
+  };
+  const bool dx = direct(x), dy = direct(y);
+  if (!dx) cuda_check(cudaMemcpyAsync(plan.in.p, x, bytes, cudaMemcpyDeviceToDevice, c.stream), "d2d");
+  run_sigma(c, plan, dx ? x : plan.in.p, dy ? y : plan.out.p);
+  if (!dy) cuda_check(cudaMemcpyAsync(y, plan.out.p, bytes, cudaMemcpyDeviceToDevice, c.stream), "d2d");
 }
 
 void compute_diag(Context& c, Tilde& lt, Tilde& rt, int k, const PsiLayout& P, double* diag) {

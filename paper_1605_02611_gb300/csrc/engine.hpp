@@ -307,6 +307,8 @@ void env_update_right(Context& c, Tilde& rt, const SiteT& B, int site, Env& out)
 
 void build_sigma_plan(Context& c, Tilde& lt, Tilde& rt, int k, SigmaPlan& plan);
 void run_sigma(Context& c, SigmaPlan& plan, const double* x, double* y);
+// the same for vectors of a caller, which need not be what a kernel can read or write in place
+void run_sigma_caller(Context& c, SigmaPlan& plan, const double* x, double* y);
 // f(0) .. f(n - 1) on the host threads, each index once in no fixed order; work: an estimate of
 // the steps in all (a thread costs about 20 us, so few of them run in the calling thread alone).
 // The first exception is thrown on to the caller after every thread has ended.
