@@ -289,7 +289,7 @@ struct TmaPlan {
     DArr<long> sfirst;
     DArr<TmStage> stages;
     DArr<TmPiece> pieces;
-    int grid = 0, ctas = 1, slots = 0, slot_bytes = 0;
+    int grid = 0, slots = 0, slot_bytes = 0;
     long total = 0;
     // the stage counts on the host (reduce mode: sets the tiles' stages and segments,
     // so it comes before the tiles are uploaded); throws on a malformed term
@@ -297,7 +297,6 @@ struct TmaPlan {
       TmListPlan lp;
       if (!tma_plan_lists(mode, nsl, tiles, terms, lp)) throw Error(ST_ECUDA, "internal: malformed TMA term list");
       grid = lp.grid;
-      ctas = lp.ctas;
       slots = lp.slots;
       slot_bytes = lp.slot_bytes;
       total = lp.total;
@@ -310,11 +309,11 @@ struct TmaPlan {
     }
     // the lists themselves, on the device, from the uploaded tiles and terms
     void fill(int mode, int nsl, const TmTile* d_tiles, int ntiles, const TmTerm* d_terms, cudaStream_t s) {
-      cuda_check(launch_fill_lists(mode, nsl, slots, d_tiles, ntiles, d_terms, tpiece0.p, sorder.p, sfirst.p, total, stages.p,
+      cuda_check(launch_fill_lists(mode, nsl, d_tiles, ntiles, d_terms, tpiece0.p, sorder.p, sfirst.p, total, stages.p,
                                    pieces.p, s),
                  "list fill");
     }
-    TmListsDev dev() const { return {grid, ctas, slots, slot_bytes, cta_stage.p, stages.p, pieces.p}; }
+    TmListsDev dev() const { return {grid, slots, slot_bytes, cta_stage.p, stages.p, pieces.p}; }
   };
   struct Chunk {
     DArr<TmTile> t1, t2;
@@ -738,32 +737,41 @@ void build_tma_plan(Context& c, Tilde& lt, Tilde& rt, int k, SigmaPlan& plan, in
     if (off < 0 || rows < 1 || cols < 1 || rows % 16 != 0 || cols % 16 != 0 || off % 8 != 0 ||
         (size_t)(off + nsl * rows * cols) > buf.n)
       throw Error(ST_ECUDA, "internal: tensor map outside its buffer");
-    // boxes of all slices, then (two or three slices) of one
-    const int first = (int)maps.size();
-    for (int bs = nsl; bs >= 1; bs -= std::max(1, nsl - 1)) {
-      CUtensorMap m;
-      if (!encode_slice_map(&m, buf.p + off, (uint64_t)rows, (uint64_t)cols, nsl, (uint32_t)box_rows, bs))
-        throw Error(ST_ECUDA, "cuTensorMapEncodeTiled failed");
-      maps.push_back(m);
-      minfo.push_back({rows, cols, box_rows});
-    }
-    return first;
+    const int id = (int)maps.size();
+    CUtensorMap m;
+    if (!encode_slice_map(&m, buf.p + off, (uint64_t)rows, (uint64_t)cols, nsl, (uint32_t)box_rows))
+      throw Error(ST_ECUDA, "cuTensorMapEncodeTiled failed");
+    maps.push_back(m);
+    minfo.push_back({rows, cols, box_rows});
+    return id;
   };
-  // width of the stage-1 N tiles: with two or three slices the largest whose ring holds the longest
-  // term with two CTAs per SM (one CTA per SM is far slower)
+  // Two or three slices: a term stays in the ring whole, so a block that is longer than
+  // tm_term_pieces is cut into equal parts (a term each).  Stage 1: the widest N tiles whose ring
+  // holds the longest part.
+  // Three and two slices, ms per sigma, against whole terms with one CTA per SM and twice the ring,
+  // and one 16-column copy of one slice per stage where they did not fit that either: K=16, M=2000
+  // (sectors of up to 238) 67.6 and 34.8 -> 15.1 and 8.8; K=16, M=1000 (121) 4.02 and 2.68 -> 2.41
+  // and 1.45; K=20, M=800 (83) 3.34 and 1.62 -> 2.72 and 1.60; K=40, M=2000 (115, three slices)
+  // 47.8 -> 33.2.
   int n1max = tm_max_n(TM_MODE_STORE_BF16, nsl);
   const int n2max = tm_max_n(TM_MODE_REDUCE_F32, nsl);
+  auto parts_of = [&](int kk, int limit) {
+    return nsl == 1 ? 1 : (kk / TM_PIECE_COLS + limit - 1) / limit;
+  };
+  // columns [first, second) of part i of `parts`
+  auto part_cols = [](int kk, int parts, int i) {
+    const int kp = kk / TM_PIECE_COLS;
+    return std::make_pair(kp * i / parts * TM_PIECE_COLS, kp * (i + 1) / parts * TM_PIECE_COLS);
+  };
   if (nsl > 1) {
     int kmax = 16;
     for (int qr = 0; qr < nR; ++qr) kmax = std::max(kmax, pad16(Rb.dim[qr]));
-    for (int n = n1max; n >= 64; n -= 16)
-      if (tm_fit_slots(nsl, n, 2) >= kmax / TM_PIECE_COLS) {
-        n1max = n;
-        break;
-      }
+    const int parts = parts_of(kmax, TM_TERM_PIECES), len = (kmax / TM_PIECE_COLS + parts - 1) / parts;
+    while (n1max > 64 && tm_term_pieces(nsl, n1max) < len) n1max -= 16;
   }
   std::vector<std::vector<std::array<int, 3>>> nt1(ng);  // per g': (row0, width, Psi map) of the stage-1 N tiles
   std::vector<int> a1map(ng, -1);
+  int n1wide = 16, n2wide = 16;
   for (int gp = 0; gp < ng; ++gp) {
     if (a1rows[gp] == 0) continue;
     const int parts = (gR[gp] + n1max - 1) / n1max;
@@ -772,9 +780,12 @@ void build_tma_plan(Context& c, Tilde& lt, Tilde& rt, int k, SigmaPlan& plan, in
       const int w = std::min(gR[gp] - r0, pad16((gR[gp] - r0 + (parts - p) - 1) / (parts - p)));
       nt1[gp].push_back({r0, w, add_map(tp->psi_b, goff[gp] * nsl, gR[gp], gC[gp], w)});
       r0 += w;
+      n1wide = std::max(n1wide, w);
     }
     a1map[gp] = add_map(tp->a1, a1off[gp] * nsl, a1rows[gp], gC[gp], 128);
   }
+  for (int ql = 0; ql < nL; ++ql) n2wide = std::max(n2wide, std::min(n2max, pad16(Lb.dim[ql])));
+  const int limit1 = tm_term_pieces(nsl, n1wide), limit2 = tm_term_pieces(nsl, n2wide);
   // X^T region of (chunk, g')
   std::vector<std::vector<int>> xtmap(nch, std::vector<int>(ng, -1));
   for (int ci = 0; ci < nch; ++ci)
@@ -806,11 +817,17 @@ void build_tma_plan(Context& c, Tilde& lt, Tilde& rt, int k, SigmaPlan& plan, in
     std::vector<std::array<size_t, 3>> at1(ng + 1, std::array<size_t, 3>{0, 0, rowmap.size()});  // tiles, terms, rows
     for (int gp = 0; gp < ng; ++gp) {
       at1[gp + 1] = at1[gp];
+      size_t nterm[4];  // terms of the K block of n2'
+      for (int n2p = 0; n2p < 4; ++n2p) {
+        const int qrp = Rb.find(gq[gp].first + LQA[n2p], gq[gp].second + LQB[n2p]);
+        nterm[n2p] = qrp < 0 ? 0 : (size_t)parts_of(pad16(Rb.dim[qrp]), limit1);
+      }
       for (const Run& run : runs[gp]) {
         if (run.chunk != ci) continue;
         const size_t nrow = (size_t)((run.r1 - run.r0 + 127) / 128);
         at1[gp + 1][0] += nrow * nt1[gp].size();
-        at1[gp + 1][1] += nrow * nt1[gp].size() * (size_t)__builtin_popcount((unsigned)run.mask);
+        for (int n2p = 0; n2p < 4; ++n2p)
+          if ((run.mask >> n2p) & 1) at1[gp + 1][1] += nrow * nt1[gp].size() * nterm[n2p];
         at1[gp + 1][2] += nrow * 128;
       }
     }
@@ -835,7 +852,12 @@ void build_tma_plan(Context& c, Tilde& lt, Tilde& rt, int k, SigmaPlan& plan, in
               const int qrp = Rb.find(gq[gp].first + LQA[n2p], gq[gp].second + LQB[n2p]);
               const int coff = cpos[qrp * 4 + n2p][1];
               const int kk = pad16(Rb.dim[qrp]);
-              m1[im++] = {a1map[gp], nt[2], coff, (int)r0, coff, nt[0], kk, nsl << 4};
+              const int parts = parts_of(kk, limit1);
+              for (int p = 0; p < parts; ++p) {
+                const auto cols = part_cols(kk, parts, p);
+                m1[im++] = {a1map[gp], nt[2], coff + cols.first, (int)r0, coff + cols.first, nt[0],
+                            cols.second - cols.first, nsl << 4};
+              }
               ksum += kk * npair;
               st1[gp][0] += (kk + 63) / 64 * npair;
             }
@@ -909,8 +931,13 @@ void build_tma_plan(Context& c, Tilde& lt, Tilde& rt, int k, SigmaPlan& plan, in
               if (rpp[0] != gp) continue;
               const int mid_ = lmid[beta][n1 * 4 + n1p];
               const int wc = wcls.at(pad16(Lb.dim[qlp]));
-              base.push_back({xtmap[ci][gp], lmap[wc][nw / 16], rpp[1], (int)xrow[(size_t)beta * ng + gp], 0,
-                              (int)(mblk_row[mid_][bl] + c0), pad16(Lb.dim[qlp]), (int)lneg[beta][n1 * 4 + n1p]});
+              const int kk = pad16(Lb.dim[qlp]), parts = parts_of(kk, limit2);
+              for (int p = 0; p < parts; ++p) {
+                const auto cols = part_cols(kk, parts, p);
+                base.push_back({xtmap[ci][gp], lmap[wc][nw / 16], rpp[1] + cols.first, (int)xrow[(size_t)beta * ng + gp],
+                                cols.first, (int)(mblk_row[mid_][bl] + c0), cols.second - cols.first,
+                                (int)lneg[beta][n1 * 4 + n1p]});
+              }
             }
           }
           if (base.empty()) continue;
@@ -979,8 +1006,8 @@ void build_tma_plan(Context& c, Tilde& lt, Tilde& rt, int k, SigmaPlan& plan, in
             throw Error(ST_ECUDA, "internal: malformed TMA tile");
           for (int t = tl.t0; t < tl.t1; ++t) {
             const TmTerm& m = mm[t];
-            if (((m.neg >> 4) & 15) != nsl || m.amap < 0 || m.amap + (nsl > 1) >= (int)minfo.size() || m.bmap < 0 ||
-                m.bmap + (nsl > 1) >= (int)minfo.size() || minfo[m.amap].box != 128 || minfo[m.bmap].box != tl.n || m.k < 16 ||
+            if (((m.neg >> 4) & 15) != nsl || m.amap < 0 || m.amap >= (int)minfo.size() || m.bmap < 0 ||
+                m.bmap >= (int)minfo.size() || minfo[m.amap].box != 128 || minfo[m.bmap].box != tl.n || m.k < 16 ||
                 m.k % 16 || m.ax % 8 || m.bx % 8 || m.ay % 16 || m.by % 16 || m.ax < 0 || m.bx < 0 || m.ay < 0 ||
                 m.by < 0 || m.ay >= minfo[m.amap].rows || m.by >= minfo[m.bmap].rows ||
                 m.ax + m.k > minfo[m.amap].cols || m.bx + m.k > minfo[m.bmap].cols)
@@ -1815,8 +1842,8 @@ void env_update_exact(Context& c, Tilde& t, const SiteT& A, int site, Env& out, 
 // maps and row maps are concatenated, so one persistent kernel walks the tiles of
 // every problem (one launch per slice count where the problems differ in it).  Optionally the
 // whole sequence (conversions, stage launches, gathers) is captured once in a CUDA graph and
-// replayed.  (Eight problems, K 12-20, M 64-256, three slices: 1.29 ms; 9.04 ms on per-sector
-// tiles staged by cp.async.)
+// replayed.  (Eight problems, three slices, device time batched and one by one: K 12-20, M 64-256
+// 1.03 and 1.20 ms; K 16-32, M 362-992 16.4 and 16.7 ms.)
 struct BatchPlan {
   std::vector<Context*> ctx;
   cudaStream_t stream = nullptr;
@@ -1847,9 +1874,50 @@ struct BatchPlan {
   }
 };
 
-// chunk ch of the problems with nsl slices as one launch per stage; map0, row0: every problem's first
-// tensor map and row-map entry in the concatenated arrays
-static void batch_launch(BatchPlan& b, size_t ch, int nsl, const std::vector<int>& map0, const std::vector<long>& row0) {
+// Chunk ch of the problems with nsl slices, in groups that share a launch per stage.  With two or
+// three slices a launch's ring follows from its widest tile and has to hold its longest term, which
+// may come from different problems: a problem joins the first group whose ring then still does.
+static std::vector<std::vector<size_t>> batch_groups(const BatchPlan& b, size_t ch, int nsl) {
+  struct Need {
+    int n[2] = {16, 16}, k[2] = {16, 16};  // widest tile and longest term of the stages
+  };
+  std::vector<std::vector<size_t>> groups;
+  std::vector<Need> needs;
+  for (size_t p = 0; p < b.ctx.size(); ++p) {
+    const TmaPlan& tp = *b.ctx[p]->plan.tm;
+    if (tp.nsl != nsl || ch >= tp.chunks.size()) continue;
+    const TmaPlan::Chunk& c = tp.chunks[ch];
+    Need own;
+    for (const TmTile& t : c.ht1) own.n[0] = std::max(own.n[0], t.n);
+    for (const TmTile& t : c.ht2) own.n[1] = std::max(own.n[1], t.n);
+    for (const TmTerm& m : c.hm1) own.k[0] = std::max(own.k[0], m.k);
+    for (const TmTerm& m : c.hm2) own.k[1] = std::max(own.k[1], m.k);
+    size_t g = 0;
+    for (; g < groups.size(); ++g) {
+      Need both = needs[g];
+      bool fits = true;
+      for (int i = 0; i < 2; ++i) {
+        both.n[i] = std::max(both.n[i], own.n[i]);
+        both.k[i] = std::max(both.k[i], own.k[i]);
+        fits = fits && (nsl == 1 || both.k[i] / TM_PIECE_COLS <= tm_term_pieces(nsl, both.n[i]));
+      }
+      if (!fits) continue;
+      needs[g] = both;
+      break;
+    }
+    if (g == groups.size()) {
+      groups.emplace_back();
+      needs.push_back(own);
+    }
+    groups[g].push_back(p);
+  }
+  return groups;
+}
+
+// chunk ch of the problems `group` (of nsl slices) as one launch per stage; map0, row0: every problem's
+// first tensor map and row-map entry in the concatenated arrays
+static void batch_launch(BatchPlan& b, size_t ch, int nsl, const std::vector<size_t>& group,
+                         const std::vector<int>& map0, const std::vector<long>& row0) {
   std::vector<TmTile> t1, t2;
   std::vector<TmTerm> m1, m2;
   std::vector<ZeroJob> zj;
@@ -1870,9 +1938,8 @@ static void batch_launch(BatchPlan& b, size_t ch, int nsl, const std::vector<int
       terms.push_back(m);
     }
   };
-  for (size_t p = 0; p < b.ctx.size(); ++p) {
+  for (size_t p : group) {
     const TmaPlan& tp = *b.ctx[p]->plan.tm;
-    if (tp.nsl != nsl || ch >= tp.chunks.size()) continue;
     const TmaPlan::Chunk& c = tp.chunks[ch];
     if (!L.out1) {
       L.out1 = tp.xt.p;
@@ -1937,7 +2004,8 @@ BatchPlan* batch_create(const std::vector<Context*>& ctxs) {
   b->maps.upload(maps, b->stream);
   b->rowmap.upload(rowmap, b->stream);
   for (size_t ch = 0; ch < nch; ++ch)
-    for (int nsl = 1; nsl <= 3; ++nsl) batch_launch(*b, ch, nsl, map0, row0);
+    for (int nsl = 1; nsl <= 3; ++nsl)
+      for (const auto& group : batch_groups(*b, ch, nsl)) batch_launch(*b, ch, nsl, group, map0, row0);
   for (int i = 0; i < 3; ++i) {
     b->conv[i].upload(cj[i], b->stream);
     b->nconv[i] = (int)cj[i].size();

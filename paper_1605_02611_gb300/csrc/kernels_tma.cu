@@ -10,7 +10,7 @@
 // before the launch into per-CTA copy lists (stage word, expected bytes, box coordinates:
 // fill_lists_kernel), so the producer does no term arithmetic.
 //
-// Persistent and warp-specialised, one or two CTAs per SM in the sigma modes (256 tensor-memory
+// Persistent and warp-specialised, two CTAs per SM in the sigma modes (256 tensor-memory
 // columns each), one in the exact mode:
 //   warp 0     fetches its CTA's copy lists 32 stages at a time into shared memory
 //              (1D bulk copies, double-buffered); per stage lane 0 waits for the ring
@@ -36,7 +36,8 @@
 // keep the order term, slice pair, column (they are rounded into the accumulator one by one, and
 // a Davidson solve magnifies another order's rounding), so a term's pieces stay in the ring until
 // its last pair.  Two CTAs per SM: with one, the copies, the products and the epilogue of a tile wait
-// for each other (K=24, one CTA: 3.1 ms).
+// for each other (K=24, one CTA: 3.1 ms).  Blocks of more columns than a term may have
+// (tm_term_pieces) are cut into several terms by the plan.
 // Measured against one pair of swizzled boxes per slice product (16-column boxes in the
 // reduce mode), one CTA per SM: three slices at K=24, M=512 3.19 -> 1.53 ms per sigma, K=40, M=1200
 // 23.1 -> 12.6 ms, K=10, M=150 0.240 -> 0.144 ms; one pass at K=32, M=1024 2.71 -> 1.60 ms.  (Without
@@ -67,14 +68,14 @@ constexpr int TM_BOX_K = 64;                    // exact mode: columns per box (
 constexpr int TM_A_BYTES = 128 * TM_BOX_K * 2;  // 16 KB
 constexpr int TM_REC_BATCH = 32;  // stages of the copy lists fetched per bulk copy
 
-// CTAS: CTAs per SM the launch is made for (the sigma modes; the exact mode has one)
-template <int MODE, int NSL, int CTAS>
+template <int MODE, int NSL>
 struct TmCfg {
   static constexpr bool STORE = MODE == TM_MODE_STORE_BF16;
   static constexpr bool EXACT = MODE == TM_MODE_EXACT_F64;
   // two or three slices: a term's 16-column pieces, one per ring slot, stay until all slice
   // products of the term have been issued
   static constexpr bool CHAIN = !EXACT && NSL > 1;
+  static constexpr int CTAS = tm_ctas(MODE);
   static constexpr int NMAX = tm_max_n(MODE, NSL);
   static constexpr int TMEM = EXACT ? 512 : 256;
   static constexpr int NACC = TMEM / NMAX;
@@ -84,7 +85,7 @@ struct TmCfg {
   static constexpr int B_BYTES = EXACT ? NMAX * TM_BOX_K * 2 : NMAX * TM_PIECE_COLS * 2 * NSL;
   static constexpr int STAGE_BYTES = SLOTS * (A_BYTES + B_BYTES);  // (chains: a launch's own slot size)
   static constexpr int STAGES = EXACT ? 8 : (STORE ? 4 : 6);       // (chains: a launch's own count)
-  static constexpr int SMEM = (CHAIN ? tm_ring_bytes(CTAS) : STAGES * STAGE_BYTES) + 1024;
+  static constexpr int SMEM = (CHAIN ? TM_RING_BYTES : STAGES * STAGE_BYTES) + 1024;
 };
 constexpr int TM_MAX_STAGES = TM_MAX_SLOTS, TM_MAX_ACC = 8;
 constexpr int TM_TERMS = 32;  // term barriers of the chains (a power of two, more than twice the slots)
@@ -109,13 +110,12 @@ __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map
       : "memory");
 }
 
-// box of a column-group map: all of dimension 0, row group y, slices from sl, column group x
-__device__ __forceinline__ void tma_load_groups(uint32_t dst, const CUtensorMap* map, int x, int y, int sl,
-                                                uint64_t* bar) {
+// box of a column-group map: all of dimension 0, row group y, every slice, column group x
+__device__ __forceinline__ void tma_load_groups(uint32_t dst, const CUtensorMap* map, int x, int y, uint64_t* bar) {
   asm volatile(
       "cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5}], "
       "[%6];\n" ::"r"(dst),
-      "l"(map), "r"(0), "r"(y), "r"(sl), "r"(x), "r"(smem_u32(bar))
+      "l"(map), "r"(0), "r"(y), "r"(0), "r"(x), "r"(smem_u32(bar))
       : "memory");
 }
 
@@ -142,14 +142,14 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&v)[16]) {
   asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
 }
 
-template <int MODE, int NSL, int CTAS>
-__global__ void __launch_bounds__(TM_THREADS, CTAS)
+template <int MODE, int NSL>
+__global__ void __launch_bounds__(TM_THREADS, tm_ctas(MODE))
     gemm_tma_kernel(const TmTile* __restrict__ tiles, int ntiles, const TmTerm* __restrict__ terms,
                     const CUtensorMap* __restrict__ maps, const long* __restrict__ rowmap, void* __restrict__ out,
                     int* __restrict__ err, const int* __restrict__ expo, const int* __restrict__ cta_stage,
                     const TmStage* __restrict__ stg, const TmPiece* __restrict__ pcs, int ring_slots,
                     int slot_bytes) {
-  using Cfg = TmCfg<MODE, NSL, CTAS>;
+  using Cfg = TmCfg<MODE, NSL>;
   constexpr bool CHAIN = Cfg::CHAIN;
   const int S = CHAIN ? ring_slots : Cfg::STAGES;
   const int STAGE_BYTES = CHAIN ? slot_bytes : Cfg::STAGE_BYTES;
@@ -272,8 +272,8 @@ __global__ void __launch_bounds__(TM_THREADS, CTAS)
             tma_load_2d(da, maps + q.amap, q.ax, q.ay, &full_b[st]);
             tma_load_2d(db, maps + q.bmap, q.bx, q.by, &full_b[st]);
           } else {
-            tma_load_groups(da, maps + q.amap, q.ax, q.ay, q.as, &full_b[st]);
-            tma_load_groups(db, maps + q.bmap, q.bx, q.by, q.bs, &full_b[st]);
+            tma_load_groups(da, maps + q.amap, q.ax, q.ay, &full_b[st]);
+            tma_load_groups(db, maps + q.bmap, q.bx, q.by, &full_b[st]);
           }
         }
         ++j;
@@ -324,7 +324,7 @@ __global__ void __launch_bounds__(TM_THREADS, CTAS)
         // accumulator.  The pieces' slots are released during the last pair.
         // One thread issues them all and needs several clocks per instruction, so what it executes
         // per product bounds the kernel once its loops, branches and commits outnumber the products.
-        // Terms of up to six pieces (96 columns) that end inside the open segment are straight-line
+        // Terms (up to TM_TERM_PIECES pieces) that end inside the open segment are straight-line
         // code with one commit for all their slots (term barriers, in order), short ones that cross
         // its end too, with a check per product; the others go product by product in a loop.
         // Measured at K=24, M=512 (stage 2): all in loops 1.20-1.50 ms, whatever was moved out of
@@ -355,12 +355,11 @@ __global__ void __launch_bounds__(TM_THREADS, CTAS)
             const uint64_t mw = meta[st];
             const uint32_t fl = (uint32_t)(mw >> 32), id = (uint32_t)mw | ((fl >> 9 & 1u) << 13);
             const uint32_t n = ((uint32_t)mw >> 17 & 63u) << 3;  // rows of B: 8 columns of a slice are n * 16 bytes
-            const bool single = (fl & 256u) != 0;  // one slice of each operand
             tile_done = (fl & 1024u) != 0;
-            const int kp = (int)(fl & 255u), npair = single ? 1 : NPAIR;
-            const uint32_t a0 = al0 | (uint32_t)(single ? 128 : 128 * NSL) << 16, b0 = bl0 | (single ? n : n * NSL) << 16;
-            // the term's pieces: slot offsets of the first six, and their arrival
-            uint32_t off[6];
+            const int kp = (int)(fl & 255u);
+            const uint32_t a0 = al0 | (uint32_t)(128 * NSL) << 16, b0 = bl0 | (n * NSL) << 16;
+            // the term's pieces: their slot offsets and their arrival
+            uint32_t off[TM_TERM_PIECES];
             {
               int s2 = st;
               uint32_t p2 = par;
@@ -374,7 +373,7 @@ __global__ void __launch_bounds__(TM_THREADS, CTAS)
               }
               if (!ok) break;
 #pragma unroll
-              for (int c = 0; c < 6; ++c) off[c] = (uint32_t)(st + c < S ? st + c : st + c - S) * step;
+              for (int c = 0; c < TM_TERM_PIECES; ++c) off[c] = (uint32_t)(st + c < S ? st + c : st + c - S) * step;
             }
             asm volatile("tcgen05.fence::after_thread_sync;\n" ::);
             if (cnt == 0 && !(ok = open())) break;
@@ -402,7 +401,7 @@ __global__ void __launch_bounds__(TM_THREADS, CTAS)
                   }
             };
             using std::integral_constant;
-            if (!single && kp <= 6 && after <= SEG) {
+            if (after <= SEG) {
               const integral_constant<bool, false> no{};
               switch (kp) {
                 case 1: term(integral_constant<int, 1>{}, no); break;
@@ -410,11 +409,11 @@ __global__ void __launch_bounds__(TM_THREADS, CTAS)
                 case 3: term(integral_constant<int, 3>{}, no); break;
                 case 4: term(integral_constant<int, 4>{}, no); break;
                 case 5: term(integral_constant<int, 5>{}, no); break;
-                default: term(integral_constant<int, 6>{}, no); break;
+                default: term(integral_constant<int, TM_TERM_PIECES>{}, no); break;
               }
               cnt = after;
               if (cnt == SEG || tile_done) close();
-            } else if (!single && kp <= 3) {
+            } else if (kp <= 3) {
               const integral_constant<bool, true> yes{};
               switch (kp) {
                 case 1: term(integral_constant<int, 1>{}, yes); break;
@@ -425,14 +424,14 @@ __global__ void __launch_bounds__(TM_THREADS, CTAS)
               if (cnt == SEG || tile_done) close();
             } else {
 #pragma unroll 1
-              for (int q = 0; q < npair && ok; ++q) {
+              for (int q = 0; q < NPAIR && ok; ++q) {
                 uint32_t a = a0 + off[0] + (PAIR_I >> (4 * q) & 15u) * 128u, b = b0 + off[0] + (PAIR_J >> (4 * q) & 15u) * n;
                 int s2 = st;
 #pragma unroll 1
                 for (int c = 0; c < kp; ++c) {
                   if (cnt == 0 && !(ok = open())) break;
                   mma(dacc, sdesc_groups(a), sdesc_groups(b), id, cnt > 0);
-                  if (++cnt == SEG || (tile_done && q == npair - 1 && c == kp - 1)) close();
+                  if (++cnt == SEG || (tile_done && q == NPAIR - 1 && c == kp - 1)) close();
                   a += step;
                   b += step;
                   if (++s2 == S) {
@@ -652,23 +651,23 @@ __global__ void __launch_bounds__(TM_THREADS, CTAS)
   }
 }
 
-template <int MODE, int NSL, int CTAS>
+template <int MODE, int NSL>
 cudaError_t launch_mode(const TmTile* d_tiles, int ntiles, const TmTerm* d_terms, const CUtensorMap* d_maps,
                         const long* d_rowmap, void* out, int* d_err, cudaStream_t s, const int* d_expo,
                         const TmListsDev& lists) {
-  using Cfg = TmCfg<MODE, NSL, CTAS>;
+  using Cfg = TmCfg<MODE, NSL>;
   static const bool attr_ok =
-      cudaFuncSetAttribute(gemm_tma_kernel<MODE, NSL, CTAS>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::SMEM) ==
+      cudaFuncSetAttribute(gemm_tma_kernel<MODE, NSL>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::SMEM) ==
       cudaSuccess;
   if (!attr_ok) return cudaErrorInvalidValue;
   // the lists were built for this grid (every CTA's tiles and stages) and ring
-  if (lists.grid != tma_grid(CTAS, ntiles) || !lists.cta_stage || !lists.stages || !lists.pieces)
+  if (lists.grid != tma_grid(Cfg::CTAS, ntiles) || !lists.cta_stage || !lists.stages || !lists.pieces)
     return cudaErrorInvalidValue;
   if (Cfg::CHAIN && (lists.slots < 1 || lists.slots > TM_MAX_SLOTS || lists.slot_bytes % 1024 != 0 ||
-                     lists.slots * lists.slot_bytes > tm_ring_bytes(CTAS)))
+                     lists.slots * lists.slot_bytes > TM_RING_BYTES))
     return cudaErrorInvalidValue;
   count_tc_launches(1);
-  gemm_tma_kernel<MODE, NSL, CTAS><<<lists.grid, TM_THREADS, Cfg::SMEM, s>>>(
+  gemm_tma_kernel<MODE, NSL><<<lists.grid, TM_THREADS, Cfg::SMEM, s>>>(
       d_tiles, ntiles, d_terms, d_maps, d_rowmap, out, d_err, d_expo, lists.cta_stage, lists.stages, lists.pieces,
       lists.slots, lists.slot_bytes);
   return cudaGetLastError();
@@ -763,16 +762,15 @@ cudaError_t launch_gemm_slices(int mode, int nsl, const TmTile* d_tiles, int nti
                                const long* d_rowmap, void* out, int* d_err, cudaStream_t s, const TmListsDev& lists) {
   if (ntiles <= 0) return cudaSuccess;
   auto go = [&](auto fn) { return fn(d_tiles, ntiles, nullptr, d_maps, d_rowmap, out, d_err, s, nullptr, lists); };
-  const bool two = lists.ctas == 2;
   if (mode == TM_MODE_STORE_BF16) {
-    if (nsl == 1) return go(launch_mode<TM_MODE_STORE_BF16, 1, 2>);
-    if (nsl == 2) return two ? go(launch_mode<TM_MODE_STORE_BF16, 2, 2>) : go(launch_mode<TM_MODE_STORE_BF16, 2, 1>);
-    if (nsl == 3) return two ? go(launch_mode<TM_MODE_STORE_BF16, 3, 2>) : go(launch_mode<TM_MODE_STORE_BF16, 3, 1>);
+    if (nsl == 1) return go(launch_mode<TM_MODE_STORE_BF16, 1>);
+    if (nsl == 2) return go(launch_mode<TM_MODE_STORE_BF16, 2>);
+    if (nsl == 3) return go(launch_mode<TM_MODE_STORE_BF16, 3>);
   }
   if (mode == TM_MODE_REDUCE_F32) {
-    if (nsl == 1) return go(launch_mode<TM_MODE_REDUCE_F32, 1, 2>);
-    if (nsl == 2) return two ? go(launch_mode<TM_MODE_REDUCE_F32, 2, 2>) : go(launch_mode<TM_MODE_REDUCE_F32, 2, 1>);
-    if (nsl == 3) return two ? go(launch_mode<TM_MODE_REDUCE_F32, 3, 2>) : go(launch_mode<TM_MODE_REDUCE_F32, 3, 1>);
+    if (nsl == 1) return go(launch_mode<TM_MODE_REDUCE_F32, 1>);
+    if (nsl == 2) return go(launch_mode<TM_MODE_REDUCE_F32, 2>);
+    if (nsl == 3) return go(launch_mode<TM_MODE_REDUCE_F32, 3>);
   }
   return cudaErrorInvalidValue;
 }
@@ -781,7 +779,7 @@ cudaError_t launch_gemm_exact(const TmTile* d_tiles, int ntiles, const TmTerm* d
                               double* out, int* d_err, cudaStream_t s, const TmListsDev& lists, const int* d_expo) {
   if (ntiles <= 0) return cudaSuccess;
   if (!d_expo || !d_terms) return cudaErrorInvalidValue;
-  return launch_mode<TM_MODE_EXACT_F64, 1, 1>(d_tiles, ntiles, d_terms, d_maps, nullptr, out, d_err, s, d_expo, lists);
+  return launch_mode<TM_MODE_EXACT_F64, 1>(d_tiles, ntiles, d_terms, d_maps, nullptr, out, d_err, s, d_expo, lists);
 }
 
 int tma_grid(int ctas, int ntiles) {
@@ -800,13 +798,9 @@ int tma_pieces(int mode, int nsl) { return mode == TM_MODE_EXACT_F64 ? 1 : tm_sl
 namespace {
 __host__ __device__ inline int slice_pairs(int nsl) { return nsl * (nsl + 1) / 2; }
 
-// pieces of a term: 16 columns each; 16 columns of every slice pair where a term of two or three
-// slices has more pieces than the ring has slots; or (exact mode) 64 columns of every slice pair
-__host__ __device__ inline long term_pieces(const TmTerm& m, bool exact, int nslices, int slots) {
-  if (!exact) {
-    const int kp = m.k / TM_PIECE_COLS;
-    return nslices > 1 && kp > slots ? (long)kp * slice_pairs(nslices) : kp;
-  }
+// pieces of a term: 16 columns each, or (exact mode) 64 columns of every slice pair
+__host__ __device__ inline long term_pieces(const TmTerm& m, bool exact) {
+  if (!exact) return m.k / TM_PIECE_COLS;
   const int nsl = ((m.neg >> 4) & 15) > 1 ? ((m.neg >> 4) & 15) : 1;
   return (long)((m.k + TM_BOX_K - 1) / TM_BOX_K) * slice_pairs(nsl);
 }
@@ -829,7 +823,7 @@ __device__ __forceinline__ void slice_pair(int q, int& l, int& i) {
 // tensor memory over a segment only and the epilogue adds the segments in FP32 with
 // round-to-nearest, so the rounding toward zero of the tensor-core accumulation acts on
 // short sums); exact mode one per level of every term.
-__global__ void fill_lists_kernel(int mode, int nslices, int slots, const TmTile* __restrict__ tiles, int ntiles,
+__global__ void fill_lists_kernel(int mode, int nslices, const TmTile* __restrict__ tiles, int ntiles,
                                   const TmTerm* __restrict__ terms, const int* __restrict__ tpiece0,
                                   const int* __restrict__ sorder, const long* __restrict__ sfirst, long total,
                                   TmStage* __restrict__ stages, TmPiece* __restrict__ pieces) {
@@ -851,32 +845,23 @@ __global__ void fill_lists_kernel(int mode, int nslices, int slots, const TmTile
     const int mid = (t + th + 1) >> 1;
     if (tpiece0[mid] <= p0) t = mid; else th = mid - 1;
   }
-  const long tile_pieces = tpiece0[tl.t1 - 1] + term_pieces(terms[tl.t1 - 1], exact, nslices, slots);
+  const long tile_pieces = tpiece0[tl.t1 - 1] + term_pieces(terms[tl.t1 - 1], exact);
   const int np = (int)min((long)P, tile_pieces - p0);
-  uint32_t piece_bytes = (uint32_t)(128 + tl.n) * bc * 2 * (exact ? 1 : nslices);
+  const uint32_t piece_bytes = (uint32_t)(128 + tl.n) * bc * 2 * (exact ? 1 : nslices);
   const bool last = sl == nst - 1;
   TmTerm m = terms[t];
   long r = p0 - tpiece0[t];
   uint32_t negm = 0, fl = 0, id = 0;
   for (int slot = 0; slot < np; ++slot, ++r) {
-    if (r >= term_pieces(m, exact, nslices, slots)) {
+    if (r >= term_pieces(m, exact)) {
       m = terms[++t];
       r = 0;
     }
     if (!exact) {
-      const int kp = m.k / bc, q = (int)r / kp, k0 = ((int)r - q * kp) * bc;
-      const bool single = nslices > 1 && kp > slots;  // one slice of each operand: the maps after the term's
-      int l = 0, i = 0;
-      if (single) slice_pair(q, l, i);
-      pieces[g * P + slot] = TmPiece{m.amap + single, (m.ax + k0) / 8, m.ay / 16, m.bmap + single, (m.bx + k0) / 8,
-                                     m.by / 16, i, l - i};
+      const int k0 = (int)r * bc;
+      pieces[g * P + slot] = TmPiece{m.amap, (m.ax + k0) / 8, m.ay / 16, m.bmap, (m.bx + k0) / 8, m.by / 16, {0, 0}};
       negm |= (uint32_t)(m.neg & 1) << slot;
-      if (nslices > 1) {
-        const bool term_last = t == tl.t1 - 1;
-        if (single) piece_bytes = (uint32_t)(128 + tl.n) * bc * 2;
-        fl = (single ? 256u + 1u : (uint32_t)kp) | (negm & 1u) << 9;
-        fl |= (single ? last : term_last) ? 1024u : 0u;
-      }
+      if (nslices > 1) fl = (uint32_t)(m.k / bc) | (negm & 1u) << 9 | (t == tl.t1 - 1 ? 1024u : 0u);
       continue;
     }
     const int nsl = max(1, (m.neg >> 4) & 15);
@@ -884,13 +869,13 @@ __global__ void fill_lists_kernel(int mode, int nslices, int slots, const TmTile
     const int q = (int)(r / kp), kk = (int)(r - (long)q * kp), k0 = kk * bc;
     int l, i;
     slice_pair(q, l, i);
-    pieces[g * P + slot] = TmPiece{m.amap + i, m.ax + k0, m.ay, m.bmap + (l - i), m.bx + k0, m.by, 0, 0};
+    pieces[g * P + slot] = TmPiece{m.amap + i, m.ax + k0, m.ay, m.bmap + (l - i), m.bx + k0, m.by, {0, 0}};
     fl = (uint32_t)min(bc / 16, (m.k - k0) / 16);
     fl |= (i == 0 && kk == 0) ? 8u : 0u;
     fl |= (i == l && kk == kp - 1) ? 16u : 0u;
     id = tm_idesc_bf16(tl.n, (m.neg & 1) != 0);
   }
-  for (int p = np; p < P; ++p) pieces[g * P + p] = TmPiece{0, 0, 0, 0, 0, 0, 0, 0};
+  for (int p = np; p < P; ++p) pieces[g * P + p] = TmPiece{0, 0, 0, 0, 0, 0, {0, 0}};
   if (!exact) id = tm_idesc_bf16(tl.n, false);
   if (!exact && nslices == 1) {
     const long seg = mode == TM_MODE_REDUCE_F32 ? TM_SEG_PRODUCTS / tm_slots(1) : nst;
@@ -960,18 +945,16 @@ bool tma_plan_lists(int mode, int nsl, std::vector<TmTile>& tiles, const std::ve
     if (m.k < 16 || m.k % 16) return false;
     max_k = std::max(max_k, m.k);
   }
-  // ring of a launch with two or three slices: slots of one piece of all slices.  Two CTAs per SM
-  // where the longest term fits the ring of each, else one with a ring twice as large (and terms
-  // that do not fit that go slice pair by slice pair).
-  out.ctas = exact ? 1 : 2;
+  // ring of a launch with two or three slices: slots of one piece of all slices, enough for the
+  // longest term
   out.slots = 0;
   out.slot_bytes = 0;
   if (chain) {
     out.slot_bytes = tm_slot_bytes(nsl, max_n);
-    if (tm_fit_slots(nsl, max_n, 2) < max_k / TM_PIECE_COLS) out.ctas = 1;
-    out.slots = tm_fit_slots(nsl, max_n, out.ctas);
+    out.slots = tm_fit_slots(nsl, max_n);
+    if (max_k / TM_PIECE_COLS > tm_term_pieces(nsl, max_n)) return false;
   }
-  const int grid = ntiles > 0 ? tma_grid(out.ctas, ntiles) : 0;
+  const int grid = ntiles > 0 ? tma_grid(tm_ctas(mode), ntiles) : 0;
   for (const TmTile& tl : tiles)
     if (tl.t0 < 0 || tl.t1 <= tl.t0 || tl.t1 > (int)terms.size()) return false;
   if (grid > 0) level_rounds(tiles, terms, grid);
@@ -984,7 +967,7 @@ bool tma_plan_lists(int mode, int nsl, std::vector<TmTile>& tiles, const std::ve
     for (int t = tl.t0; t < tl.t1; ++t) {
       if (out.tpiece0[(size_t)t] >= 0 || pc >= (1L << 31)) return false;
       out.tpiece0[(size_t)t] = (int)pc;
-      pc += term_pieces(terms[(size_t)t], exact, nsl, out.slots);
+      pc += term_pieces(terms[(size_t)t], exact);
       pr += (long)terms[(size_t)t].k / TM_PIECE_COLS * slice_pairs(nsl);
     }
     tst[(size_t)ti] = (pc + P - 1) / P;
@@ -1015,12 +998,12 @@ bool tma_plan_lists(int mode, int nsl, std::vector<TmTile>& tiles, const std::ve
   return true;
 }
 
-cudaError_t launch_fill_lists(int mode, int nsl, int slots, const TmTile* d_tiles, int ntiles, const TmTerm* d_terms,
+cudaError_t launch_fill_lists(int mode, int nsl, const TmTile* d_tiles, int ntiles, const TmTerm* d_terms,
                               const int* d_tpiece0, const int* d_sorder, const long* d_sfirst, long total,
                               TmStage* d_stages, TmPiece* d_pieces, cudaStream_t s) {
   if (ntiles <= 0 || total <= 0) return cudaSuccess;
   count_tc_launches(1);
-  fill_lists_kernel<<<(unsigned)((total + 255) / 256), 256, 0, s>>>(mode, nsl, slots, d_tiles, ntiles, d_terms, d_tpiece0,
+  fill_lists_kernel<<<(unsigned)((total + 255) / 256), 256, 0, s>>>(mode, nsl, d_tiles, ntiles, d_terms, d_tpiece0,
                                                                     d_sorder, d_sfirst, total, d_stages, d_pieces);
   return cudaGetLastError();
 }
@@ -1040,15 +1023,14 @@ bool encode_bf16_map(CUtensorMap* out, const void* base, uint64_t rows, uint64_t
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-bool encode_slice_map(CUtensorMap* out, const void* base, uint64_t rows, uint64_t cols, int nsl, uint32_t box_rows,
-                      int box_slices) {
+bool encode_slice_map(CUtensorMap* out, const void* base, uint64_t rows, uint64_t cols, int nsl, uint32_t box_rows) {
   EncodeTiledFn fn = encoder();
-  if (!fn || rows == 0 || rows % 16 != 0 || cols == 0 || cols % 8 != 0 || nsl < 1 || nsl > 3 || box_slices < 1 || box_slices > nsl ||
+  if (!fn || rows == 0 || rows % 16 != 0 || cols == 0 || cols % 8 != 0 || nsl < 1 || nsl > 3 ||
       ((uintptr_t)base & 15) != 0 || box_rows == 0 || box_rows % 16 != 0 || box_rows > 256)
     return false;
   const cuuint64_t dims[4] = {128, rows / 16, (cuuint64_t)nsl, cols / 8};
   const cuuint64_t strides[3] = {256, rows * 16, rows * 16 * nsl};
-  const cuuint32_t box[4] = {128, box_rows / 16, (cuuint32_t)box_slices, TM_PIECE_COLS / 8};
+  const cuuint32_t box[4] = {128, box_rows / 16, (cuuint32_t)nsl, TM_PIECE_COLS / 8};
   const cuuint32_t estr[4] = {1, 1, 1, 1};
   return fn(out, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(base), dims, strides, box, estr,
             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,

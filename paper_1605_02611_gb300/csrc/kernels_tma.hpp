@@ -73,13 +73,19 @@ __host__ __device__ constexpr int tm_slots(int nsl) { return nsl == 1 ? 2 : 1; }
 // K=16 products accumulated in tensor memory before the reduce-mode epilogue takes the partial
 // sum over (the tensor cores round their running sum toward zero)
 constexpr int TM_SEG_PRODUCTS = 64;
-// ring of two or three slices: at most TM_MAX_SLOTS slots of one piece in tm_ring_bytes(CTAs per SM)
-constexpr int TM_MAX_SLOTS = 12;
-constexpr int tm_ring_bytes(int ctas) { return ctas == 2 ? 108 * 1024 : 216 * 1024; }
+// CTAs per SM of a mode
+constexpr int tm_ctas(int mode) { return mode == TM_MODE_EXACT_F64 ? 1 : 2; }
+// ring of two or three slices: at most TM_MAX_SLOTS slots of one piece in TM_RING_BYTES
+constexpr int TM_MAX_SLOTS = 12, TM_RING_BYTES = 108 * 1024;
 constexpr int tm_slot_bytes(int nsl, int n) { return ((128 + n) * TM_PIECE_COLS * 2 * nsl + 1023) / 1024 * 1024; }
-constexpr int tm_fit_slots(int nsl, int n, int ctas) {
-  return tm_ring_bytes(ctas) / tm_slot_bytes(nsl, n) < TM_MAX_SLOTS ? tm_ring_bytes(ctas) / tm_slot_bytes(nsl, n)
-                                                                     : TM_MAX_SLOTS;
+constexpr int tm_fit_slots(int nsl, int n) {
+  return TM_RING_BYTES / tm_slot_bytes(nsl, n) < TM_MAX_SLOTS ? TM_RING_BYTES / tm_slot_bytes(nsl, n) : TM_MAX_SLOTS;
+}
+// most pieces of a term of two or three slices in a launch whose widest tile has n columns: what its
+// ring holds and the straight-line code takes
+constexpr int TM_TERM_PIECES = 6;
+constexpr int tm_term_pieces(int nsl, int n) {
+  return tm_fit_slots(nsl, n) < TM_TERM_PIECES ? tm_fit_slots(nsl, n) : TM_TERM_PIECES;
 }
 // maximum MMA width of a mode
 constexpr int tm_max_n(int mode, int nsl) {
@@ -90,8 +96,8 @@ constexpr int tm_max_n(int mode, int nsl) {
 // up to tma_pieces(mode, nsl) pieces.  In the sigma modes a piece is 16 columns of one term
 // with all slices of both operands: the slice products i + j < nsl come from one pair of
 // copies, and a term's pieces stay in the ring until all its products have been issued (slice pair
-// by slice pair, each over all pieces).  A term with more pieces than the ring has slots
-// expands into 16 columns of one slice of each operand instead, pair by pair.  In the exact mode a term expands into its slice pairs (i, j), i + j < nsl, in the
+// by slice pair, each over all pieces), so a term has at most tm_term_pieces of them.
+// In the exact mode a term expands into its slice pairs (i, j), i + j < nsl, in the
 // order of the level l = i + j (A map amap + i, B map bmap + j), each into boxes of 64
 // columns along K, one to a stage.  CTA c of a launch of `grid` CTAs takes the tiles c,
 // c + grid, ... and issues the stages [cta_stage[c], cta_stage[c + 1]), stage s with the
@@ -99,14 +105,14 @@ constexpr int tm_max_n(int mode, int nsl) {
 // A piece's coordinates are columns and rows in the exact mode, column groups (8) and row
 // groups (16) in the sigma modes.
 struct TmPiece {  // 32 bytes, so that any run of pieces is a bulk copy of 16-byte multiples
-  int amap, ax, ay, bmap, bx, by, as, bs;  // as, bs: first slice (sigma modes)
+  int amap, ax, ay, bmap, bx, by, pad[2];
 };
 // word: the stage word the MMA issuer reads, the instruction descriptor (negation of A in
 // the exact mode) in the low half.  High half, exact mode and one slice: the K=16 instructions
 // (exact) or pieces in bits 0-2, flags first of a segment (bit 3), end of a segment (4), last
 // stage of the tile (5), with one slice the negation of slot p in bit 8 + p.  Two or three slices:
-// the term's pieces in bits 0-7 (read from its first), a piece of single slices (bit 8),
-// negation (9), last term (or single-slice piece) of the tile (10).  bytes: the stage's expected
+// the term's pieces in bits 0-7 (read from its first),
+// negation (9), last term of the tile (10).  bytes: the stage's expected
 // copy bytes.
 struct TmStage {
   uint64_t word;
@@ -114,16 +120,16 @@ struct TmStage {
   int np;
 };
 struct TmListsDev {  // device copies, kept alive by the caller for the launches
-  int grid = 0, ctas = 1, slots = 0, slot_bytes = 0;
+  int grid = 0, slots = 0, slot_bytes = 0;
   const int* cta_stage = nullptr;
   const TmStage* stages = nullptr;
   const TmPiece* pieces = nullptr;
 };
-// host side of a launch's lists: its grid, CTAs per SM and (two or three slices) ring, every CTA's first stage (grid + 1 entries),
+// host side of a launch's lists: its grid and (two or three slices) ring, every CTA's first stage (grid + 1 entries),
 // the tiles in stage order (sorder) with their first stages (sfirst), and every term's
 // first piece within its tile (tpiece0; a term belongs to one tile)
 struct TmListPlan {
-  int grid = 0, ctas = 1, slots = 0, slot_bytes = 0;
+  int grid = 0, slots = 0, slot_bytes = 0;
   long total = 0;
   std::vector<int> cta_stage;
   std::vector<int> sorder;
@@ -147,12 +153,12 @@ __host__ __device__ inline uint32_t tm_idesc_bf16(int n, bool negA) {
 // Host: the stage counts of a launch of `mode` (operands of nsl slices) over these tiles
 // (for the grid the launch will use).  The tiles are put in an order that levels the work of the
 // CTAs; reduce mode: every tile's pad (its stages) and nseg are set.  Returns false if a term is malformed (k not a positive
-// multiple of 16), belongs to two tiles, or the lists would be too long.
+// multiple of 16, or longer than tm_term_pieces allows), belongs to two tiles, or the lists would be too long.
 bool tma_plan_lists(int mode, int nsl, std::vector<TmTile>& tiles, const std::vector<TmTerm>& terms, TmListPlan& out);
 // Device: fills the copy lists (stages: total entries, pieces: total * tma_pieces(mode,
 // nsl)), one thread per stage, from the tiles and terms the plan was made from and the plan's
 // tpiece0, sorder and sfirst (all on the device).
-cudaError_t launch_fill_lists(int mode, int nsl, int slots, const TmTile* d_tiles, int ntiles, const TmTerm* d_terms,
+cudaError_t launch_fill_lists(int mode, int nsl, const TmTile* d_tiles, int ntiles, const TmTerm* d_terms,
                               const int* d_tpiece0, const int* d_sorder, const long* d_sfirst, long total,
                               TmStage* d_stages, TmPiece* d_pieces, cudaStream_t s);
 // CTAs of a launch over ntiles tiles (at most ctas per SM of the current device)
@@ -191,8 +197,7 @@ cudaError_t launch_split_exact(const SplitJob* d_jobs, int njobs, int nsl, int* 
 bool encode_bf16_map(CUtensorMap* out, const void* base, uint64_t rows, uint64_t cols, uint64_t ld, uint32_t box_rows);
 // Host: encode the 4D map of a matrix in the layout of the sigma modes (rows a multiple of
 // 16, cols of 8, nsl slices), boxes of box_rows rows (a multiple of 16, at
-// most 256), TM_PIECE_COLS columns and box_slices slices.  Returns false on failure.
-bool encode_slice_map(CUtensorMap* out, const void* base, uint64_t rows, uint64_t cols, int nsl, uint32_t box_rows,
-                      int box_slices);
+// most 256), TM_PIECE_COLS columns and all slices.  Returns false on failure.
+bool encode_slice_map(CUtensorMap* out, const void* base, uint64_t rows, uint64_t cols, int nsl, uint32_t box_rows);
 
 }  // namespace gbdmrg
