@@ -27,6 +27,7 @@ namespace gbdmrg {
 
 void cuda_check(cudaError_t e, const char* what) {
   if (e == cudaSuccess) return;
+  cudaGetLastError();  // reported here, it must not meet the launch check of the next call
   if (e == cudaErrorMemoryAllocation)
     throw Error(ST_ENOMEM, std::string(what) + ": " + cudaGetErrorString(e));
   throw Error(ST_ECUDA, std::string(what) + ": " + cudaGetErrorString(e));
