@@ -75,8 +75,9 @@ struct DArr {
   ~DArr() { release(); }
   void release() { if (p) dev_free(p, s); p = nullptr; n = 0; }
   void alloc(size_t cnt, cudaStream_t st) {
-    release(); s = st; n = cnt;
+    release(); s = st;
     if (cnt) p = (T*)dev_alloc(cnt * sizeof(T), st);
+    n = cnt;  // 0 where the allocation failed
   }
   void upload(const std::vector<T>& h, cudaStream_t st) {
     alloc(h.size(), st);

@@ -745,10 +745,11 @@ static int dw2_parts(long rows) { return (int)std::max<long>(1, std::min<long>(S
 
 static void ensure_cap(Mlp& m, long B) {
   if (B <= m.cap) return;
-  m.cap = B;
+  m.cap = 0;  // until all of them are there
   m.H1.alloc((size_t)B * MLP_H, m.stream);
   m.dA2.alloc((size_t)B * MLP_H, m.stream);
   m.part.alloc((size_t)dw2_parts(B) * MLP_H * MLP_H, m.stream);
+  m.cap = B;
 }
 
 template <bool GRAD>

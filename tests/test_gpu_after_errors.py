@@ -30,3 +30,25 @@ def test_an_error_is_reported_once():
     got, _ = ctx.sigma(x)
     assert np.abs(got - ref).max() <= 1e-5 * np.abs(ref).max()
     ctx.close()
+
+
+@pytest.mark.parametrize("batch", [32, 64])
+def test_training_after_a_batch_that_does_not_fit(batch):
+    """The next step trains: its loss is that of a network that never saw the failure (to the bit: one
+    sum per thread block of 32 samples, and two of them commute), and it moves the parameters."""
+    require_gpu()
+    rng = np.random.default_rng(44)
+    F = rng.normal(size=(batch, 5)).astype(np.float32)
+    P, T = rng.normal(size=batch).astype(np.float32), rng.normal(size=batch).astype(np.float32)
+    net, other = G.Mlp(seed=3), G.Mlp(seed=3)
+    with pytest.raises(G.GbdmrgError, match="ENOMEM"):
+        net.train(F, P, T, epochs=1, batch=2 ** 31 - 1)  # 2.2 TB of activations
+    start = net.get_params()
+    first, _ = net.train(F, P, T, epochs=1, batch=batch, seed=5)
+    assert first == other.train(F, P, T, epochs=1, batch=batch, seed=5)[0]
+    moved = net.get_params()
+    assert np.all(np.isfinite(moved)) and np.any(moved != start)
+    L, g = net.loss_grad(F, P, T)
+    assert np.isfinite(L) and np.all(np.isfinite(g))
+    net.close()
+    other.close()
