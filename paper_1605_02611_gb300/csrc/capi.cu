@@ -841,7 +841,7 @@ gbdmrg_status gbdmrg_set_harvest(gbdmrg_ctx* ctx, int64_t capacity, int32_t per_
   if (!ctx || capacity < 0 || per_iteration < 0) return GBDMRG_EINVAL;
   return guard(ctx, [&] {
     auto& H = ctx->c.harvest;
-    H.cap = capacity;
+    H.cap = 0;  // until the buffers are there
     H.count = 0;
     H.per_iter = per_iteration;
     H.seed = seed;
@@ -849,6 +849,7 @@ gbdmrg_status gbdmrg_set_harvest(gbdmrg_ctx* ctx, int64_t capacity, int32_t per_
     H.F.alloc((size_t)capacity * gbdmrg::MLP_F, ctx->c.stream);
     H.P.alloc(capacity, ctx->c.stream);
     H.T.alloc(capacity, ctx->c.stream);
+    H.cap = capacity;
     gbdmrg::cuda_check(cudaStreamSynchronize(ctx->c.stream), "sync");
   });
 }

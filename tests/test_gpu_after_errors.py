@@ -52,3 +52,17 @@ def test_training_after_a_batch_that_does_not_fit(batch):
     assert np.isfinite(L) and np.all(np.isfinite(g))
     net.close()
     other.close()
+
+
+def test_harvest_that_does_not_fit_collects_nothing():
+    require_gpu()
+    ctx = _context()
+    with pytest.raises(G.GbdmrgError, match="ENOMEM"):
+        ctx.set_harvest(1 << 40, 16, 0)
+    ctx.step(2, 0, 30, 1e-8, 20)
+    assert len(ctx.get_harvest()[0]) == 0
+    ctx.set_harvest(64, 16, 0)
+    ctx.prepare(2)
+    ctx.step(2, 0, 30, 1e-8, 20)
+    assert len(ctx.get_harvest()[0]) > 0
+    ctx.close()
