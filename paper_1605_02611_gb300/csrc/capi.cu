@@ -389,6 +389,7 @@ gbdmrg_status gbdmrg_plan(gbdmrg_ctx* ctx, int32_t k) {
     if (k < 0 || k + 1 >= c.K) throw gbdmrg::Error(gbdmrg::ST_EINVAL, "two-site position out of range");
     if (!c.left[k].valid || !c.right[k + 2].valid)
       throw gbdmrg::Error(gbdmrg::ST_ESTATE, "environments of bonds k and k+2 are not built");
+    c.prepared = -1;  // the old work lists go; if making the new ones fails there are none
     gbdmrg::build_tilde_left(c, c.left[k], k, c.lt, true);
     gbdmrg::build_tilde_right(c, c.right[k + 2], k + 1, c.rt, true);
     gbdmrg::build_sigma_plan(c, c.lt, c.rt, k, c.plan);

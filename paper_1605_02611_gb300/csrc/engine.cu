@@ -1108,6 +1108,7 @@ void prepare_two_site(Context& c, int k) {
   if (k < 0 || k + 1 >= c.K) throw Error(ST_EINVAL, "two-site position out of range");
   for (int j = 0; j < c.K; ++j)
     if (!c.site_set[j]) throw Error(ST_ESTATE, "MPS tensor of site " + std::to_string(j) + " not set");
+  c.prepared = -1;  // the old work lists go; if making the new ones fails there are none
   env_boundary_left(c, c.left[0]);
   for (int j = 0; j < k; ++j) {
     Tilde t;

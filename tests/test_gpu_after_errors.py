@@ -1,4 +1,8 @@
 """What a call leaves behind when a device allocation fails: an error status, and objects that work."""
+import os
+import subprocess
+import sys
+
 import numpy as np
 import pytest
 
@@ -66,3 +70,50 @@ def test_harvest_that_does_not_fit_collects_nothing():
     ctx.step(2, 0, 30, 1e-8, 20)
     assert len(ctx.get_harvest()[0]) > 0
     ctx.close()
+
+
+PLAN_OUT_OF_MEMORY = """
+import numpy as np, torch
+import paper_1605_02611_gb300 as G
+from paper_1605_02611_gb300 import synth
+K, M, k = 24, 1500, 11
+h, eri = synth.integrals(K, 45)
+bonds, T = synth.random_isometric_mps(K, K, 0, M, 46, k, 1.0)
+ctx = G.Context(h, eri, K, 0)
+ctx.set_mps(T, [b.labels() for b in bonds])
+ctx.set_env_precision(3)
+ctx.prepare(k)
+x = torch.zeros(ctx.nnz, dtype=torch.float64, device="cuda")
+y = torch.zeros_like(x)
+torch.cuda.synchronize()
+ctx.set_precision(5)
+hold = torch.empty(torch.cuda.mem_get_info()[0] - (256 << 20), dtype=torch.uint8, device="cuda")
+
+def status(f):
+    try:
+        f()
+    except G.GbdmrgError as e:
+        return e.status
+    return "OK"
+
+a = status(lambda: ctx.plan(k))
+b = status(lambda: ctx.sigma_device(x.data_ptr(), y.data_ptr()))
+del hold
+torch.cuda.empty_cache()
+c = status(lambda: ctx.plan(k))
+d = status(lambda: ctx.sigma_device(x.data_ptr(), y.data_ptr()))
+print(a, "|", b, "|", c, "|", d)
+"""
+
+
+def test_a_plan_that_does_not_fit_leaves_no_plan():
+    """In a process of its own: what other tests left in the memory pool would change what fits.  The
+    work lists of this problem (three slices) take more than 20 GB, a few of them are there to be
+    had."""
+    require_gpu()
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    p = subprocess.run([sys.executable, "-c", PLAN_OUT_OF_MEMORY], cwd=root, capture_output=True, text=True,
+                       timeout=300)
+    assert p.returncode == 0, p.stderr[-2000:]
+    a, b, c, d = [s.strip() for s in p.stdout.strip().splitlines()[-1].split("|")]
+    assert "ENOMEM" in a and "ESTATE" in b and c == "OK" and d == "OK", p.stdout
