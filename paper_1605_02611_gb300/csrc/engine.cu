@@ -1273,18 +1273,18 @@ double davidson(Context& c, SigmaPlan& plan, const double* diag, double* psi, co
         }
       }
       if (use_mlp) {
+        // the fallback is the diagonal correction: the one computed above when the residual did
+        // not decrease; when the network produced a non-finite value, which is in t now, it is
+        // computed again
         bool learned = false;
-        if (rn < prev_rn) learned = mlp_precondition(*c.mlp, *c.mlp_s, r.p, diag, theta, rn, t.p, c.stream);
-        if (learned) {
-          ++c.mlp_applied;
+        if (rn < prev_rn) {
+          learned = mlp_precondition(*c.mlp, *c.mlp_s, r.p, diag, theta, rn, t.p, c.stream);
+          if (!learned) launch_precond(n, r.p, diag, theta, 1e-8, t.p, c.stream);
           orthogonalise(mb);
           read(2, 1, h3 + 2);
           tn = std::sqrt(h3[2]);
-        } else {
-          // the diagonal correction computed above is the fallback when the residual
-          // did not decrease or the network produced a non-finite value
-          ++c.mlp_fallbacks;
         }
+        ++(learned ? c.mlp_applied : c.mlp_fallbacks);
       }
       prev_rn = rn;
       m = mb;
