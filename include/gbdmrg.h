@@ -303,6 +303,15 @@ int64_t gbdmrg_kernel_launches(void);
 gbdmrg_status gbdmrg_gemm_bf16_selftest(const int64_t* tasks, int32_t ntasks, const int64_t* terms, int32_t nterms,
                                         void* stream);
 
+/* Self-test of the eigensolvers of the small matrices (Jacobi, one thread block): which = 0, all
+ * eigenpairs of the symmetric n x n matrix A (n <= 32; the decimation's sectors), w[n] ascending
+ * and row i of V[n*n] the vector of w[i]; which = 1, the lowest pair (n <= 48; the Rayleigh-Ritz
+ * step of Davidson), w[1] and V[n].  A, w and V are host arrays, row-major.  At most max_sweeps
+ * sweeps over all rotations (the solves use 60); GBDMRG_ENOCONV if that is too few or A is not
+ * finite, GBDMRG_EINVAL for n out of range. */
+gbdmrg_status gbdmrg_eigen_selftest(int32_t which, int32_t n, const double* A, int32_t max_sweeps, double* w,
+                                    double* V, void* stream);
+
 /* Host only: algorithmic flop count of one sigma at sites (k, k+1) when bond k
  * has labels qn_l[2*Dl] and bond k+2 has qn_r[2*Dr] (sum 2mnk over non-zero
  * blocks, the count gbdmrg_sigma reports). */

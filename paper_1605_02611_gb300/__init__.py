@@ -72,6 +72,7 @@ SIGNATURES = {
     "gbdmrg_step": (C.c_int, [_P, _I32, _I32, _I32, C.c_double, _I32, _P, _P, _I32, _PD, _PD, _PI32]),
     "gbdmrg_counters": (C.c_int, [_P, _PD, _PD, _PI64, _PD]),
     "gbdmrg_kernel_launches": (C.c_int64, []),
+    "gbdmrg_eigen_selftest": (C.c_int, [_I32, _I32, _PD, _I32, _PD, _PD, _P]),
     "gbdmrg_gemm_bf16_selftest": (C.c_int, [_PI64, _I32, _PI64, _I32, _P]),
     "gbdmrg_phase_times": (C.c_int, [_P, _PD]),
     "gbdmrg_phase_flops": (C.c_int, [_P, _PD]),
@@ -159,6 +160,20 @@ def gemm_bf16_selftest(tasks: np.ndarray, terms: np.ndarray, stream: int = 0) ->
                                        len(terms), _P(stream))
     if st != 0:
         raise GbdmrgError(f"gbdmrg_gemm_bf16_selftest failed: {STATUS.get(st, st)}")
+
+
+def eigen_selftest(which: int, A: np.ndarray, max_sweeps: int = 60):
+    """Small eigensolvers of the library (see include/gbdmrg.h): (w, V), vectors in rows; which = 1
+    returns the lowest pair."""
+    lib = load()
+    A = np.ascontiguousarray(A, dtype=np.float64)
+    n = len(A)
+    w = np.zeros(n if which == 0 else 1)
+    V = np.zeros((n, n) if which == 0 else n)
+    st = lib.gbdmrg_eigen_selftest(which, n, _dptr(A), max_sweeps, _dptr(w), _dptr(V), _P(0))
+    if st != 0:
+        raise GbdmrgError(f"gbdmrg_eigen_selftest failed: {STATUS.get(st, st)}", STATUS.get(st, str(st)))
+    return w, V
 
 
 def sigma_flops_host(h1, eri, N: int, two_sz: int, k: int, lab_l, lab_r) -> float:

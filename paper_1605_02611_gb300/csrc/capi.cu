@@ -584,6 +584,42 @@ gbdmrg_status gbdmrg_gemm_bf16_selftest(const int64_t* tasks, int32_t ntasks, co
   });
 }
 
+gbdmrg_status gbdmrg_eigen_selftest(int32_t which, int32_t n, const double* A, int32_t max_sweeps, double* w,
+                                    double* V, void* stream) {
+  if (!A || !w || !V || max_sweeps < 0 || (which != 0 && which != 1) || n < 1 ||
+      n > (which == 0 ? gbdmrg::EIGH_MAX : gbdmrg::RR_MAX_SUB))
+    return GBDMRG_EINVAL;
+  return guard(nullptr, [&] {
+    using namespace gbdmrg;
+    cudaStream_t st = (cudaStream_t)stream;
+    const size_t nn = (size_t)n * n, nw = which == 0 ? (size_t)n : 1, nv = which == 0 ? nn : (size_t)n;
+    DArr<double> a, dw, dv;
+    DArr<int> info;
+    DArr<EighJob> job;
+    const std::vector<double> ah(A, A + nn);
+    std::vector<EighJob> j;
+    a.upload(ah, st);
+    dw.alloc(nw, st);
+    dv.alloc((size_t)n, st);
+    info.alloc(1, st);
+    cuda_check(cudaMemsetAsync(info.p, 0, sizeof(int), st), "memset");
+    if (which == 0) {
+      j.push_back({a.p, dw.p, info.p, n});
+      job.upload(j, st);
+      launch_eigh(job.p, 1, st, max_sweeps);
+    } else {
+      launch_rr(a.p, n, n, dv.p, dw.p, st, max_sweeps);
+    }
+    cuda_check(cudaGetLastError(), "eigen kernel");
+    int h = 0;
+    cuda_check(cudaMemcpyAsync(w, dw.p, nw * sizeof(double), cudaMemcpyDeviceToHost, st), "d2h");
+    cuda_check(cudaMemcpyAsync(V, which == 0 ? a.p : dv.p, nv * sizeof(double), cudaMemcpyDeviceToHost, st), "d2h");
+    cuda_check(cudaMemcpyAsync(&h, info.p, sizeof(int), cudaMemcpyDeviceToHost, st), "d2h");
+    cuda_check(cudaStreamSynchronize(st), "sync");
+    if (h != 0 || !std::isfinite(w[0])) throw Error(ST_ENOCONV, "eigen kernel: not converged");
+  });
+}
+
 gbdmrg_status gbdmrg_counters(gbdmrg_ctx* ctx, double* sigma_flops, double* sigma_seconds, int64_t* sigma_calls,
                               double* other_flops) {
   if (!ctx) return GBDMRG_EINVAL;

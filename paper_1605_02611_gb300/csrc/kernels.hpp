@@ -108,12 +108,12 @@ void launch_diag_extract(const DiagJob* d_jobs, int njobs, int max_rows, cudaStr
 
 // Davidson on the device (FP64).  Rayleigh-Ritz: lowest eigenpair of the symmetric
 // part of the m x m projected matrix G (m <= 48) by parallel cyclic Jacobi in one
-// thread block; eigenvalue to scal[0], eigenvector to y[0..m).  false (nothing
-// launched) if m is outside [1, RR_MAX_SUB]
-constexpr int RR_MAX_SUB = 48;
+// thread block; eigenvalue to scal[0] (NaN where it does not converge in max_sweeps sweeps),
+// eigenvector to y[0..m).  false (nothing launched) if m is outside [1, RR_MAX_SUB]
+constexpr int RR_MAX_SUB = 48, JAC_SWEEPS = 60;
 // Eigen-decompositions of symmetric d x d matrices (row-major, d <= EIGH_MAX), one thread block
 // each: w the eigenvalues in ascending order, row i of G the eigenvector of w[i]; *info is set to
-// 1 (and w to NaN) if the matrix is not finite
+// 1 (and w to NaN) if the matrix is not finite or does not converge in max_sweeps sweeps
 constexpr int EIGH_MAX = 32;
 struct EighJob {
   double* G;
@@ -121,8 +121,8 @@ struct EighJob {
   int* info;
   int d;
 };
-void launch_eigh(const EighJob* d_jobs, int njobs, cudaStream_t s);
-bool launch_rr(const double* G, int ldg, int m, double* y, double* scal, cudaStream_t s);
+void launch_eigh(const EighJob* d_jobs, int njobs, cudaStream_t s, int max_sweeps = JAC_SWEEPS);
+bool launch_rr(const double* G, int ldg, int m, double* y, double* scal, cudaStream_t s, int max_sweeps = JAC_SWEEPS);
 // One Davidson iteration's vectors from the subspace V, its sigma vectors S and the Ritz
 // coefficients c: x = sum_j c_j V_j, hx = sum_j c_j S_j, r = hx - theta x (theta on device), the
 // diagonal correction t = r / (theta - diag) with |denominator| >= eps, and *rr = |r|^2
