@@ -746,12 +746,18 @@ gbdmrg_status gbdmrg_mlp_forward(gbdmrg_mlp* mlp, const float* features, int64_t
     gbdmrg::DArr<float> tf, tg;
     const float* F = to_device(features, (size_t)n * gbdmrg::MLP_F, on_device, tf, s);
     float* G = g;
-    if (!on_device) {
+    // thread blocks write their values of g while others still read features: where the two overlap,
+    // g is copied to its place at the end
+    const bool apart = g >= features + n * gbdmrg::MLP_F || features >= g + n;
+    if (!on_device || !apart) {
       tg.alloc(n, s);
       G = tg.p;
     }
     gbdmrg::mlp_forward(mlp->m, F, n, G, inference != 0);
-    if (!on_device) gbdmrg::cuda_check(cudaMemcpyAsync(g, G, n * sizeof(float), cudaMemcpyDeviceToHost, s), "d2h");
+    if (G != g)
+      gbdmrg::cuda_check(cudaMemcpyAsync(g, G, n * sizeof(float),
+                                         on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, s),
+                         "copy of g");
     gbdmrg::cuda_check(cudaStreamSynchronize(s), "sync");
   });
 }
