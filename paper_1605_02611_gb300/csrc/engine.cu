@@ -3,17 +3,16 @@
 // in the kernels of kernels.cu (cuSOLVER syevd serves the dense symmetric
 // eigenproblems of the decimation step).
 #include <algorithm>
-#include <atomic>
 #include <cstdint>
 #include <cstdio>
 #include <chrono>
 #include <cmath>
 #include <cstring>
 #include <exception>
+#include <limits>
 #include <map>
 #include <mutex>
 #include <numeric>
-#include <system_error>
 #include <thread>
 #include <tuple>
 
@@ -489,27 +488,13 @@ void env_boundary_right(Context& c, Env& e) {
   cuda_check(cudaStreamSynchronize(c.stream), "sync");
 }
 
-// f(lo, hi) over contiguous parts of [0, n) on up to 16 host threads (the calling
-// thread takes the first part); the first exception of any part is rethrown
+// f(lo, hi) over contiguous parts of [0, n) on up to 16 host threads
 template <class F>
 static void parallel_ranges(size_t n, F&& f) {
   const size_t hw = std::max(1u, std::thread::hardware_concurrency());
   const size_t nt = std::max<size_t>(1, std::min<size_t>({hw, 16, n / 1024 + 1}));
-  std::exception_ptr fail;
-  std::mutex mu;
-  auto part = [&](size_t t) {
-    try {
-      f(n * t / nt, n * (t + 1) / nt);
-    } catch (...) {
-      std::lock_guard<std::mutex> lk(mu);
-      if (!fail) fail = std::current_exception();
-    }
-  };
-  std::vector<std::thread> pool;
-  for (size_t t = 1; t < nt; ++t) pool.emplace_back(part, t);
-  part(0);
-  for (auto& th : pool) th.join();
-  if (fail) std::rethrow_exception(fail);
+  host_parallel((long)nt, std::numeric_limits<long>::max(),
+                [&](long t) { f(n * (size_t)t / nt, n * ((size_t)t + 1) / nt); });
 }
 
 // The blocking sums of one side: for every (bond state beta, site slot nn) the list
@@ -818,38 +803,6 @@ void env_update_right(Context& c, Tilde& rt, const SiteT& B, int site, Env& out)
     run_builder(c, g2);
     b0 = b1;
   }
-}
-
-// ---------------------------------------------------------------- host threads
-
-void host_parallel(long n, long work, const std::function<void(long)>& f) {
-  const unsigned hw = std::max(1u, std::thread::hardware_concurrency());
-  const long nth = std::min({n, (long)std::min(16u, hw), work / 4000 + 1});
-  if (nth <= 1) {
-    for (long i = 0; i < n; ++i) f(i);
-    return;
-  }
-  std::atomic<long> next{0};
-  std::exception_ptr err;
-  std::mutex mu;
-  auto run = [&] {
-    try {
-      for (long i = next.fetch_add(1); i < n; i = next.fetch_add(1)) f(i);
-    } catch (...) {
-      next = n;
-      std::lock_guard<std::mutex> lk(mu);
-      if (!err) err = std::current_exception();
-    }
-  };
-  std::vector<std::thread> th;
-  try {
-    for (long w = 1; w < nth; ++w) th.emplace_back(run);
-  } catch (const std::system_error&) {
-    // no more threads to be had: the ones there are do it
-  }
-  run();
-  for (auto& t : th) t.join();
-  if (err) std::rethrow_exception(err);
 }
 
 // ---------------------------------------------------------------- sigma

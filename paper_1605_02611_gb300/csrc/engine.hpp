@@ -6,12 +6,12 @@
 
 #include <array>
 #include <cstdint>
-#include <functional>
 #include <memory>
 #include <stdexcept>
 #include <string>
 #include <vector>
 
+#include "host_parallel.hpp"
 #include "kernels.hpp"
 #include "mpo.hpp"
 
@@ -310,10 +310,6 @@ void build_sigma_plan(Context& c, Tilde& lt, Tilde& rt, int k, SigmaPlan& plan);
 void run_sigma(Context& c, SigmaPlan& plan, const double* x, double* y);
 // the same for vectors of a caller, which need not be what a kernel can read or write in place
 void run_sigma_caller(Context& c, SigmaPlan& plan, const double* x, double* y);
-// f(0) .. f(n - 1) on the host threads, each index once in no fixed order; work: an estimate of
-// the steps in all (a thread costs about 20 us, so few of them run in the calling thread alone).
-// The first exception is thrown on to the caller after every thread has ended.
-void host_parallel(long n, long work, const std::function<void(long)>& f);
 void build_tma_plan(Context& c, Tilde& lt, Tilde& rt, int k, SigmaPlan& plan, int nslices);
 void run_tma_sigma(Context& c, SigmaPlan& plan, const double* x, double* y);
 // non-zero if a tensor-core launch of the plan reported a bounded wait that ran out
