@@ -33,6 +33,7 @@
 #include <atomic>
 #include <cstdint>
 
+#include "device_once.hpp"
 #include "kernels_tc.hpp"
 
 namespace gbdmrg {
@@ -431,17 +432,14 @@ void count_tc_launches(long n) { g_tc_launches += n; }
 template <int NSL>
 static cudaError_t launch_nsl(const TcTile* d_tiles, int ntiles, const TcTask* d_tasks, const TcTerm* d_terms,
                               int* d_err, cudaStream_t s) {
-  // one-time set-up per instantiation, thread-safe (function-local static)
+  static DeviceOnce once;
+  if (!allow_shared_memory(once, gemm_bf16_tc_kernel<NSL>, TcCfg<NSL>::SMEM)) return cudaErrorInvalidValue;
   static const int nsm = [] {
-    if (cudaFuncSetAttribute(gemm_bf16_tc_kernel<NSL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             TcCfg<NSL>::SMEM) != cudaSuccess)
-      return -1;
     int dev = 0, n = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
     return n > 0 ? n : 148;
   }();
-  if (nsm < 0) return cudaErrorInvalidValue;
   // persistent: one wave of resident CTAs (256 TMEM columns each)
   const int resident = TcCfg<NSL>::CTAS_PER_SM * nsm;
   const int grid = ntiles < resident ? ntiles : resident;

@@ -44,6 +44,7 @@
 // the fixed order, four instructions of up to 2 n columns per piece and slots released piece by
 // piece: 1.27 and 9.2 ms.)  The X intermediates' round trip and the stacked operators, 6.3 GB at
 // K=24, take 0.93 ms of that at the measured copy rate.
+#include "device_once.hpp"
 #include "kernels_tma.hpp"
 #include "ptx.cuh"
 
@@ -656,10 +657,8 @@ cudaError_t launch_mode(const TmTile* d_tiles, int ntiles, const TmTerm* d_terms
                         const long* d_rowmap, void* out, int* d_err, cudaStream_t s, const int* d_expo,
                         const TmListsDev& lists) {
   using Cfg = TmCfg<MODE, NSL>;
-  static const bool attr_ok =
-      cudaFuncSetAttribute(gemm_tma_kernel<MODE, NSL>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::SMEM) ==
-      cudaSuccess;
-  if (!attr_ok) return cudaErrorInvalidValue;
+  static DeviceOnce once;
+  if (!allow_shared_memory(once, gemm_tma_kernel<MODE, NSL>, Cfg::SMEM)) return cudaErrorInvalidValue;
   // the lists were built for this grid (every CTA's tiles and stages) and ring
   if (lists.grid != tma_grid(Cfg::CTAS, ntiles) || !lists.cta_stage || !lists.stages || !lists.pieces)
     return cudaErrorInvalidValue;

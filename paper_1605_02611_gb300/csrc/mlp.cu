@@ -8,6 +8,7 @@
 #include <random>
 #include <vector>
 
+#include "device_once.hpp"
 #include "kernels_tma.hpp"
 #include "mlp.hpp"
 #include "ptx.cuh"
@@ -755,9 +756,8 @@ static void ensure_cap(Mlp& m, long B) {
 template <bool GRAD>
 static void launch_train(Mlp& m, long rows, long n, uint64_t key, bool draw, const float* F, const float* P,
                          const float* T, float* g, double scale, double* loss_acc) {
-  static const bool attr_ok = cudaFuncSetAttribute(train_kernel<GRAD>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                   (int)sizeof(TrSmem)) == cudaSuccess;
-  if (!attr_ok) throw Error(ST_ECUDA, "mlp: shared memory attribute");
+  static DeviceOnce once;
+  if (!allow_shared_memory(once, train_kernel<GRAD>, (int)sizeof(TrSmem))) throw Error(ST_ECUDA, "mlp: shared memory attribute");
   const int grid = (int)std::min<long>((rows + TR_ROWS - 1) / TR_ROWS, SM_COUNT);
   train_kernel<GRAD><<<grid, TR_THREADS, sizeof(TrSmem), m.stream>>>(rows, n, key, draw ? 1 : 0, F, P, T, m.wq.p,
                                                                      m.w2b.p, g, m.H1.p, m.dA2.p, scale, loss_acc,
@@ -798,9 +798,8 @@ double mlp_loss_grad(Mlp& m, const float* F, const float* P, const float* T, lon
 template <int MODE>
 static void launch_infer(Mlp& m, long n, const float* F, const double* r, const double* d, double theta, double rn,
                          const MlpScratch* s, float* g, double* t, cudaStream_t st) {
-  static const bool attr_ok = cudaFuncSetAttribute(infer_kernel<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                   (int)sizeof(InSmem)) == cudaSuccess;
-  if (!attr_ok) throw Error(ST_ECUDA, "mlp: shared memory attribute");
+  static DeviceOnce once;
+  if (!allow_shared_memory(once, infer_kernel<MODE>, (int)sizeof(InSmem))) throw Error(ST_ECUDA, "mlp: shared memory attribute");
   const int grid = (int)std::min<long>((n + IN_ROWS - 1) / IN_ROWS, SM_COUNT);
   infer_kernel<MODE><<<grid, IN_THREADS, sizeof(InSmem), st>>>(
       n, F, r, d, theta, rn, s ? s->boff.p : nullptr, s ? s->nb : 0, s ? s->bsum.p : nullptr, s ? s->bmean.p : nullptr,
