@@ -137,8 +137,13 @@ gbdmrg_status gbdmrg_set_refinement(gbdmrg_ctx* ctx, int32_t precision, int32_t 
 gbdmrg_status gbdmrg_plan_stats(gbdmrg_ctx* ctx, double* out);
 
 /* Device memory (MB) for the per-chunk intermediates X_beta of one H_eff.psi
- * (default 2048): the operator terms are processed in chunks whose
- * intermediates fit this budget.  Takes effect at the next gbdmrg_prepare. */
+ * (default 2048) in precisions 0 to 3: the operator terms are processed in chunks whose
+ * intermediates fit this budget.  Takes effect at the next gbdmrg_prepare.  Beside them
+ * the work lists of precisions 1 to 6 hold the stacked right operators, a block for every
+ * bond state and site block that reads it (BF16, per slice: 3.7 GB at K=24, M=1500, 12.3 GB at
+ * K=40, M=2000).  Precisions 1 to 3 hold those of one chunk at a time, and make them in every
+ * H_eff.psi, where all of them and the vectors of a solve would take more than half of the
+ * device memory that is left when the lists are made. */
 gbdmrg_status gbdmrg_set_chunk_budget(gbdmrg_ctx* ctx, int32_t megabytes);
 
 /* Keep host copies of the tensor-core work lists built by later gbdmrg_prepare

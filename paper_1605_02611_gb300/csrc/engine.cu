@@ -46,6 +46,19 @@ void dev_free(void* p, cudaStream_t s) {
   if (p) cudaFreeAsync(p, s);
 }
 
+size_t device_memory_left() {
+  size_t free = 0, total = 0;
+  int dev = 0;
+  cudaMemPool_t pool;
+  uint64_t reserved = 0, used = 0;
+  cuda_check(cudaMemGetInfo(&free, &total), "memory info");
+  cuda_check(cudaGetDevice(&dev), "device");
+  cuda_check(cudaDeviceGetDefaultMemPool(&pool, dev), "mem pool");
+  cuda_check(cudaMemPoolGetAttribute(pool, cudaMemPoolAttrReservedMemCurrent, &reserved), "mem pool");
+  cuda_check(cudaMemPoolGetAttribute(pool, cudaMemPoolAttrUsedMemCurrent, &used), "mem pool");
+  return free + (size_t)(reserved - std::min(reserved, used));
+}
+
 int Bond::find(int a, int b) const {
   int lo = 0, hi = nsec() - 1;
   while (lo <= hi) {

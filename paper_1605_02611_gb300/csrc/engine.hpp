@@ -58,6 +58,8 @@ OpLayout make_op_layout(const Bond& b, int da, int db);
 // stream-ordered device allocation
 void* dev_alloc(size_t bytes, cudaStream_t s);
 void dev_free(void* p, cudaStream_t s);
+// device memory that allocations could still get: what is free, and unused in the default pool
+size_t device_memory_left();
 
 template <class T>
 struct DArr {

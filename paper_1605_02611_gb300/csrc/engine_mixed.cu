@@ -323,10 +323,15 @@ struct TmaPlan {
     DArr<ZeroJob> z;
     int nz = 0;
     long zmax = 0;
+    // the chunk's stacked right operators, where not all of them are held (n_a1_jobs == 0)
+    DArr<GroupJob> a1;
+    int n_a1 = 0;
+    long a1_maxel = 0;
     // host copies, kept when the plan may be fused into a batched launch
     std::vector<TmTile> ht1, ht2;
     std::vector<TmTerm> hm1, hm2;
     std::vector<ZeroJob> hz;
+    std::vector<GroupJob> ha1;
   };
   std::vector<Chunk> chunks;
   bool host_copies = false;
@@ -540,15 +545,47 @@ void build_tma_plan(Context& c, Tilde& lt, Tilde& rt, int k, SigmaPlan& plan, in
       if (xhas[(size_t)beta * ng + gp]) xsz[beta] += (size_t)gC[gout[(size_t)beta * ng + gp]] * gR[gp];
   const long budget_mb = c.precision >= 4 ? c.tma_budget_mb : (long)c.chunk_budget_mb;
   const size_t budget = (size_t)std::max<long>(1, budget_mb) * (1u << 20) / (sizeof(__nv_bfloat16) * nsl);
+  // The stacked right operators hold a block once for every bond state and site block that reads it
+  // (K=40, M=2000: 12 GB a slice, of a 3.5 GB environment) and are made once per plan, which is
+  // quicker than to make those of a chunk in every sigma.  Precisions 1-3 bound their intermediates
+  // to leave room for other problems: they do the latter where the whole stack and the vectors of a
+  // solve would take more than half of the memory that there is (K=24, M=1500, three
+  // slices: 12.9 ms per sigma and 13 GB with the whole stack, 24.9 ms and 5 GB chunk by chunk).
+  std::vector<size_t> ssz(nmid, 0);
+  for (int gp = 0; gp < ng; ++gp)
+    for (const RowBlk& x : rb[gp]) ssz[x.beta] += (size_t)x.rows * gC[gp];
+  bool held = true;
+  size_t stack_max = std::numeric_limits<size_t>::max();
+  if (c.precision <= 3) {
+    const size_t el = sizeof(__nv_bfloat16) * nsl;
+    size_t x = 0, stack = 0;
+    for (int beta = 0; beta < nmid; ++beta) {
+      x += xsz[beta];
+      stack += ssz[beta];
+    }
+    const size_t vectors = (size_t)P.nnz * sizeof(double) * 56;  // subspace, its sigma vectors, the others
+    const size_t need = (stack + std::min(x, budget)) * el + vectors;
+    if (need > (256u << 20)) {  // (the question takes longer than a small plan)
+      const size_t left = device_memory_left();
+      held = need <= left / 2;
+      if (!held) stack_max = left / 8 / el;
+    }
+  }
   std::vector<std::pair<int, int>> chunks;
   for (int b0 = 0; b0 < nmid;) {
     int b1 = b0;
-    size_t tot = 0;
-    while (b1 < nmid && (b1 == b0 || tot + xsz[b1] <= budget)) tot += xsz[b1++];
+    size_t tot = 0, stack = 0;
+    while (b1 < nmid && (b1 == b0 || (tot + xsz[b1] <= budget && (held || stack + ssz[b1] <= stack_max)))) {
+      tot += xsz[b1];
+      stack += ssz[b1++];
+    }
     chunks.push_back({b0, b1});
     b0 = b1;
   }
   const int nch = (int)chunks.size();
+  // stacks of their own layout: one, or one per chunk
+  const int nstack = held ? 1 : nch;
+  auto stack_of = [&](int ci) { return held ? 0 : ci; };
   std::vector<int> chunk_of(nmid, 0);
   for (int ci = 0; ci < nch; ++ci)
     for (int b = chunks[ci].first; b < chunks[ci].second; ++b) chunk_of[b] = ci;
@@ -583,21 +620,23 @@ void build_tma_plan(Context& c, Tilde& lt, Tilde& rt, int k, SigmaPlan& plan, in
     });
   });
   // (a run starts on a row group of 16, as the boxes of its tiles have to)
-  std::vector<long> a1off(ng), a1rows(ng);
-  long a1tot = 0;
+  std::vector<std::vector<long>> a1off(nstack, std::vector<long>(ng, 0)), a1rows(nstack, std::vector<long>(ng, 0));
+  std::vector<long> stack_el(nstack, 0);
   for (int gp = 0; gp < ng; ++gp) {
-    long rows = 0;
     const RowBlk* prev = nullptr;
     for (const RowBlk& x : rb[gp]) {
+      long& rows = a1rows[stack_of(chunk_of[x.beta])][gp];
       if (prev && (chunk_of[prev->beta] != chunk_of[x.beta] || prev->mask != x.mask)) rows = (rows + 15) / 16 * 16;
       rows += x.rows;
       prev = &x;
     }
-    rows = (rows + 15) / 16 * 16;
-    a1off[gp] = a1tot;
-    a1rows[gp] = rows;
-    a1tot += rows * gC[gp];
+    for (int st = 0; st < nstack; ++st) {
+      a1rows[st][gp] = (a1rows[st][gp] + 15) / 16 * 16;
+      a1off[st][gp] = stack_el[st];
+      stack_el[st] += a1rows[st][gp] * gC[gp];
+    }
   }
+  const long a1tot = *std::max_element(stack_el.begin(), stack_el.end());
   tp->a1.alloc(std::max<long>(a1tot, 8) * nsl, c.stream);
   cuda_check(cudaMemsetAsync(tp->a1.p, 0, tp->a1.n * sizeof(__nv_bfloat16), c.stream), "memset");
   struct Run {
@@ -607,44 +646,67 @@ void build_tma_plan(Context& c, Tilde& lt, Tilde& rt, int k, SigmaPlan& plan, in
   std::vector<std::vector<Run>> runs(ng);
   // per A1 row: its row in the X^T region of its chunk (columns: blocks of g', each its
   // own submatrix of the region)
-  std::vector<std::vector<long>> rowdst(ng);
-  std::vector<size_t> ajob0(ng + 1, 0);  // first conversion job of every group
-  for (int gp = 0; gp < ng; ++gp) {
-    ajob0[gp + 1] = ajob0[gp];
-    for (const RowBlk& x : rb[gp]) ajob0[gp + 1] += (size_t)__builtin_popcount((unsigned)x.mask);
-  }
-  std::vector<GroupJob> aconv(ajob0[ng]);
-  std::vector<long> amaxel(ng, 0);
+  std::vector<std::vector<std::vector<long>>> rowdst(nstack, std::vector<std::vector<long>>(ng));
+  // conversion jobs stack by stack, in each group by group: job0[stack * ng + group] the first
+  std::vector<size_t> job0((size_t)nstack * ng + 1, 0);
+  for (int gp = 0; gp < ng; ++gp)
+    for (const RowBlk& x : rb[gp])
+      job0[(size_t)stack_of(chunk_of[x.beta]) * ng + gp + 1] += (size_t)__builtin_popcount((unsigned)x.mask);
+  for (size_t i = 1; i < job0.size(); ++i) job0[i] += job0[i - 1];
+  std::vector<GroupJob> aconv(job0.back());
+  std::vector<long> amaxel((size_t)nstack * ng, 0);
   host_parallel(ng, (long)aconv.size(), [&](long gp) {
     long row = 0;
-    GroupJob* job = aconv.data() + ajob0[gp];
-    rowdst[gp].assign((size_t)a1rows[gp], -1);
+    int st = -1;
+    GroupJob* job = nullptr;
+    for (int s = 0; s < nstack; ++s) rowdst[s][gp].assign((size_t)a1rows[s][gp], -1);
     for (const RowBlk& x : rb[gp]) {
       const int ci = chunk_of[x.beta];
+      if (stack_of(ci) != st) {
+        st = stack_of(ci);
+        row = 0;
+        job = aconv.data() + job0[(size_t)st * ng + gp];
+      }
       if (runs[gp].empty() || runs[gp].back().chunk != ci || runs[gp].back().mask != x.mask) {
         row = (row + 15) / 16 * 16;
         runs[gp].push_back({ci, x.mask, row, row});
       }
       runs[gp].back().r1 = row + x.rows;
       const long xr0 = xrow[(size_t)x.beta * ng + gp] + (long)cpos[x.qr * 4 + x.n2][1];
-      for (int i = 0; i < x.rows; ++i) rowdst[gp][(size_t)(row + i)] = xr0 + i;
+      for (int i = 0; i < x.rows; ++i) rowdst[st][gp][(size_t)(row + i)] = xr0 + i;
       for (int n2p = 0; n2p < 4; ++n2p) {
         if (!((x.mask >> n2p) & 1)) continue;
         const TRef& r = rt.ref[x.beta][x.n2 * 4 + n2p];
         const Block& B = Renv.cls[r.cls].blocks[x.bl[n2p]];
         // the K block (n2', qr') of g': columns coff .. coff + pad16(d(qr')) of A1
         const int coff = cpos[B.cs * 4 + n2p][1];
-        *job++ = {r.p + B.off, tp->a1.p + (a1off[gp] + a1rows[gp] * coff) * nsl + row * 8, a1rows[gp] * 8,
-                  a1rows[gp] * 8 * nsl, B.rows, B.cols, B.cols, pad16(B.cols), r.coef};
-        amaxel[gp] = std::max<long>(amaxel[gp], (long)B.rows * pad16(B.cols));
+        const long rows = a1rows[st][gp];
+        *job++ = {r.p + B.off, tp->a1.p + (a1off[st][gp] + rows * coff) * nsl + row * 8, rows * 8,
+                  rows * 8 * nsl, B.rows, B.cols, B.cols, pad16(B.cols), r.coef};
+        long& most = amaxel[(size_t)st * ng + gp];
+        most = std::max<long>(most, (long)B.rows * pad16(B.cols));
       }
       row += x.rows;
     }
   });
-  for (long m : amaxel) tp->a1_maxel = std::max(tp->a1_maxel, m);
   check_group_jobs(aconv, nsl, tp->a1);
-  tp->a1_jobs.upload(aconv, c.stream);
-  tp->n_a1_jobs = (int)aconv.size();
+  tp->chunks.resize(nch);
+  if (held) {
+    for (long m : amaxel) tp->a1_maxel = std::max(tp->a1_maxel, m);
+    tp->a1_jobs.upload(aconv, c.stream);
+    tp->n_a1_jobs = (int)aconv.size();
+  } else {
+    for (int ci = 0; ci < nch; ++ci) {
+      TmaPlan::Chunk& ch = tp->chunks[ci];
+      for (int gp = 0; gp < ng; ++gp) ch.a1_maxel = std::max(ch.a1_maxel, amaxel[(size_t)ci * ng + gp]);
+      ch.ha1.assign(aconv.begin() + (long)job0[(size_t)ci * ng], aconv.begin() + (long)job0[(size_t)(ci + 1) * ng]);
+      ch.a1.upload(ch.ha1, c.stream);
+      ch.n_a1 = (int)ch.ha1.size();
+    }
+    cuda_check(cudaStreamSynchronize(c.stream), "sync");
+    if (!tp->host_copies)
+      for (auto& ch : tp->chunks) std::vector<GroupJob>().swap(ch.ha1);
+  }
   // ---- left mirror: every distinct (operator, scale) referenced by Lt, all its blocks,
   // each padded to 16 rows and columns; blocks of one padded width w share one matrix of
   // w columns
@@ -770,10 +832,10 @@ void build_tma_plan(Context& c, Tilde& lt, Tilde& rt, int k, SigmaPlan& plan, in
     while (n1max > 64 && tm_term_pieces(nsl, n1max) < len) n1max -= 16;
   }
   std::vector<std::vector<std::array<int, 3>>> nt1(ng);  // per g': (row0, width, Psi map) of the stage-1 N tiles
-  std::vector<int> a1map(ng, -1);
+  std::vector<std::vector<int>> a1map(nstack, std::vector<int>(ng, -1));
   int n1wide = 16, n2wide = 16;
   for (int gp = 0; gp < ng; ++gp) {
-    if (a1rows[gp] == 0) continue;
+    if (rb[gp].empty()) continue;
     const int parts = (gR[gp] + n1max - 1) / n1max;
     int r0 = 0;
     for (int p = 0; p < parts; ++p) {
@@ -782,7 +844,8 @@ void build_tma_plan(Context& c, Tilde& lt, Tilde& rt, int k, SigmaPlan& plan, in
       r0 += w;
       n1wide = std::max(n1wide, w);
     }
-    a1map[gp] = add_map(tp->a1, a1off[gp] * nsl, a1rows[gp], gC[gp], 128);
+    for (int st = 0; st < nstack; ++st)
+      if (a1rows[st][gp] > 0) a1map[st][gp] = add_map(tp->a1, a1off[st][gp] * nsl, a1rows[st][gp], gC[gp], 128);
   }
   for (int ql = 0; ql < nL; ++ql) n2wide = std::max(n2wide, std::min(n2max, pad16(Lb.dim[ql])));
   const int limit1 = tm_term_pieces(nsl, n1wide), limit2 = tm_term_pieces(nsl, n2wide);
@@ -806,7 +869,6 @@ void build_tma_plan(Context& c, Tilde& lt, Tilde& rt, int k, SigmaPlan& plan, in
   // ---- work lists per chunk
   std::vector<long> rowmap;
   double st1_tiles = 0, st1_steps = 0, st2_tiles = 0, st2_steps = 0, st1_fl = 0, st2_fl = 0;
-  tp->chunks.resize(nch);
   for (int ci = 0; ci < nch; ++ci) {
     TmaPlan::Chunk& ch = tp->chunks[ci];
     std::vector<TmTile> t1, t2;
@@ -841,7 +903,7 @@ void build_tma_plan(Context& c, Tilde& lt, Tilde& rt, int k, SigmaPlan& plan, in
         if (run.chunk != ci) continue;
         for (long r0 = run.r0; r0 < run.r1; r0 += 128) {
           const long moff = (long)ir;
-          for (long i = 0; i < 128; ++i) rowmap[ir++] = r0 + i < run.r1 ? rowdst[gp][(size_t)(r0 + i)] : -1;
+          for (long i = 0; i < 128; ++i) rowmap[ir++] = r0 + i < run.r1 ? rowdst[stack_of(ci)][gp][(size_t)(r0 + i)] : -1;
           for (const auto& nt : nt1[gp]) {
             TmTile tl{};
             tl.t0 = (int)im;
@@ -855,7 +917,7 @@ void build_tma_plan(Context& c, Tilde& lt, Tilde& rt, int k, SigmaPlan& plan, in
               const int parts = parts_of(kk, limit1);
               for (int p = 0; p < parts; ++p) {
                 const auto cols = part_cols(kk, parts, p);
-                m1[im++] = {a1map[gp], nt[2], coff + cols.first, (int)r0, coff + cols.first, nt[0],
+                m1[im++] = {a1map[stack_of(ci)][gp], nt[2], coff + cols.first, (int)r0, coff + cols.first, nt[0],
                             cols.second - cols.first, nsl << 4};
               }
               ksum += kk * npair;
@@ -1069,7 +1131,7 @@ void build_tma_plan(Context& c, Tilde& lt, Tilde& rt, int k, SigmaPlan& plan, in
   }
   tp->rowmap.upload(rowmap, c.stream);
   if (tp->host_copies) tp->hrowmap = rowmap;
-  // the operator stacks depend only on the environments: filled once per plan
+  // the operator stacks depend only on the environments: filled once per plan if all are held
   if (tp->n_a1_jobs) launch_conv_groups(tp->a1_jobs, tp->n_a1_jobs, nsl, tp->a1_maxel, c.stream);
   if (tp->n_l_jobs) launch_conv_groups(tp->l_jobs, tp->n_l_jobs, nsl, tp->l_maxel, c.stream);
   tp->err.alloc(1, c.stream);
@@ -1093,6 +1155,7 @@ void run_tma_sigma(Context& c, SigmaPlan& plan, const double* x, double* y) {
   if (tp.n_psi_jobs) launch_conv_groups(tp.psi_jobs, tp.n_psi_jobs, tp.nsl, tp.psi_maxel, c.stream, x - plan.in.p);
   cuda_check(cudaMemsetAsync(tp.sig_t.p, 0, tp.sig_total * sizeof(float), c.stream), "memset");
   for (auto& ch : tp.chunks) {
+    if (ch.n_a1) launch_conv_groups(ch.a1, ch.n_a1, tp.nsl, ch.a1_maxel, c.stream);
     if (ch.nz) launch_zero(ch.z.p, ch.nz, ch.zmax, c.stream);
     cuda_check(launch_gemm_slices(TM_MODE_STORE_BF16, tp.nsl, ch.t1.p, ch.n1, tp.maps.p, tp.rowmap.p, tp.xt.p, tp.err.p,
                                   c.stream, ch.l1.dev()),
@@ -1848,12 +1911,13 @@ struct BatchPlan {
   std::vector<Context*> ctx;
   cudaStream_t stream = nullptr;
   struct Launch {
-    int nsl = 1, n1 = 0, n2 = 0, nz = 0;
-    long zmax = 0;
+    int nsl = 1, n1 = 0, n2 = 0, nz = 0, n_a1 = 0;
+    long zmax = 0, a1_maxel = 0;
     DArr<TmTile> t1, t2;
     DArr<TmTerm> m1, m2;
     TmaPlan::Lists l1, l2;
     DArr<ZeroJob> z;
+    DArr<GroupJob> a1;
     void *out1 = nullptr, *out2 = nullptr;  // what the tiles' offsets count from
   };
   std::vector<Launch> launches;  // chunk by chunk
@@ -1921,6 +1985,7 @@ static void batch_launch(BatchPlan& b, size_t ch, int nsl, const std::vector<siz
   std::vector<TmTile> t1, t2;
   std::vector<TmTerm> m1, m2;
   std::vector<ZeroJob> zj;
+  std::vector<GroupJob> aj;
   BatchPlan::Launch L;
   L.nsl = nsl;
   auto add = [&](std::vector<TmTile>& tiles, std::vector<TmTerm>& terms, const std::vector<TmTile>& pt,
@@ -1954,6 +2019,8 @@ static void batch_launch(BatchPlan& b, size_t ch, int nsl, const std::vector<siz
     add(t2, m2, c.ht2, c.hm2, map0[p], [&](TmTile& t) { t.out_off += ds; });
     zj.insert(zj.end(), c.hz.begin(), c.hz.end());
     L.zmax = std::max(L.zmax, c.zmax);
+    aj.insert(aj.end(), c.ha1.begin(), c.ha1.end());
+    L.a1_maxel = std::max(L.a1_maxel, c.a1_maxel);
   }
   if (t1.empty() && t2.empty()) return;
   longest_first(t1, m1);
@@ -1968,6 +2035,8 @@ static void batch_launch(BatchPlan& b, size_t ch, int nsl, const std::vector<siz
   L.t2.upload(t2, b.stream);
   L.m2.upload(m2, b.stream);
   L.z.upload(zj, b.stream);
+  L.n_a1 = (int)aj.size();
+  L.a1.upload(aj, b.stream);
   L.l1.fill(TM_MODE_STORE_BF16, nsl, L.t1.p, L.n1, L.m1.p, b.stream);
   L.l2.fill(TM_MODE_REDUCE_F32, nsl, L.t2.p, L.n2, L.m2.p, b.stream);
   cuda_check(cudaStreamSynchronize(b.stream), "sync");
@@ -2034,6 +2103,7 @@ static void batch_enqueue(BatchPlan& b) {
   for (int i = 0; i < 3; ++i)
     if (b.nconv[i]) launch_conv_groups(b.conv[i], b.nconv[i], i + 1, b.conv_maxel, s);
   for (const BatchPlan::Launch& L : b.launches) {
+    if (L.n_a1) launch_conv_groups(L.a1, L.n_a1, L.nsl, L.a1_maxel, s);
     if (L.nz) launch_zero(L.z.p, L.nz, L.zmax, s);
     cuda_check(launch_gemm_slices(TM_MODE_STORE_BF16, L.nsl, L.t1.p, L.n1, b.maps.p, b.rowmap.p, L.out1, b.err.p, s,
                                   L.l1.dev()),
