@@ -35,6 +35,7 @@
 
 #include "device_once.hpp"
 #include "kernels_tc.hpp"
+#include "ptx.cuh"
 
 namespace gbdmrg {
 
@@ -50,9 +51,8 @@ constexpr int TC_EPI_BYTES = 4 * 32 * TC_EPI_LD * 2;
 // With three slices a stage holds every BF16 slice of both operands for one
 // 64-wide K step, so each loaded slice serves all the slice products it takes
 // part in (six products from six tiles instead of twelve), at two stages and
-// one CTA per SM.  With one or two slices a stage holds one A and one B slice
-// (one slice pair), three stages, two CTAs per SM: measured faster for two
-// slices, where reuse saves only a third of the loads but halves the CTAs.
+// one CTA per SM.  With one slice a stage holds one A and one B tile, three stages,
+// two CTAs per SM.
 template <int NSL>
 struct TcCfg {
   static constexpr bool REUSE = NSL == 3;
@@ -69,25 +69,11 @@ struct TcCfg {
 constexpr int TC_THREADS = 288;
 constexpr int TC_PRODUCERS = 128;  // warps 4-7
 constexpr int TC_MAXACC = 4;  // tensor-memory accumulators of 128 columns (at most)
-constexpr long TC_WAIT_LIMIT = 1L << 24;
 
 // slice pairs (i, j) with i + j < nsl, largest products first
 __constant__ int PAIR_I[6] = {0, 0, 1, 0, 1, 2};
 __constant__ int PAIR_J[6] = {0, 1, 0, 2, 1, 0};
 __device__ __forceinline__ int npairs(int nsl) { return nsl <= 1 ? 1 : (nsl == 2 ? 3 : 6); }
-
-__device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-
-// shared-memory matrix descriptor: K-major, 128-byte swizzle, 8-row groups 1024 B apart
-__device__ __forceinline__ uint64_t sdesc(uint32_t saddr) {
-  uint64_t d = 0;
-  d |= (uint64_t)((saddr >> 4) & 0x3FFFu);
-  d |= (uint64_t)1 << 16;            // leading byte offset (unused for swizzled K-major)
-  d |= (uint64_t)(1024 >> 4) << 32;  // stride byte offset
-  d |= (uint64_t)1 << 46;            // descriptor version
-  d |= (uint64_t)2 << 61;            // SWIZZLE_128B
-  return d;
-}
 
 // instruction descriptor: D f32, A/B bf16, both K-major, M = 128, N = n
 __device__ __forceinline__ uint32_t idesc_bf16(int n, bool negA) {
@@ -109,37 +95,7 @@ __device__ __forceinline__ void cp_async_wait() {
   asm volatile("cp.async.wait_group %0;\n" ::"n"(N));
 }
 
-__device__ __forceinline__ void mbar_init(uint64_t* b, int count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(smem_u32(b)), "r"(count));
-}
-__device__ __forceinline__ void mbar_arrive(uint64_t* b) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(smem_u32(b)) : "memory");
-}
-// bounded parity wait; gives up when the CTA-wide abort flag is raised
-__device__ __forceinline__ bool mbar_wait(uint64_t* b, uint32_t parity, volatile int* abort_flag) {
-  const uint32_t a = smem_u32(b);
-  for (long it = 0; it < TC_WAIT_LIMIT; ++it) {
-    uint32_t done;
-    asm volatile(
-        "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
-        : "=r"(done)
-        : "r"(a), "r"(parity)
-        : "memory");
-    if (done) return true;
-    if ((it & 1023) == 1023 && *abort_flag) return false;
-  }
-  *abort_flag = 1;
-  return false;
-}
-
 __device__ __forceinline__ int round16(int x) { return (x + 15) & ~15; }
-
-// four FP32 atomic adds in one vector reduction (16-byte aligned address)
-__device__ __forceinline__ void red_add_v4(float* p, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
-  asm volatile("red.relaxed.gpu.global.add.v4.f32 [%0], {%1, %2, %3, %4};\n" ::"l"(p), "f"(__uint_as_float(a)),
-               "f"(__uint_as_float(b)), "f"(__uint_as_float(c)), "f"(__uint_as_float(d))
-               : "memory");
-}
 
 // BF16 slice s of x: x = s0 + s1 + s2 + O(2^-24 |x|)
 __device__ __forceinline__ __nv_bfloat16 bf16_slice(float x, int s) {
@@ -452,7 +408,6 @@ cudaError_t launch_gemm_bf16_tc(const TcTile* d_tiles, int ntiles, const TcTask*
                                 int* d_err, cudaStream_t s, int nsl) {
   if (ntiles <= 0) return cudaSuccess;
   if (nsl <= 1) return launch_nsl<1>(d_tiles, ntiles, d_tasks, d_terms, d_err, s);
-  if (nsl == 2) return launch_nsl<2>(d_tiles, ntiles, d_tasks, d_terms, d_err, s);
   if (nsl == 3) return launch_nsl<3>(d_tiles, ntiles, d_tasks, d_terms, d_err, s);
   return cudaErrorInvalidValue;
 }

@@ -685,7 +685,7 @@ inline int blocks_for(long n, int threads = 256, int cap = 4096) {
 
 Mlp::~Mlp() {
   // the arrays are freed on the network's stream: release them before it goes
-  for (DArr<float>* a : {&w, &wq, &grad, &am, &av, &H1, &dA2, &G, &part}) a->release();
+  for (DArr<float>* a : {&w, &wq, &grad, &am, &av, &H1, &dA2, &part}) a->release();
   w2b.release();
   err.release();
   acc.release();

@@ -48,7 +48,7 @@ struct Mlp {
   DArr<int> err;                 // tensor-core kernel wait flag
   // training scratch, sized for `cap` samples
   long cap = 0;
-  DArr<float> H1, dA2, G;
+  DArr<float> H1, dA2;
   DArr<float> part;  // partial sums of dL/dW2
   DArr<double> acc;
   ~Mlp();

@@ -9,6 +9,17 @@ constexpr long WAIT_LIMIT = 1L << 24;  // polls of a barrier before a wait gives
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
+// shared-memory matrix descriptor: K-major, 128-byte swizzle, 8-row groups 1024 B apart
+__device__ __forceinline__ uint64_t sdesc(uint32_t saddr) {
+  uint64_t d = 0;
+  d |= (uint64_t)((saddr >> 4) & 0x3FFFu);
+  d |= (uint64_t)1 << 16;            // leading byte offset (unused for swizzled K-major)
+  d |= (uint64_t)(1024 >> 4) << 32;  // stride byte offset
+  d |= (uint64_t)1 << 46;            // descriptor version
+  d |= (uint64_t)2 << 61;            // SWIZZLE_128B
+  return d;
+}
+
 // shared-memory matrix descriptor of the column-group layout: K-major without swizzle, core matrices of 8 rows x
 // 16 bytes contiguous along the rows (128 B apart), the second 8 columns `rows` rows further.
 // lo: address and rows in 16-byte units, (saddr >> 4) | rows << 16.
@@ -45,6 +56,13 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* b, uint32_t parity, volatile
   }
   *abort_flag = 1;
   return false;
+}
+
+// four FP32 atomic adds in one vector reduction (16-byte aligned address)
+__device__ __forceinline__ void red_add_v4(float* p, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
+  asm volatile("red.relaxed.gpu.global.add.v4.f32 [%0], {%1, %2, %3, %4};\n" ::"l"(p), "f"(__uint_as_float(a)),
+               "f"(__uint_as_float(b)), "f"(__uint_as_float(c)), "f"(__uint_as_float(d))
+               : "memory");
 }
 
 // 32 consecutive FP32 columns of this warp's 32 tensor-memory lanes
