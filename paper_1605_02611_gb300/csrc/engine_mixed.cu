@@ -21,7 +21,6 @@
 #include <map>
 #include <numeric>
 #include <unordered_map>
-#include <unordered_set>
 
 #include "engine.hpp"
 #include "kernels_tc.hpp"
@@ -673,7 +672,8 @@ void build_tma_plan(Context& c, Tilde& lt, Tilde& rt, int k, SigmaPlan& plan, in
       }
       runs[gp].back().r1 = row + x.rows;
       const long xr0 = xrow[(size_t)x.beta * ng + gp] + (long)cpos[x.qr * 4 + x.n2][1];
-      for (int i = 0; i < x.rows; ++i) rowdst[st][gp][(size_t)(row + i)] = xr0 + i;
+      std::vector<long>& dst = rowdst[st][gp];
+      for (int i = 0; i < x.rows; ++i) dst[(size_t)(row + i)] = xr0 + i;
       for (int n2p = 0; n2p < 4; ++n2p) {
         if (!((x.mask >> n2p) & 1)) continue;
         const TRef& r = rt.ref[x.beta][x.n2 * 4 + n2p];
@@ -899,11 +899,12 @@ void build_tma_plan(Context& c, Tilde& lt, Tilde& rt, int k, SigmaPlan& plan, in
     std::vector<std::array<double, 2>> st1(ng, {0, 0});  // steps, flops
     host_parallel(ng, (long)rowmap.size() / 16, [&](long gp) {
       size_t it = at1[gp][0], im = at1[gp][1], ir = at1[gp][2];
+      const std::vector<long>& dst = rowdst[stack_of(ci)][gp];
       for (const Run& run : runs[gp]) {
         if (run.chunk != ci) continue;
         for (long r0 = run.r0; r0 < run.r1; r0 += 128) {
           const long moff = (long)ir;
-          for (long i = 0; i < 128; ++i) rowmap[ir++] = r0 + i < run.r1 ? rowdst[stack_of(ci)][gp][(size_t)(r0 + i)] : -1;
+          for (long i = 0; i < 128; ++i) rowmap[ir++] = r0 + i < run.r1 ? dst[(size_t)(r0 + i)] : -1;
           for (const auto& nt : nt1[gp]) {
             TmTile tl{};
             tl.t0 = (int)im;
@@ -945,22 +946,28 @@ void build_tma_plan(Context& c, Tilde& lt, Tilde& rt, int k, SigmaPlan& plan, in
     // X^T rows of this chunk that stage 1 does not write: zero them before the chunk
     // (with one chunk the buffer is zero from the start)
     if (nch > 1) {
-      for (int gp = 0; gp < ng; ++gp) {
-        std::unordered_set<long> written;
-        for (const RowBlk& x : rb[gp])
-          if (chunk_of[x.beta] == ci) written.insert(((long)x.beta * 4 + x.n2) * nR + x.qr);
-        for (int beta = chunks[ci].first; beta < chunks[ci].second; ++beta) {
+      std::vector<std::vector<ZeroJob>> zg(ng);
+      const int b0 = chunks[ci].first, b1 = chunks[ci].second;
+      host_parallel(ng, (long)(b1 - b0) * ng * 4, [&](long gp) {
+        std::vector<char> written((size_t)(b1 - b0) * 4 * nR, 0);  // [beta][n2][qr]
+        auto at = [&](int beta, int n2, int qr) { return ((size_t)(beta - b0) * 4 + n2) * nR + qr; };
+        // the row blocks are sorted by chunk
+        auto x = std::lower_bound(rb[gp].begin(), rb[gp].end(), ci,
+                                  [&](const RowBlk& a, int c2) { return chunk_of[a.beta] < c2; });
+        for (; x != rb[gp].end() && chunk_of[x->beta] == ci; ++x) written[at(x->beta, x->n2, x->qr)] = 1;
+        for (int beta = b0; beta < b1; ++beta) {
           if (!xhas[(size_t)beta * ng + gp]) continue;
           const int g = gout[(size_t)beta * ng + gp];
           for (const auto& cb : gcol[g]) {
-            if (written.count(((long)beta * 4 + cb[0]) * nR + cb[1])) continue;
+            if (written[at(beta, cb[0], cb[1])]) continue;
             // the block's rows in every column group
             const long r0 = xrow[(size_t)beta * ng + gp] + cb[2], rows = xregrows[ci][gp];
-            zj.push_back({tp->xt.p + xreg[ci][gp] * nsl + r0 * 8, (long)pad16(Rb.dim[cb[1]]) * 8, rows * 8, nsl,
-                          gR[gp] / 8, rows * 8 * nsl});
+            zg[gp].push_back({tp->xt.p + xreg[ci][gp] * nsl + r0 * 8, (long)pad16(Rb.dim[cb[1]]) * 8, rows * 8, nsl,
+                              gR[gp] / 8, rows * 8 * nsl});
           }
         }
-      }
+      });
+      for (const auto& z : zg) zj.insert(zj.end(), z.begin(), z.end());
     }
     // stage 2: per output block (g, (ql, n1) column block, N part), 128-row tiles, terms
     // over the chunk's bond states; long term lists cut into parts (split-K)
