@@ -36,11 +36,6 @@ ROOT = os.path.dirname(os.path.abspath(__file__))
 sys.path.insert(0, ROOT)
 
 METRIC = "H_eff·ψ TFLOP/s & sweep s at K=40 M=2000, mixed vs FP64 GPU at |ΔE|≤1e-6 Eh"
-# DRAM bytes (read + write) of one H_eff.psi of the K=40 centre workload, both stages,
-# per precision, from one ncu capture of dram__bytes_read.sum + dram__bytes_write.sum
-# (profiles/gemm_tma_kernel_sigma_k40_m2000.md); absent where not captured for the
-# current kernels
-TRAFFIC = {5: 28.06e9 + 37.76e9 + 74.70e9 + 0.05e9}
 
 WORKLOADS = {
     # name: K, N, two_sz, M, spread of the synthetic sector dimensions, integral seed, h off-diagonal std,
@@ -411,11 +406,11 @@ def run_ours(args, rank, world, local_rank):
         fp64_cmp["fullsize_checks"] = checks
     ach_k = kern["primary"]["tflops"]
     if args.precision == 0:
-        peak = peaks["bf16_tflops_sustained"] * 1.25 / 2250.0
+        peak = 1.25
         roof = {"bound": "alu", "achieved": ach_k, "peak": peak, "unit": "TFLOP/s",
                 "frac": ach_k / peak, "traffic": None,
                 "kernel": "gemm_f64_kernel (sigma stages 1+2)",
-                "peak_note": f"FP64 = {src} bf16 sustained x 1.25/2250 (nominal FP64/BF16)"}
+                "peak_note": "FP64 nominal: two multiply-adds per clock and SM, 152 SMs at 2.07 GHz"}
         dtype = "f64"
     else:
         peak = peaks["bf16_tflops_sustained"]
@@ -423,7 +418,7 @@ def run_ours(args, rank, world, local_rank):
         # split-precision products) / event-timed sigma time; the products the tensor
         # cores actually execute for the slices are reported beside it, not in frac
         roof = {"bound": "tensor", "achieved": ach_k, "peak": peak, "unit": "TFLOP/s",
-                "frac": ach_k / peak, "traffic": TRAFFIC.get(args.precision) if args.workload == "k40_m2000" else None,
+                "frac": ach_k / peak, "traffic": None,  # counters are read on small cases only (profiles/)
                 "kernel": f"gemm_tma_kernel<1>+<2> (sigma stages 1+2, TMA-staged), precision {args.precision}",
                 "executed_tflops": ach_k * nprod,
                 "products_per_multiply_add": nprod,
@@ -625,7 +620,7 @@ def main():
     ap.add_argument("--autotune", action="store_true",
                     help="with --batched: choose the split-K granularity of the fused work lists by timing")
     ap.add_argument("--profiler-range", action="store_true",
-                    help="bracket the timed steps with cudaProfilerStart/Stop (for ncu --profile-from-start off)")
+                    help="bracket the timed steps with cudaProfilerStart/Stop (for ncu --profile-from-start off on a small workload)")
     ap.add_argument("--profile-sigma", type=int, default=0,
                     help="after setup run this many H_eff.psi calls only (for ncu captures) and exit")
     args = ap.parse_args()
