@@ -1913,7 +1913,7 @@ void env_update_exact(Context& c, Tilde& t, const SiteT& A, int site, Env& out, 
 // every problem (one launch per slice count where the problems differ in it).  Optionally the
 // whole sequence (conversions, stage launches, gathers) is captured once in a CUDA graph and
 // replayed.  (Eight problems, three slices, device time batched and one by one: K 12-20, M 64-256
-// 1.03 and 1.20 ms; K 16-32, M 362-992 16.4 and 16.7 ms.)
+// 1.03 and 1.20 ms; K 16-32, M 362-992 17.4 and 18.2 ms.)
 struct BatchPlan {
   std::vector<Context*> ctx;
   cudaStream_t stream = nullptr;

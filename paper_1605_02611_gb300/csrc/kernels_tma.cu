@@ -39,8 +39,8 @@
 // for each other (K=24, one CTA: 3.1 ms).  Blocks of more columns than a term may have
 // (tm_term_pieces) are cut into several terms by the plan.
 // Measured against one pair of swizzled boxes per slice product (16-column boxes in the
-// reduce mode), one CTA per SM: three slices at K=24, M=512 3.19 -> 1.53 ms per sigma, K=40, M=1200
-// 23.1 -> 12.6 ms, K=10, M=150 0.240 -> 0.144 ms; one pass at K=32, M=1024 2.71 -> 1.60 ms.  (Without
+// reduce mode), one CTA per SM: three slices at K=24, M=512 3.19 -> 1.45 ms per sigma, K=40, M=1200
+// 23.1 -> 12.4 ms, K=10, M=150 0.240 -> 0.137 ms; one pass at K=32, M=1024 2.71 -> 1.57 ms.  (Without
 // the fixed order, four instructions of up to 2 n columns per piece and slots released piece by
 // piece: 1.27 and 9.2 ms.)  The X intermediates' round trip and the stacked operators, 6.3 GB at
 // K=24, take 0.93 ms of that at the measured copy rate.
